@@ -109,11 +109,15 @@ typedef struct {
                            the tensor cores.  Reflector generation, the TSQR
                            R-merges and the in-panel products stay FP64. */
     int32_t batch_streams; /* gbqr_factor_batched: streams to spread over (1..128) */
-    int32_t fp64_gemm;  /* FP64 GEMM tiles of 64 x 64 outputs: 0 or GBQR_GEMM_DFMA
-                           = CUDA-core FMA (default, measured faster);
-                           GBQR_GEMM_DMMA = FP64 tensor cores (mma.sync
-                           m8n8k4).  Both are deterministic and differ by
-                           rounding only. */
+    int32_t fp64_gemm;  /* FP64 GEMM engine.  0 or GBQR_GEMM_DFMA (default):
+                           large products on the BF16 tensor cores by exact
+                           digit splitting (FP64 accuracy, no larger error
+                           than the FMA kernel), the others - and all of
+                           them where the workspace has no room for the
+                           digits - on CUDA-core FMA; GBQR_GEMM_DMMA = FMA
+                           kernels with 64 x 64 tiles on the FP64 tensor
+                           cores (mma.sync m8n8k4).  All are deterministic
+                           and differ by rounding only. */
 } gbqr_opts;
 
 /* Device-side record of one or more calls since the last gbqr_sync(). */

@@ -32,6 +32,8 @@ constexpr int kKrylov = 100;          // GMRES refinement: Arnoldi steps per cor
 constexpr int kInPanelTcMinCols = 32;  // mixed path: in-panel updates on the tensor cores from n1 >= 32 (16 measured slower) ...
 constexpr int64_t kInPanelTcMinRows = 2048;   // ... and m >= 2048
 constexpr int kMaxBatchLanes = 128;
+constexpr size_t kOzMainBytes = (size_t)448 << 20;   // digit scratch of the trailing updates (8192^2: up to three column chunks)
+constexpr int64_t kOzChunkCols = 512;              // ... never less than this many columns' worth
 
 struct DeviceInfo {
     unsigned long long nonfinite;
@@ -83,6 +85,7 @@ struct Params {
     bool lookahead = true;
     int nsplit = 0;        // 0: FP64 updates; 1..3: split-BF16 tensor-core updates
     bool dmma = false;     // FP64 GEMM engine of 64 x 64 tiles: DFMA (0.94 vs 0.83 TFLOP/s on 8192^2)
+    bool oz = true;        // scratch for digit-split FP64 products (off: a caller's workspace without room for it)
 };
 
 bool resolve(const gbqr_opts *o, int64_t m, int64_t n, Params *p) {
@@ -117,6 +120,7 @@ struct Layout {
     size_t partial2 = 0, gcount2 = 0, M1b = 0, M2b = 0;   // second lane (look-ahead panel stream)
     size_t tc = 0, n_tc = 0;                              // tensor-core slices (mixed updates)
     size_t tc2 = 0, n_tc2 = 0;                            // ... of the look-ahead lane's in-panel updates
+    size_t oz = 0, n_oz = 0, oz2 = 0, n_oz2 = 0;          // digit-split FP64 products, main and look-ahead lane
     size_t kry = 0, n_kry = 0;                            // least squares, mixed: Krylov basis of the refinement
     size_t dinv = 0, n_dinv = 0;                          // ... and inverses of R's diagonal blocks
     size_t total = 0;
@@ -172,6 +176,19 @@ Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num
         const int64_t h = std::max<int64_t>(nb / 2, 1);
         L.n_tc2 = pr.lookahead ? tc_gemm_scratch_bytes(h, h, std::max<int64_t>(m, 1), num_sms) : 0;
         if (L.n_tc2) L.tc2 = take(L.n_tc2);
+    }
+    if (pr.oz && !pr.dmma) {
+        // digits of the trailing columns (the mixed path: of the T product
+        // only) and of V, up to kOzMainBytes - wider updates go in column
+        // chunks - and of a panel's halves on the look-ahead lane
+        const int64_t mm = std::max<int64_t>(m, 1), nn = std::max<int64_t>(n, 1), kv = t_layout == GBQR_T_FULL ? (nn + 1) / 2 : nb;
+        auto need = [&](int64_t cols) { return std::max(oz_gemm_scratch_bytes(kv, cols, mm), oz_gemm_scratch_bytes(mm, cols, kv)); };
+        L.n_oz = pr.nsplit > 0 ? oz_gemm_scratch_bytes(kv, nn, kv)
+                               : std::max(need(std::min(nn, kOzChunkCols)), std::min(need(nn), kOzMainBytes));
+        L.oz = take(L.n_oz);
+        const int64_t h = std::max<int64_t>((nb + 1) / 2, 1);
+        L.n_oz2 = pr.lookahead && nn > nb ? std::max(oz_gemm_scratch_bytes(h, h, mm), oz_gemm_scratch_bytes(mm, h, h)) : 0;
+        if (L.n_oz2) L.oz2 = take(L.n_oz2);
     }
     L.bigA = take(L.n_bigA * 8);
     L.bigT = take(L.n_bigT * 8);
@@ -318,6 +335,7 @@ struct Work {
         g.partial_elems = gs.partial_elems * (sizeof(double) / sizeof(Real));
         g.counters = gs.counters;
         g.ncounters = gs.ncounters;
+        g.oz = gs.oz;
         return g;
     }
     template <class Real> TsqrWorkT<Real> twr() const {
@@ -379,6 +397,7 @@ void carve_work(gbqr_ctx *cx, char *base, const Layout &L, const Params &pr, con
     w->tw.Y = (double *)(base + w->L.tY);
     w->tw.X = (double *)(base + w->L.tX);
     w->tw.counters = (unsigned *)(base + w->L.tcount);
+    w->gs.oz = {w->L.n_oz ? (void *)(base + w->L.oz) : nullptr, w->L.n_oz, &cx->dinfo->timeout};
     w->M1 = (double *)(base + w->L.M1);
     w->M2 = (double *)(base + w->L.M2);
     w->bigA = (double *)(base + w->L.bigA);
@@ -391,6 +410,7 @@ void carve_work(gbqr_ctx *cx, char *base, const Layout &L, const Params &pr, con
     w->gs2.partial_elems = pr.lookahead ? w->L.n_partial : 0;
     w->gs2.counters = (unsigned *)(base + w->L.gcount2);
     w->gs2.ncounters = w->L.n_gcount;
+    w->gs2.oz = {w->L.n_oz2 ? (void *)(base + w->L.oz2) : nullptr, w->L.n_oz2, &cx->dinfo->timeout};
     w->M1b = (double *)(base + w->L.M1b);
     w->M2b = (double *)(base + w->L.M2b);
     w->tcs.base = w->L.n_tc ? (void *)(base + w->L.tc) : nullptr;
@@ -412,7 +432,13 @@ gbqr_status zero_counters(const Work &w, cudaStream_t s) {
 gbqr_status begin_work(gbqr_ctx *cx, int64_t m, int64_t n, int t_layout, const Params &pr, Work *w,
                        size_t min_M = 0) {
     if (cudaSetDevice(cx->device) != cudaSuccess) return GBQR_ECUDA;
-    const Layout L = make_layout(m, n, t_layout, pr, cx->num_sms, true, min_M);
+    Layout L = make_layout(m, n, t_layout, pr, cx->num_sms, true, min_M);
+    if (!cx->ws_owned && L.total > cx->ws_bytes) {
+        // a caller's workspace without room for the digits: FMA products only
+        Params p0 = pr;
+        p0.oz = false;
+        L = make_layout(m, n, t_layout, p0, cx->num_sms, true, min_M);
+    }
     gbqr_status st = ensure_workspace(cx, L.total);
     if (st != GBQR_OK) return st;
     carve_work(cx, cx->ws, L, pr, cx->exec(), w);
@@ -951,6 +977,7 @@ gbqr_status gbqr_factor_f32(gbqr_ctx *cx, int64_t m, int64_t n, float *A, int64_
     if (!cx) return GBQR_EINVAL;
     Params pr;
     if (!resolve(opts, m, n, &pr) || pr.nsplit != 0) return GBQR_EINVAL;
+    pr.oz = false;
     TRY(check_layout_args(m, n, lda, ldt, t_layout, pr.nb));
     if (n == 0) return GBQR_OK;
     if (!A || !T) return GBQR_EINVAL;
@@ -1299,6 +1326,7 @@ gbqr_status gbqr::factor_batched_untuned(gbqr_ctx *cx, int count, const int64_t 
     Params pr;
     if (!resolve(opts, mmax, nmax, &pr)) return GBQR_EINVAL;
     pr.lookahead = false;                       // one stream per lane
+    pr.oz = false;
     if (!opts || opts->cutoff_b == 0) pr.b = kBatchCutoff;
     const int S = std::min(count, opts && opts->batch_streams > 0 ? std::min(opts->batch_streams, kMaxBatchLanes) : kBatchLanes);
     const int lane_sms = std::max(8, (2 * cx->num_sms + S - 1) / S);
@@ -1390,6 +1418,7 @@ size_t gbqr_batched_workspace_bytes(int count, const int64_t *m, const int64_t *
     Params pr;
     if (!resolve(opts, mmax, nmax, &pr)) return 0;
     pr.lookahead = false;
+    pr.oz = false;
     if (!opts || opts->cutoff_b == 0) pr.b = kBatchCutoff;
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {

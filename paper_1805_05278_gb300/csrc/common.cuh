@@ -64,12 +64,19 @@ struct GemmOpT {
 };
 using GemmOp = GemmOpT<double>;
 
+// Scratch of the digit-split FP64 products (oz_gemm): digits and partials.
+struct OzScratch {
+    void *base = nullptr; size_t bytes = 0;
+    int *err = nullptr;                       // device flag raised on a timed-out wait
+};
+
 // Scratch for split-K: partial tiles and self-resetting per-tile counters
 // (must be zero before the first use; every launch leaves them zero).
 template <class Real>
 struct GemmScratchT {
     Real *partial = nullptr; size_t partial_elems = 0;
     unsigned *counters = nullptr; size_t ncounters = 0;
+    OzScratch oz;                             // FP64: none = FMA kernels only
 };
 using GemmScratch = GemmScratchT<double>;
 
@@ -82,6 +89,13 @@ gbqr_status gemm(const Exec &ex, const GemmOpT<Real> &op, const GemmScratchT<Rea
 // Algorithmic flops of op (structural zeros of masked operands excluded).
 template <class Real>
 double gemm_algorithmic_flops(const GemmOpT<Real> &op);
+
+// FP64 products on the BF16 tensor cores by exact digit splitting: gemm()
+// takes this path where it is estimated faster and the scratch holds it.
+// oz_gemm_scratch_bytes: enough for any product of these sizes or smaller.
+size_t oz_gemm_scratch_bytes(int64_t M, int64_t N, int64_t K);
+bool oz_gemm_wanted(const GemmOp &op, const OzScratch &sc, int num_sms);
+gbqr_status oz_gemm(const Exec &ex, const GemmOp &op, const OzScratch &sc);
 
 #define TRY_ST(x) do { gbqr_status _s = (x); if (_s != GBQR_OK) return _s; } while (0)
 
