@@ -34,6 +34,7 @@ constexpr int64_t kInPanelTcMinRows = 2048;   // ... and m >= 2048
 constexpr int kMaxBatchLanes = 128;
 constexpr size_t kOzMainBytes = (size_t)448 << 20;   // digit scratch of the trailing updates (8192^2: up to three column chunks)
 constexpr int64_t kOzChunkCols = 512;              // ... never less than this many columns' worth
+constexpr int kGramFallbackB = 64;   // TSQR width behind a Gram-matrix panel: few launches, which mostly return at once
 
 struct DeviceInfo {
     unsigned long long nonfinite;
@@ -85,6 +86,7 @@ struct Params {
     bool lookahead = true;
     int nsplit = 0;        // 0: FP64 updates; 1..3: split-BF16 tensor-core updates
     bool dmma = false;     // FP64 GEMM engine of 64 x 64 tiles: DFMA (0.94 vs 0.83 TFLOP/s on 8192^2)
+    bool gram = false;     // Gram-matrix panels (default TSQR parameters only)
     bool oz = true;        // scratch for digit-split FP64 products (off: a caller's workspace without room for it)
 };
 
@@ -109,6 +111,8 @@ bool resolve(const gbqr_opts *o, int64_t m, int64_t n, Params *p) {
         else if (o->fp64_gemm != 0 && o->fp64_gemm != GBQR_GEMM_DFMA) return false;
     }
     r.nb = std::max<int64_t>(1, r.nb);
+    // a caller who sets the TSQR's parameters gets the TSQR
+    r.gram = r.b == kDefaultCutoff && r.leaf_rows == 0 && r.fanout == kDefaultFanout && !r.dmma;
     *p = r;
     return true;
 }
@@ -121,6 +125,7 @@ struct Layout {
     size_t tc = 0, n_tc = 0;                              // tensor-core slices (mixed updates)
     size_t tc2 = 0, n_tc2 = 0;                            // ... of the look-ahead lane's in-panel updates
     size_t oz = 0, n_oz = 0, oz2 = 0, n_oz2 = 0;          // digit-split FP64 products, main and look-ahead lane
+    size_t gram = 0, n_gram = 0;                          // Gram-matrix panels: w x w arrays and the flag
     size_t kry = 0, n_kry = 0;                            // least squares, mixed: Krylov basis of the refinement
     size_t dinv = 0, n_dinv = 0;                          // ... and inverses of R's diagonal blocks
     size_t total = 0;
@@ -140,7 +145,8 @@ Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num
                            std::max(gemm_partial_elems_min(num_sms),
                                     (size_t)std::max<int64_t>(m, 1) * (size_t)std::max<int64_t>(n, 1) / 4));
     L.n_gcount = gemm_counters_max(num_sms);
-    const int w = (int)std::max<int64_t>(1, std::min<int64_t>(pr.b, n));
+    const bool gram = pr.gram && pr.oz && n >= kGramMinW && m >= 4 * kGramMinW;
+    const int w = (int)std::max<int64_t>(1, std::min<int64_t>(gram ? std::max(pr.b, kGramFallbackB) : pr.b, n));
     L.tsqr = tsqr_plan_bound(std::max<int64_t>(m, 1), w, pr.leaf_rows, pr.fanout, num_sms);
     const int64_t nb = std::min<int64_t>(pr.nb, std::max<int64_t>(n, 1));
     // temporaries of the update / T-assembly products and of applying Q
@@ -185,10 +191,17 @@ Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num
         auto need = [&](int64_t cols) { return std::max(oz_gemm_scratch_bytes(kv, cols, mm), oz_gemm_scratch_bytes(mm, cols, kv)); };
         L.n_oz = pr.nsplit > 0 ? oz_gemm_scratch_bytes(kv, nn, kv)
                                : std::max(need(std::min(nn, kOzChunkCols)), std::min(need(nn), kOzMainBytes));
+        // a panel: its Gram matrix and V, or the products of its halves
+        const int64_t h = gram ? std::min<int64_t>(nb, kGramMaxW) : std::max<int64_t>((nb + 1) / 2, 1);
+        const size_t panel = std::max(oz_gemm_scratch_bytes(h, h, mm), oz_gemm_scratch_bytes(mm, h, h));
+        if (gram || !pr.lookahead) L.n_oz = std::max(L.n_oz, panel);
         L.oz = take(L.n_oz);
-        const int64_t h = std::max<int64_t>((nb + 1) / 2, 1);
-        L.n_oz2 = pr.lookahead && nn > nb ? std::max(oz_gemm_scratch_bytes(h, h, mm), oz_gemm_scratch_bytes(mm, h, h)) : 0;
+        L.n_oz2 = pr.lookahead && nn > nb ? panel : 0;
         if (L.n_oz2) L.oz2 = take(L.n_oz2);
+        if (gram) {
+            L.n_gram = gram_work_elems();
+            L.gram = take(L.n_gram * 8 + 16);
+        }
     }
     L.bigA = take(L.n_bigA * 8);
     L.bigT = take(L.n_bigT * 8);
@@ -324,6 +337,8 @@ struct Work {
     TcScratch tcs2;                  // ... of the look-ahead lane
     GemmScratch gs2;
     double *M1b, *M2b;
+    double *gram = nullptr;          // Gram-matrix panels: work, and the flag behind it (null: TSQR only)
+    int *gram_flag = nullptr;
 
     // Typed views of the workspace (regions are sized for FP64; an FP32 call
     // uses the same bytes).
@@ -411,6 +426,8 @@ void carve_work(gbqr_ctx *cx, char *base, const Layout &L, const Params &pr, con
     w->gs2.counters = (unsigned *)(base + w->L.gcount2);
     w->gs2.ncounters = w->L.n_gcount;
     w->gs2.oz = {w->L.n_oz2 ? (void *)(base + w->L.oz2) : nullptr, w->L.n_oz2, &cx->dinfo->timeout};
+    w->gram = w->L.n_gram ? (double *)(base + w->L.gram) : nullptr;
+    w->gram_flag = w->L.n_gram ? (int *)(w->gram + w->L.n_gram) : nullptr;
     w->M1b = (double *)(base + w->L.M1b);
     w->M2b = (double *)(base + w->L.M2b);
     w->tcs.base = w->L.n_tc ? (void *)(base + w->L.tc) : nullptr;
@@ -517,6 +534,21 @@ gbqr_status base_qr(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, Real *T
 template <class Real>
 gbqr_status qr_eg(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, Real *T, int64_t ldt) {
     if (n <= 0) return GBQR_OK;
+    if constexpr (std::is_same<Real, double>::value) {
+        if (w.gram && !w.ex.pred && gram_qr_fits(w.gs.oz, m, n)) {
+            TRY(gram_qr(w.ex, m, n, A, lda, T, ldt, w.gram, w.gram_flag, w.gs.oz));
+            // ill-conditioned panels: the flag is up and A as it was, and
+            // the same recursion on FMA products and wide TSQRs runs
+            Work f = w;
+            f.ex.pred = w.gram_flag;
+            TsqrPlan pl;
+            const int64_t n1 = n <= kGramFallbackB ? n : n / 2;
+            const bool wide = tsqr_plan(m, (int)n1, 0, 0, w.ex.num_sms, &pl) &&
+                              (n1 == n || tsqr_plan(m - n1, (int)(n - n1), 0, 0, w.ex.num_sms, &pl));
+            f.pr.b = wide ? kGramFallbackB : kGramFallbackB / 2;
+            return qr_eg(f, m, n, A, lda, T, ldt);
+        }
+    }
     if (n <= w.pr.b) return base_qr(w, m, n, A, lda, T, ldt);
     const int64_t n1 = n / 2, n2 = n - n1;
     Real *AR = A + n1 * lda;
@@ -527,7 +559,7 @@ gbqr_status qr_eg(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, Real *T, 
     // two tall products go to the tensor cores once they are large enough to
     // beat the FP64 kernel's latency (the T-assembly below stays FP64, so T
     // stays consistent with V and Q = I - V T V^T orthogonal to FP64 accuracy).
-    const int nsplit_in = (w.pr.nsplit > 0 && n1 >= kInPanelTcMinCols && m >= kInPanelTcMinRows) ? w.pr.nsplit : 0;
+    const int nsplit_in = (w.pr.nsplit > 0 && !w.ex.pred && n1 >= kInPanelTcMinCols && m >= kInPanelTcMinRows) ? w.pr.nsplit : 0;
     TRY(apply_block(w, true, m, n2, n1, A, lda, T, ldt, AR, lda, nsplit_in));
     // right recursion on B22
     Real *TR = T + n1 + n1 * ldt;

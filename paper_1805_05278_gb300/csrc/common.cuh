@@ -31,6 +31,7 @@ struct Exec {
     int num_sms = 152;
     int device = 0;
     bool dmma = false;          // 64 x 64 FP64 GEMM tiles on the FP64 tensor cores (else DFMA)
+    const int *pred = nullptr;  // device flag: the kernels of gemm() and tsqr_run() return at once while it is zero
 };
 
 inline void trace_begin(const Exec &ex, Family f) {
@@ -38,7 +39,7 @@ inline void trace_begin(const Exec &ex, Family f) {
 }
 inline gbqr_status trace_end(const Exec &ex, Family f, double flops, double bytes) {
     if (ex.launches) ++*ex.launches;
-    if (ex.tracer) ex.tracer->end(ex.stream, f, flops, bytes);
+    if (ex.tracer) ex.tracer->end(ex.stream, f, ex.pred ? 0.0 : flops, ex.pred ? 0.0 : bytes);
     return cudaPeekAtLastError() == cudaSuccess ? GBQR_OK : GBQR_ECUDA;
 }
 
@@ -61,6 +62,9 @@ struct GemmOpT {
     const Real *B = nullptr; int64_t ldb = 1; int maskB = MASK_NONE;
     Real *C = nullptr; int64_t ldc = 1;
     Real alpha = Real(1), beta = Real(0);
+    const int *skip = nullptr;   // digit-split products only: device flag, non-zero = do nothing
+    const int *kexp = nullptr;   // ... and K exponents that balance op(A)'s columns against B's rows:
+                                 // op(A)(:, k) 2^-kexp[k] and 2^kexp[k] B(k, :) are split
 };
 using GemmOp = GemmOpT<double>;
 
@@ -96,6 +100,16 @@ double gemm_algorithmic_flops(const GemmOpT<Real> &op);
 size_t oz_gemm_scratch_bytes(int64_t M, int64_t N, int64_t K);
 bool oz_gemm_wanted(const GemmOp &op, const OzScratch &sc, int num_sms);
 gbqr_status oz_gemm(const Exec &ex, const GemmOp &op, const OzScratch &sc);
+
+// Householder QR of a well-conditioned panel from its Gram matrix
+// (gram_qr.cu): V \ R over A, T (w x w).  Where the condition does not allow
+// it, *flag (device) is set, else cleared, and A and T are left alone.
+// work: gram_work_elems() doubles.  oz holds the panel's digits.
+constexpr int kGramMaxW = 128, kGramMinW = 16;
+size_t gram_work_elems();
+bool gram_qr_fits(const OzScratch &oz, int64_t m, int64_t w);
+gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, double *A, int64_t lda, double *T, int64_t ldt,
+                    double *work, int *flag, const OzScratch &oz);
 
 #define TRY_ST(x) do { gbqr_status _s = (x); if (_s != GBQR_OK) return _s; } while (0)
 

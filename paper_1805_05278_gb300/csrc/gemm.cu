@@ -36,6 +36,7 @@ struct GemmParamsT {
     Real *partial;            // per tile: slots_per_tile * BM*BN elements
     unsigned *counters;       // per tile: counters_per_tile
     int slots_per_tile, counters_per_tile;
+    const int *pred;          // non-null: run only while *pred != 0
 };
 using GemmParams = GemmParamsT<double>;
 
@@ -76,6 +77,7 @@ __global__ void __launch_bounds__(kThreads) dgemm_kernel(GemmParamsT<Real> p) {
     __shared__ Real As[BK][BM + 1];
     __shared__ Real Bs[BK][BN + 1];
     __shared__ int s_last;
+    if (p.pred && *(volatile const int *)p.pred == 0) return;
 
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int64_t m0 = (int64_t)blockIdx.x * BM, n0 = (int64_t)blockIdx.y * BN;
@@ -212,6 +214,7 @@ __global__ void __launch_bounds__(kThreads) dgemm_dmma_kernel(GemmParams p) {
     __shared__ double As[BK][BM + 4];
     __shared__ double Bs[BK][BN + 4];
     __shared__ int s_last;
+    if (p.pred && *(volatile const int *)p.pred == 0) return;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wm = warp & 1, wn = warp >> 1;
@@ -408,7 +411,7 @@ gbqr_status gemm(const Exec &ex, const GemmOpT<Real> &op, const GemmScratchT<Rea
         if (op.beta == Real(1)) return GBQR_OK;
     }
     if constexpr (std::is_same<Real, double>::value)
-        if (!ex.dmma && oz_gemm_wanted(op, sc.oz, ex.num_sms)) return oz_gemm(ex, op, sc.oz);
+        if (!ex.dmma && !ex.pred && oz_gemm_wanted(op, sc.oz, ex.num_sms)) return oz_gemm(ex, op, sc.oz);
     // A small output (the T products of Algorithm 2 are 64 x 64 x 64 at the
     // panel's top node) on 64 x 64 tiles would run on a handful of SMs at one
     // SM's FP64 rate (2 FMA/clock: ~60 us for 64^3): shrink the tiles until
@@ -458,6 +461,7 @@ gbqr_status gemm(const Exec &ex, const GemmOpT<Real> &op, const GemmScratchT<Rea
     p.C = op.C; p.ldc = op.ldc; p.alpha = op.alpha; p.beta = op.beta;
     p.partial = sc.partial; p.counters = sc.counters;
     p.slots_per_tile = 1; p.counters_per_tile = 1;
+    p.pred = ex.pred;
     if (S > 1) {
         tree_shape(S, &p.slots_per_tile, &p.counters_per_tile);
         size_t need_p = (size_t)tiles * p.slots_per_tile * BM * BN;

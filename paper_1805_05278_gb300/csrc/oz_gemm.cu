@@ -106,6 +106,8 @@ struct OzOperand {
     int64_t ldk;
     int *exps;                 // per operand row
     unsigned blocks;           // CTAs working on it
+    const int *skip;           // non-null: nothing to do while *skip != 0
+    const int *kexp; int ksign;   // entries of index k scaled by 2^(ksign kexp[k]) first
 };
 
 // x 2^e, exact unless it leaves the normal range.
@@ -123,7 +125,8 @@ __device__ __forceinline__ double oz_load(const OzOperand &o, int64_t r, int64_t
     if (k >= o.K || r >= o.R) return 0.0;
     if (o.mask == MASK_UNIT_LOWER && i <= j) return 0.0;
     if (o.mask == MASK_UPPER && i > j) return 0.0;
-    return o.X[i + j * o.ld];
+    const double x = o.X[i + j * o.ld];
+    return o.kexp ? mul_pow2(x, o.ksign * __ldcg(o.kexp + k)) : x;
 }
 
 __device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
@@ -165,6 +168,7 @@ __global__ void __launch_bounds__(kThreads) oz_slice_kernel(const OzOperand a, c
     __shared__ int red[8][32];
     const bool isB = blockIdx.x >= a.blocks;
     const OzOperand &o = isB ? b : a;
+    if (o.skip && *(volatile const int *)o.skip) return;
     const int64_t blk = isB ? blockIdx.x - a.blocks : blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int ex = 0;
@@ -249,6 +253,7 @@ struct OzParams {
     double *C; int64_t ldc;
     double alpha, beta;
     const double *add; int64_t ldadd; int add_rows;   // unit diagonal of op(A): + alpha * B(i, j), i < add_rows
+    const int *skip;           // non-null: nothing to do while *skip != 0
     int *err;
 };
 
@@ -282,6 +287,7 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     oz_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const OzParams p) {
     extern __shared__ uint8_t smem_raw[];
+    if (p.skip && *(volatile const int *)p.skip) return;
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *sA = smem, *sB = sA + OZ_STAGES * OZ_A_STAGE;
     uint64_t *bars = (uint64_t *)(sB + OZ_STAGES * OZ_B_STAGE);
@@ -458,6 +464,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 // C = beta C + alpha (2^(ea + eb - 54) sum_z P[z] + unit-diagonal term): the
 // sum is exact (high and low halves in 64 bits each), one rounding.
 __global__ void __launch_bounds__(kThreads) oz_reduce_kernel(const OzParams p, int S) {
+    if (p.skip && *(volatile const int *)p.skip) return;
     const size_t total = (size_t)p.M * p.N;
     for (size_t e = blockIdx.x * (size_t)kThreads + threadIdx.x; e < total; e += (size_t)gridDim.x * kThreads) {
         const int i = (int)(e % (unsigned)p.M), j = (int)(e / (unsigned)p.M);
@@ -596,6 +603,14 @@ static gbqr_status oz_chunk(const Exec &ex, const GemmOp &op, const OzScratch &s
     };
     a.blocks = slice_a ? blocks(a) : 0;
     b.blocks = blocks(b);
+    if (op.ta && op.A == op.B && op.lda == op.ldb && op.M == op.N && op.maskA == op.maskB) {
+        b = a;                         // X^T X: one set of digits
+        b.blocks = 0;
+    }
+    a.skip = b.skip = op.skip;
+    a.kexp = b.kexp = op.kexp;
+    a.ksign = -1;
+    b.ksign = 1;
     trace_begin(ex, FAM_OTHER);
     if (a.blocks + b.blocks) oz_slice_kernel<<<a.blocks + b.blocks, kThreads, 0, ex.stream>>>(a, b);
     TRY_ST(trace_end(ex, FAM_OTHER, 0.0, 22.0 * ((double)op.M + op.N) * op.K));
@@ -611,6 +626,7 @@ static gbqr_status oz_chunk(const Exec &ex, const GemmOp &op, const OzScratch &s
     p.C = op.C; p.ldc = op.ldc; p.alpha = op.alpha; p.beta = op.beta;
     p.add = op.B; p.ldadd = op.ldb;
     p.add_rows = op.maskA == MASK_UNIT_LOWER ? (int)std::min(op.M, op.K) : 0;
+    p.skip = op.skip;
     p.err = sc.err;
     CUtensorMap mA, mB;
     if (!oz_map(&mA, a.dst, op.M, L.ldk, OZ_BM) || !oz_map(&mB, b.dst, op.N, L.ldk, OZ_BN)) return GBQR_ECUDA;

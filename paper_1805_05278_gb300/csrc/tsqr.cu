@@ -44,6 +44,7 @@ struct TsqrParamsT {
     Real *wsR, *wsT, *wsY, *wsX;
     unsigned *counters;
     Real *Tout; int64_t ldt;
+    const int *pred;          // non-null: run only while *pred != 0
 };
 
 // The cnt consecutive w x w slots at src (slot i, entry (row, col) at
@@ -86,6 +87,7 @@ __global__ void __launch_bounds__(kThreads) tsqr_up_kernel(TsqrParamsT<Real> p) 
     Real *aux = G + w * w;
     const Refl<Real> rf{aux, aux + w, aux + 2 * w, aux + 3 * w, aux + 4 * w, aux + 5 * w};
     __shared__ int s_last;
+    if (p.pred && *(volatile const int *)p.pred == 0) return;
 
     const int leaf = blockIdx.x;
     const int64_t r0 = leaf_begin(p.mp, p.P, leaf), r1 = leaf_begin(p.mp, p.P, leaf + 1);
@@ -272,6 +274,7 @@ __global__ void __launch_bounds__(kThreads) tsqr_down_kernel(TsqrParamsT<Real> p
     Real *Sg = Li + ww;      // w signs
     Real *rU = Sg + w;       // w reciprocals of diag(U)
     Real *Vs = rU + w;       // ldS x w: this leaf's rows of V, then of W and V
+    if (p.pred && *(volatile const int *)p.pred == 0) return;
 
     const int leaf = blockIdx.x;
     // X = [B_0; 0] top rows - V0 Z0, V0 = leaf 0's unit lower top block
@@ -489,6 +492,7 @@ gbqr_status tsqr_run(const Exec &ex, const TsqrPlan &pl, Real *A, int64_t lda,
     p.wsR = work.R; p.wsT = work.T; p.wsY = work.Y; p.wsX = work.X;
     p.counters = work.counters;
     p.Tout = Tout; p.ldt = ldt;
+    p.pred = ex.pred;
 
     // per device and scalar type, once (server workers launch from several threads)
     static std::atomic<bool> attr_done[64];
