@@ -28,13 +28,19 @@
 // while the flag is zero, factor it.
 //
 // The w x w work runs in 32-wide blocks, three launches a block:
-//   diag   one CTA: Cholesky and LU of the diagonal block with their inverses
-//          (Gauss-Jordan: the inverses cost columns, not steps),
-//   row    block row k of R and U, block column k of L, ...
+//   diag   one CTA: Cholesky and LU of the diagonal block
+//   row    triangular solves with it: block row k of R and U, block column k
+//          of L, the diagonal blocks of R^{-1}, U^{-1} and V1^{-1}, ...
 //   trail  the trailing blocks of G and A1; R^{-1}, U^{-1} and V1^{-1} grow by
 //          one block column or row.
-// FP64 issues one instruction per warp per 64 cycles on this part, so a 32^3
-// product on one SM takes 9 us: row and trail spread every block over 8 CTAs.
+// FP64 issues one instruction per warp per 64 cycles and per SM sub-partition
+// per 76 on this part, so diag is bound by its 64 dependent pivots (a
+// reciprocal, a multiply-add and a barrier each) and does nothing else: with
+// the block's inverses formed in it by augmented columns, it took 75 us, the
+// columns' FP64 issue delaying the chain; without them 20 us.  A 32^3 product
+// on one SM would take 9 us, so row and trail spread every block over 8 CTAs;
+// a triangular solve with a unit diagonal is 32 shuffles and multiply-adds,
+// no longer than a product with the inverse.
 #include "tsqr_dev.cuh"
 
 #include <algorithm>
@@ -53,6 +59,8 @@ struct GramArgs {
     double *Tout; int64_t ldt;
     int w, nblk;
     double *G, *R, *RI, *A1, *L, *U, *LI, *X, *YX, *YR, *YL, *K, *sgn, *gd;
+    double *M;                       // the block's unit triangular factors, M[t][lane]: see UnitFactor
+    double *sc;                      // ... and the reciprocals of R's and U's diagonal
     int *flag, *kexp;                // kexp: exponents of the column norms
 };
 
@@ -65,147 +73,154 @@ __device__ __forceinline__ double a1_at(const GramArgs &p, int i, int j, int k) 
     return (i < p.w && j < p.w) ? p.A[i + (int64_t)j * p.lda] : (i == j ? 1.0 : 0.0);
 }
 
-// Diagonal block k.  In both eliminations warp 0 carries the chain (update of
-// the next column, pivot, reciprocal, multipliers) one step ahead of the
-// other warps, which update the remaining columns and the augmented identity;
-// in the LU warp 1 carries the next row of U the same way.
+// 1/d by the reciprocal approximation and one third-order Newton step
+// (r + r (e + e^2), e = 1 - d r): three dependent FP64 instructions, where
+// the correctly rounded reciprocal takes about twice as long.
+__device__ __forceinline__ double quick_rcp(double d) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    const double e = rfma(-d, r, 1.0);
+    return rfma(r, rfma(e, e, e), r);
+}
+
+// Unit triangular factors of the diagonal block, row t holding the
+// coefficients of step t of a substitution: Cholesky's L (M[t][i] = L(i, t),
+// i > t), V1's diagonal block the same way, and U scaled to a unit diagonal
+// (M[t][j] = U(t, j) / U(t, t), j > t).
+enum UnitFactor { UF_CHOL = 0, UF_L = 1, UF_U = 2 };
+
+// Diagonal block k: S = D^{1/2}-free Cholesky G_kk = Lc D Lc^T, then the LU of
+// A1_kk - S R_kk.  Warp 0 carries the chain: it brings the next column up to
+// date, takes its pivot's reciprocal and publishes both, while the other
+// warps apply the current column to the ones behind; in the LU warp 1 carries
+// the next row of U the same way.  One barrier a step.
 __global__ void __launch_bounds__(kThreads) gram_diag_kernel(const GramArgs p, int k) {
-    __shared__ double S[GB][GB + 1], E[GB][GB + 1], Rb[GB][GB + 1];   // [column][row]
-    __shared__ double cb[2][GB], lb[2][GB], rd[GB], sg[GB];
+    __shared__ double S[GB][GB + 1], Rb[GB][GB + 1];     // [column][row]; Rb: R(row, column)
+    __shared__ double cb[2][GB], ub[2][GB], rb[2], rd[GB], sg[GB];
     __shared__ int bad;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, b0 = k * GB;
     if (k > 0 && *(volatile int *)p.flag) return;
-    for (int c = warp; c < GB; c += 8) {
+    double a1[GB / 8];                                   // the LU's block, loaded behind the Cholesky's
+#pragma unroll
+    for (int q = 0; q < GB / 8; ++q) {
+        const int c = warp + 8 * q;
         S[c][lane] = lane <= c ? g_at(p, b0 + lane, b0 + c, k) : g_at(p, b0 + c, b0 + lane, k);
-        E[c][lane] = lane == c ? 1.0 : 0.0;
+        a1[q] = a1_at(p, b0 + lane, b0 + c, k);
     }
-    if (k == 0) {
+    if (k == 0)
         for (int i = tid; i < p.nblk * GB; i += kThreads) {
             const double g = i < p.w ? __ldcg(p.G + i + i * GLD) : 1.0;
             p.gd[i] = g;
             p.kexp[i] = (((__double2hiint(g) >> 20) & 0x7ff) - 1023) >> 1;
         }
-        if (tid == 0) *p.flag = 0;
-    }
     if (tid == 0) bad = 0;
     __syncthreads();
-    // ---- Cholesky: S = L D L^T, E -> L^{-1}
+    // ---- Cholesky
+    double v = 0.0, r = 0.0;                             // warp 0: column t below (and at) its pivot, 1 / pivot
     if (warp == 0) {
-        const double v = S[0][lane];
-        const double r = real_rcp(__shfl_sync(kFull, v, 0));
+        v = S[0][lane];
+        r = quick_rcp(__shfl_sync(kFull, v, 0));
         cb[0][lane] = v;
-        lb[0][lane] = v * r;
+        if (lane == 0) rb[0] = rd[0] = r;
     }
     __syncthreads();
-    for (int t = 0; t < GB; ++t) {
-        const double *c = cb[t & 1], *l = lb[t & 1];
-        const double li = lane > t ? l[lane] : 0.0;
+    for (int t = 0; t + 1 < GB; ++t) {
         if (warp == 0) {
-            if (t + 1 < GB) {
-                const double v = rfma(-li, c[t + 1], S[t + 1][lane]);
-                const double r = real_rcp(__shfl_sync(kFull, v, t + 1));
-                S[t + 1][lane] = v;
-                cb[(t + 1) & 1][lane] = v;
-                lb[(t + 1) & 1][lane] = v * r;
-            }
-        } else {
-            for (int q = warp - 1; q < GB - 1; q += 7) {
-                // columns 0..t of E, then t+2.. of S
-                if (q <= t) E[q][lane] = rfma(-li, E[q][t], E[q][lane]);
-                else S[q + 1][lane] = rfma(-li, c[q + 1], S[q + 1][lane]);
-            }
-            if (t == GB - 1 && warp == 1) E[GB - 1][lane] = rfma(-li, E[GB - 1][t], E[GB - 1][lane]);
+            v = rfma(-r, v * __shfl_sync(kFull, v, t + 1), S[t + 1][lane]);
+            r = quick_rcp(__shfl_sync(kFull, v, t + 1));
+            S[t + 1][lane] = v;
+            cb[(t + 1) & 1][lane] = v;
+            if (lane == 0) rb[(t + 1) & 1] = rd[t + 1] = r;
+        } else if (t + 1 + warp < GB) {
+            const double *c = cb[t & 1];
+            const double li = lane > t ? c[lane] * rb[t & 1] : 0.0;
+            for (int j = t + 1 + warp; j < GB; j += 7) S[j][lane] = rfma(-li, c[j], S[j][lane]);
         }
         __syncthreads();
     }
-    // R = D^{1/2} L^T, R^{-1} = L^{-T} D^{-1/2}; S[t][i] = d_t L(i, t)
+    // R = D^{1/2} Lc^T; column t of S holds d_t Lc(:, t)
     if (warp == 0) {
         const double d = S[lane][lane];
+        if (!(d > 0.0 && d < 1e300)) bad = 1;
         const double s = sqrt(d);
-        rd[lane] = real_rcp(s);
-        if (!(d > 0.0)) bad = 1;
-    }
-    __syncthreads();
-    for (int c = warp; c < GB; c += 8) {
-        // column c: R(lane, c) = S[lane][c] rd[lane], RI(lane, c) = E[lane][c] rd[c]
-        const double rv = lane <= c ? S[lane][c] * rd[lane] : 0.0;
-        const double ri = lane <= c ? E[lane][c] * rd[c] : 0.0;
-        Rb[c][lane] = rv;
-        p.R[(b0 + lane) + (b0 + c) * GLD] = rv;
-        p.RI[(b0 + lane) + (b0 + c) * GLD] = ri;
-        const double g = k == 0 ? (b0 + lane < p.w ? __ldcg(p.G + (b0 + lane) * (GLD + 1)) : 1.0) : __ldcg(p.gd + b0 + lane);
-        if (!(ri * ri * g <= kGramBound2)) bad = 1;
+        sg[lane] = s;
+        p.sc[lane] = s * rd[lane];                       // 1 / r_tt
     }
     __syncthreads();
     if (bad) {
         if (tid == 0) *p.flag = 1;
         return;
     }
-    // ---- LU of A1 - S R: E -> V1^{-1} (diagonal block)
-    for (int c = warp; c < GB; c += 8) {
-        S[c][lane] = a1_at(p, b0 + lane, b0 + c, k);
-        E[c][lane] = lane == c ? 1.0 : 0.0;
+    if (k == 0 && tid == 0) *p.flag = 0;
+#pragma unroll
+    for (int q = 0; q < GB / 8; ++q) {
+        // row t = c of the factor, lane = i
+        const int c = warp + 8 * q;
+        const double lc = S[c][lane] * rd[c];
+        p.M[c * GB + lane] = lane > c ? lc : 0.0;
+        const double rv = lane > c ? lc * sg[c] : (lane == c ? sg[c] : 0.0);
+        Rb[lane][c] = rv;
     }
     __syncthreads();
-    // cb: row t of U (entry j at [j]); lb: multipliers
+#pragma unroll
+    for (int q = 0; q < GB / 8; ++q) {
+        const int c = warp + 8 * q;
+        p.R[(b0 + lane) + (b0 + c) * GLD] = Rb[c][lane];
+        S[c][lane] = a1[q];
+    }
+    __syncthreads();
+    // ---- LU of A1 - S R.  v: column t; ub: row t of U
     if (warp == 0) {
-        const double v = S[0][lane], al = __shfl_sync(kFull, v, 0);
-        const double u = al - (al < 0.0 ? Rb[0][0] : -Rb[0][0]);
-        const double r = real_rcp(u);
-        if (lane == 0) rd[0] = r;
-        lb[0][lane] = v * r;
+        v = S[0][lane];
+        const double al = __shfl_sync(kFull, v, 0), rr = Rb[0][0];
+        r = quick_rcp(al - (al < 0.0 ? rr : -rr));
+        cb[0][lane] = v;
+        if (lane == 0) rb[0] = rd[0] = r;
     } else if (warp == 1) {
-        const double x = S[lane][0], al = __shfl_sync(kFull, x, 0);
-        const double s = al < 0.0 ? 1.0 : -1.0;
+        const double x = S[lane][0], s = __shfl_sync(kFull, x, 0) < 0.0 ? 1.0 : -1.0;
         if (lane == 0) sg[0] = s;
-        cb[0][lane] = x - s * Rb[lane][0];
+        const double u = x - s * Rb[lane][0];
+        ub[0][lane] = u;
+        p.U[b0 + (b0 + lane) * GLD] = u;
     }
     __syncthreads();
-    for (int t = 0; t < GB; ++t) {
-        const double *u = cb[t & 1], *l = lb[t & 1];
-        const double li = lane > t ? l[lane] : 0.0;
+    for (int t = 0; t + 1 < GB; ++t) {
+        const double *u = ub[t & 1];
         if (warp == 0) {
-            double v = 0.0;
-            if (t + 1 < GB) {
-                v = rfma(-li, u[t + 1], S[t + 1][lane]);
-                const double al = __shfl_sync(kFull, v, t + 1), rr = Rb[t + 1][t + 1];
-                const double r = real_rcp(al - (al < 0.0 ? rr : -rr));
-                if (lane == 0) rd[t + 1] = r;
-                lb[(t + 1) & 1][lane] = v * r;
-            }
-            S[t][lane] = lane > t ? li : S[t][lane];                    // L below the diagonal
+            // (the product first: the same bits as in warp 1, so that both see one pivot)
+            v = rfma(-r, v * u[t + 1], S[t + 1][lane]);
+            const double al = __shfl_sync(kFull, v, t + 1), rr = Rb[t + 1][t + 1];
+            r = quick_rcp(al - (al < 0.0 ? rr : -rr));
+            if (lane > t + 1) S[t + 1][lane] = v;           // (warp 1 reads the pivot entry)
+            cb[(t + 1) & 1][lane] = v;
+            if (lane == 0) rb[(t + 1) & 1] = rd[t + 1] = r;
         } else if (warp == 1) {
-            if (t + 1 < GB) {
-                const double x = rfma(-l[t + 1], u[lane], S[lane][t + 1]);
-                const double al = __shfl_sync(kFull, x, t + 1);
-                const double s = al < 0.0 ? 1.0 : -1.0;
-                if (lane == 0) sg[t + 1] = s;
-                cb[(t + 1) & 1][lane] = lane > t ? x - s * Rb[lane][t + 1] : 0.0;
-            }
-            if (lane >= t) p.U[(b0 + t) + (b0 + lane) * GLD] = u[lane];  // row t of U
-        } else {
-            for (int q = warp - 2; q < GB - 1; q += 6) {
-                if (q <= t) E[q][lane] = rfma(-li, E[q][t], E[q][lane]);
-                else if (lane != t + 1) S[q + 1][lane] = rfma(-li, u[q + 1], S[q + 1][lane]);
-            }
-            if (t == GB - 1 && warp == 2) E[GB - 1][lane] = rfma(-li, E[GB - 1][t], E[GB - 1][lane]);
+            const double x = rfma(-rb[t & 1], cb[t & 1][t + 1] * u[lane], S[lane][t + 1]);
+            const double s = __shfl_sync(kFull, x, t + 1) < 0.0 ? 1.0 : -1.0;
+            if (lane == 0) sg[t + 1] = s;
+            const double un = lane > t ? x - s * Rb[lane][t + 1] : 0.0;
+            ub[(t + 1) & 1][lane] = un;
+            p.U[(b0 + t + 1) + (b0 + lane) * GLD] = un;
+        } else if (t + warp < GB) {
+            const double li = cb[t & 1][lane] * rb[t & 1];
+            if (lane > t + 1)
+                for (int j = t + warp; j < GB; j += 6) S[j][lane] = rfma(-li, u[j], S[j][lane]);
         }
         __syncthreads();
     }
-    for (int c = warp; c < GB; c += 8) {
-        p.L[(b0 + lane) + (b0 + c) * GLD] = lane > c ? S[c][lane] : (lane == c ? 1.0 : 0.0);
-        p.LI[(b0 + lane) + (b0 + c) * GLD] = E[c][lane];
-        if (lane > c) p.U[(b0 + lane) + (b0 + c) * GLD] = 0.0;
+    // L(i, t) = column t times 1 / u_tt
+#pragma unroll
+    for (int q = 0; q < GB / 8; ++q) {
+        const int c = warp + 8 * q;
+        const double l = S[c][lane] * rd[c];
+        p.L[(b0 + lane) + (b0 + c) * GLD] = lane > c ? l : (lane == c ? 1.0 : 0.0);
+        p.M[(UF_L * GB + c) * GB + lane] = lane > c ? l : 0.0;
+        p.M[(UF_U * GB + c) * GB + lane] = lane > c ? __ldcg(p.U + (b0 + c) + (b0 + lane) * GLD) * rd[c] : 0.0;
     }
-    if (tid < GB) p.sgn[b0 + tid] = sg[tid];
-    __syncthreads();
-    // X = U^{-1}: upper triangular inverse, diagonal 1 / u_tt in rd
-    double *Gs = &E[0][0], *Ts = &S[0][0], *Ms = &Rb[0][0];
-    for (int idx = tid; idx < GB * GB; idx += kThreads)
-        Gs[idx] = __ldcg(p.U + (b0 + idx % GB) + (b0 + idx / GB) * GLD);
-    __syncthreads();
-    build_t(Ts, Gs, rd, Ms, GB);
-    for (int idx = tid; idx < GB * GB; idx += kThreads) p.X[(b0 + idx % GB) + (b0 + idx / GB) * GLD] = Ts[idx];
+    if (tid < GB) {
+        p.sgn[b0 + tid] = sg[tid];
+        p.sc[GB + tid] = rd[tid];
+    }
 }
 
 // acc += sum_kk A(i, kk) B(kk, c) over one 32-wide step; A staged in sA
@@ -238,57 +253,88 @@ struct Tile {
 __device__ __forceinline__ const double *blk(const double *M, int i, int j) { return M + i * GB + j * GB * GLD; }
 __device__ __forceinline__ double *blk(double *M, int i, int j) { return M + i * GB + j * GB * GLD; }
 
-// Block row k of R and U (tasks 0 .. n-k-2), block column k of L (the next
-// n-k-1), then for l < k: YX_l = U_lk X_kk, YR_l = R_lk RI_kk and YL_l =
-// sum_j L_kj LI_jl.  blockIdx.x = task * 8 + column group.
+// y <- the solution of a unit triangular system by substitution, one warp,
+// lane = unknown: y_i -= M[t][i] y_t for t = 0, 1, ...
+__device__ __forceinline__ double unit_solve(const double (*M)[GB + 1], double y) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll 8
+    for (int t = 0; t + 1 < GB; ++t) y = rfma(-M[t][lane], __shfl_sync(kFull, y, t), y);
+    return y;
+}
+__device__ __forceinline__ void load_unit(double (*M)[GB + 1], const double *src, int which) {
+    for (int t = threadIdx.x >> 5; t < GB; t += GT / 32)
+        M[t][threadIdx.x & 31] = __ldcg(src + (which * GB + t) * GB + (threadIdx.x & 31));
+}
+
+// Solves with diagonal block k, a warp per column or row: block row k of R and
+// U (tasks 0 .. n-k-2), block column k of L (the next n-k-1), the diagonal
+// blocks of U^{-1}, R^{-1} and V1^{-1} (3 tasks); then for l < k: YX_l = U_lk
+// U_kk^{-1}, YR_l = R_lk R_kk^{-1} and YL_l = sum_j L_kj LI_jl.
+// blockIdx.x = task * 8 + column (row) group.
 __global__ void __launch_bounds__(GT) gram_row_kernel(const GramArgs p, int k) {
     __shared__ double sA[GB][GB + 1], sB[4][GB];
     if (*(volatile int *)p.flag) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    Tile tl{sA, sB, warp, lane};
-    const int task = blockIdx.x >> 3, c0 = (blockIdx.x & 7) * 4, rest = p.nblk - k - 1;
-    const int c = c0 + warp;
+    int task = blockIdx.x >> 3;
+    const int c0 = (blockIdx.x & 7) * 4, rest = p.nblk - k - 1, c = c0 + warp;
+    const double rinv = __ldcg(p.sc + lane), uinv = __ldcg(p.sc + GB + lane);
     if (task < rest) {
         const int j = k + 1 + task;
-        tl.load_a(blk(p.RI, k, k), true);                      // R_kj = RI_kk^T G_kj
-        sB[warp][lane] = g_at(p, k * GB + lane, j * GB + c, k);
-        const double a = a1_at(p, k * GB + lane, j * GB + c, k);
+        const double g = g_at(p, k * GB + lane, j * GB + c, k), a = a1_at(p, k * GB + lane, j * GB + c, k);
+        load_unit(sA, p.M, UF_CHOL);                           // R_kk^T R_kj = G_kj
         __syncthreads();
-        const double r = tl.dot(0.0);
-        __syncthreads();
+        const double r = unit_solve(sA, g) * rinv;
         blk(p.R, k, j)[lane + c * GLD] = r;
-        tl.load_a(blk(p.LI, k, k), false);                     // U_kj = V1_kk^{-1} (A1_kj - S R_kj)
-        sB[warp][lane] = rfma(-__ldcg(p.sgn + k * GB + lane), r, a);
         __syncthreads();
-        blk(p.U, k, j)[lane + c * GLD] = tl.dot(0.0);
+        load_unit(sA, p.M, UF_L);                              // V1_kk U_kj = A1_kj - S R_kj
+        __syncthreads();
+        blk(p.U, k, j)[lane + c * GLD] = unit_solve(sA, rfma(-__ldcg(p.sgn + k * GB + lane), r, a));
         return;
     }
-    if (task < 2 * rest) {
-        const int i = k + 1 + task - rest;                     // L_ik = A1_ik X_kk
-        for (int kk = warp; kk < GB; kk += 4) sA[kk][lane] = a1_at(p, i * GB + lane, k * GB + kk, k);
-        tl.load_b(blk(p.X, k, k) + c0 * GLD);
+    task -= rest;
+    if (task < rest) {
+        const int i = k + 1 + task;                            // L_ik U_kk = A1_ik, row c
+        const double a = a1_at(p, i * GB + c, k * GB + lane, k);
+        load_unit(sA, p.M, UF_U);
         __syncthreads();
-        blk(p.L, i, k)[lane + c * GLD] = tl.dot(0.0);
+        blk(p.L, i, k)[c + lane * GLD] = unit_solve(sA, a) * uinv;
         return;
     }
-    const int e = task - 2 * rest, l = e / 3, what = e % 3;
-    double *out = what == 0 ? p.YX : (what == 1 ? p.YR : p.YL);
-    double acc = 0.0;
-    if (what < 2) {
-        tl.load_a(blk(what == 0 ? p.U : p.R, l, k), false);
-        tl.load_b(blk(what == 0 ? p.X : p.RI, k, k) + c0 * GLD);
+    task -= rest;
+    if (task < 3) {
+        load_unit(sA, p.M, task == 0 ? UF_U : (task == 1 ? UF_CHOL : UF_L));
         __syncthreads();
-        acc = tl.dot(0.0);
-    } else {
-        for (int j = l; j < k; ++j) {
-            __syncthreads();
-            tl.load_a(blk(p.L, k, j), false);
-            tl.load_b(blk(p.LI, j, l) + c0 * GLD);
-            __syncthreads();
-            acc = tl.dot(acc);
+        double y = unit_solve(sA, lane == c ? 1.0 : 0.0);      // row c of U^{-1}, R^{-1}; column c of V1^{-1}
+        if (task == 0) {
+            blk(p.X, k, k)[c + lane * GLD] = y * uinv;
+        } else if (task == 1) {
+            y *= rinv;
+            blk(p.RI, k, k)[c + lane * GLD] = y;
+            // the row is scaled by the norm of column b0 + c of the panel
+            if (!(y * y * __ldcg(p.gd + k * GB + c) <= kGramBound2)) *(volatile int *)p.flag = 1;
+        } else {
+            blk(p.LI, k, k)[lane + c * GLD] = y;
         }
+        return;
     }
-    out[l * GB + lane + c * GLD] = acc;                        // Y_l: block row l of a w x 32 array
+    const int e = task - 3, l = e / 3, what = e % 3;
+    if (what < 2) {
+        const double a = __ldcg(blk(what == 0 ? p.U : p.R, l, k) + c + lane * GLD);   // row c
+        load_unit(sA, p.M, what == 0 ? UF_U : UF_CHOL);
+        __syncthreads();
+        (what == 0 ? p.YX : p.YR)[l * GB + c + lane * GLD] = unit_solve(sA, a) * (what == 0 ? uinv : rinv);
+        return;
+    }
+    Tile tl{sA, sB, warp, lane};
+    double acc = 0.0;
+    for (int j = l; j < k; ++j) {
+        __syncthreads();
+        tl.load_a(blk(p.L, k, j), false);
+        tl.load_b(blk(p.LI, j, l) + c0 * GLD);
+        __syncthreads();
+        acc = tl.dot(acc);
+    }
+    p.YL[l * GB + lane + c * GLD] = acc;                       // Y_l: block row l of a w x 32 array
 }
 
 // Trailing blocks of G (upper) and A1, then for l < k: X_lk = -sum X_lj YX_j,
@@ -333,32 +379,47 @@ __global__ void __launch_bounds__(GT) gram_trail_kernel(const GramArgs p, int k)
     if (what == 1 && !(acc * acc * __ldcg(p.gd + l * GB + lane) <= kGramBound2)) *(volatile int *)p.flag = 1;
 }
 
-// K = U R^{-1} (step 0), then T = -K S' ... (step 1): T = -U (S R)^{-1} V1^{-T}
-// = -U R^{-1} S V1^{-T}.  Step 1 also writes V1 \ R over the panel's top block.
+// K = (U R^{-1}) S (step 0), then T = -K V1^{-T} (step 1): T = -U (S R)^{-1}
+// V1^{-T}, both products upper triangular.  A CTA takes 32 x 2 outputs of
+// block (i, j), a warp one column and the even or odd 32-wide steps; all
+// operands are staged at once.  Step 1 also writes V1 \ R over the panel's
+// top block.  blockIdx.x = task * 16 + column pair.
 __global__ void __launch_bounds__(GT) gram_t_kernel(const GramArgs p, int step) {
-    __shared__ double sA[GB][GB + 1], sB[4][GB];
+    __shared__ double sA[4][GB][GB + 1], sB[2][4 * GB], part[2][GB];
     if (*(volatile int *)p.flag) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    Tile tl{sA, sB, warp, lane};
-    const int c0 = (blockIdx.x & 7) * 4, c = c0 + warp, task = blockIdx.x >> 3;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, col = warp & 1, half = warp >> 1;
+    const int c0 = (blockIdx.x & 15) * 2, c = c0 + col, task = blockIdx.x >> 4;
     const int i = task % p.nblk, j = task / p.nblk;
     const int gi = i * GB + lane, gj = j * GB + c;
     double acc = 0.0;
-    if (i <= j)
+    if (i <= j) {
+        const double *A = step == 0 ? p.U : p.K;
         for (int l = i; l <= j; ++l) {
-            __syncthreads();
-            if (step == 0) {
-                tl.load_a(blk(p.U, i, l), false);
-                tl.load_b(blk(p.RI, l, j) + c0 * GLD);
-            } else {
-                tl.load_a(blk(p.K, i, l), false);
-                tl.load_b(blk(p.LI, j, l) + c0, true);         // (V1^{-T})(l, j) = LI(j, l)^T
-            }
-            __syncthreads();
-            acc = tl.dot(acc);
+#pragma unroll
+            for (int q = 0; q < GB / 4; ++q) sA[l - i][warp + 4 * q][lane] = __ldcg(blk(A, i, l) + lane + (warp + 4 * q) * GLD);
+            // B(l, c): R^{-1} block (l, j), or V1^{-T}(l, j) = LI(j, l)^T
+            if (half == ((l - i) & 1))
+                sB[col][(l - i) * GB + lane] = step == 0 ? __ldcg(blk(p.RI, l, j) + lane + c * GLD)
+                                                         : __ldcg(blk(p.LI, j, l) + c + lane * GLD);
         }
+        __syncthreads();
+        double a0 = 0.0, a1 = 0.0;
+        for (int l = half; l <= j - i; l += 2)
+#pragma unroll
+            for (int kk = 0; kk < GB; kk += 2) {
+                a0 = rfma(sA[l][kk][lane], sB[col][l * GB + kk], a0);
+                a1 = rfma(sA[l][kk + 1][lane], sB[col][l * GB + kk + 1], a1);
+            }
+        acc = a0 + a1;
+        if (half) part[col][lane] = acc;
+        __syncthreads();
+        if (half) return;
+        acc += part[col][lane];
+    } else if (half) {
+        return;
+    }
     if (step == 0) {
-        if (i <= j) blk(p.K, i, j)[lane + c * GLD] = acc * __ldcg(p.sgn + gj);   // (U R^{-1}) S
+        if (i <= j) blk(p.K, i, j)[lane + c * GLD] = acc * __ldcg(p.sgn + gj);
         return;
     }
     if (gi >= p.w || gj >= p.w) return;
@@ -369,7 +430,7 @@ __global__ void __launch_bounds__(GT) gram_t_kernel(const GramArgs p, int step) 
 
 }  // namespace
 
-size_t gram_work_elems() { return (size_t)13 * GLD * GLD + 4 * GLD; }
+size_t gram_work_elems() { return (size_t)12 * GLD * GLD + 3 * GB * GB + 2 * GB + 4 * GLD; }
 
 bool gram_qr_fits(const OzScratch &oz, int64_t m, int64_t w) {
     return w >= kGramMinW && w <= kGramMaxW && m >= 4 * w && oz.base &&
@@ -384,7 +445,9 @@ gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, double *A, int64_t lda
     double **slots[] = {&p.G, &p.R, &p.RI, &p.A1, &p.L, &p.U, &p.LI, &p.X, &p.YX, &p.YR, &p.YL, &p.K};
     double *at = work;
     for (double **s : slots) { *s = at; at += (size_t)GLD * GLD; }
-    p.sgn = at;
+    p.M = at;
+    p.sc = p.M + 3 * GB * GB;
+    p.sgn = p.sc + 2 * GB;
     p.gd = p.sgn + GLD;
     p.flag = flag;
     p.kexp = (int *)(p.gd + GLD);
@@ -398,11 +461,11 @@ gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, double *A, int64_t lda
         trace_begin(ex, FAM_OTHER);
         gram_diag_kernel<<<1, kThreads, 0, ex.stream>>>(p, k);
         TRY_ST(mark(3.0 * f3));
-        const int rest = p.nblk - k - 1, row = 2 * rest + 3 * k, trail = 2 * rest * rest + 3 * k;
-        if (row) {
-            trace_begin(ex, FAM_OTHER);
-            gram_row_kernel<<<row * 8, GT, 0, ex.stream>>>(p, k);
-            TRY_ST(mark(row * f3));
+        const int rest = p.nblk - k - 1, row = 2 * rest + 3 + 3 * k, trail = 2 * rest * rest + 3 * k;
+        trace_begin(ex, FAM_OTHER);
+        gram_row_kernel<<<row * 8, GT, 0, ex.stream>>>(p, k);
+        TRY_ST(mark(row * f3));
+        if (trail) {
             trace_begin(ex, FAM_OTHER);
             gram_trail_kernel<<<trail * 8, GT, 0, ex.stream>>>(p, k);
             TRY_ST(mark(trail * f3));
@@ -410,7 +473,7 @@ gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, double *A, int64_t lda
     }
     for (int step = 0; step < 2; ++step) {
         trace_begin(ex, FAM_OTHER);
-        gram_t_kernel<<<p.nblk * p.nblk * 8, GT, 0, ex.stream>>>(p, step);
+        gram_t_kernel<<<p.nblk * p.nblk * 16, GT, 0, ex.stream>>>(p, step);
         TRY_ST(mark(p.nblk * p.nblk * f3));
     }
     if (m > w) {

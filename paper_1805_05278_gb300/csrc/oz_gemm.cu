@@ -157,15 +157,31 @@ __device__ __forceinline__ void store_digits(const OzOperand &o, int64_t r, int6
     }
 }
 
+// Four consecutive entries of operand row r (a column of X) from k0 on.
+__device__ __forceinline__ void load_quad(const OzOperand &o, bool plain, int64_t r, int64_t k0, double (&v)[4]) {
+    if (plain && k0 + 4 <= o.K) {
+        const double *x = o.X + k0 + r * o.ld;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = x[q];
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = oz_load(o, r, k0 + q);
+    }
+}
+
 // Digits of both operands of a product: the first a.blocks CTAs work on A.
-// Bound by HBM (8 bytes read, 14 written per entry; the second read of a
-// column comes from L2) and, for few rows, by latency.
+// Bound by HBM (8 bytes read, 14 written per entry) and, for few rows, by
+// latency, so every entry is read once where registers hold the row between
+// the search for its maximum and the split: NT threads keep NQ quads each
+// (256 x 8: rows of 8192; 1024 x 4: 16384; what lies beyond is read again).
 //   by column: a warp per operand row (K <= 1024) or a CTA per row; a thread
 //              takes 4 consecutive k (8-byte stores, a warp 256 bytes).
 //   by row:    a CTA takes 32 rows, lane = row, a warp 16 consecutive k (reads
 //              are coalesced along the rows, a store is one 32-byte sector).
-__global__ void __launch_bounds__(kThreads) oz_slice_kernel(const OzOperand a, const OzOperand b) {
-    __shared__ int red[8][32];
+template <int NT, int NQ>
+__global__ void __launch_bounds__(NT) oz_slice_kernel(const OzOperand a, const OzOperand b) {
+    __shared__ int red[NT / 32][32];
+    constexpr int NW = NT / 32;
     const bool isB = blockIdx.x >= a.blocks;
     const OzOperand &o = isB ? b : a;
     if (o.skip && *(volatile const int *)o.skip) return;
@@ -174,8 +190,8 @@ __global__ void __launch_bounds__(kThreads) oz_slice_kernel(const OzOperand a, c
     int ex = 0;
     if (o.by_row) {
         const int64_t r = blk * 32 + lane;
-        for (int64_t k0 = warp * 16; k0 < o.K; k0 += 128) {
-            double v[16];
+        double v[16];
+        for (int64_t k0 = warp * 16; k0 < o.K; k0 += 16 * NW) {
 #pragma unroll
             for (int q = 0; q < 16; ++q) v[q] = oz_load(o, r, k0 + q);
 #pragma unroll
@@ -184,41 +200,66 @@ __global__ void __launch_bounds__(kThreads) oz_slice_kernel(const OzOperand a, c
         red[warp][lane] = ex;
         __syncthreads();
 #pragma unroll
-        for (int w = 0; w < 8; ++w) ex = max(ex, red[w][lane]);
+        for (int w = 0; w < NW; ++w) ex = max(ex, red[w][lane]);
         ex = max(ex, 1);
         if (r >= o.R) return;
         if (warp == 0) o.exps[r] = ex == 0x7ff ? kExpNan : ex - 1022;
-        for (int64_t k0 = warp * 16; k0 < o.ldk; k0 += 128) {
-            double v[16];
+        const bool kept = o.K <= 16 * NW;                       // v holds this warp's only 16 k
+        for (int64_t k0 = warp * 16; k0 < o.ldk; k0 += 16 * NW) {
 #pragma unroll
-            for (int q = 0; q < 16; ++q) v[q] = ex == 0x7ff ? 0.0 : oz_load(o, r, k0 + q);
+            for (int q = 0; q < 16; ++q) {
+                if (ex == 0x7ff || (kept && k0 >= o.K)) v[q] = 0.0;
+                else if (!kept) v[q] = oz_load(o, r, k0 + q);
+            }
             store_digits(o, r, k0, v, ex);
         }
         return;
     }
     const bool wide = o.K > 1024;
-    const int64_t r = wide ? blk : blk * 8 + warp;
-    const int t = wide ? (int)threadIdx.x : lane, nt = wide ? kThreads : 32;
-    if (r < o.R)
-        for (int64_t k0 = t * 4; k0 < o.K; k0 += nt * 4) {
+    const int64_t r = wide ? blk : blk * NW + warp;
+    const int t = wide ? (int)threadIdx.x : lane, nt = wide ? NT : 32;
+    const bool plain = o.mask == MASK_NONE && !o.kexp;
+    double v[NQ][4];
+    if (r < o.R) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) ex = max(ex, exp_field(oz_load(o, r, k0 + q)));
+        for (int q = 0; q < NQ; ++q) load_quad(o, plain, r, (int64_t)(t + q * nt) * 4, v[q]);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) ex = max(ex, exp_field(v[q][i]));
+        for (int64_t k0 = (int64_t)(t + NQ * nt) * 4; k0 < o.K; k0 += nt * 4) {
+            double x[4];
+            load_quad(o, plain, r, k0, x);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) ex = max(ex, exp_field(x[i]));
         }
+    }
     ex = __reduce_max_sync(0xffffffffu, ex);
     if (wide) {
         if (lane == 0) red[0][warp] = ex;
         __syncthreads();
 #pragma unroll
-        for (int w = 0; w < 8; ++w) ex = max(ex, red[0][w]);
+        for (int w = 0; w < NW; ++w) ex = max(ex, red[0][w]);
     }
     if (r >= o.R) return;
     ex = max(ex, 1);
     if (t == 0) o.exps[r] = ex == 0x7ff ? kExpNan : ex - 1022;
-    for (int64_t k0 = t * 4; k0 < o.ldk; k0 += nt * 4) {
-        double v[4];
+    if (ex == 0x7ff) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = ex == 0x7ff ? 0.0 : oz_load(o, r, k0 + q);
-        store_digits(o, r, k0, v, ex);
+        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[q][i] = 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+        if ((int64_t)(t + q * nt) * 4 < o.ldk) store_digits(o, r, (int64_t)(t + q * nt) * 4, v[q], ex);
+    for (int64_t k0 = (int64_t)(t + NQ * nt) * 4; k0 < o.ldk; k0 += nt * 4) {
+        double x[4];
+        load_quad(o, plain, r, k0, x);
+        if (ex == 0x7ff)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[i] = 0.0;
+        store_digits(o, r, k0, x, ex);
     }
 }
 
@@ -598,8 +639,10 @@ static gbqr_status oz_chunk(const Exec &ex, const GemmOp &op, const OzScratch &s
     a.dst = (__nv_bfloat16 *)(base + L.a); a.ldk = L.ldk; a.exps = (int *)(base + L.ea);
     b.X = op.B; b.ld = op.ldb; b.R = op.N; b.K = op.K; b.mask = op.maskB; b.by_row = 0;
     b.dst = (__nv_bfloat16 *)(base + L.b); b.ldk = L.ldk; b.exps = (int *)(base + L.eb);
-    auto blocks = [](const OzOperand &o) {
-        return (unsigned)(o.by_row ? (o.R + 31) / 32 : (o.K > 1024 ? o.R : (o.R + 7) / 8));
+    const bool tall = op.K > 8192;                               // 1024 threads per row, else 256
+    const int warps = tall ? 32 : 8;
+    auto blocks = [&](const OzOperand &o) {
+        return (unsigned)(o.by_row ? (o.R + 31) / 32 : (o.K > 1024 ? o.R : (o.R + warps - 1) / warps));
     };
     a.blocks = slice_a ? blocks(a) : 0;
     b.blocks = blocks(b);
@@ -612,7 +655,9 @@ static gbqr_status oz_chunk(const Exec &ex, const GemmOp &op, const OzScratch &s
     a.ksign = -1;
     b.ksign = 1;
     trace_begin(ex, FAM_OTHER);
-    if (a.blocks + b.blocks) oz_slice_kernel<<<a.blocks + b.blocks, kThreads, 0, ex.stream>>>(a, b);
+    const unsigned nblk = a.blocks + b.blocks;
+    if (nblk && tall) oz_slice_kernel<1024, 4><<<nblk, 1024, 0, ex.stream>>>(a, b);
+    else if (nblk) oz_slice_kernel<kThreads, 8><<<nblk, kThreads, 0, ex.stream>>>(a, b);
     TRY_ST(trace_end(ex, FAM_OTHER, 0.0, 22.0 * ((double)op.M + op.N) * op.K));
 
     OzParams p{};
