@@ -8,6 +8,7 @@
 // All device work is enqueued on the context's stream; nothing here computes
 // on the host.
 #include "common.cuh"
+#include "oz.cuh"
 
 #include <algorithm>
 #include <climits>
@@ -32,8 +33,9 @@ constexpr int kKrylov = 100;          // GMRES refinement: Arnoldi steps per cor
 constexpr int kInPanelTcMinCols = 32;  // mixed path: in-panel updates on the tensor cores from n1 >= 32 (16 measured slower) ...
 constexpr int64_t kInPanelTcMinRows = 2048;   // ... and m >= 2048
 constexpr int kMaxBatchLanes = 128;
-constexpr size_t kOzMainBytes = (size_t)448 << 20;   // digit scratch of the trailing updates (8192^2: up to three column chunks)
+constexpr size_t kOzMainBytes = (size_t)384 << 20;   // digit scratch of the trailing updates (8192^2: up to three column chunks)
 constexpr int64_t kOzChunkCols = 512;              // ... never less than this many columns' worth
+constexpr int64_t kFusedMinRows = 256;             // shorter matrices update by separate products
 constexpr int kGramFallbackB = 64;   // TSQR width behind a Gram-matrix panel: few launches, which mostly return at once
 
 struct DeviceInfo {
@@ -126,6 +128,7 @@ struct Layout {
     size_t tc2 = 0, n_tc2 = 0;                            // ... of the look-ahead lane's in-panel updates
     size_t oz = 0, n_oz = 0, oz2 = 0, n_oz2 = 0;          // digit-split FP64 products, main and look-ahead lane
     size_t gram = 0, n_gram = 0;                          // Gram-matrix panels: w x w arrays and the flag
+    size_t Y = 0, n_Y = 0, vy = 0, n_vy = 0;              // fused updates: Y = V T, and two panels' digits of V and Y
     size_t kry = 0, n_kry = 0;                            // least squares, mixed: Krylov basis of the refinement
     size_t dinv = 0, n_dinv = 0;                          // ... and inverses of R's diagonal blocks
     size_t total = 0;
@@ -188,16 +191,25 @@ Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num
         // only) and of V, up to kOzMainBytes - wider updates go in column
         // chunks - and of a panel's halves on the look-ahead lane
         const int64_t mm = std::max<int64_t>(m, 1), nn = std::max<int64_t>(n, 1), kv = t_layout == GBQR_T_FULL ? (nn + 1) / 2 : nb;
-        auto need = [&](int64_t cols) { return std::max(oz_gemm_scratch_bytes(kv, cols, mm), oz_gemm_scratch_bytes(mm, cols, kv)); };
-        L.n_oz = pr.nsplit > 0 ? oz_gemm_scratch_bytes(kv, nn, kv)
+        auto need = [&](int64_t cols) {
+            return std::max(oz_gemm_scratch_bytes<double>(kv, cols, mm), oz_gemm_scratch_bytes<double>(mm, cols, kv));
+        };
+        L.n_oz = pr.nsplit > 0 ? oz_gemm_scratch_bytes<double>(kv, nn, kv)
                                : std::max(need(std::min(nn, kOzChunkCols)), std::min(need(nn), kOzMainBytes));
-        // a panel: its Gram matrix and V, or the products of its halves
+        // a panel: its Gram matrix, V and Y, or the products of its halves
         const int64_t h = gram ? std::min<int64_t>(nb, kGramMaxW) : std::max<int64_t>((nb + 1) / 2, 1);
-        const size_t panel = std::max(oz_gemm_scratch_bytes(h, h, mm), oz_gemm_scratch_bytes(mm, h, h));
+        const size_t panel = gram ? std::max(gram_scratch_bytes<double>(mm, h), oz_gemm_scratch_bytes<double>(mm, h, h))
+                                  : std::max(oz_gemm_scratch_bytes<double>(h, h, mm), oz_gemm_scratch_bytes<double>(mm, h, h));
         if (gram || !pr.lookahead) L.n_oz = std::max(L.n_oz, panel);
         L.oz = take(L.n_oz);
         L.n_oz2 = pr.lookahead && nn > nb ? panel : 0;
         if (L.n_oz2) L.oz2 = take(L.n_oz2);
+        if (gram && t_layout == GBQR_T_PANEL && pr.nsplit == 0 && nn > nb && nb <= kGramMaxW && mm >= kFusedMinRows) {
+            L.n_Y = (size_t)mm * nb;
+            L.Y = take(L.n_Y * 8);
+            L.n_vy = 2 * (oz_digit_bytes(kOzDigits64, mm, nb, kOzTileA) + oz_digit_bytes(kOzDigits64, nb, mm, kOzTileA));
+            L.vy = take(L.n_vy);
+        }
         if (gram) {
             L.n_gram = gram_work_elems();
             L.gram = take(L.n_gram * 8 + 16);
@@ -339,6 +351,8 @@ struct Work {
     double *M1b, *M2b;
     double *gram = nullptr;          // Gram-matrix panels: work, and the flag behind it (null: TSQR only)
     int *gram_flag = nullptr;
+    double *Y = nullptr;             // fused updates (null: none)
+    char *vy = nullptr;
 
     // Typed views of the workspace (regions are sized for FP64; an FP32 call
     // uses the same bytes).
@@ -427,6 +441,8 @@ void carve_work(gbqr_ctx *cx, char *base, const Layout &L, const Params &pr, con
     w->gs2.ncounters = w->L.n_gcount;
     w->gs2.oz = {w->L.n_oz2 ? (void *)(base + w->L.oz2) : nullptr, w->L.n_oz2, &cx->dinfo->timeout};
     w->gram = w->L.n_gram ? (double *)(base + w->L.gram) : nullptr;
+    w->Y = w->L.n_vy ? (double *)(base + w->L.Y) : nullptr;
+    w->vy = w->L.n_vy ? base + w->L.vy : nullptr;
     w->gram_flag = w->L.n_gram ? (int *)(w->gram + w->L.n_gram) : nullptr;
     w->M1b = (double *)(base + w->L.M1b);
     w->M2b = (double *)(base + w->L.M2b);
@@ -530,25 +546,44 @@ gbqr_status base_qr(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, Real *T
     return tsqr_run(w.ex, pl, A, lda, T, ldt, w.twr<Real>());
 }
 
+template <class Real>
+gbqr_status qr_eg(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, Real *T, int64_t ldt);
+
+// Y (m x n) = V T for the panel V \ R of A.
+template <class Real>
+gbqr_status form_y(const Exec &ex, const GemmScratchT<Real> &gs, int64_t m, int64_t n, const Real *A, int64_t lda,
+                   const Real *T, int64_t ldt, Real *Y, int64_t ldy) {
+    GemmOpT<Real> y;
+    y.M = m; y.N = n; y.K = n;
+    y.A = A; y.lda = lda; y.maskA = MASK_UNIT_LOWER;
+    y.B = T; y.ldb = ldt; y.maskB = MASK_UPPER;
+    y.C = Y; y.ldc = ldy;
+    return gemm(ex, y, gs);
+}
+
+// A panel from its Gram matrix.  Where that is too ill-conditioned the flag is
+// up and A as it was, and the recursion on FMA products and wide TSQRs, whose
+// launches return at once while the flag is zero, does it.  Y: V T, or null.
+template <class Real>
+gbqr_status gram_or_tsqr(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, Real *T, int64_t ldt, Real *Y, int64_t ldy) {
+    TRY(gram_qr(w.ex, m, n, A, lda, T, ldt, Y, ldy, w.gram, w.gram_flag, w.gs.oz));
+    Work f = w;
+    f.ex.pred = w.gram_flag;
+    TsqrPlan pl;
+    const int64_t n1 = n <= kGramFallbackB ? n : n / 2;
+    const bool wide = tsqr_plan(m, (int)n1, 0, 0, w.ex.num_sms, &pl) &&
+                      (n1 == n || tsqr_plan(m - n1, (int)(n - n1), 0, 0, w.ex.num_sms, &pl));
+    f.pr.b = wide ? kGramFallbackB : kGramFallbackB / 2;
+    TRY(qr_eg(f, m, n, A, lda, T, ldt));
+    return Y ? form_y(f.ex, f.gsr<Real>(), m, n, A, lda, T, ldt, Y, ldy) : GBQR_OK;
+}
+
 // Algorithm 2: (V, T, R) = QR-EG(A, b), V\R in place over A, T (n x n) at T.
 template <class Real>
 gbqr_status qr_eg(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, Real *T, int64_t ldt) {
     if (n <= 0) return GBQR_OK;
-    if constexpr (std::is_same<Real, double>::value) {
-        if (w.gram && !w.ex.pred && gram_qr_fits(w.gs.oz, m, n)) {
-            TRY(gram_qr(w.ex, m, n, A, lda, T, ldt, w.gram, w.gram_flag, w.gs.oz));
-            // ill-conditioned panels: the flag is up and A as it was, and
-            // the same recursion on FMA products and wide TSQRs runs
-            Work f = w;
-            f.ex.pred = w.gram_flag;
-            TsqrPlan pl;
-            const int64_t n1 = n <= kGramFallbackB ? n : n / 2;
-            const bool wide = tsqr_plan(m, (int)n1, 0, 0, w.ex.num_sms, &pl) &&
-                              (n1 == n || tsqr_plan(m - n1, (int)(n - n1), 0, 0, w.ex.num_sms, &pl));
-            f.pr.b = wide ? kGramFallbackB : kGramFallbackB / 2;
-            return qr_eg(f, m, n, A, lda, T, ldt);
-        }
-    }
+    if (w.gram && !w.ex.pred && gram_qr_fits<Real>(w.gs.oz, m, n))
+        return gram_or_tsqr<Real>(w, m, n, A, lda, T, ldt, nullptr, 0);
     if (n <= w.pr.b) return base_qr(w, m, n, A, lda, T, ldt);
     const int64_t n1 = n / 2, n2 = n - n1;
     Real *AR = A + n1 * lda;
@@ -584,6 +619,91 @@ gbqr_status qr_eg(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, Real *T, 
     g5.B = M2; g5.ldb = n1;
     g5.C = T + n1 * ldt; g5.ldc = ldt; g5.alpha = Real(-1); g5.beta = Real(0);
     return gemm(w.ex, g5, gsr);
+}
+
+// ---- fused updates of the right-looking top level.  With Y = V T the update
+// C -= V T^T V^T C is W = Y^T C, C -= V W: two digit-split products, the T
+// product gone, W going from the first one's integer sums straight to the
+// second one's digits, and the digits of V and Y taken once per panel for the
+// look-ahead update and the trailing one.
+template <class Real>
+struct PanelDigits { OzOperand<Real> v, y; };
+
+// Panel [0, wd) of the m-row A, and its digits in buffer `buf`.
+template <class Real>
+gbqr_status factor_panel(Work &w, int64_t m, int64_t wd, Real *A, int64_t lda, Real *T, int64_t ldt, int buf,
+                         PanelDigits<Real> *pd) {
+    Real *Y = reinterpret_cast<Real *>(w.Y);
+    if (w.gram && gram_qr_fits<Real>(w.gs.oz, m, wd)) {
+        TRY(gram_or_tsqr(w, m, wd, A, lda, T, ldt, Y, m));
+    } else {
+        TRY(qr_eg(w, m, wd, A, lda, T, ldt));
+        TRY(form_y(w.ex, w.gsr<Real>(), m, wd, A, lda, T, ldt, Y, m));
+    }
+    constexpr int D = oz_digits<Real>();
+    char *base = w.vy + (size_t)buf * (w.L.n_vy / 2);
+    pd->v = oz_operand(D, (const Real *)A, lda, m, wd, true, MASK_UNIT_LOWER, kOzTileA, base);
+    pd->y = oz_operand(D, (const Real *)Y, m, wd, m, false, MASK_NONE, kOzTileA, base + oz_digit_bytes(D, m, wd, kOzTileA));
+    OzOperand<Real> ops[2] = {pd->v, pd->y};
+    return oz_slice(w.ex, D, ops, 2);
+}
+
+// C (m x nc) <- (I - V T^T V^T) C from the panel's digits, in column chunks
+// whose digits fit the scratch.
+template <class Real>
+gbqr_status update_fused(Work &w, const PanelDigits<Real> &pd, int64_t m, int64_t nc, int64_t wd, Real *C, int64_t ldc) {
+    constexpr int D = oz_digits<Real>();
+    const OzScratch &sc = w.gs.oz;
+    const size_t splits = (size_t)(oz_ktiles(m) + 15) / 16;
+    const size_t per64 = oz_digit_bytes(D, 64, m, kOzTileB) + oz_digit_bytes(D, 64, wd, kOzTileB) + (splits + 1) * 64 * wd * 8;
+    const int64_t most = (int64_t)((sc.bytes - sc.bytes / 16) / per64) * 64;
+    if (most < 64) return GBQR_ENOMEM;
+    const int64_t chunks = (nc + most - 1) / most, step = ((nc + chunks - 1) / chunks + 63) / 64 * 64;
+    for (int64_t j = 0; j < nc; j += step) {
+        const int64_t n = std::min(step, nc - j);
+        char *base = (char *)sc.base;
+        const size_t nb_c = oz_digit_bytes(D, n, m, kOzTileB), nb_w = oz_digit_bytes(D, n, wd, kOzTileB);
+        const size_t nb_f = align_up((size_t)n * wd * sizeof(Real), 256), used = nb_c + nb_w + nb_f;
+        if (used >= sc.bytes) return GBQR_ENOMEM;
+        OzOperand<Real> c = oz_operand(D, (const Real *)(C + j * ldc), ldc, n, m, false, MASK_NONE, kOzTileB, base);
+        TRY(oz_slice(w.ex, D, &c, 1));
+        const OzOperand<Real> wq = oz_operand(D, (const Real *)nullptr, 1, n, wd, false, MASK_NONE, kOzTileB, base + nb_c);
+        Real *wf = reinterpret_cast<Real *>(base + nb_c + nb_w);
+        OzMmaArgs<Real> g{};
+        g.prob[0] = oz_problem<Real>(pd.y, c);
+        if (!oz_choose_split(g.prob[0], w.ex.num_sms, sc.bytes - used, true)) return GBQR_ENOMEM;
+        g.prob[0].partial = (long long *)(base + used);
+        g.prob[0].C = wf;
+        g.prob[0].ldc = wd;
+        g.prob[0].qdst = wq.dst;
+        g.prob[0].qexp = wq.exps;
+        g.n = 1;
+        g.items = oz_items((int)wd, (int)n, g.prob[0].S);
+        g.err = sc.err;
+        TRY(oz_mma_launch(w.ex, g, (double)wd * n * m));
+        TRY(oz_requant_launch(w.ex, g, (int)n));
+        OzMmaArgs<Real> u{};
+        u.prob[0] = oz_problem<Real>(pd.v, wq);
+        u.prob[0].C = C + j * ldc;
+        u.prob[0].ldc = ldc;
+        u.prob[0].alpha = Real(-1);
+        u.prob[0].beta = Real(1);
+        u.prob[0].add = wf;
+        u.prob[0].ldadd = wd;
+        u.prob[0].add_rows = (int)wd;
+        u.n = 1;
+        u.items = oz_items((int)m, (int)n, 1);
+        u.err = sc.err;
+        TRY(oz_mma_launch(w.ex, u, (double)wd * n * m));
+    }
+    return GBQR_OK;
+}
+
+// Whether an update is large enough for the fused products (four launches)
+// rather than three FMA ones: FP64 FMA reaches 1.15 TFLOP/s, FP32 about 9.
+template <class Real>
+bool update_large(int64_t m, int64_t nc, int64_t wd) {
+    return nc >= 8 && 4.0 * (double)m * nc * wd > (std::is_same<Real, double>::value ? 2e7 : 2e8);
 }
 
 // Zero T(i, j) for i > (j mod nb) (the strict lower part of every block).
@@ -657,15 +777,28 @@ gbqr_status factor_device(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, R
     TRY(zero_below_blocks(w, nb, n, nb, T, ldt));
     const int64_t npan = (n + nb - 1) / nb;
     gbqr_ctx *cx = w.cx;
+    // panel k with its digits where any update of it is large enough to use them
+    PanelDigits<Real> pd[2];
+    bool fused[2] = {false, false};
+    auto panel = [&](Work &wp, int64_t j0) -> gbqr_status {
+        const int64_t wd = std::min<int64_t>(nb, n - j0), k = j0 / nb;
+        Real *Ap = A + j0 + j0 * lda;
+        fused[k & 1] = w.vy && w.gs.oz.base && update_large<Real>(m - j0, n - j0 - wd, wd);
+        if (fused[k & 1]) return factor_panel(wp, m - j0, wd, Ap, lda, T + j0 * ldt, ldt, (int)(k & 1), &pd[k & 1]);
+        return qr_eg(wp, m - j0, wd, Ap, lda, T + j0 * ldt, ldt);
+    };
+    // panel k applied to columns [c0, c0 + nc)
+    auto update = [&](int64_t j0, int64_t c0, int64_t nc) -> gbqr_status {
+        const int64_t wd = std::min<int64_t>(nb, n - j0), k = j0 / nb;
+        Real *C = A + j0 + c0 * lda;
+        if (fused[k & 1] && update_large<Real>(m - j0, nc, wd)) return update_fused(w, pd[k & 1], m - j0, nc, wd, C, lda);
+        return apply_block(w, true, m - j0, nc, wd, A + j0 + j0 * lda, lda, T + j0 * ldt, ldt, C, lda, w.pr.nsplit);
+    };
     if (!w.pr.lookahead || npan == 1 || !cx->side) {
         for (int64_t j0 = 0; j0 < n; j0 += nb) {
             const int64_t wd = std::min<int64_t>(nb, n - j0);
-            Real *Ap = A + j0 + j0 * lda;
-            Real *Tk = T + j0 * ldt;
-            TRY(qr_eg(w, m - j0, wd, Ap, lda, Tk, ldt));
-            if (j0 + wd < n)
-                TRY(apply_block(w, true, m - j0, n - j0 - wd, wd, Ap, lda, Tk, ldt, A + j0 + (j0 + wd) * lda, lda,
-                                w.pr.nsplit));
+            TRY(panel(w, j0));
+            if (j0 + wd < n) TRY(update(j0, j0 + wd, n - j0 - wd));
         }
         return GBQR_OK;
     }
@@ -696,7 +829,7 @@ gbqr_status factor_device(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, R
     };
     if (cudaEventRecord(cx->ev_fork, ms) != cudaSuccess || cudaStreamWaitEvent(ss, cx->ev_fork, 0) != cudaSuccess)
         return GBQR_ECUDA;
-    TRY(qr_eg(wp, m, std::min<int64_t>(nb, n), A, lda, T, ldt));
+    TRY(panel(wp, 0));
     if (cudaEventRecord(cx->ev_panel, ss) != cudaSuccess) return GBQR_ECUDA;
     TRY(panel_out(0, std::min<int64_t>(nb, n)));
     for (int64_t k = 0; k < npan; ++k) {
@@ -704,21 +837,17 @@ gbqr_status factor_device(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, R
         if (cudaStreamWaitEvent(ms, cx->ev_panel, 0) != cudaSuccess) return GBQR_ECUDA;   // panel k done
         if (k + 1 == npan) break;
         const int64_t j1 = j0 + wd, w1 = std::min<int64_t>(nb, n - j1);
-        const Real *Vk = A + j0 + j0 * lda;
-        const Real *Tk = T + j0 * ldt;
         if (io && k == 0 && cudaStreamWaitEvent(ms, cx->ev_in1, 0) != cudaSuccess) return GBQR_ECUDA;
         // panel k+1's columns first ...
-        TRY(apply_block(w, true, m - j0, w1, wd, Vk, lda, Tk, ldt, A + j0 + j1 * lda, lda, w.pr.nsplit));
+        TRY(update(j0, j1, w1));
         if (cudaEventRecord(cx->ev_ready, ms) != cudaSuccess || cudaStreamWaitEvent(ss, cx->ev_ready, 0) != cudaSuccess)
             return GBQR_ECUDA;
         // ... then panel k+1 on the side stream, concurrently with the rest of the update
-        TRY(qr_eg(wp, m - j1, w1, A + j1 + j1 * lda, lda, T + j1 * ldt, ldt));
+        TRY(panel(wp, j1));
         if (cudaEventRecord(cx->ev_panel, ss) != cudaSuccess) return GBQR_ECUDA;
         TRY(panel_out(j1, w1));
         if (io && k == 0 && cudaStreamWaitEvent(ms, cx->ev_in, 0) != cudaSuccess) return GBQR_ECUDA;
-        if (j1 + w1 < n)
-            TRY(apply_block(w, true, m - j0, n - j1 - w1, wd, Vk, lda, Tk, ldt, A + j0 + (j1 + w1) * lda, lda,
-                            w.pr.nsplit));
+        if (j1 + w1 < n) TRY(update(j0, j1 + w1, n - j1 - w1));
     }
     return GBQR_OK;
 }
@@ -1009,7 +1138,6 @@ gbqr_status gbqr_factor_f32(gbqr_ctx *cx, int64_t m, int64_t n, float *A, int64_
     if (!cx) return GBQR_EINVAL;
     Params pr;
     if (!resolve(opts, m, n, &pr) || pr.nsplit != 0) return GBQR_EINVAL;
-    pr.oz = false;
     TRY(check_layout_args(m, n, lda, ldt, t_layout, pr.nb));
     if (n == 0) return GBQR_OK;
     if (!A || !T) return GBQR_EINVAL;

@@ -62,9 +62,6 @@ struct GemmOpT {
     const Real *B = nullptr; int64_t ldb = 1; int maskB = MASK_NONE;
     Real *C = nullptr; int64_t ldc = 1;
     Real alpha = Real(1), beta = Real(0);
-    const int *skip = nullptr;   // digit-split products only: device flag, non-zero = do nothing
-    const int *kexp = nullptr;   // ... and K exponents that balance op(A)'s columns against B's rows:
-                                 // op(A)(:, k) 2^-kexp[k] and 2^kexp[k] B(k, :) are split
 };
 using GemmOp = GemmOpT<double>;
 
@@ -97,18 +94,21 @@ double gemm_algorithmic_flops(const GemmOpT<Real> &op);
 // FP64 products on the BF16 tensor cores by exact digit splitting: gemm()
 // takes this path where it is estimated faster and the scratch holds it.
 // oz_gemm_scratch_bytes: enough for any product of these sizes or smaller.
-size_t oz_gemm_scratch_bytes(int64_t M, int64_t N, int64_t K);
-bool oz_gemm_wanted(const GemmOp &op, const OzScratch &sc, int num_sms);
-gbqr_status oz_gemm(const Exec &ex, const GemmOp &op, const OzScratch &sc);
+template <class Real> size_t oz_gemm_scratch_bytes(int64_t M, int64_t N, int64_t K);
+template <class Real> bool oz_gemm_wanted(const GemmOpT<Real> &op, const OzScratch &sc, int num_sms);
+template <class Real> gbqr_status oz_gemm(const Exec &ex, const GemmOpT<Real> &op, const OzScratch &sc);
 
 // Householder QR of a well-conditioned panel from its Gram matrix
-// (gram_qr.cu): V \ R over A, T (w x w).  Where the condition does not allow
-// it, *flag (device) is set, else cleared, and A and T are left alone.
-// work: gram_work_elems() doubles.  oz holds the panel's digits.
+// (gram_qr.cu): V \\ R over A, T (w x w) and, if Y is not null, Y = V T (m x w).
+// Where the condition does not allow it, *flag (device) is set, else cleared,
+// and A, T and Y are left alone.  work: gram_work_elems() doubles; oz holds
+// the panel's digits.
 constexpr int kGramMaxW = 128, kGramMinW = 16;
 size_t gram_work_elems();
-bool gram_qr_fits(const OzScratch &oz, int64_t m, int64_t w);
-gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, double *A, int64_t lda, double *T, int64_t ldt,
+template <class Real> size_t gram_scratch_bytes(int64_t m, int64_t w);
+template <class Real> bool gram_qr_fits(const OzScratch &oz, int64_t m, int64_t w);
+template <class Real>
+gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, Real *A, int64_t lda, Real *T, int64_t ldt, Real *Y, int64_t ldy,
                     double *work, int *flag, const OzScratch &oz);
 
 #define TRY_ST(x) do { gbqr_status _s = (x); if (_s != GBQR_OK) return _s; } while (0)

@@ -410,8 +410,7 @@ gbqr_status gemm(const Exec &ex, const GemmOpT<Real> &op, const GemmScratchT<Rea
     if (op.K <= 0) {
         if (op.beta == Real(1)) return GBQR_OK;
     }
-    if constexpr (std::is_same<Real, double>::value)
-        if (!ex.dmma && !ex.pred && oz_gemm_wanted(op, sc.oz, ex.num_sms)) return oz_gemm(ex, op, sc.oz);
+    if (!ex.dmma && !ex.pred && oz_gemm_wanted(op, sc.oz, ex.num_sms)) return oz_gemm(ex, op, sc.oz);
     // A small output (the T products of Algorithm 2 are 64 x 64 x 64 at the
     // panel's top node) on 64 x 64 tiles would run on a handful of SMs at one
     // SM's FP64 rate (2 FMA/clock: ~60 us for 64^3): shrink the tiles until

@@ -9,8 +9,9 @@
 //   R+^T R+ = G                   Cholesky
 //   A1 - S R+ = V1 U              LU without pivoting of the top w x w block,
 //                                 S_jj = -sgn(pivot before the subtraction)
-//   V2 = A2 U^{-1}                the rows below, one tall product
-//   T = -U R+^{-1} S V1^{-T}
+//   Z = -R+^{-1} S V1^{-T},  T = U Z
+//   V2 = A2 U^{-1}                the rows below, one tall product,
+//   Y2 = A2 Z                     and where the caller asks, Y = V T beside it
 //
 // R = S R+.  Why this is the Householder QR: with Q = I - V T V^T and Q^T A =
 // [R; 0], A - [R; 0] = -V (T V1^T R), a unit lower trapezoidal matrix times
@@ -41,10 +42,12 @@
 // on one SM would take 9 us, so row and trail spread every block over 8 CTAs;
 // a triangular solve with a unit diagonal is 32 shuffles and multiply-adds,
 // no longer than a product with the inverse.
+#include "oz.cuh"
 #include "tsqr_dev.cuh"
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 namespace gbqr {
 namespace {
@@ -54,23 +57,27 @@ constexpr int GLD = kGramMaxW;       // leading dimension of every w x w array
 constexpr int GT = 128;              // threads of the row / trail kernels: 32 x 4 outputs
 constexpr double kGramBound2 = 16.0; // largest accepted (R^-1)_ij^2 g_ii
 
+template <class Real>
 struct GramArgs {
-    double *A; int64_t lda;          // panel
-    double *Tout; int64_t ldt;
+    Real *A; int64_t lda;            // panel
+    Real *Tout; int64_t ldt;
+    Real *Y; int64_t ldy;            // V T (null: not wanted)
     int w, nblk;
-    double *G, *R, *RI, *A1, *L, *U, *LI, *X, *YX, *YR, *YL, *K, *sgn, *gd;
+    double *G, *R, *RI, *A1, *L, *U, *LI, *X, *YX, *YR, *YL, *B1, *Z, *sgn, *gd;
     double *M;                       // the block's unit triangular factors, M[t][lane]: see UnitFactor
     double *sc;                      // ... and the reciprocals of R's and U's diagonal
     int *flag, *kexp;                // kexp: exponents of the column norms
 };
 
-__device__ __forceinline__ double g_at(const GramArgs &p, int i, int j, int k) {
+template <class Real>
+__device__ __forceinline__ double g_at(const GramArgs<Real> &p, int i, int j, int k) {
     if (k > 0) return __ldcg(p.G + i + j * GLD);
     return (i < p.w && j < p.w) ? __ldcg(p.G + i + j * GLD) : (i == j ? 1.0 : 0.0);
 }
-__device__ __forceinline__ double a1_at(const GramArgs &p, int i, int j, int k) {
+template <class Real>
+__device__ __forceinline__ double a1_at(const GramArgs<Real> &p, int i, int j, int k) {
     if (k > 0) return __ldcg(p.A1 + i + j * GLD);
-    return (i < p.w && j < p.w) ? p.A[i + (int64_t)j * p.lda] : (i == j ? 1.0 : 0.0);
+    return (i < p.w && j < p.w) ? (double)p.A[i + (int64_t)j * p.lda] : (i == j ? 1.0 : 0.0);
 }
 
 // 1/d by the reciprocal approximation and one third-order Newton step
@@ -94,7 +101,8 @@ enum UnitFactor { UF_CHOL = 0, UF_L = 1, UF_U = 2 };
 // date, takes its pivot's reciprocal and publishes both, while the other
 // warps apply the current column to the ones behind; in the LU warp 1 carries
 // the next row of U the same way.  One barrier a step.
-__global__ void __launch_bounds__(kThreads) gram_diag_kernel(const GramArgs p, int k) {
+template <class Real>
+__global__ void __launch_bounds__(kThreads) gram_diag_kernel(const GramArgs<Real> p, int k) {
     __shared__ double S[GB][GB + 1], Rb[GB][GB + 1];     // [column][row]; Rb: R(row, column)
     __shared__ double cb[2][GB], ub[2][GB], rb[2], rd[GB], sg[GB];
     __shared__ int bad;
@@ -271,7 +279,8 @@ __device__ __forceinline__ void load_unit(double (*M)[GB + 1], const double *src
 // blocks of U^{-1}, R^{-1} and V1^{-1} (3 tasks); then for l < k: YX_l = U_lk
 // U_kk^{-1}, YR_l = R_lk R_kk^{-1} and YL_l = sum_j L_kj LI_jl.
 // blockIdx.x = task * 8 + column (row) group.
-__global__ void __launch_bounds__(GT) gram_row_kernel(const GramArgs p, int k) {
+template <class Real>
+__global__ void __launch_bounds__(GT) gram_row_kernel(const GramArgs<Real> p, int k) {
     __shared__ double sA[GB][GB + 1], sB[4][GB];
     if (*(volatile int *)p.flag) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -339,7 +348,8 @@ __global__ void __launch_bounds__(GT) gram_row_kernel(const GramArgs p, int k) {
 
 // Trailing blocks of G (upper) and A1, then for l < k: X_lk = -sum X_lj YX_j,
 // RI_lk = -sum RI_lj YR_j, LI_kl = -LI_kk YL_l.
-__global__ void __launch_bounds__(GT) gram_trail_kernel(const GramArgs p, int k) {
+template <class Real>
+__global__ void __launch_bounds__(GT) gram_trail_kernel(const GramArgs<Real> p, int k) {
     __shared__ double sA[GB][GB + 1], sB[4][GB];
     if (*(volatile int *)p.flag) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -379,32 +389,35 @@ __global__ void __launch_bounds__(GT) gram_trail_kernel(const GramArgs p, int k)
     if (what == 1 && !(acc * acc * __ldcg(p.gd + l * GB + lane) <= kGramBound2)) *(volatile int *)p.flag = 1;
 }
 
-// K = (U R^{-1}) S (step 0), then T = -K V1^{-T} (step 1): T = -U (S R)^{-1}
-// V1^{-T}, both products upper triangular.  A CTA takes 32 x 2 outputs of
-// block (i, j), a warp one column and the even or odd 32-wide steps; all
-// operands are staged at once.  Step 1 also writes V1 \ R over the panel's
-// top block.  blockIdx.x = task * 16 + column pair.
-__global__ void __launch_bounds__(GT) gram_t_kernel(const GramArgs p, int step) {
+// Z = X T = -R+^{-1} S V1^{-T} (step 0), then T = U Z, the top block of Y = V T
+// = (A - [R; 0]) Z and V1 \\ R over the panel's top block (step 1).  A CTA
+// takes 32 x 2 outputs of block (i, j), a warp one column and the even or odd
+// 32-wide steps; all operands are staged at once.  blockIdx.x = block * 16 +
+// column pair, blockIdx.y = 1: Y.
+template <class Real>
+__global__ void __launch_bounds__(GT) gram_t_kernel(const GramArgs<Real> p, int step) {
     __shared__ double sA[4][GB][GB + 1], sB[2][4 * GB], part[2][GB];
     if (*(volatile int *)p.flag) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, col = warp & 1, half = warp >> 1;
     const int c0 = (blockIdx.x & 15) * 2, c = c0 + col, task = blockIdx.x >> 4;
-    const int i = task % p.nblk, j = task / p.nblk;
+    const bool top = blockIdx.y == 1;
+    const int i = task % p.nblk, j = task / p.nblk, l0 = top ? 0 : i;
     const int gi = i * GB + lane, gj = j * GB + c;
     double acc = 0.0;
-    if (i <= j) {
-        const double *A = step == 0 ? p.U : p.K;
-        for (int l = i; l <= j; ++l) {
+    if (l0 <= j) {
+        const double *A = step == 0 ? p.RI : (top ? p.B1 : p.U);
+        for (int l = l0; l <= j; ++l) {
 #pragma unroll
-            for (int q = 0; q < GB / 4; ++q) sA[l - i][warp + 4 * q][lane] = __ldcg(blk(A, i, l) + lane + (warp + 4 * q) * GLD);
-            // B(l, c): R^{-1} block (l, j), or V1^{-T}(l, j) = LI(j, l)^T
-            if (half == ((l - i) & 1))
-                sB[col][(l - i) * GB + lane] = step == 0 ? __ldcg(blk(p.RI, l, j) + lane + c * GLD)
-                                                         : __ldcg(blk(p.LI, j, l) + c + lane * GLD);
+            for (int q = 0; q < GB / 4; ++q) sA[l - l0][warp + 4 * q][lane] = __ldcg(blk(A, i, l) + lane + (warp + 4 * q) * GLD);
+            // step 0: (S V1^{-T})(l, j) = S_l LI(j, l)^T; step 1: Z block (l, j)
+            if (half == ((l - l0) & 1))
+                sB[col][(l - l0) * GB + lane] =
+                    step == 0 ? __ldcg(p.sgn + l * GB + lane) * __ldcg(blk(p.LI, j, l) + c + lane * GLD)
+                              : __ldcg(blk(p.Z, l, j) + lane + c * GLD);
         }
         __syncthreads();
         double a0 = 0.0, a1 = 0.0;
-        for (int l = half; l <= j - i; l += 2)
+        for (int l = half; l <= j - l0; l += 2)
 #pragma unroll
             for (int kk = 0; kk < GB; kk += 2) {
                 a0 = rfma(sA[l][kk][lane], sB[col][l * GB + kk], a0);
@@ -419,30 +432,64 @@ __global__ void __launch_bounds__(GT) gram_t_kernel(const GramArgs p, int step) 
         return;
     }
     if (step == 0) {
-        if (i <= j) blk(p.K, i, j)[lane + c * GLD] = acc * __ldcg(p.sgn + gj);
+        blk(p.Z, i, j)[lane + c * GLD] = i <= j ? -acc : 0.0;
+        if (p.Y) {
+            const double a = a1_at(p, gi, gj, 0);
+            blk(p.B1, i, j)[lane + c * GLD] = gi <= gj ? rfma(-__ldcg(p.sgn + gi), __ldcg(p.R + gi + gj * GLD), a) : a;
+        }
         return;
     }
     if (gi >= p.w || gj >= p.w) return;
-    p.Tout[gi + (int64_t)gj * p.ldt] = gi <= gj ? -acc : 0.0;
+    if (top) {
+        p.Y[gi + (int64_t)gj * p.ldy] = (Real)acc;
+        return;
+    }
+    p.Tout[gi + (int64_t)gj * p.ldt] = gi <= gj ? (Real)acc : Real(0);
     p.A[gi + (int64_t)gj * p.lda] =
-        gi <= gj ? __ldcg(p.sgn + gi) * __ldcg(p.R + gi + gj * GLD) : __ldcg(p.L + gi + gj * GLD);
+        (Real)(gi <= gj ? __ldcg(p.sgn + gi) * __ldcg(p.R + gi + gj * GLD) : __ldcg(p.L + gi + gj * GLD));
 }
 
 }  // namespace
 
-size_t gram_work_elems() { return (size_t)12 * GLD * GLD + 3 * GB * GB + 2 * GB + 4 * GLD; }
+size_t gram_work_elems() { return (size_t)13 * GLD * GLD + 3 * GB * GB + 2 * GB + 4 * GLD; }
 
-bool gram_qr_fits(const OzScratch &oz, int64_t m, int64_t w) {
-    return w >= kGramMinW && w <= kGramMaxW && m >= 4 * w && oz.base &&
-           std::max(oz_gemm_scratch_bytes(w, w, m), oz_gemm_scratch_bytes(m - w, w, w)) <= oz.bytes;
+namespace {
+
+// Scratch of one panel: the digits of P (later of A2), of X and Z, and the
+// partials of the Gram matrix's split.
+struct GramScratch { size_t p, xz, total; };
+GramScratch gram_scratch(int D, int64_t m, int64_t w, bool with_y) {
+    GramScratch s;
+    s.p = std::max(oz_digit_bytes(D, w, m, kOzTileA), oz_digit_bytes(D, m, w, kOzTileA));
+    s.xz = oz_digit_bytes(D, w, w, kOzTileB) * (with_y ? 2 : 1);
+    const size_t splits = std::min<size_t>(oz_ktiles(m), 128);
+    s.total = s.p + std::max(s.xz, splits * w * w * 8);
+    return s;
 }
 
-gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, double *A, int64_t lda, double *T, int64_t ldt,
+}  // namespace
+
+template <class Real>
+size_t gram_scratch_bytes(int64_t m, int64_t w) { return gram_scratch(oz_digits<Real>(), m, w, true).total; }
+template size_t gram_scratch_bytes<double>(int64_t, int64_t);
+template size_t gram_scratch_bytes<float>(int64_t, int64_t);
+
+template <class Real>
+bool gram_qr_fits(const OzScratch &oz, int64_t m, int64_t w) {
+    return w >= kGramMinW && w <= kGramMaxW && m >= 4 * w && m <= (1 << 30) && oz.base &&
+           gram_scratch(oz_digits<Real>(), m, w, true).total <= oz.bytes;
+}
+template bool gram_qr_fits<double>(const OzScratch &, int64_t, int64_t);
+template bool gram_qr_fits<float>(const OzScratch &, int64_t, int64_t);
+
+template <class Real>
+gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, Real *A, int64_t lda, Real *T, int64_t ldt, Real *Y, int64_t ldy,
                     double *work, int *flag, const OzScratch &oz) {
-    GramArgs p{};
-    p.A = A; p.lda = lda; p.Tout = T; p.ldt = ldt;
+    constexpr int D = oz_digits<Real>();
+    GramArgs<Real> p{};
+    p.A = A; p.lda = lda; p.Tout = T; p.ldt = ldt; p.Y = Y; p.ldy = ldy;
     p.w = (int)w; p.nblk = (int)((w + GB - 1) / GB);
-    double **slots[] = {&p.G, &p.R, &p.RI, &p.A1, &p.L, &p.U, &p.LI, &p.X, &p.YX, &p.YR, &p.YL, &p.K};
+    double **slots[] = {&p.G, &p.R, &p.RI, &p.A1, &p.L, &p.U, &p.LI, &p.X, &p.YX, &p.YR, &p.YL, &p.B1, &p.Z};
     double *at = work;
     for (double **s : slots) { *s = at; at += (size_t)GLD * GLD; }
     p.M = at;
@@ -451,42 +498,82 @@ gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, double *A, int64_t lda
     p.gd = p.sgn + GLD;
     p.flag = flag;
     p.kexp = (int *)(p.gd + GLD);
-    GemmOp g;
-    g.M = w; g.N = w; g.K = m;
-    g.A = A; g.lda = lda; g.ta = true; g.B = A; g.ldb = lda; g.C = p.G; g.ldc = GLD;
-    TRY_ST(oz_gemm(ex, g, oz));
+    const GramScratch sc = gram_scratch(D, m, w, Y != nullptr);
+    if (sc.total > oz.bytes) return GBQR_ENOMEM;
+    char *base = (char *)oz.base;
+    // G = P^T P
+    OzOperand<Real> pc = oz_operand(D, (const Real *)A, lda, w, m, false, MASK_NONE, kOzTileA, base);
+    TRY_ST(oz_slice(ex, D, &pc, 1));
+    OzMmaArgs<Real> g{};
+    g.prob[0] = oz_problem<Real>(pc, pc);
+    g.prob[0].partial = (long long *)(base + sc.p);
+    g.prob[0].Cd = p.G;
+    g.prob[0].ldc = GLD;
+    if (!oz_choose_split(g.prob[0], ex.num_sms, sc.total - sc.p, true)) return GBQR_ENOMEM;
+    g.n = 1;
+    g.items = oz_items((int)w, (int)w, g.prob[0].S);
+    g.err = oz.err;
+    TRY_ST(oz_mma_launch(ex, g, (double)w * w * m));
+    TRY_ST(oz_reduce_launch(ex, g, (size_t)w * w));
     auto mark = [&](double flops) { return trace_end(ex, FAM_OTHER, flops, 0.0); };
     const double f3 = 2.0 * GB * GB * GB;
     for (int k = 0; k < p.nblk; ++k) {
         trace_begin(ex, FAM_OTHER);
-        gram_diag_kernel<<<1, kThreads, 0, ex.stream>>>(p, k);
-        TRY_ST(mark(3.0 * f3));
+        gram_diag_kernel<Real><<<1, kThreads, 0, ex.stream>>>(p, k);
+        TRY_ST(mark(f3));
         const int rest = p.nblk - k - 1, row = 2 * rest + 3 + 3 * k, trail = 2 * rest * rest + 3 * k;
         trace_begin(ex, FAM_OTHER);
-        gram_row_kernel<<<row * 8, GT, 0, ex.stream>>>(p, k);
+        gram_row_kernel<Real><<<row * 8, GT, 0, ex.stream>>>(p, k);
         TRY_ST(mark(row * f3));
         if (trail) {
             trace_begin(ex, FAM_OTHER);
-            gram_trail_kernel<<<trail * 8, GT, 0, ex.stream>>>(p, k);
+            gram_trail_kernel<Real><<<trail * 8, GT, 0, ex.stream>>>(p, k);
             TRY_ST(mark(trail * f3));
         }
     }
     for (int step = 0; step < 2; ++step) {
         trace_begin(ex, FAM_OTHER);
-        gram_t_kernel<<<p.nblk * p.nblk * 16, GT, 0, ex.stream>>>(p, step);
+        gram_t_kernel<Real><<<dim3(p.nblk * p.nblk * 16, step == 1 && Y ? 2 : 1), GT, 0, ex.stream>>>(p, step);
         TRY_ST(mark(p.nblk * p.nblk * f3));
     }
     if (m > w) {
-        // V2 = A2 X, in place: the digits of A2 are taken before C is written
-        GemmOp v;
-        v.M = m - w; v.N = w; v.K = w;
-        v.A = A + w; v.lda = lda; v.ta = false; v.B = p.X; v.ldb = GLD; v.maskB = MASK_UPPER;
-        v.C = A + w; v.ldc = lda;
-        v.skip = flag;
-        v.kexp = p.kexp;                 // columns of A2 may differ by any scale, so may X's rows
-        TRY_ST(oz_gemm(ex, v, oz));
+        // V2 = A2 X in place (the digits of A2 are taken before C is written)
+        // and Y2 = A2 Z; columns of A2 may differ by any scale, so may the
+        // rows of X and Z: kexp
+        OzOperand<Real> a2 = oz_operand(D, (const Real *)(A + w), lda, m - w, w, true, MASK_NONE, kOzTileA, base);
+        OzOperand<double> xz[2];
+        const size_t xb = oz_digit_bytes(D, w, w, kOzTileB);
+        xz[0] = oz_operand(D, (const double *)p.X, GLD, w, w, false, MASK_UPPER, kOzTileB, base + sc.p);
+        xz[1] = oz_operand(D, (const double *)p.Z, GLD, w, w, false, MASK_UPPER, kOzTileB, base + sc.p + xb);
+        a2.skip = xz[0].skip = xz[1].skip = flag;
+        a2.kexp = xz[0].kexp = xz[1].kexp = p.kexp;
+        a2.ksign = -1;
+        xz[0].ksign = xz[1].ksign = 1;
+        const int nb = Y ? 2 : 1;
+        if constexpr (std::is_same<Real, double>::value) {
+            OzOperand<double> ops[3] = {a2, xz[0], xz[1]};
+            TRY_ST(oz_slice(ex, D, ops, 1 + nb));
+        } else {
+            TRY_ST(oz_slice(ex, D, &a2, 1));
+            TRY_ST(oz_slice(ex, D, xz, nb));
+        }
+        OzMmaArgs<Real> v{};
+        for (int q = 0; q < nb; ++q) {
+            v.prob[q] = oz_problem<Real>(a2, xz[q]);
+            v.prob[q].C = q == 0 ? A + w : Y + w;
+            v.prob[q].ldc = q == 0 ? lda : ldy;
+            v.prob[q].first = v.items;
+            v.items += oz_items((int)(m - w), (int)w, 1);
+        }
+        v.n = nb;
+        v.err = oz.err;
+        TRY_ST(oz_mma_launch(ex, v, (double)nb * w * w * (m - w)));
     }
     return GBQR_OK;
 }
+template gbqr_status gram_qr(const Exec &, int64_t, int64_t, double *, int64_t, double *, int64_t, double *, int64_t,
+                             double *, int *, const OzScratch &);
+template gbqr_status gram_qr(const Exec &, int64_t, int64_t, float *, int64_t, float *, int64_t, float *, int64_t,
+                             double *, int *, const OzScratch &);
 
 }  // namespace gbqr

@@ -32,19 +32,28 @@
 // tensor cores' accumulation truncates, and its bias grows with K.
 //
 // Kernels of one product:
-//   oz_slice_kernel   digits of both operands, K-major (HBM: 8 B read, 14
-//                     written per entry), one launch
-//   oz_mma_kernel     TMA -> shared memory -> tcgen05.mma -> TMEM -> C, or
-//                     integer partials where K is split
-//   oz_reduce_kernel  sums the partials and rounds (only where K is split)
+//   oz_slice_kernel   digits of the operands (HBM: 8 B read, 14 written per
+//                     entry), one launch
+//   oz_mma_kernel     bulk copies -> shared memory -> tcgen05.mma -> TMEM ->
+//                     C, or integer partials where K is split
+//   oz_reduce_kernel  sums the partials and rounds (only where K is split), or
+//                     oz_requant_kernel, which writes them as the digits of
+//                     the next product's operand
+//
+// FP32 (the FP32 factorizations) is the same with four digits (31 bits), ten
+// digit products and an accumulator for each of the weights 2 to 5.
+//
+// Digits lie in memory as the shared-memory images of their tiles: 128 (the M
+// side) or 64 rows x 32 k of every digit, rows of 64 bytes with the 64-byte
+// swizzle the MMA descriptors name, so a stage is filled by one bulk copy an
+// operand and a product needs no tensor map.
 //
 // Measured (one factorization with the FMA kernel against this one): graded
 // 8192^2 687 -> 157 ms, 32768 x 2048 256 -> 65 ms; the thin Q of 16001 x 1000
 // 31.3 -> 3.3 ms.
-#include "common.cuh"
+#include "oz.cuh"
 #include "tc_ptx.cuh"
 
-#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -54,29 +63,54 @@
 namespace gbqr {
 namespace {
 
-constexpr int OZ_D = 7;              // digits per operand
-constexpr int OZ_ACC = 7;            // accumulators: weights 2 .. 7, and 8 and 9 together
 constexpr int OZ_BM = 128;
-constexpr int OZ_BN = 64;            // 7 x 64 FP32 columns: 448 of the 512 of TMEM
-constexpr int OZ_TOP = 9;            // largest i + j of the digit products taken
-constexpr int OZ_BK = 32;            // one 64-byte swizzle row of BF16
+constexpr int OZ_BN = 64;
+constexpr int OZ_BK = 32;            // one 64-byte row of BF16
+constexpr uint32_t OZ_PIECE = 4096;  // bytes per bulk copy
 constexpr int OZ_CHUNK = 8;          // K tiles per drain (256 k: the accumulators stay exact)
-constexpr int OZ_MAX_KT = 16;        // K tiles per CTA (512 k: the 64-bit sum stays exact)
-constexpr int OZ_STAGES = 2;
-constexpr int OZ_EPI_WARPS = 8;
+constexpr int OZ_EPI_WARPS = 16;
 constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;
 constexpr int OZ_COLS = OZ_BN / (OZ_EPI_WARPS / 4);   // columns per epilogue thread
-static_assert(OZ_COLS % 8 == 0, "the epilogue works in groups of 8 columns");
-constexpr uint32_t OZ_A_TILE = OZ_BM * OZ_BK * 2, OZ_B_TILE = OZ_BN * OZ_BK * 2;
-constexpr uint32_t OZ_A_STAGE = OZ_D * OZ_A_TILE, OZ_B_STAGE = OZ_D * OZ_B_TILE;
-constexpr size_t OZ_SMEM = 1024 + OZ_STAGES * (size_t)(OZ_A_STAGE + OZ_B_STAGE) + 256;
 constexpr int kExpNan = 1 << 20;     // exponent of a row with a NaN or an infinity
+constexpr uint32_t OZ_A_TILE = OZ_BM * OZ_BK * 2, OZ_B_TILE = OZ_BN * OZ_BK * 2;   // one digit
+static_assert(OZ_COLS <= 32 && OZ_COLS % 8 == 0, "a lane per column's exponent, groups of 8 columns");
+static_assert(OZ_BM == kOzTileA && OZ_BN == kOzTileB, "digit tiles");
+
+// Digits, the largest i + j of the digit products taken, accumulators (one per
+// weight from 2 on, the last shared by the rest: 7 x 64 of TMEM's 512
+// columns), the unit 2^-UNIT of the integer sums and the K tiles per CTA that
+// keep them in 64 bits.
+template <class Real> struct OzTraits;
+template <> struct OzTraits<double> {
+    static constexpr int D = 7, TOP = 9, ACC = 7, UNIT = 40, STAGES = 2, MAX_KT = 16;
+};
+template <> struct OzTraits<float> {
+    static constexpr int D = 4, TOP = 5, ACC = 4, UNIT = 24, STAGES = 4, MAX_KT = 64;
+};
+constexpr int kD64 = OzTraits<double>::D, kD32 = OzTraits<float>::D;
+template <class Real> constexpr uint32_t oz_stage_bytes() { return OzTraits<Real>::D * (OZ_A_TILE + OZ_B_TILE); }
+template <class Real> constexpr size_t oz_smem() { return 1024 + OzTraits<Real>::STAGES * (size_t)oz_stage_bytes<Real>() + 256; }
+template <class Real> constexpr int oz_products() {
+    int n = 0;
+    for (int i = 1; i <= OzTraits<Real>::D; ++i)
+        for (int j = 1; j <= OzTraits<Real>::D; ++j) n += i + j <= OzTraits<Real>::TOP;
+    return n;
+}
+static_assert(kD64 == kOzDigits64 && kD32 == kOzDigits32, "digits");
+static_assert(oz_products<double>() == 34 && oz_products<float>() == 10, "digit products");
 
 // ------------------------------------------------------------- digits
 
-// x 2^(55 - e) rounded to an integer, e = exmax - 1022 (exmax: the largest
-// biased exponent of the row, so |x| < 2^e).
-__device__ __forceinline__ long long fixed55(double x, int exmax) {
+__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ int exp_field(float x) { return (__float_as_int(x) >> 23) & 0xff; }
+template <class Real> struct ExpOf;
+template <> struct ExpOf<double> { static constexpr int INF = 0x7ff, BIAS = 1022; };
+template <> struct ExpOf<float> { static constexpr int INF = 0xff, BIAS = 126; };
+
+// x 2^(8 D - 1 - e) rounded to an integer, e = exmax - BIAS (exmax: the
+// largest biased exponent of the row, so |x| < 2^e).
+template <int D>
+__device__ __forceinline__ long long fixed_of(double x, int exmax) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int ex = (int)((b >> 52) & 0x7ff);
     unsigned long long mant = b & 0xfffffffffffffull;
@@ -86,29 +120,35 @@ __device__ __forceinline__ long long fixed55(double x, int exmax) {
     if (d <= 2) f = mant << (2 - d);
     else if (d < 58) f = (mant + (1ull << (d - 3))) >> (d - 2);
     else f = 0;
+    if (D == kD32) f = (f + (1ull << 23)) >> 24;   // 31 bits
     return (long long)b < 0 ? -(long long)f : (long long)f;
+}
+template <int D>
+__device__ __forceinline__ long long fixed_of(float x, int exmax) {
+    const uint32_t b = (uint32_t)__float_as_int(x);
+    const int ex = (int)((b >> 23) & 0xff);
+    uint32_t mant = b & 0x7fffffu;
+    if (ex) mant |= 0x800000u;
+    const int d = exmax - max(ex, 1);
+    uint32_t f;
+    if (d <= 7) f = mant << (7 - d);
+    else if (d < 33) f = (mant + (1u << (d - 8))) >> (d - 7);
+    else f = 0;
+    return (int)b < 0 ? -(long long)f : (long long)f;
 }
 
 // Digit i (0-based) of the biased fixed-point number u, with its weight.
+template <int D>
 __device__ __forceinline__ float digit_of(unsigned long long u, int i) {
-    constexpr float w[OZ_D] = {1.0f, 0x1p-8f, 0x1p-16f, 0x1p-24f, 0x1p-32f, 0x1p-40f, 0x1p-48f};
-    const uint32_t v = (uint32_t)(u >> (8 * (OZ_D - 1 - i))) & (i == 0 ? 0x1ffu : 0xffu);
+    constexpr float w[7] = {1.0f, 0x1p-8f, 0x1p-16f, 0x1p-24f, 0x1p-32f, 0x1p-40f, 0x1p-48f};
+    const uint32_t v = (uint32_t)(u >> (8 * (D - 1 - i))) & (i == 0 ? 0x1ffu : 0xffu);
     return (__uint_as_float(0x4b000000u | v) - 8388736.0f) * w[i];   // (2^23 + v) - (2^23 + 128)
 }
-constexpr unsigned long long kDigitBias = 0x80808080808080ull;
-
-struct OzOperand {
-    const double *X; int64_t ld;
-    int64_t R, K;              // operand rows and their length
-    int mask;                  // MASK_UNIT_LOWER: the strict lower part only (the diagonal is added apart)
-    int by_row;                // 0: operand row r is column r of X; 1: row r of X
-    __nv_bfloat16 *dst;        // [digit][r][ldk]
-    int64_t ldk;
-    int *exps;                 // per operand row
-    unsigned blocks;           // CTAs working on it
-    const int *skip;           // non-null: nothing to do while *skip != 0
-    const int *kexp; int ksign;   // entries of index k scaled by 2^(ksign kexp[k]) first
-};
+template <int D> constexpr unsigned long long digit_bias() {
+    unsigned long long b = 0;
+    for (int i = 0; i < D; ++i) b = (b << 8) | 0x80;
+    return b;
+}
 
 // x 2^e, exact unless it leaves the normal range.
 __device__ __forceinline__ double mul_pow2(double x, int e) {
@@ -119,48 +159,59 @@ __device__ __forceinline__ double mul_pow2(double x, int e) {
         return __hiloint2double(hi + (e << 20), __double2loint(x));
     return scalbn(x, e);
 }
+__device__ __forceinline__ float mul_pow2(float x, int e) {
+    const int b = __float_as_int(x), ex = (b >> 23) & 0xff;
+    if (ex == 0xff || x == 0.0f) return x;
+    if (ex > 0 && ex + e > 0 && ex + e < 0xff && e > -512 && e < 512) return __int_as_float(b + (e << 23));
+    return scalbnf(x, e);
+}
 
-__device__ __forceinline__ double oz_load(const OzOperand &o, int64_t r, int64_t k) {
+// Entry k of operand row r.
+template <class Real>
+__device__ __forceinline__ Real oz_load(const OzOperand<Real> &o, int64_t r, int64_t k) {
     const int64_t i = o.by_row ? r : k, j = o.by_row ? k : r;
-    if (k >= o.K || r >= o.R) return 0.0;
-    if (o.mask == MASK_UNIT_LOWER && i <= j) return 0.0;
-    if (o.mask == MASK_UPPER && i > j) return 0.0;
-    const double x = o.X[i + j * o.ld];
+    if (k >= o.K || r >= o.R) return Real(0);
+    if (o.mask == MASK_UNIT_LOWER && i <= j) return i == j && o.unit ? Real(1) : Real(0);
+    if (o.mask == MASK_UPPER && i > j) return Real(0);
+    const Real x = o.X[i + j * o.ld];
     return o.kexp ? mul_pow2(x, o.ksign * __ldcg(o.kexp + k)) : x;
 }
 
-__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-
-// n consecutive digits of every weight for the values v (n = 4 or 16).
-template <int NV>
-__device__ __forceinline__ void store_digits(const OzOperand &o, int64_t r, int64_t k0, const double (&v)[NV], int exmax) {
+// Digits of the NV = 4 or 16 consecutive entries v of operand row r from k0.
+template <int D, class Real, int NV>
+__device__ __forceinline__ void store_digits(uint8_t *dst, int KT, int rt, int64_t r, int64_t k0, const Real (&v)[NV],
+                                             int exmax) {
     unsigned long long u[NV];
 #pragma unroll
-    for (int q = 0; q < NV; ++q) u[q] = (unsigned long long)(fixed55(v[q], exmax) + (long long)kDigitBias);
-    const size_t slice = (size_t)o.R * o.ldk;
-    __nv_bfloat16 *p = o.dst + (size_t)r * o.ldk + k0;
+    for (int q = 0; q < NV; ++q) u[q] = (unsigned long long)(fixed_of<D>(v[q], exmax) + (long long)digit_bias<D>());
+    const int rr = (int)(r & (rt - 1)), swz = (rr >> 1) & 3;          // rt: rows per tile, 64 or 128
+    const uint32_t dig = (uint32_t)rt * 64;
+    uint8_t *p = dst + ((size_t)(r >> (rt == OZ_BM ? 7 : 6)) * KT + (size_t)(k0 >> 5)) * (D * dig) + rr * 64;
+    const int ch = (int)(k0 >> 3) & 3;
 #pragma unroll
-    for (int i = 0; i < OZ_D; ++i) {
+    for (int i = 0; i < D; ++i) {
         uint32_t w[NV / 2];
 #pragma unroll
         for (int q = 0; q < NV / 2; ++q) {
-            const __nv_bfloat162 h = __floats2bfloat162_rn(digit_of(u[2 * q], i), digit_of(u[2 * q + 1], i));
+            const __nv_bfloat162 h = __floats2bfloat162_rn(digit_of<D>(u[2 * q], i), digit_of<D>(u[2 * q + 1], i));
             w[q] = *reinterpret_cast<const uint32_t *>(&h);
         }
         if constexpr (NV == 4) {
-            *reinterpret_cast<uint2 *>(p + i * slice) = make_uint2(w[0], w[1]);
+            *reinterpret_cast<uint2 *>(p + i * dig + ((ch ^ swz) << 4) + (k0 & 4) * 2) = make_uint2(w[0], w[1]);
         } else {
 #pragma unroll
             for (int q = 0; q < NV / 8; ++q)
-                reinterpret_cast<uint4 *>(p + i * slice)[q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+                *reinterpret_cast<uint4 *>(p + i * dig + (((ch + q) ^ swz) << 4)) =
+                    make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
         }
     }
 }
 
 // Four consecutive entries of operand row r (a column of X) from k0 on.
-__device__ __forceinline__ void load_quad(const OzOperand &o, bool plain, int64_t r, int64_t k0, double (&v)[4]) {
+template <class Real>
+__device__ __forceinline__ void load_quad(const OzOperand<Real> &o, bool plain, int64_t r, int64_t k0, Real (&v)[4]) {
     if (plain && k0 + 4 <= o.K) {
-        const double *x = o.X + k0 + r * o.ld;
+        const Real *x = o.X + k0 + r * o.ld;
 #pragma unroll
         for (int q = 0; q < 4; ++q) v[q] = x[q];
     } else {
@@ -169,28 +220,46 @@ __device__ __forceinline__ void load_quad(const OzOperand &o, bool plain, int64_
     }
 }
 
-// Digits of both operands of a product: the first a.blocks CTAs work on A.
-// Bound by HBM (8 bytes read, 14 written per entry) and, for few rows, by
-// latency, so every entry is read once where registers hold the row between
-// the search for its maximum and the split: NT threads keep NQ quads each
-// (256 x 8: rows of 8192; 1024 x 4: 16384; what lies beyond is read again).
+template <class Real>
+__device__ __forceinline__ void store_exp(const OzOperand<Real> &o, int64_t r, int ex) {
+    o.exps[r] = ex == ExpOf<Real>::INF ? kExpNan : ex - ExpOf<Real>::BIAS;
+}
+
+// Digits of up to kOzOps operands (or of a list of them): operand i works on
+// CTAs [first[i], first[i + 1]).  Bound by HBM (8 bytes read, 14 written per
+// entry) and, for few rows, by latency, so every entry is read once where
+// registers hold the row between the search for its maximum and the split:
+// NT threads keep NQ quads each (256 x 8: rows of 8192; 1024 x 4: 16384; what
+// lies beyond is read again).
 //   by column: a warp per operand row (K <= 1024) or a CTA per row; a thread
-//              takes 4 consecutive k (8-byte stores, a warp 256 bytes).
+//              takes 4 consecutive k (8-byte stores, 64 bytes a row tile).
 //   by row:    a CTA takes 32 rows, lane = row, a warp 16 consecutive k (reads
-//              are coalesced along the rows, a store is one 32-byte sector).
-template <int NT, int NQ>
-__global__ void __launch_bounds__(NT) oz_slice_kernel(const OzOperand a, const OzOperand b) {
+//              are coalesced along the rows, stores are 16 bytes).
+template <class Real, int D, int NT, int NQ>
+__global__ void __launch_bounds__(NT) oz_slice_kernel(const __grid_constant__ OzSliceArgs<Real> args) {
     __shared__ int red[NT / 32][32];
-    constexpr int NW = NT / 32;
-    const bool isB = blockIdx.x >= a.blocks;
-    const OzOperand &o = isB ? b : a;
+    constexpr int NW = NT / 32, INF = ExpOf<Real>::INF;
+    int which = 0;
+    if (args.list) {
+        int lo = 0, hi = args.n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (__ldg(&args.list[mid].first) <= blockIdx.x) lo = mid;
+            else hi = mid - 1;
+        }
+        which = lo;
+    } else {
+        while (which + 1 < args.n && blockIdx.x >= args.op[which + 1].first) ++which;
+    }
+    const OzOperand<Real> o = args.list ? args.list[which] : args.op[which];
     if (o.skip && *(volatile const int *)o.skip) return;
-    const int64_t blk = isB ? blockIdx.x - a.blocks : blockIdx.x;
+    const int64_t blk = blockIdx.x - o.first;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t kpad = (int64_t)o.KT * OZ_BK;
     int ex = 0;
     if (o.by_row) {
         const int64_t r = blk * 32 + lane;
-        double v[16];
+        Real v[16];
         for (int64_t k0 = warp * 16; k0 < o.K; k0 += 16 * NW) {
 #pragma unroll
             for (int q = 0; q < 16; ++q) v[q] = oz_load(o, r, k0 + q);
@@ -203,15 +272,15 @@ __global__ void __launch_bounds__(NT) oz_slice_kernel(const OzOperand a, const O
         for (int w = 0; w < NW; ++w) ex = max(ex, red[w][lane]);
         ex = max(ex, 1);
         if (r >= o.R) return;
-        if (warp == 0) o.exps[r] = ex == 0x7ff ? kExpNan : ex - 1022;
+        if (warp == 0) store_exp(o, r, ex);
         const bool kept = o.K <= 16 * NW;                       // v holds this warp's only 16 k
-        for (int64_t k0 = warp * 16; k0 < o.ldk; k0 += 16 * NW) {
+        for (int64_t k0 = warp * 16; k0 < kpad; k0 += 16 * NW) {
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
-                if (ex == 0x7ff || (kept && k0 >= o.K)) v[q] = 0.0;
+                if (ex == INF || (kept && k0 >= o.K)) v[q] = Real(0);
                 else if (!kept) v[q] = oz_load(o, r, k0 + q);
             }
-            store_digits(o, r, k0, v, ex);
+            store_digits<D>(o.dst, o.KT, o.rt, r, k0, v, ex);
         }
         return;
     }
@@ -219,7 +288,7 @@ __global__ void __launch_bounds__(NT) oz_slice_kernel(const OzOperand a, const O
     const int64_t r = wide ? blk : blk * NW + warp;
     const int t = wide ? (int)threadIdx.x : lane, nt = wide ? NT : 32;
     const bool plain = o.mask == MASK_NONE && !o.kexp;
-    double v[NQ][4];
+    Real v[NQ][4];
     if (r < o.R) {
 #pragma unroll
         for (int q = 0; q < NQ; ++q) load_quad(o, plain, r, (int64_t)(t + q * nt) * 4, v[q]);
@@ -228,7 +297,7 @@ __global__ void __launch_bounds__(NT) oz_slice_kernel(const OzOperand a, const O
 #pragma unroll
             for (int i = 0; i < 4; ++i) ex = max(ex, exp_field(v[q][i]));
         for (int64_t k0 = (int64_t)(t + NQ * nt) * 4; k0 < o.K; k0 += nt * 4) {
-            double x[4];
+            Real x[4];
             load_quad(o, plain, r, k0, x);
 #pragma unroll
             for (int i = 0; i < 4; ++i) ex = max(ex, exp_field(x[i]));
@@ -243,63 +312,52 @@ __global__ void __launch_bounds__(NT) oz_slice_kernel(const OzOperand a, const O
     }
     if (r >= o.R) return;
     ex = max(ex, 1);
-    if (t == 0) o.exps[r] = ex == 0x7ff ? kExpNan : ex - 1022;
-    if (ex == 0x7ff) {
+    if (t == 0) store_exp(o, r, ex);
+    if (ex == INF) {
 #pragma unroll
         for (int q = 0; q < NQ; ++q)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v[q][i] = 0.0;
+            for (int i = 0; i < 4; ++i) v[q][i] = Real(0);
     }
 #pragma unroll
     for (int q = 0; q < NQ; ++q)
-        if ((int64_t)(t + q * nt) * 4 < o.ldk) store_digits(o, r, (int64_t)(t + q * nt) * 4, v[q], ex);
-    for (int64_t k0 = (int64_t)(t + NQ * nt) * 4; k0 < o.ldk; k0 += nt * 4) {
-        double x[4];
+        if ((int64_t)(t + q * nt) * 4 < kpad) store_digits<D>(o.dst, o.KT, o.rt, r, (int64_t)(t + q * nt) * 4, v[q], ex);
+    for (int64_t k0 = (int64_t)(t + NQ * nt) * 4; k0 < kpad; k0 += nt * 4) {
+        Real x[4];
         load_quad(o, plain, r, k0, x);
-        if (ex == 0x7ff)
+        if (ex == INF)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) x[i] = 0.0;
-        store_digits(o, r, k0, x, ex);
+            for (int i = 0; i < 4; ++i) x[i] = Real(0);
+        store_digits<D>(o.dst, o.KT, o.rt, r, k0, x, ex);
     }
 }
 
 // ------------------------------------------------------------ conversion
 
-// X 2^e rounded to FP64 with integer instructions (an FP64 instruction takes
-// a warp 64 cycles here, and a conversion by FP64 adds needs two).
-__device__ __forceinline__ double fixed_to_double(long long X, int e) {
-    if (X == 0) return 0.0;
-    unsigned long long m = (unsigned long long)(X < 0 ? -X : X);
-    const int lz = __clzll((long long)m);
-    m <<= lz;
-    unsigned long long r = (m >> 11) + ((m >> 10) & 1);       // 53 bits, round half up
-    const int ex = 1022 + 63 - lz + e;                         // + 1 from the leading bit of r
-    if (ex <= 0 || ex >= 0x7fe) {
-        const double d = scalbn((double)r, 11 - lz + e);
-        return X < 0 ? -d : d;
-    }
-    r += (unsigned long long)(uint32_t)ex << 52;
-    if (X < 0) r |= 0x8000000000000000ull;
-    return __longlong_as_double((long long)r);
+// X 2^e, X rounded to Real once.  e comes from exponents of operand rows: in
+// the everyday range the scaling is an integer addition (an FP64 instruction
+// takes a warp 64 cycles here); beyond it, and for rows with a NaN or an
+// infinity (exponent kExpNan), scalbn.
+__device__ __noinline__ double scaled_far(double d, int e) {
+    return e > kExpNan / 2 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(d, e);
+}
+__device__ __forceinline__ double scaled(long long X, int e, double) {
+    const double d = __ll2double_rn(X);
+    if ((unsigned)(e + 900) > 1800u) return scaled_far(d, e);
+    return __hiloint2double(__double2hiint(d) + (X == 0 ? 0 : e << 20), __double2loint(d));
+}
+__device__ __forceinline__ float scaled(long long X, int e, float) {
+    const float f = __ll2float_rn(X);
+    if ((unsigned)(e + 60) > 120u) return (float)scaled_far(__ll2double_rn(X), e);
+    return __int_as_float(__float_as_int(f) + (X == 0 ? 0 : e << 23));
 }
 
-__device__ __forceinline__ double nan_value() { return __longlong_as_double(0x7ff8000000000000ll); }
+template <class Real> __device__ __forceinline__ Real nan_value();
+template <> __device__ __forceinline__ double nan_value<double>() { return __longlong_as_double(0x7ff8000000000000ll); }
+template <> __device__ __forceinline__ float nan_value<float>() { return __int_as_float(0x7fc00000); }
 
-struct OzParams {
-    int M, N, K;
-    int ktiles, kt_per;        // K tiles in all and per CTA
-    int clipA;                 // op(A) strict lower: 1 K x M stored (k > i), 2 M x K stored (k < i); 0 dense
-    const int *ea, *eb;
-    long long *partial;        // K split: [z][M x N] column-major
-    double *C; int64_t ldc;
-    double alpha, beta;
-    const double *add; int64_t ldadd; int add_rows;   // unit diagonal of op(A): + alpha * B(i, j), i < add_rows
-    const int *skip;           // non-null: nothing to do while *skip != 0
-    int *err;
-};
-
-// Shared-memory descriptor of a K-major BF16 tile written by TMA with 64-byte
-// swizzle: rows of 64 bytes, 8-row atoms 512 bytes apart.
+// Shared-memory descriptor of a K-major BF16 tile with 64-byte swizzle: rows
+// of 64 bytes, 8-row atoms 512 bytes apart.
 __device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
     uint64_t d = 0;
     d |= (uint64_t)((saddr >> 4) & 0x3FFF);
@@ -320,32 +378,97 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&r)[8]) {
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// One CTA per 128 x 64 tile and K range, 10 warps: TMA producer (a box brings
-// all 7 digits of a 32-k step: 56 KB of A, 28 KB of B, two stages), MMA issuer
-// (34 products x 2 instructions per stage), 8 epilogue warps (warp w reads
-// TMEM lanes 32 (w % 4) .. + 31 and half of the columns).  Waits are bounded
-// as in the mixed-precision kernel.
-__global__ void __launch_bounds__(OZ_THREADS, 1)
-    oz_mma_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const OzParams p) {
-    extern __shared__ uint8_t smem_raw[];
-    if (p.skip && *(volatile const int *)p.skip) return;
-    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *sA = smem, *sB = sA + OZ_STAGES * OZ_A_STAGE;
-    uint64_t *bars = (uint64_t *)(sB + OZ_STAGES * OZ_B_STAGE);
-    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * OZ_STAGES + 2);
-    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + OZ_STAGES);
-    const uint32_t acc_full = smem_u32(bars + 2 * OZ_STAGES), acc_empty = smem_u32(bars + 2 * OZ_STAGES + 1);
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t mbar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(mbar)
+                 : "memory");
+}
 
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+    long long d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
+
+// The accumulators of one output as an integer in units of 2^-UNIT: weight i
+// (0-based) counts 2^-8i; FP64's last two share a[6], rounded to 2^-40.
+template <int ACC>
+__device__ __forceinline__ long long collect(const float (&a)[ACC]) {
+    // the two leading ones fit 32 bits together: K = 256 gives 2^22 and 2^23
+    const int top = __float2int_rn(a[0]) * 256 + __float2int_rn(a[1] * 0x1p8f);
+    const int r2 = __float2int_rn(a[2] * 0x1p16f), r3 = __float2int_rn(a[3] * 0x1p24f);
+    if constexpr (ACC == 7) {
+        long long x = (long long)((unsigned long long)(uint32_t)top << 32);
+        x = mad_wide(r2, 1 << 24, x);
+        x = mad_wide(r3, 1 << 16, x);
+        x = mad_wide(__float2int_rn(a[4] * 0x1p32f), 1 << 8, x);
+        return x + (long long)(__float2int_rn(a[5] * 0x1p40f) + __float2int_rn(a[6] * 0x1p40f));
+    } else {
+        return mad_wide(top, 1 << 16, mad_wide(r2, 1 << 8, (long long)r3));
+    }
+}
+
+// One work item: a 128 x 64 tile of a problem's output and a K range.
+struct OzItem { int prob, m0, n0, z, kt0, kt1; };
+
+template <class Real>
+__device__ __forceinline__ OzItem oz_item(const OzMmaArgs<Real> &args, int item, OzProblem<Real> &p) {
+    OzItem t;
+    int which = 0;
+    if (args.list) {
+        int lo = 0, hi = args.n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (__ldg(&args.list[mid].first) <= item) lo = mid;
+            else hi = mid - 1;
+        }
+        which = lo;
+        p = args.list[which];
+    } else {
+        while (which + 1 < args.n && item >= args.prob[which + 1].first) ++which;
+        p = args.prob[which];
+    }
+    t.prob = which;
+    int e = item - p.first;
+    const int tm = (p.M + OZ_BM - 1) / OZ_BM, tn = (p.N + OZ_BN - 1) / OZ_BN;
+    t.m0 = (e % tm) * OZ_BM;
+    e /= tm;
+    t.n0 = (e % tn) * OZ_BN;
+    t.z = e / tn;
+    t.kt0 = t.z * p.kt_per;
+    t.kt1 = min(p.KT, t.kt0 + p.kt_per);
+    if (p.clip == 1) t.kt0 = max(t.kt0, t.m0 / OZ_BK);
+    else if (p.clip == 2) t.kt1 = min(t.kt1, (t.m0 + OZ_BM + OZ_BK - 1) / OZ_BK);
+    if (p.clipB == 2) t.kt1 = min(t.kt1, (t.n0 + OZ_BN + OZ_BK - 1) / OZ_BK);
+    if (p.skip && *(volatile const int *)p.skip) t.kt1 = -1;        // nothing at all
+    return t;
+}
+
+// 10 warps per CTA: bulk-copy producer (per 32-k step all digits of a tile of
+// A, 56 KB in FP64, and of one of B, 28 KB), MMA issuer (two instructions
+// per digit product and stage), 16 epilogue warps (warp w reads TMEM lanes 32
+// (w % 4) .. + 31 and a quarter of the columns; with 8 warps the epilogue, a
+// chain of dependent integer instructions an output, took 48000 cycles an
+// item where the MMAs take 13000).  A CTA takes items blockIdx.x,
+// + gridDim.x, ...: once an item's accumulators are in the epilogue's
+// registers, the MMAs of the next one run while C is updated.  Waits are
+// bounded as in the mixed-precision kernel.
+template <class Real>
+__global__ void __launch_bounds__(OZ_THREADS, 1) oz_mma_kernel(const __grid_constant__ OzMmaArgs<Real> args) {
+    using Tr = OzTraits<Real>;
+    constexpr int D = Tr::D, STAGES = Tr::STAGES;
+    constexpr uint32_t A_STAGE = D * OZ_A_TILE, B_STAGE = D * OZ_B_TILE;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t *sA = smem, *sB = sA + STAGES * A_STAGE;
+    uint64_t *bars = (uint64_t *)(sB + STAGES * B_STAGE);
+    uint32_t *tmem_slot = (uint32_t *)(bars + 2 * STAGES + 2);
+    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES);
+    const uint32_t acc_full = smem_u32(bars + 2 * STAGES), acc_empty = smem_u32(bars + 2 * STAGES + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * OZ_BM, n0 = blockIdx.y * OZ_BN, z = blockIdx.z;
-    int kt0 = z * p.kt_per, kt1 = min(p.ktiles, kt0 + p.kt_per);
-    if (p.clipA == 1) kt0 = max(kt0, m0 / OZ_BK);
-    else if (p.clipA == 2) kt1 = min(kt1, (m0 + OZ_BM + OZ_BK - 1) / OZ_BK);
-    const int total = max(0, kt1 - kt0);
-    const int nchunk = (total + OZ_CHUNK - 1) / OZ_CHUNK;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < OZ_STAGES; ++s) {
+        for (int s = 0; s < STAGES; ++s) {
             mbar_init(full0 + 8 * s, 1);
             mbar_init(empty0 + 8 * s, 1);
         }
@@ -354,9 +477,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    constexpr uint32_t TCOLS = Tr::ACC * OZ_BN <= 256 ? 256 : 512;
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(512u));
+                     "r"(TCOLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     tc_fence_before();
@@ -366,214 +490,278 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 
     if (warp == 0) {
         if (lane == 0) {
-            int issued = 0;
-            for (int it = 0; it < total; ++it) {
-                const int s = it % OZ_STAGES, r = it / OZ_STAGES;
-                if (!mbar_wait(empty0 + 8 * s, (uint32_t)((r & 1) ^ 1), p.err)) break;
-                mbar_expect_tx(full0 + 8 * s, OZ_A_STAGE + OZ_B_STAGE);
-                tma_load_3d(smem_u32(sA + s * OZ_A_STAGE), &tmA, (kt0 + it) * OZ_BK, m0, 0, full0 + 8 * s);
-                tma_load_3d(smem_u32(sB + s * OZ_B_STAGE), &tmB, (kt0 + it) * OZ_BK, n0, 0, full0 + 8 * s);
-                issued = it + 1;
+            int it = 0;
+            bool ok = true;
+            for (int item = blockIdx.x; item < args.items && ok; item += gridDim.x) {
+                OzProblem<Real> p;
+                const OzItem t = oz_item(args, item, p);
+                // A in tiles of 128 rows; B in tiles of 64, or (X^T X) half a tile of 128
+                const uint8_t *a = p.a + (size_t)(t.m0 / OZ_BM) * p.KT * A_STAGE;
+                const uint8_t *b = p.b128 ? p.b + (size_t)(t.n0 / OZ_BM) * p.KT * A_STAGE + (t.n0 & OZ_BN ? OZ_B_TILE : 0)
+                                          : p.b + (size_t)(t.n0 / OZ_BN) * p.KT * B_STAGE;
+                for (int kt = t.kt0; kt < t.kt1; ++kt, ++it) {
+                    const int s = it % STAGES, r = it / STAGES;
+                    ok = mbar_wait(empty0 + 8 * s, (uint32_t)((r & 1) ^ 1), args.err);
+                    if (!ok) break;
+                    const uint32_t fb = full0 + 8 * s, db = smem_u32(sB + s * B_STAGE);
+                    mbar_expect_tx(fb, A_STAGE + B_STAGE);
+#pragma unroll
+                    for (uint32_t o = 0; o < A_STAGE; o += OZ_PIECE)
+                        bulk_load(smem_u32(sA + s * A_STAGE) + o, a + (size_t)kt * A_STAGE + o, OZ_PIECE, fb);
+                    if (p.b128) {
+#pragma unroll
+                        for (int i = 0; i < D; ++i)
+                            bulk_load(db + i * OZ_B_TILE, b + (size_t)kt * A_STAGE + i * OZ_A_TILE, OZ_B_TILE, fb);
+                    } else {
+#pragma unroll
+                        for (uint32_t o = 0; o < B_STAGE; o += OZ_PIECE)
+                            bulk_load(db + o, b + (size_t)kt * B_STAGE + o, OZ_PIECE, fb);
+                    }
+                }
             }
             // after an abort, let the loads already issued land before the CTA exits
-            if (issued < total)
-                for (int it = max(0, issued - OZ_STAGES); it < issued; ++it)
-                    mbar_wait(full0 + 8 * (it % OZ_STAGES), (uint32_t)((it / OZ_STAGES) & 1), p.err);
+            if (!ok)
+                for (int q = max(0, it - STAGES); q < it; ++q)
+                    mbar_wait(full0 + 8 * (q % STAGES), (uint32_t)((q / STAGES) & 1), args.err);
         }
     } else if (warp == 1) {
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_bf16(OZ_BM, OZ_BN);
             bool ok = true;
-            for (int c = 0, it = 0; c < nchunk && ok; ++c) {
-                if (c > 0) {
-                    ok = mbar_wait(acc_empty, (uint32_t)((c - 1) & 1), p.err);
-                    if (!ok) break;
-                    tc_fence_after();
-                }
-                const int end = min(total, it + OZ_CHUNK);
-                for (bool first = true; it < end; ++it, first = false) {
-                    const int s = it % OZ_STAGES, r = it / OZ_STAGES;
-                    ok = mbar_wait(full0 + 8 * s, (uint32_t)(r & 1), p.err);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint64_t ad = sw64_desc(smem_u32(sA + s * OZ_A_STAGE));
-                    const uint64_t bd = sw64_desc(smem_u32(sB + s * OZ_B_STAGE));
-                    // lowest weight first: i + j = 8 down to 2 (1-based digits)
-#pragma unroll
-                    for (int w = OZ_TOP - 2; w >= 0; --w) {
-                        const uint32_t acc = tmem + (uint32_t)((w < OZ_ACC - 1 ? w : OZ_ACC - 1) * OZ_BN);
-                        const int i0 = w < OZ_D ? 0 : w - OZ_D + 1;
-#pragma unroll
-                        for (int i = i0; i <= w - i0; ++i) {
-                            const int j = w - i;
-                            const bool fresh = first && i == i0 && (w < OZ_ACC - 1 || w == OZ_TOP - 2);
-#pragma unroll
-                            for (int kk = 0; kk < OZ_BK / 16; ++kk)
-                                mma_bf16(acc, ad + (uint64_t)(i * (OZ_A_TILE >> 4) + 2 * kk),
-                                         bd + (uint64_t)(j * (OZ_B_TILE >> 4) + 2 * kk), idesc,
-                                         (fresh && kk == 0) ? 0u : 1u);
-                        }
+            int it = 0, ch = 0;
+            for (int item = blockIdx.x; item < args.items && ok; item += gridDim.x) {
+                OzProblem<Real> p;
+                const OzItem t = oz_item(args, item, p);
+                for (int kt = t.kt0; kt < t.kt1 && ok; ++ch) {
+                    if (ch > 0) {
+                        ok = mbar_wait(acc_empty, (uint32_t)((ch - 1) & 1), args.err);
+                        if (!ok) break;
+                        tc_fence_after();
                     }
-                    mma_commit(empty0 + 8 * s);
+                    const int end = min(t.kt1, kt + OZ_CHUNK);
+                    for (bool first = true; kt < end; ++kt, ++it, first = false) {
+                        const int s = it % STAGES, r = it / STAGES;
+                        ok = mbar_wait(full0 + 8 * s, (uint32_t)(r & 1), args.err);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint64_t ad = sw64_desc(smem_u32(sA + s * A_STAGE));
+                        const uint64_t bd = sw64_desc(smem_u32(sB + s * B_STAGE));
+                        // lowest weight first: i + j = TOP down to 2 (1-based digits)
+#pragma unroll
+                        for (int w = Tr::TOP - 2; w >= 0; --w) {
+                            const uint32_t acc = tmem + (uint32_t)((w < Tr::ACC - 1 ? w : Tr::ACC - 1) * OZ_BN);
+                            const int i0 = w < D ? 0 : w - D + 1;
+#pragma unroll
+                            for (int i = i0; i <= w - i0; ++i) {
+                                const int j = w - i;
+                                const bool fresh = first && i == i0 && (w < Tr::ACC - 1 || w == Tr::TOP - 2);
+#pragma unroll
+                                for (int kk = 0; kk < OZ_BK / 16; ++kk)
+                                    mma_bf16(acc, ad + (uint64_t)(i * (OZ_A_TILE >> 4) + 2 * kk),
+                                             bd + (uint64_t)(j * (OZ_B_TILE >> 4) + 2 * kk), idesc,
+                                             (fresh && kk == 0) ? 0u : 1u);
+                            }
+                        }
+                        mma_commit(empty0 + 8 * s);
+                    }
+                    mma_commit(acc_full);
                 }
-                mma_commit(acc_full);
             }
         }
     } else {
-        const int q = warp & 3, half = (warp - 2) >> 2;
-        const int row = q * 32 + lane, m = m0 + row;
-        const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * OZ_COLS);
-        long long X[OZ_COLS];
-#pragma unroll
-        for (int c = 0; c < OZ_COLS; ++c) X[c] = 0;
+        const int q = warp & 3, part = (warp - 2) >> 2;     // lane quadrant, column quarter
+        const int row = q * 32 + lane;
+        const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(part * OZ_COLS);
         bool ok = true;
-        for (int ch = 0; ch < nchunk; ++ch) {
-            ok = mbar_wait(acc_full, (uint32_t)(ch & 1), p.err);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            tc_fence_after();
-#pragma unroll
-            for (int g = 0; g < OZ_COLS / 8; ++g) {
-                float a[OZ_ACC][8];
-#pragma unroll
-                for (int s = 0; s < OZ_ACC; ++s) tmem_ld8(tbase + (uint32_t)(s * OZ_BN + g * 8), a[s]);
-                tmem_wait_ld();
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    // the weights 2 .. 7 in units of their own; the last rounded to the unit 2^-40
-                    const long long hi = ((long long)__float2int_rn(a[0][c]) << 24) +
-                                         ((long long)__float2int_rn(a[1][c] * 0x1p8f) << 16) +
-                                         ((long long)__float2int_rn(a[2][c] * 0x1p16f) << 8) +
-                                         (long long)__float2int_rn(a[3][c] * 0x1p24f);
-                    const int lo = __float2int_rn(a[5][c] * 0x1p40f) + __float2int_rn(a[6][c] * 0x1p40f);
-                    X[g * 8 + c] += (hi << 16) + ((long long)__float2int_rn(a[4][c] * 0x1p32f) << 8) + (long long)lo;
-                }
+        int ch = 0;
+        for (int item = blockIdx.x; item < args.items && ok; item += gridDim.x) {
+            OzProblem<Real> p;
+            const OzItem t = oz_item(args, item, p);
+            if (t.kt1 < 0) continue;
+            // exponents (column nb + lane's in this lane) and C on its way to
+            // L2 while the MMAs run
+            const int nb = t.n0 + part * OZ_COLS, m = t.m0 + row;
+            const int ea = m < p.M ? __ldcg(p.ea + m) : 0, eb = nb + lane < p.N ? __ldcg(p.eb + nb + lane) : 0;
+            if (!p.partial && p.beta != Real(0) && nb + lane < p.N) {
+                const Real *c = p.C + (int64_t)(nb + lane) * p.ldc + t.m0 + q * 32;
+                const int rows = min(32, p.M - (t.m0 + q * 32));
+                for (int r = 0; r < rows; r += 128 / (int)sizeof(Real)) asm volatile("prefetch.global.L2 [%0];" ::"l"(c + r));
+                if (rows > 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(c + rows - 1));
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty) : "memory");
-        }
-        const int nb = n0 + half * OZ_COLS;
-        if (ok && m < p.M) {
-            if (p.partial) {
-                long long *pp = p.partial + (size_t)z * p.M * p.N + m;
+            long long X[OZ_COLS];
 #pragma unroll
-                for (int c = 0; c < OZ_COLS; ++c)
-                    if (nb + c < p.N) pp[(size_t)(nb + c) * p.M] = X[c];
-            } else {
-                const int ea = p.ea[m];
-                const bool sub = p.beta == 1.0 && p.alpha == -1.0;
-                double *cp = p.C + m + (int64_t)nb * p.ldc;
-                const double *ap = (m < p.add_rows) ? p.add + m + (int64_t)nb * p.ldadd : nullptr;
+            for (int c = 0; c < OZ_COLS; ++c) X[c] = 0;
+            for (int kt = t.kt0; kt < t.kt1; kt += OZ_CHUNK, ++ch) {
+                ok = mbar_wait_warp(acc_full, (uint32_t)(ch & 1), args.err);
+                if (!ok) break;
+                tc_fence_after();
 #pragma unroll
                 for (int g = 0; g < OZ_COLS / 8; ++g) {
-                    double cv[8];
+                    float a[Tr::ACC][8];
 #pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        cv[c] = (p.beta != 0.0 && nb + g * 8 + c < p.N) ? cp[(int64_t)(g * 8 + c) * p.ldc] : 0.0;
+                    for (int s = 0; s < Tr::ACC; ++s) tmem_ld8(tbase + (uint32_t)(s * OZ_BN + g * 8), a[s]);
+                    tmem_wait_ld();
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
-                        const int n = nb + g * 8 + c;
-                        if (n < p.N) {
-                            const int eb = p.eb[n];
-                            double d = (ea == kExpNan || eb == kExpNan) ? nan_value()
-                                                                        : fixed_to_double(X[g * 8 + c], ea + eb - 54);
-                            if (ap) {
-                                const double u = ap[(int64_t)(g * 8 + c) * p.ldadd];
-                                if (sub) cv[c] -= u;
-                                else d += u;
-                            }
-                            double out;
-                            if (sub) out = cv[c] - d;
-                            else if (p.beta == 0.0) out = p.alpha == 1.0 ? d : p.alpha * d;
-                            else out = fma(p.beta, cv[c], p.alpha * d);
-                            cp[(int64_t)(g * 8 + c) * p.ldc] = out;
+                        float f[Tr::ACC];
+#pragma unroll
+                        for (int i = 0; i < Tr::ACC; ++i) f[i] = a[i][c];
+                        X[g * 8 + c] += collect<Tr::ACC>(f);
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty) : "memory");
+            }
+            // (every lane takes the same branch: the loops below shuffle)
+            if (ok && p.partial) {
+                if (m < p.M) {
+                    long long *pp = p.partial + (size_t)t.z * p.M * p.N + m;
+#pragma unroll
+                    for (int c = 0; c < OZ_COLS; ++c)
+                        if (nb + c < p.N) pp[(size_t)(nb + c) * p.M] = X[c];
+                }
+            } else if (ok) {
+                const bool sub = p.beta == Real(1) && p.alpha == Real(-1) && t.m0 >= p.add_rows;
+                if (sub && t.m0 + OZ_BM <= p.M && nb + OZ_COLS <= p.N) {
+                    // a whole tile of C -= V W
+                    Real *cp = p.C + m + (int64_t)nb * p.ldc;
+#pragma unroll
+                    for (int g = 0; g < OZ_COLS; g += 8) {
+                        Real cv[8], *cg = cp;
+#pragma unroll
+                        for (int c = 0; c < 8; ++c, cg += p.ldc) cv[c] = __ldcg(cg);
+#pragma unroll
+                        for (int c = 0; c < 8; ++c, cp += p.ldc)
+                            *cp = cv[c] - scaled(X[g + c], ea + __shfl_sync(0xffffffffu, eb, g + c) - 14 - Tr::UNIT, Real(0));
+                    }
+                } else {
+                    Real *cp = p.C + m + (int64_t)nb * p.ldc;
+                    const Real *ap = m < min(p.add_rows, p.M) ? p.add + m + (int64_t)nb * p.ldadd : nullptr;
+#pragma unroll
+                    for (int c = 0; c < OZ_COLS; ++c) {
+                        Real d = scaled(X[c], ea + __shfl_sync(0xffffffffu, eb, c) - 14 - Tr::UNIT, Real(0));
+                        if (nb + c < p.N && m < p.M) {
+                            const Real old = p.beta != Real(0) ? __ldcg(cp + (int64_t)c * p.ldc) : Real(0);
+                            const Real u = ap ? __ldcg(ap + (int64_t)c * p.ldadd) : Real(0);
+                            Real out;
+                            if (p.beta == Real(1) && p.alpha == Real(-1)) out = (old - u) - d;
+                            else if (p.beta == Real(0)) out = p.alpha == Real(1) ? d + u : p.alpha * (d + u);
+                            else out = p.beta * old + p.alpha * (d + u);
+                            cp[(int64_t)c * p.ldc] = out;
                         }
                     }
                 }
             }
+            __syncwarp();
         }
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS));
     }
 }
 
-// C = beta C + alpha (2^(ea + eb - 54) sum_z P[z] + unit-diagonal term): the
-// sum is exact (high and low halves in 64 bits each), one rounding.
-__global__ void __launch_bounds__(kThreads) oz_reduce_kernel(const OzParams p, int S) {
+// sum_z P[z][e]: exact, high and low halves in 64 bits each, then FP64.
+__device__ __forceinline__ double sum_partials(const long long *P, size_t stride, int S) {
+    long long H = 0;
+    unsigned long long L = 0;
+#pragma unroll 8
+    for (int z = 0; z < S; ++z) {
+        const long long v = __ldcg(P + (size_t)z * stride);
+        H += v >> 32;
+        L += (unsigned long long)v & 0xffffffffull;
+    }
+    return fma((double)H, 4294967296.0, (double)L);
+}
+
+template <class Real>
+__device__ __forceinline__ const OzProblem<Real> &nth_problem(const OzMmaArgs<Real> &args, int which) {
+    return args.list ? args.list[which] : args.prob[which];
+}
+
+// C = beta C + alpha 2^(ea + eb - 14 - UNIT) sum_z P[z], one rounding to FP64
+// (FP32: and one to FP32).  blockIdx.y: the problem.
+template <class Real>
+__global__ void __launch_bounds__(kThreads) oz_reduce_kernel(const __grid_constant__ OzMmaArgs<Real> args) {
+    const OzProblem<Real> p = nth_problem(args, blockIdx.y);
     if (p.skip && *(volatile const int *)p.skip) return;
     const size_t total = (size_t)p.M * p.N;
     for (size_t e = blockIdx.x * (size_t)kThreads + threadIdx.x; e < total; e += (size_t)gridDim.x * kThreads) {
         const int i = (int)(e % (unsigned)p.M), j = (int)(e / (unsigned)p.M);
-        long long H = 0;
-        unsigned long long L = 0;
-        const long long *P = p.partial + e;
-#pragma unroll 8
-        for (int z = 0; z < S; ++z) {
-            const long long v = P[(size_t)z * total];
-            H += v >> 32;
-            L += (unsigned long long)v & 0xffffffffull;
+        const double s = sum_partials(p.partial + e, total, p.S);
+        const int ea = __ldcg(p.ea + i), eb = __ldcg(p.eb + j);
+        double d = (ea == kExpNan || eb == kExpNan) ? nan_value<double>()
+                                                    : mul_pow2(s, ea + eb - 14 - OzTraits<Real>::UNIT);
+        if (i < p.add_rows) d += (double)p.add[i + (int64_t)j * p.ldadd];
+        if (p.Cd) {                                        // FP64 result of an FP32 product
+            p.Cd[i + (int64_t)j * p.ldc] = d;
+            continue;
         }
-        const int ea = p.ea[i], eb = p.eb[j];
-        double d = (ea == kExpNan || eb == kExpNan)
-                       ? nan_value()
-                       : mul_pow2(fma((double)H, 4294967296.0, (double)L), ea + eb - 54);
-        double *cp = p.C + i + (int64_t)j * p.ldc;
-        if (i < p.add_rows) d += p.add[i + (int64_t)j * p.ldadd];
-        double out;
-        if (p.beta == 0.0) out = p.alpha == 1.0 ? d : p.alpha * d;
-        else if (p.beta == 1.0 && p.alpha == -1.0) out = *cp - d;
-        else out = fma(p.beta, *cp, p.alpha * d);
+        Real *cp = p.C + i + (int64_t)j * p.ldc;
+        Real out;
+        if (p.beta == Real(0)) out = p.alpha == Real(1) ? (Real)d : p.alpha * (Real)d;
+        else if (p.beta == Real(1) && p.alpha == Real(-1)) out = *cp - (Real)d;
+        else out = p.beta * *cp + p.alpha * (Real)d;
         *cp = out;
     }
 }
 
-bool oz_map(CUtensorMap *map, const void *base, int64_t rows, int64_t ldk, int box_rows) {
-    auto enc = (PFN_cuTensorMapEncodeTiled_v12000)tensor_map_encoder();
-    if (!enc) return false;
-    cuuint64_t dims[3] = {(cuuint64_t)ldk, (cuuint64_t)rows, (cuuint64_t)OZ_D};
-    cuuint64_t strides[2] = {(cuuint64_t)ldk * 2, (cuuint64_t)ldk * (cuuint64_t)rows * 2};
-    cuuint32_t box[3] = {(cuuint32_t)OZ_BK, (cuuint32_t)box_rows, (cuuint32_t)OZ_D};
-    cuuint32_t estr[3] = {1, 1, 1};
-    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+// The M x N sums (M <= 128) as the digits of the next product's B operand:
+// column j becomes operand row j with M entries, and (for the unit diagonal
+// of a V basis, which no digits carry) the rounded sums.  A warp per column, 4
+// consecutive rows per lane.
+template <class Real>
+__global__ void __launch_bounds__(kThreads) oz_requant_kernel(const __grid_constant__ OzMmaArgs<Real> args) {
+    const OzProblem<Real> p = nth_problem(args, blockIdx.y);
+    const int lane = threadIdx.x & 31, KT = (p.M + OZ_BK - 1) / OZ_BK;
+    const size_t total = (size_t)p.M * p.N;
+    for (int j = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); j < p.N; j += gridDim.x * (kThreads / 32)) {
+        const int eb = __ldcg(p.eb + j);
+        Real v[4];
+        int ex = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = lane * 4 + q;
+            v[q] = Real(0);
+            if (i < p.M) {
+                const double s = sum_partials(p.partial + i + (size_t)j * p.M, total, p.S);
+                const int ea = __ldcg(p.ea + i);
+                v[q] = (ea == kExpNan || eb == kExpNan) ? nan_value<Real>()
+                                                        : (Real)mul_pow2(s, ea + eb - 14 - OzTraits<Real>::UNIT);
+            }
+            ex = max(ex, exp_field(v[q]));
+            if (p.C && i < p.M) p.C[i + (int64_t)j * p.ldc] = v[q];
+        }
+        ex = max(__reduce_max_sync(0xffffffffu, ex), 1);
+        if (lane == 0) p.qexp[j] = ex == ExpOf<Real>::INF ? kExpNan : ex - ExpOf<Real>::BIAS;
+        if (ex == ExpOf<Real>::INF)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = Real(0);
+        if (lane * 4 < KT * OZ_BK) store_digits<OzTraits<Real>::D>(p.qdst, KT, OZ_BN, j, lane * 4, v, ex);
+    }
 }
 
 size_t a256(size_t x) { return (x + 255) / 256 * 256; }
-int64_t pad_k(int64_t K) { return (K + 15) / 16 * 16; }
 
-// Scratch layout of one product.
-struct OzLayout { int64_t ldk; size_t a, b, ea, eb, part, total; };
-OzLayout oz_layout(int64_t M, int64_t N, int64_t K, int64_t S) {
-    OzLayout L;
-    L.ldk = pad_k(K);
-    L.a = 0;                       // A first: its place does not depend on N
-    L.ea = L.a + a256((size_t)OZ_D * M * L.ldk * 2);
-    L.b = L.ea + a256((size_t)M * 4);
-    L.eb = L.b + a256((size_t)OZ_D * N * L.ldk * 2);
-    L.part = L.eb + a256((size_t)N * 4);
-    L.total = L.part + (S > 1 ? a256((size_t)S * M * N * 8) : 0);
-    return L;
-}
-
-// Split of a product: K tiles per CTA, splits and the estimated time (us).
-// Per-CTA cycles are those of the kernel's parts: about 2900 per 32-k step (68
-// MMAs of 128 x 64 x 16), 3500 per drain, 9000 for an FP64 epilogue.
+// Split of a product: K tiles per item, splits and the estimated time (us).
+// Cycles per item are those of the kernel's parts: about 2900 (FP32: 900) per
+// 32-k step, 3500 per drain; the FP64 epilogue, 9000, runs beside the next
+// item's MMAs where a CTA has one.
 struct OzSplit { int kt_per, S; double us; };
-OzSplit oz_split(int64_t M, int64_t N, int64_t K, int num_sms, size_t part_cap_elems) {
+template <class Real>
+OzSplit oz_split(int64_t M, int64_t N, int64_t K, int num_sms, size_t part_cap_elems, bool force_partial) {
     const int64_t tiles = ((M + OZ_BM - 1) / OZ_BM) * ((N + OZ_BN - 1) / OZ_BN);
     const int kt = (int)((K + OZ_BK - 1) / OZ_BK);
+    const double step = std::is_same<Real, double>::value ? 2900.0 : 900.0;
     OzSplit best{0, 0, 1e30};
-    for (int per = 1; per <= std::min(kt, OZ_MAX_KT); ++per) {
+    for (int per = 1; per <= std::min(kt, OzTraits<Real>::MAX_KT); ++per) {
         const int S = (kt + per - 1) / per;
-        if (S > 1 && ((size_t)S * M * N > part_cap_elems || S > 65535)) continue;
-        const double cta = 3000.0 + 2900.0 * per + 3500.0 * ((per + OZ_CHUNK - 1) / OZ_CHUNK) + (S == 1 ? 9000.0 : 2500.0);
-        double clk = std::ceil((double)tiles * S / num_sms) * cta;
+        if ((S > 1 || force_partial) && ((size_t)S * M * N > part_cap_elems || S > 65535)) continue;
+        const double item = 1000.0 + step * per + 3500.0 * ((per + OZ_CHUNK - 1) / OZ_CHUNK) + (S == 1 && !force_partial ? 3000.0 : 1500.0);
+        double clk = 4000.0 + std::ceil((double)tiles * S / num_sms) * item;
         if (S > 1) clk += 6000.0 + (double)S * M * N * 16.0 / 2500.0;
         if (clk / 1900.0 < best.us) best = {per, S, clk / 1900.0};
     }
@@ -582,126 +770,236 @@ OzSplit oz_split(int64_t M, int64_t N, int64_t K, int num_sms, size_t part_cap_e
 
 }  // namespace
 
+int oz_ktiles(int64_t K) { return (int)((K + OZ_BK - 1) / OZ_BK); }
+
+size_t oz_digit_bytes(int D, int64_t R, int64_t K, int rt) {
+    return a256((size_t)((R + rt - 1) / rt) * oz_ktiles(K) * D * rt * 64) + a256((size_t)R * 4);
+}
+
+template <class Src>
+OzOperand<Src> oz_operand(int D, const Src *X, int64_t ld, int64_t R, int64_t K, bool by_row, int mask, int rt,
+                          void *mem) {
+    OzOperand<Src> o{};
+    o.X = X; o.ld = ld; o.R = R; o.K = K; o.by_row = by_row ? 1 : 0; o.mask = mask;
+    o.KT = oz_ktiles(K);
+    o.rt = rt;
+    o.dst = (uint8_t *)mem;
+    o.exps = (int *)((char *)mem + oz_digit_bytes(D, R, K, rt) - a256((size_t)R * 4));
+    return o;
+}
+template OzOperand<double> oz_operand(int, const double *, int64_t, int64_t, int64_t, bool, int, int, void *);
+template OzOperand<float> oz_operand(int, const float *, int64_t, int64_t, int64_t, bool, int, int, void *);
+
+template <class Real>
+unsigned oz_slice_blocks(const OzOperand<Real> &o, bool tall) {
+    const int warps = tall ? 32 : 8;
+    return (unsigned)(o.by_row ? (o.R + 31) / 32 : (o.K > 1024 ? o.R : (o.R + warps - 1) / warps));
+}
+template unsigned oz_slice_blocks(const OzOperand<double> &, bool);
+template unsigned oz_slice_blocks(const OzOperand<float> &, bool);
+
+template <class Src>
+gbqr_status oz_slice_launch(const Exec &ex, int D, const OzSliceArgs<Src> &args, unsigned blocks, bool tall, double elems) {
+    if (!blocks) return GBQR_OK;
+    if (D != kD32 && (D != kD64 || std::is_same<Src, float>::value)) return GBQR_EINVAL;
+    trace_begin(ex, FAM_OTHER);
+    if (D == kD32) {
+        if (tall) oz_slice_kernel<Src, kD32, 1024, 4><<<blocks, 1024, 0, ex.stream>>>(args);
+        else oz_slice_kernel<Src, kD32, kThreads, 8><<<blocks, kThreads, 0, ex.stream>>>(args);
+    } else if constexpr (std::is_same<Src, double>::value) {
+        if (tall) oz_slice_kernel<Src, kD64, 1024, 4><<<blocks, 1024, 0, ex.stream>>>(args);
+        else oz_slice_kernel<Src, kD64, kThreads, 8><<<blocks, kThreads, 0, ex.stream>>>(args);
+    }
+    return trace_end(ex, FAM_OTHER, 0.0, ((double)sizeof(Src) + 2.0 * D) * elems);
+}
+template gbqr_status oz_slice_launch(const Exec &, int, const OzSliceArgs<double> &, unsigned, bool, double);
+template gbqr_status oz_slice_launch(const Exec &, int, const OzSliceArgs<float> &, unsigned, bool, double);
+
+template <class Src>
+gbqr_status oz_slice(const Exec &ex, int D, OzOperand<Src> *ops, int n) {
+    OzSliceArgs<Src> args{};
+    unsigned blocks = 0;
+    bool tall = false;
+    double elems = 0.0;
+    if (n > kOzOps) return GBQR_EINVAL;
+    for (int i = 0; i < n; ++i) tall = tall || (!ops[i].by_row && ops[i].K > 8192);
+    for (int i = 0; i < n; ++i) {
+        ops[i].first = blocks;
+        blocks += oz_slice_blocks(ops[i], tall);
+        elems += (double)ops[i].R * ops[i].K;
+        args.op[i] = ops[i];
+    }
+    args.n = n;
+    return oz_slice_launch(ex, D, args, blocks, tall, elems);
+}
+template gbqr_status oz_slice(const Exec &, int, OzOperand<double> *, int);
+template gbqr_status oz_slice(const Exec &, int, OzOperand<float> *, int);
+
+template <class Real, class SA, class SB>
+OzProblem<Real> oz_problem(const OzOperand<SA> &a, const OzOperand<SB> &b) {
+    OzProblem<Real> p{};
+    p.a = a.dst; p.b = b.dst; p.ea = a.exps; p.eb = b.exps;
+    p.M = (int)a.R; p.N = (int)b.R; p.KT = a.KT;
+    p.kt_per = p.KT; p.S = 1;
+    p.alpha = Real(1);
+    p.skip = a.skip;
+    p.b128 = b.rt == OZ_BM;
+    // op(A) lower: zero for k < i (stored K x M) or k > i; B upper: zero for k > j
+    if (a.mask == MASK_UNIT_LOWER) p.clip = a.by_row ? 2 : 1;
+    if (b.mask == MASK_UPPER && !b.by_row) p.clipB = 2;
+    return p;
+}
+template OzProblem<double> oz_problem<double>(const OzOperand<double> &, const OzOperand<double> &);
+template OzProblem<float> oz_problem<float>(const OzOperand<float> &, const OzOperand<float> &);
+template OzProblem<float> oz_problem<float>(const OzOperand<float> &, const OzOperand<double> &);
+
+int oz_items(int M, int N, int S) { return ((M + OZ_BM - 1) / OZ_BM) * ((N + OZ_BN - 1) / OZ_BN) * S; }
+
+// Chooses the split of a product whose partials fit part_bytes.
+template <class Real>
+bool oz_choose_split(OzProblem<Real> &p, int num_sms, size_t part_bytes, bool force_partial) {
+    const OzSplit s = oz_split<Real>(p.M, p.N, (int64_t)p.KT * OZ_BK, num_sms, part_bytes / 8, force_partial);
+    p.kt_per = s.kt_per;
+    p.S = s.S;
+    return s.S > 0;
+}
+template bool oz_choose_split(OzProblem<double> &, int, size_t, bool);
+template bool oz_choose_split(OzProblem<float> &, int, size_t, bool);
+
+template <class Real>
+gbqr_status oz_mma_launch(const Exec &ex, const OzMmaArgs<Real> &args, double elems) {
+    if (args.items <= 0) return GBQR_OK;
+    static std::atomic<bool> attr[64];
+    const bool cached = ex.device >= 0 && ex.device < 64;
+    if (!cached || !attr[ex.device].load(std::memory_order_acquire)) {
+        if (cudaFuncSetAttribute(oz_mma_kernel<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)oz_smem<Real>()) != cudaSuccess)
+            return GBQR_ECUDA;
+        if (cached) attr[ex.device].store(true, std::memory_order_release);
+    }
+    // a few items per CTA, so that epilogues overlap MMAs; no more, so that a
+    // look-ahead panel's launches on another stream find free SMs soon
+    const int grid = std::min(args.items, std::max(ex.num_sms, (args.items + kOzItemsPerCta - 1) / kOzItemsPerCta));
+    trace_begin(ex, FAM_TC_GEMM);
+    oz_mma_kernel<Real><<<grid, OZ_THREADS, oz_smem<Real>(), ex.stream>>>(args);
+    return trace_end(ex, FAM_TC_GEMM, 2.0 * oz_products<Real>() * elems, 0.0);
+}
+template gbqr_status oz_mma_launch(const Exec &, const OzMmaArgs<double> &, double);
+template gbqr_status oz_mma_launch(const Exec &, const OzMmaArgs<float> &, double);
+
+template <class Real>
+gbqr_status oz_reduce_launch(const Exec &ex, const OzMmaArgs<Real> &args, size_t largest) {
+    trace_begin(ex, FAM_OTHER);
+    const unsigned g = (unsigned)std::min<size_t>((largest + kThreads - 1) / kThreads, (size_t)ex.num_sms * 16);
+    oz_reduce_kernel<Real><<<dim3(g, (unsigned)args.n), kThreads, 0, ex.stream>>>(args);
+    return trace_end(ex, FAM_OTHER, 0.0, 0.0);
+}
+template gbqr_status oz_reduce_launch(const Exec &, const OzMmaArgs<double> &, size_t);
+template gbqr_status oz_reduce_launch(const Exec &, const OzMmaArgs<float> &, size_t);
+
+template <class Real>
+gbqr_status oz_requant_launch(const Exec &ex, const OzMmaArgs<Real> &args, int widest) {
+    trace_begin(ex, FAM_OTHER);
+    const unsigned g = (unsigned)std::min((widest + 7) / 8, ex.num_sms * 16);
+    oz_requant_kernel<Real><<<dim3(g, (unsigned)args.n), kThreads, 0, ex.stream>>>(args);
+    return trace_end(ex, FAM_OTHER, 0.0, 0.0);
+}
+template gbqr_status oz_requant_launch(const Exec &, const OzMmaArgs<double> &, int);
+template gbqr_status oz_requant_launch(const Exec &, const OzMmaArgs<float> &, int);
+
 // Digits of op(A) and of up to N columns of B, and the partials of a split
-// that gives every CTA at most 512 k and a small output two CTAs per SM.
+// that gives every item at most 512 k and a small output two CTAs per SM.
+template <class Real>
 size_t oz_gemm_scratch_bytes(int64_t M, int64_t N, int64_t K) {
     const int64_t tiles = std::max<int64_t>(1, ((M + OZ_BM - 1) / OZ_BM) * ((N + OZ_BN - 1) / OZ_BN));
-    const int64_t S = std::max((K + OZ_MAX_KT * OZ_BK - 1) / (OZ_MAX_KT * OZ_BK),
+    const int64_t S = std::max((K + 16 * OZ_BK - 1) / (16 * OZ_BK),
                                std::min<int64_t>({(K + OZ_BK - 1) / OZ_BK, (304 + tiles - 1) / tiles, 64}));
-    return oz_layout(M, N, K, S).total;
+    return oz_digit_bytes(OzTraits<Real>::D, M, K, OZ_BM) + oz_digit_bytes(OzTraits<Real>::D, N, K, OZ_BN) + (S > 1 ? a256((size_t)S * M * N * 8) : 0);
 }
+template size_t oz_gemm_scratch_bytes<double>(int64_t, int64_t, int64_t);
+template size_t oz_gemm_scratch_bytes<float>(int64_t, int64_t, int64_t);
 
 // How C = alpha op(A) B + beta C is done here, if at all: the columns of B in
 // chunks whose digits fit the scratch, where the estimated time beats the
-// FMA kernel's (1.15 TFLOP/s on large products).
+// FMA kernel's (1.15 TFLOP/s on large products; FP32 about 9).
 struct OzPlan { int64_t nc; OzSplit split; };
-static bool oz_plan(const GemmOp &op, const OzScratch &sc, int num_sms, OzPlan *plan, double *gain_us) {
+template <class Real>
+static bool oz_plan(const GemmOpT<Real> &op, const OzScratch &sc, int num_sms, OzPlan *plan, double *gain_us) {
     if (!sc.base || op.M < 8 || op.N < 8 || op.K < 8) return false;
     if (op.M > (1 << 30) || op.N > (1 << 30) || op.K > (1 << 30)) return false;
-    if (op.maskB == MASK_UNIT_LOWER) return false;
-    int64_t nc = std::min<int64_t>(op.N, (int64_t)OZ_BN * 65535);
+    int64_t nc = op.N;
     const size_t room = sc.bytes - sc.bytes / 8;                 // an eighth for partials
-    if (oz_layout(op.M, nc, op.K, 1).total > room) {
-        const size_t fixed = oz_layout(op.M, 0, op.K, 1).total + 1024, col = (size_t)OZ_D * pad_k(op.K) * 2 + 4;
-        const int64_t most = fixed < room ? (int64_t)((room - fixed) / col) / OZ_BN * OZ_BN : 0;
+    const size_t fixed = oz_digit_bytes(OzTraits<Real>::D, op.M, op.K, OZ_BM) + 512;
+    if (fixed + oz_digit_bytes(OzTraits<Real>::D, nc, op.K, OZ_BN) > room) {
+        const size_t col = oz_digit_bytes(OzTraits<Real>::D, OZ_BN, op.K, OZ_BN);
+        const int64_t most = fixed < room ? (int64_t)((room - fixed) / col) * OZ_BN : 0;
         if (most >= OZ_BN) {                                     // equal chunks of whole tiles
             const int64_t chunks = (nc + most - 1) / most;
             nc = ((nc + chunks - 1) / chunks + OZ_BN - 1) / OZ_BN * OZ_BN;
         }
     }
-    const OzLayout L = oz_layout(op.M, nc, op.K, 1);
-    if (L.total > sc.bytes) return false;
-    if ((size_t)op.M * nc >= ((size_t)1 << 32)) return false;
+    const size_t digits = oz_digit_bytes(OzTraits<Real>::D, op.M, op.K, OZ_BM) + oz_digit_bytes(OzTraits<Real>::D, nc, op.K, OZ_BN);
+    if (digits > sc.bytes) return false;
+    if ((size_t)op.M * nc >= ((size_t)1 << 32) || oz_items((int)op.M, (int)nc, 1) < 0) return false;
     plan->nc = nc;
-    plan->split = oz_split(op.M, nc, op.K, num_sms, (sc.bytes - L.total) / 8);
+    plan->split = oz_split<Real>(op.M, nc, op.K, num_sms, (sc.bytes - digits) / 8, false);
     if (plan->split.S == 0) return false;
     const double chunks = std::ceil((double)op.N / nc);
-    const double slice_us = 22.0 * ((double)op.M + nc) * op.K / 4.0e6;
-    *gain_us = gemm_algorithmic_flops(op) / 1.15e6 - chunks * (plan->split.us + slice_us + 10.0);
+    const double slice_us = (sizeof(Real) + 2.0 * OzTraits<Real>::D) * ((double)op.M + nc) * op.K / 4.0e6;
+    const double rate = std::is_same<Real, double>::value ? 1.15e6 : 9.0e6;
+    *gain_us = gemm_algorithmic_flops(op) / rate - chunks * (plan->split.us + slice_us + 10.0);
     return true;
 }
 
-bool oz_gemm_wanted(const GemmOp &op, const OzScratch &sc, int num_sms) {
+template <class Real>
+bool oz_gemm_wanted(const GemmOpT<Real> &op, const OzScratch &sc, int num_sms) {
     OzPlan p;
     double gain = 0.0;
     return sc.base && gemm_algorithmic_flops(op) > 1.4e7 && oz_plan(op, sc, num_sms, &p, &gain) && gain > 0.0;
 }
+template bool oz_gemm_wanted(const GemmOpT<double> &, const OzScratch &, int);
+template bool oz_gemm_wanted(const GemmOpT<float> &, const OzScratch &, int);
 
 // One chunk of columns; slice_a: op(A)'s digits are not in the scratch yet.
-static gbqr_status oz_chunk(const Exec &ex, const GemmOp &op, const OzScratch &sc, bool slice_a) {
-    OzLayout L = oz_layout(op.M, op.N, op.K, 1);
-    if (L.total > sc.bytes) return GBQR_ENOMEM;
-    const OzSplit sp = oz_split(op.M, op.N, op.K, ex.num_sms, (sc.bytes - L.total) / 8);
-    if (sp.S == 0) return GBQR_ENOMEM;
+template <class Real>
+static gbqr_status oz_chunk(const Exec &ex, const GemmOpT<Real> &op, const OzScratch &sc, bool slice_a) {
     char *base = (char *)sc.base;
-    OzOperand a{}, b{};
-    a.X = op.A; a.ld = op.lda; a.R = op.M; a.K = op.K; a.mask = op.maskA; a.by_row = op.ta ? 0 : 1;
-    a.dst = (__nv_bfloat16 *)(base + L.a); a.ldk = L.ldk; a.exps = (int *)(base + L.ea);
-    b.X = op.B; b.ld = op.ldb; b.R = op.N; b.K = op.K; b.mask = op.maskB; b.by_row = 0;
-    b.dst = (__nv_bfloat16 *)(base + L.b); b.ldk = L.ldk; b.exps = (int *)(base + L.eb);
-    const bool tall = op.K > 8192;                               // 1024 threads per row, else 256
-    const int warps = tall ? 32 : 8;
-    auto blocks = [&](const OzOperand &o) {
-        return (unsigned)(o.by_row ? (o.R + 31) / 32 : (o.K > 1024 ? o.R : (o.R + warps - 1) / warps));
-    };
-    a.blocks = slice_a ? blocks(a) : 0;
-    b.blocks = blocks(b);
-    if (op.ta && op.A == op.B && op.lda == op.ldb && op.M == op.N && op.maskA == op.maskB) {
-        b = a;                         // X^T X: one set of digits
-        b.blocks = 0;
-    }
-    a.skip = b.skip = op.skip;
-    a.kexp = b.kexp = op.kexp;
-    a.ksign = -1;
-    b.ksign = 1;
-    trace_begin(ex, FAM_OTHER);
-    const unsigned nblk = a.blocks + b.blocks;
-    if (nblk && tall) oz_slice_kernel<1024, 4><<<nblk, 1024, 0, ex.stream>>>(a, b);
-    else if (nblk) oz_slice_kernel<kThreads, 8><<<nblk, kThreads, 0, ex.stream>>>(a, b);
-    TRY_ST(trace_end(ex, FAM_OTHER, 0.0, 22.0 * ((double)op.M + op.N) * op.K));
-
-    OzParams p{};
-    p.M = (int)op.M; p.N = (int)op.N; p.K = (int)op.K;
-    p.ktiles = (int)((op.K + OZ_BK - 1) / OZ_BK);
-    p.kt_per = sp.kt_per;
-    // a strict lower op(A) is zero for k <= i (stored K x M) or k >= i (stored M x K)
-    p.clipA = op.maskA == MASK_UNIT_LOWER ? (op.ta ? 1 : 2) : 0;
-    p.ea = a.exps; p.eb = b.exps;
-    p.partial = sp.S > 1 ? (long long *)(base + L.part) : nullptr;
+    const size_t na = oz_digit_bytes(OzTraits<Real>::D, op.M, op.K, OZ_BM), nb = oz_digit_bytes(OzTraits<Real>::D, op.N, op.K, OZ_BN);
+    if (na + nb > sc.bytes) return GBQR_ENOMEM;
+    OzOperand<Real> a = oz_operand(OzTraits<Real>::D, op.A, op.lda, op.M, op.K, !op.ta, op.maskA, OZ_BM, base);
+    OzOperand<Real> b = oz_operand(OzTraits<Real>::D, op.B, op.ldb, op.N, op.K, false, op.maskB, OZ_BN, base + na);
+    b.unit = 1;
+    OzOperand<Real> ops[2];
+    int n = 0;
+    if (slice_a) ops[n++] = a;
+    if (op.ta && op.A == op.B && op.lda == op.ldb && op.M == op.N && op.maskA == MASK_NONE && op.maskB == MASK_NONE) b = a;   // X^T X
+    else ops[n++] = b;
+    TRY_ST(oz_slice(ex, OzTraits<Real>::D, ops, n));
+    OzMmaArgs<Real> args{};
+    OzProblem<Real> &p = args.prob[0];
+    p = oz_problem<Real>(a, b);
     p.C = op.C; p.ldc = op.ldc; p.alpha = op.alpha; p.beta = op.beta;
-    p.add = op.B; p.ldadd = op.ldb;
-    p.add_rows = op.maskA == MASK_UNIT_LOWER ? (int)std::min(op.M, op.K) : 0;
-    p.skip = op.skip;
-    p.err = sc.err;
-    CUtensorMap mA, mB;
-    if (!oz_map(&mA, a.dst, op.M, L.ldk, OZ_BM) || !oz_map(&mB, b.dst, op.N, L.ldk, OZ_BN)) return GBQR_ECUDA;
-    static std::atomic<bool> attr[64];
-    const bool cached = ex.device >= 0 && ex.device < 64;
-    if (!cached || !attr[ex.device].load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(oz_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM) != cudaSuccess)
-            return GBQR_ECUDA;
-        if (cached) attr[ex.device].store(true, std::memory_order_release);
+    if (op.maskA == MASK_UNIT_LOWER) {
+        // + B(i, j) for the unit diagonal; the strict part is split without it,
+        // whose entries it would outweigh by orders of magnitude
+        p.add = op.B; p.ldadd = op.ldb;
+        p.add_rows = (int)std::min(op.M, op.K);
     }
-    const dim3 grid((unsigned)((op.M + OZ_BM - 1) / OZ_BM), (unsigned)((op.N + OZ_BN - 1) / OZ_BN), (unsigned)sp.S);
-    trace_begin(ex, FAM_TC_GEMM);
-    oz_mma_kernel<<<grid, OZ_THREADS, OZ_SMEM, ex.stream>>>(mA, mB, p);
-    TRY_ST(trace_end(ex, FAM_TC_GEMM, 2.0 * 34.0 * (double)op.M * op.N * op.K, 14.0 * ((double)op.M + op.N) * op.K));
-    if (sp.S > 1) {
-        trace_begin(ex, FAM_OTHER);
-        const size_t total = (size_t)op.M * op.N;
-        const unsigned g = (unsigned)std::min<size_t>((total + kThreads - 1) / kThreads, (size_t)ex.num_sms * 16);
-        oz_reduce_kernel<<<g, kThreads, 0, ex.stream>>>(p, sp.S);
-        TRY_ST(trace_end(ex, FAM_OTHER, (double)sp.S * total, 8.0 * sp.S * total + 16.0 * total));
-    }
-    return GBQR_OK;
+    if (!oz_choose_split(p, ex.num_sms, sc.bytes - na - nb, false)) return GBQR_ENOMEM;
+    p.partial = p.S > 1 ? (long long *)(base + na + nb) : nullptr;
+    args.n = 1;
+    args.items = oz_items(p.M, p.N, p.S);
+    args.err = sc.err;
+    TRY_ST(oz_mma_launch(ex, args, (double)op.M * op.N * op.K));
+    return p.S > 1 ? oz_reduce_launch(ex, args, (size_t)op.M * op.N) : GBQR_OK;
 }
 
-gbqr_status oz_gemm(const Exec &ex, const GemmOp &op, const OzScratch &sc) {
+template <class Real>
+gbqr_status oz_gemm(const Exec &ex, const GemmOpT<Real> &op, const OzScratch &sc) {
     OzPlan pl;
     double gain = 0.0;
     if (!oz_plan(op, sc, ex.num_sms, &pl, &gain)) return GBQR_ENOMEM;
     for (int64_t j = 0; j < op.N; j += pl.nc) {
-        GemmOp c = op;
+        GemmOpT<Real> c = op;
         c.N = std::min(pl.nc, op.N - j);
         c.B = op.B + j * op.ldb;
         c.C = op.C + j * op.ldc;
@@ -709,5 +1007,7 @@ gbqr_status oz_gemm(const Exec &ex, const GemmOp &op, const OzScratch &sc) {
     }
     return GBQR_OK;
 }
+template gbqr_status oz_gemm(const Exec &, const GemmOpT<double> &, const OzScratch &);
+template gbqr_status oz_gemm(const Exec &, const GemmOpT<float> &, const OzScratch &);
 
 }  // namespace gbqr

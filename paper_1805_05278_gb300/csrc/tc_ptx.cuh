@@ -32,18 +32,32 @@ __device__ __forceinline__ uint64_t global_ns() {
     return t;
 }
 // Wait for the phase of the given parity; give up after ~2 s or as soon as
-// another thread of the grid has raised the error flag.
+// another thread of the grid has raised the error flag.  The flag (a load from
+// L2) and the timer are looked at once in 64 tries: a waiter that reads them
+// after every try sees its phase about a microsecond late.
 __device__ inline bool mbar_wait(uint32_t a, uint32_t parity, int *err) {
     if (mbar_try(a, parity)) return true;
     const uint64_t t0 = global_ns();
     for (;;) {
-        if (mbar_try(a, parity)) return true;
+#pragma unroll 1
+        for (int i = 0; i < 64; ++i)
+            if (mbar_try(a, parity)) return true;
         if (*(volatile int *)err) return false;
         if (global_ns() - t0 > 2000000000ull) {
             atomicExch(err, 1);
             return false;
         }
     }
+}
+// The same for a whole warp: one lane spins, the others then look once (the
+// phase is complete, the try orders their reads behind it).
+__device__ inline bool mbar_wait_warp(uint32_t a, uint32_t parity, int *err) {
+    bool ok = true;
+    if ((threadIdx.x & 31) == 0) ok = mbar_wait(a, parity, err);
+    ok = __all_sync(0xffffffffu, ok);
+    if (ok) mbar_try(a, parity);
+    __syncwarp();
+    return ok;
 }
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int x, int y, int z, uint32_t mbar) {
