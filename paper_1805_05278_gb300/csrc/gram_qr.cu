@@ -100,7 +100,9 @@ enum UnitFactor { UF_CHOL = 0, UF_L = 1, UF_U = 2 };
 // A1_kk - S R_kk.  Warp 0 carries the chain: it brings the next column up to
 // date, takes its pivot's reciprocal and publishes both, while the other
 // warps apply the current column to the ones behind; in the LU warp 1 carries
-// the next row of U the same way.  One barrier a step.
+// the next row of U the same way.  One barrier a step.  Warp 4, which shares
+// warp 0's sub-partition, stays idle, so that the chain's instructions do not
+// queue behind it.
 template <class Real>
 __global__ void __launch_bounds__(kThreads) gram_diag_kernel(const GramArgs<Real> p, int k) {
     __shared__ double S[GB][GB + 1], Rb[GB][GB + 1];     // [column][row]; Rb: R(row, column)
@@ -139,10 +141,13 @@ __global__ void __launch_bounds__(kThreads) gram_diag_kernel(const GramArgs<Real
             S[t + 1][lane] = v;
             cb[(t + 1) & 1][lane] = v;
             if (lane == 0) rb[(t + 1) & 1] = rd[t + 1] = r;
-        } else if (t + 1 + warp < GB) {
+        } else if (warp != 4) {
             const double *c = cb[t & 1];
-            const double li = lane > t ? c[lane] * rb[t & 1] : 0.0;
-            for (int j = t + 1 + warp; j < GB; j += 7) S[j][lane] = rfma(-li, c[j], S[j][lane]);
+            const int first = t + 2 + (warp > 4 ? warp - 2 : warp - 1);      // six warps share the columns
+            if (first < GB) {
+                const double li = lane > t ? c[lane] * rb[t & 1] : 0.0;
+                for (int j = first; j < GB; j += 6) S[j][lane] = rfma(-li, c[j], S[j][lane]);
+            }
         }
         __syncthreads();
     }
@@ -209,10 +214,13 @@ __global__ void __launch_bounds__(kThreads) gram_diag_kernel(const GramArgs<Real
             const double un = lane > t ? x - s * Rb[lane][t + 1] : 0.0;
             ub[(t + 1) & 1][lane] = un;
             p.U[(b0 + t + 1) + (b0 + lane) * GLD] = un;
-        } else if (t + warp < GB) {
-            const double li = cb[t & 1][lane] * rb[t & 1];
-            if (lane > t + 1)
-                for (int j = t + warp; j < GB; j += 6) S[j][lane] = rfma(-li, u[j], S[j][lane]);
+        } else if (warp != 4) {
+            const int first = t + 2 + (warp > 4 ? warp - 3 : warp - 2);      // five warps
+            if (first < GB) {
+                const double li = cb[t & 1][lane] * rb[t & 1];
+                if (lane > t + 1)
+                    for (int j = first; j < GB; j += 5) S[j][lane] = rfma(-li, u[j], S[j][lane]);
+            }
         }
         __syncthreads();
     }

@@ -334,21 +334,33 @@ __global__ void __launch_bounds__(NT) oz_slice_kernel(const __grid_constant__ Oz
 
 // ------------------------------------------------------------ conversion
 
-// X 2^e, X rounded to Real once.  e comes from exponents of operand rows: in
-// the everyday range the scaling is an integer addition (an FP64 instruction
-// takes a warp 64 cycles here); beyond it, and for rows with a NaN or an
-// infinity (exponent kExpNan), scalbn.
-__device__ __noinline__ double scaled_far(double d, int e) {
-    return e > kExpNan / 2 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(d, e);
+// X 2^e, X rounded to Real once.  To FP64 by integer instructions alone: an
+// FP64 instruction takes a warp 64 cycles here, and the conversion of a 64-bit
+// integer is several of them (it took a tile's epilogue 20 us).  e comes from
+// exponents of operand rows; outside the everyday range, and for rows with a
+// NaN or an infinity (exponent kExpNan), scalbn.
+__device__ __noinline__ double scaled_far(long long X, int e) {
+    return e > kExpNan / 2 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(__ll2double_rn(X), e);
 }
 __device__ __forceinline__ double scaled(long long X, int e, double) {
-    const double d = __ll2double_rn(X);
-    if ((unsigned)(e + 900) > 1800u) return scaled_far(d, e);
-    return __hiloint2double(__double2hiint(d) + (X == 0 ? 0 : e << 20), __double2loint(d));
+    if ((unsigned)(e + 900) > 1800u) return scaled_far(X, e);
+    const int sign = (int)(X >> 63);
+    const unsigned long long m = (unsigned long long)((X ^ (long long)sign) - (long long)sign);
+    const uint32_t hi = (uint32_t)(m >> 32), lo = (uint32_t)m;
+    const bool small = hi == 0;
+    const int lz = __clz(small ? lo : hi);                     // 32 if X == 0
+    const uint32_t th = __funnelshift_l(small ? 0u : lo, small ? lo : hi, lz);   // leading one at bit 31
+    const uint32_t tl = small ? 0u : lo << lz;
+    unsigned long long r = ((unsigned long long)(th >> 11) << 32) | __funnelshift_r(tl, th, 11);
+    r += (tl >> 10) & 1u;                                      // 53 bits, round half up
+    // biased exponent, less the one that the leading bit of r adds
+    const uint32_t ex = (uint32_t)(1022 + (small ? 31 : 63) - lz + e) << 20;
+    const uint32_t rh = m == 0 ? 0u : ((uint32_t)(r >> 32) + ex) | ((uint32_t)sign & 0x80000000u);
+    return __hiloint2double((int)rh, (int)(uint32_t)r);
 }
 __device__ __forceinline__ float scaled(long long X, int e, float) {
     const float f = __ll2float_rn(X);
-    if ((unsigned)(e + 60) > 120u) return (float)scaled_far(__ll2double_rn(X), e);
+    if ((unsigned)(e + 60) > 120u) return (float)scaled_far(X, e);
     return __int_as_float(__float_as_int(f) + (X == 0 ? 0 : e << 23));
 }
 
@@ -622,8 +634,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_mma_kernel(const __grid_cons
                         if (nb + c < p.N) pp[(size_t)(nb + c) * p.M] = X[c];
                 }
             } else if (ok) {
-                const bool sub = p.beta == Real(1) && p.alpha == Real(-1) && t.m0 >= p.add_rows;
-                if (sub && t.m0 + OZ_BM <= p.M && nb + OZ_COLS <= p.N) {
+                // compared once: an FP64 comparison costs as much as an addition
+                const bool minus = p.beta == Real(1) && p.alpha == Real(-1), read = p.beta != Real(0), plain = p.alpha == Real(1);
+                if (minus && t.m0 >= p.add_rows && t.m0 + OZ_BM <= p.M && nb + OZ_COLS <= p.N) {
                     // a whole tile of C -= V W
                     Real *cp = p.C + m + (int64_t)nb * p.ldc;
 #pragma unroll
@@ -642,12 +655,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_mma_kernel(const __grid_cons
                     for (int c = 0; c < OZ_COLS; ++c) {
                         Real d = scaled(X[c], ea + __shfl_sync(0xffffffffu, eb, c) - 14 - Tr::UNIT, Real(0));
                         if (nb + c < p.N && m < p.M) {
-                            const Real old = p.beta != Real(0) ? __ldcg(cp + (int64_t)c * p.ldc) : Real(0);
-                            const Real u = ap ? __ldcg(ap + (int64_t)c * p.ldadd) : Real(0);
+                            const Real old = read ? __ldcg(cp + (int64_t)c * p.ldc) : Real(0);
                             Real out;
-                            if (p.beta == Real(1) && p.alpha == Real(-1)) out = (old - u) - d;
-                            else if (p.beta == Real(0)) out = p.alpha == Real(1) ? d + u : p.alpha * (d + u);
-                            else out = p.beta * old + p.alpha * (d + u);
+                            if (minus) {
+                                out = (ap ? old - __ldcg(ap + (int64_t)c * p.ldadd) : old) - d;
+                            } else {
+                                if (ap) d += __ldcg(ap + (int64_t)c * p.ldadd);
+                                if (!read) out = plain ? d : p.alpha * d;
+                                else out = p.beta * old + p.alpha * d;
+                            }
                             cp[(int64_t)c * p.ldc] = out;
                         }
                     }
