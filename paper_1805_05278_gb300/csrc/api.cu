@@ -1462,12 +1462,17 @@ gbqr_status gbqr::factor_batched_untuned(gbqr_ctx *cx, int count, const int64_t 
         BatchPlan *pl = nullptr;
         TRY(batched_plan<Real>(&cx->bplan[sizeof(Real) == 8 ? 0 : 1], cx->device, cx->num_sms, count, m, n, lda, ldt,
                                b, !capturing, &pl));
-        if (capturing && cx->ws_bytes < batched_plan_bytes(pl)) return GBQR_EBUSY;
-        TRY(ensure_workspace(cx, batched_plan_bytes(pl)));
+        // a caller's workspace without room for the grouped part: the persistent kernel alone
+        size_t bytes = batched_plan_bytes(pl);
+        if (!cx->ws_owned && cx->ws_bytes < bytes) bytes = batched_plan_bytes_plain(pl);
+        if (capturing && cx->ws_bytes < bytes) return GBQR_EBUSY;
+        TRY(ensure_workspace(cx, bytes));
+        if (!capturing) TRY(batched_plan_upload(pl));
         if (prepare_only) return GBQR_OK;
         void *owned = nullptr;
         const gbqr_status st = batched_enqueue<Real>(cx->exec(), pl, A, T, m, n, lda, ldt, cx->ws, cx->ws_bytes,
-                                                     &cx->dinfo->timeout, &cx->dinfo->nonfinite, capturing, &owned);
+                                                     &cx->dinfo->timeout, &cx->dinfo->nonfinite, capturing, &owned,
+                                                     BatchSide{cx->side, cx->ev_fork, cx->ev_panel});
         if (owned) cx->capture_owned.push_back(owned);
         return st;
     }

@@ -46,6 +46,8 @@ namespace {
 
 constexpr int kUpdCols = 64;    // columns of an update task (the look-ahead block excepted)
 
+constexpr int kBesideCtas = 32;  // CTAs of the launch beside the grouped part: two per SM
+
 constexpr size_t kSmemBudget = 110 * 1024;   // two CTAs per SM
 
 template <class Real>
@@ -55,7 +57,7 @@ struct BMat {
     int64_t lda, ldt;
     int m, n;
     int state0;     // its first column-block counter
-    int pad;
+    int group;      // panel width of its grouped part in blocks of b, 0: none
 };
 
 template <class Real>
@@ -73,7 +75,19 @@ struct BParams {
     size_t tscr_stride;     // elements per CTA
     int tscr_blocks;
     long long wait_ns;
+    // per matrix: 0 = the grouped part did it, else 1 + the grouped panel it
+    // stopped at; null: not looked at (tasks of ungrouped matrices only)
+    const int *status;
 };
+
+// After the grouped part: nothing left to do (the dispenser starts at the end
+// of the list) unless some matrix stopped.
+__global__ void __launch_bounds__(kThreads) batched_rest_kernel(const int *status, int count, unsigned *next, int ntasks) {
+    int any = 0;
+    for (int i = threadIdx.x; i < count; i += kThreads) any |= status[i];
+    any = __syncthreads_or(any);
+    if (threadIdx.x == 0 && !any) *next = (unsigned)ntasks;
+}
 
 __device__ __forceinline__ int ld_acquire(const int *p) {
     int v;
@@ -564,17 +578,23 @@ __global__ void __launch_bounds__(kThreads, 2) batched_qr_kernel(BParams<Real> p
                 if (t < (unsigned)p.ntasks) {
                     const int4 tk = p.tasks[t];
                     s_task[0] = tk.x; s_task[1] = tk.y; s_task[2] = tk.z; s_task[3] = tk.w;
-                    go = wait_deps(p, p.state + p.mats[tk.x].state0, tk.y, tk.z, tk.w) ? 1 : 0;
+                    // a matrix that the grouped part finished has nothing left
+                    // to do; one that it left at some panel is done up to there
+                    const int grp = p.status ? p.mats[tk.x].group : 0, at = grp ? p.status[tk.x] : 1;
+                    if (at == 0) go = 3;
+                    else go = wait_deps(p, p.state + p.mats[tk.x].state0, tk.y, tk.z, tk.w) ? (tk.y < (at - 1) * grp ? 2 : 1) : 0;
                 }
             }
             s_go = go;
         }
         __syncthreads();
         if (!s_go) return;
+        if (s_go == 3) { __syncthreads(); continue; }
         const int mi = s_task[0], k = s_task[1], c0 = s_task[2], c1 = s_task[3];
         const BMat<Real> M = p.mats[mi];
         int bad = 0;
-        if (c0 == c1) bad = panel_task<MaxB>(p, M, k, sm, tscr);
+        if (s_go == 2) ;
+        else if (c0 == c1) bad = panel_task<MaxB>(p, M, k, sm, tscr);
         else update_task<MaxB>(p, M, k, c0, c1, sm);
         bad = __syncthreads_or(bad);
         if (threadIdx.x == 0) {
@@ -629,19 +649,26 @@ struct BatchPlan {
     uint64_t key = 0;            // shapes, leading dimensions, b, scalar size, device
     size_t real = 8;
     int b = 16, hblk = 0, hup = 64, ldS = 0, grid = 0, ntasks = 0, nstate = 0, tscr_blocks = 0, count = 0;
+    int nalone = 0;              // the first tasks: those of ungrouped matrices
     size_t smem = 0;
     size_t off_tasks = 0, off_state = 0, off_tscr = 0, total = 0, table_bytes = 0, state_bytes = 0;
     size_t tscr_stride = 0;
-    std::vector<int4> order;     // the task list, in list-schedule order
+    std::vector<int4> order;     // the task list, in list-schedule order (ungrouped matrices first)
     std::vector<int> state0;     // each matrix's first column-block counter
     std::vector<unsigned char> stage;   // pageable staging of the table for uncaptured calls
     double est_ms = 0.0;         // the list schedule's estimated makespan
+    GroupPlan *group = nullptr;  // the grouped part (b = 16), its workspace behind `total`
 };
 
-void batch_plan_free(BatchPlan *pl) { delete pl; }
+void batch_plan_free(BatchPlan *pl) {
+    if (pl) group_plan_free(pl->group);
+    delete pl;
+}
 
 double batch_plan_estimate_ms(const BatchPlan *pl) { return pl ? pl->est_ms : 0.0; }
-size_t batched_plan_bytes(const BatchPlan *pl) { return pl ? pl->total : 0; }
+size_t batched_plan_bytes_plain(const BatchPlan *pl) { return pl ? pl->total : 0; }
+size_t batched_plan_bytes(const BatchPlan *pl) { return pl ? std::max(pl->total, group_plan_bytes(pl->group)) : 0; }
+gbqr_status batched_plan_upload(BatchPlan *pl) { return group_plan_upload(pl->group); }
 
 namespace {
 
@@ -749,7 +776,7 @@ bool build_plan(BatchPlan *pl, int count, const int64_t *m, const int64_t *n, in
     pl->off_tasks = al(mat_bytes * (size_t)count);
     pl->table_bytes = pl->off_tasks + sizeof(int4) * pl->order.size();
     pl->off_state = al(pl->table_bytes);
-    pl->state_bytes = sizeof(int) * ((size_t)nstate + 2);
+    pl->state_bytes = sizeof(int) * ((size_t)nstate + 4);   // two launches: a dispenser and an abort flag each
     pl->off_tscr = al(pl->off_state + pl->state_bytes);
     pl->tscr_stride = (size_t)maxP * b * b;
     pl->total = al(pl->off_tscr + real * pl->tscr_stride * (size_t)grid);
@@ -797,6 +824,8 @@ gbqr_status batched_plan(BatchPlan **cache, int device, int num_sms, int count, 
         *cache = pl;
     }
     pl->key = 0;
+    group_plan_free(pl->group);
+    pl->group = nullptr;
     pl->real = sizeof(Real);
     pl->b = b;
     pl->hblk = hblk;
@@ -805,6 +834,13 @@ gbqr_status batched_plan(BatchPlan **cache, int device, int num_sms, int count, 
     pl->smem = smem;
     pl->grid = per_sm * num_sms;
     if (!build_plan(pl, count, m, n, b, pl->grid, sizeof(Real), sizeof(BMat<Real>))) return GBQR_ENOMEM;
+    if (b == 16) pl->group = group_plan_build<Real>(count, m, n, lda, ldt, num_sms, pl->total);
+    pl->nalone = pl->ntasks;
+    if (pl->group) {
+        const int *width = group_widths(pl->group);
+        auto mid = std::stable_partition(pl->order.begin(), pl->order.end(), [&](const int4 &t) { return width[t.x] == 0; });
+        pl->nalone = (int)(mid - pl->order.begin());
+    }
     pl->key = key;
     *out = pl;
     return GBQR_OK;
@@ -813,12 +849,14 @@ gbqr_status batched_plan(BatchPlan **cache, int device, int num_sms, int count, 
 template <class Real>
 gbqr_status batched_enqueue(const Exec &ex, BatchPlan *pl, Real *const *A, Real *const *T, const int64_t *m,
                             const int64_t *n, const int64_t *lda, const int64_t *ldt, char *ws, size_t ws_bytes,
-                            int *timeout_flag, unsigned long long *nonfinite, bool capturing, void **owned) {
+                            int *timeout_flag, unsigned long long *nonfinite, bool capturing, void **owned,
+                            const BatchSide &side) {
     *owned = nullptr;
     if (!pl || pl->real != sizeof(Real) || ws_bytes < pl->total) return GBQR_EINVAL;
     if (pl->ntasks == 0) return GBQR_OK;
     for (int i = 0; i < pl->count; ++i)
         if (n[i] > 0 && (!A[i] || !T[i])) return GBQR_EINVAL;
+    const bool group = pl->group && ws_bytes >= batched_plan_bytes(pl);
     // the matrix table and the task list, uploaded on the stream: from
     // pageable staging when running now (the copy is staged before the call
     // returns), from page-locked memory that the captured graph keeps when
@@ -835,7 +873,8 @@ gbqr_status batched_enqueue(const Exec &ex, BatchPlan *pl, Real *const *A, Real 
     for (int i = 0; i < pl->count; ++i) {
         BMat<Real> bm;
         bm.A = A[i]; bm.T = T[i]; bm.lda = lda[i]; bm.ldt = ldt[i];
-        bm.m = (int)m[i]; bm.n = (int)n[i]; bm.state0 = pl->state0[i]; bm.pad = 0;
+        bm.m = (int)m[i]; bm.n = (int)n[i]; bm.state0 = pl->state0[i];
+        bm.group = group ? group_widths(pl->group)[i] / pl->b : 0;
         memcpy(mats + i, &bm, sizeof bm);
     }
     memcpy(host + pl->off_tasks, pl->order.data(), sizeof(int4) * pl->order.size());
@@ -845,6 +884,7 @@ gbqr_status batched_enqueue(const Exec &ex, BatchPlan *pl, Real *const *A, Real 
     BParams<Real> p;
     p.mats = reinterpret_cast<const BMat<Real> *>(ws);
     p.tasks = reinterpret_cast<const int4 *>(ws + pl->off_tasks);
+    p.status = nullptr;
     p.ntasks = pl->ntasks;
     p.b = pl->b;
     p.hblk = pl->hblk;
@@ -859,10 +899,38 @@ gbqr_status batched_enqueue(const Exec &ex, BatchPlan *pl, Real *const *A, Real 
     p.tscr_stride = pl->tscr_stride;
     p.tscr_blocks = pl->tscr_blocks;
     p.wait_ns = 5000000000ll;   // 5 s: far beyond any one matrix's critical path
-    trace_begin(ex, FAM_BATCHED);
-    if (pl->b <= 16) batched_qr_kernel<16, Real><<<pl->grid, kThreads, pl->smem, ex.stream>>>(p);
-    else batched_qr_kernel<kMaxBatchB, Real><<<pl->grid, kThreads, pl->smem, ex.stream>>>(p);
-    return trace_end(ex, FAM_BATCHED, 0.0, 0.0);
+    auto launch = [&](const BParams<Real> &q, int grid, cudaStream_t st) {
+        Exec e = ex;
+        e.stream = st;
+        trace_begin(e, FAM_BATCHED);
+        if (pl->b <= 16) batched_qr_kernel<16, Real><<<grid, kThreads, pl->smem, st>>>(q);
+        else batched_qr_kernel<kMaxBatchB, Real><<<grid, kThreads, pl->smem, st>>>(q);
+        return trace_end(e, FAM_BATCHED, 0.0, 0.0);
+    };
+    if (!group) return launch(p, pl->grid, ex.stream);
+    // the ungrouped matrices (few and small: bound by their chains of steps)
+    // beside the grouped ones, on a few SMs; then whatever the grouped part
+    // left, with a T scratch of its own (the first launch is over by then)
+    const bool beside = pl->nalone > 0;
+    if (beside) {
+        BParams<Real> q = p;
+        q.ntasks = pl->nalone;
+        if (cudaEventRecord(side.fork, ex.stream) != cudaSuccess || cudaStreamWaitEvent(side.stream, side.fork, 0) != cudaSuccess)
+            return GBQR_ECUDA;
+        TRY_ST(launch(q, std::min(pl->grid, kBesideCtas), side.stream));
+        if (cudaEventRecord(side.join, side.stream) != cudaSuccess) return GBQR_ECUDA;
+    }
+    TRY_ST(group_enqueue<Real>(ex, pl->group, ws, ws, (int)sizeof(BMat<Real>), pl->count, timeout_flag));
+    if (beside && cudaStreamWaitEvent(ex.stream, side.join, 0) != cudaSuccess) return GBQR_ECUDA;
+    p.status = reinterpret_cast<const int *>(ws + group_status_offset(pl->group));
+    p.tasks += pl->nalone;
+    p.ntasks -= pl->nalone;
+    p.next += 2;
+    p.abort += 2;
+    trace_begin(ex, FAM_OTHER);
+    batched_rest_kernel<<<1, kThreads, 0, ex.stream>>>(p.status, pl->count, p.next, p.ntasks);
+    TRY_ST(trace_end(ex, FAM_OTHER, 0.0, 0.0));
+    return launch(p, pl->grid, ex.stream);
 }
 
 template gbqr_status batched_plan<double>(BatchPlan **, int, int, int, const int64_t *, const int64_t *,
@@ -871,10 +939,10 @@ template gbqr_status batched_plan<float>(BatchPlan **, int, int, int, const int6
                                          const int64_t *, const int64_t *, int, bool, BatchPlan **);
 template gbqr_status batched_enqueue<double>(const Exec &, BatchPlan *, double *const *, double *const *,
                                              const int64_t *, const int64_t *, const int64_t *, const int64_t *,
-                                             char *, size_t, int *, unsigned long long *, bool, void **);
+                                             char *, size_t, int *, unsigned long long *, bool, void **, const BatchSide &);
 template gbqr_status batched_enqueue<float>(const Exec &, BatchPlan *, float *const *, float *const *,
                                             const int64_t *, const int64_t *, const int64_t *, const int64_t *,
-                                            char *, size_t, int *, unsigned long long *, bool, void **);
+                                            char *, size_t, int *, unsigned long long *, bool, void **, const BatchSide &);
 
 }  // namespace gbqr
 
@@ -895,7 +963,7 @@ extern "C" GBQR_API gbqr_status gbqr_selftest_batched_wait(int device, int wait_
     gbqr_status st = GBQR_OK;
     BMat<double> bm;
     bm.A = reinterpret_cast<double *>(d); bm.T = reinterpret_cast<double *>(d);   // never dereferenced
-    bm.lda = 64; bm.ldt = 16; bm.m = 64; bm.n = 32; bm.state0 = 0; bm.pad = 0;
+    bm.lda = 64; bm.ldt = 16; bm.m = 64; bm.n = 32; bm.state0 = 0; bm.group = 0;
     const int4 task = make_int4(0, 0, 1, 2);
     if (cudaMemset(d, 0, bytes) != cudaSuccess || cudaMemcpy(d, &bm, sizeof bm, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(d + off_tasks, &task, sizeof task, cudaMemcpyHostToDevice) != cudaSuccess)
@@ -920,6 +988,7 @@ extern "C" GBQR_API gbqr_status gbqr_selftest_batched_wait(int device, int wait_
         p.tscr = reinterpret_cast<double *>(d);
         p.tscr_stride = 0;
         p.tscr_blocks = 0;
+        p.status = nullptr;
         p.wait_ns = (long long)wait_ms * 1000000ll;
         batched_qr_kernel<16, double><<<1, kThreads, smem>>>(p);
         if (cudaDeviceSynchronize() != cudaSuccess ||

@@ -177,6 +177,7 @@ gbqr_status tsqr_run(const Exec &ex, const TsqrPlan &plan, Real *A, int64_t lda,
 // call uploads the matrix table and the task list and launches one
 // persistent kernel.  T layout: panel kernels of width b (PANEL, nb = b).
 struct BatchPlan;
+struct BatchSide { cudaStream_t stream; cudaEvent_t fork, join; };   // for work beside the grouped part
 void batch_plan_free(BatchPlan *pl);
 double batch_plan_estimate_ms(const BatchPlan *pl);
 size_t batched_plan_bytes(const BatchPlan *pl);
@@ -186,13 +187,32 @@ template <class Real>
 gbqr_status batched_plan(BatchPlan **cache, int device, int num_sms, int count, const int64_t *m,
                          const int64_t *n, const int64_t *lda, const int64_t *ldt, int b, bool may_build,
                          BatchPlan **out);
+// Grouped part of a batch (gram_qr.cu): the well-shaped matrices' panels from
+// their Gram matrices, all matrices of a group in lockstep; the persistent
+// kernel then does the other matrices, and what stopped as ill-conditioned.
+struct GroupPlan;
+template <class Real>
+GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const int64_t *lda, const int64_t *ldt,
+                            int num_sms, size_t ws_off);
+void group_plan_free(GroupPlan *g);
+size_t group_plan_bytes(const GroupPlan *g);           // workspace, from its start
+const int *group_widths(const GroupPlan *g);           // per matrix, 0 = not grouped
+size_t group_status_offset(const GroupPlan *g);
+gbqr_status group_plan_upload(GroupPlan *g);
+template <class Real>
+gbqr_status group_enqueue(const Exec &ex, const GroupPlan *g, char *ws, const void *mats, int stride, int count, int *err);
+// The plan's workspace without the grouped part, and the upload of that part
+// (outside captures).
+size_t batched_plan_bytes_plain(const BatchPlan *pl);
+gbqr_status batched_plan_upload(BatchPlan *pl);
 // Enqueues the table upload, the counter reset and the launch on ex.stream.
 // capturing: the table is staged in page-locked memory returned in *owned,
 // which the captured graph must keep alive.
 template <class Real>
 gbqr_status batched_enqueue(const Exec &ex, BatchPlan *pl, Real *const *A, Real *const *T, const int64_t *m,
                             const int64_t *n, const int64_t *lda, const int64_t *ldt, char *ws, size_t ws_bytes,
-                            int *timeout_flag, unsigned long long *nonfinite, bool capturing, void **owned);
+                            int *timeout_flag, unsigned long long *nonfinite, bool capturing, void **owned,
+                            const BatchSide &side);
 
 // ------------------------------------------------------------ small kernels
 gbqr_status fill_identity(const Exec &ex, int64_t m, int64_t n, double *Q, int64_t ldq);

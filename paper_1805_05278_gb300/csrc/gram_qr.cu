@@ -47,7 +47,10 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
+#include <new>
 #include <type_traits>
+#include <vector>
 
 namespace gbqr {
 namespace {
@@ -67,7 +70,21 @@ struct GramArgs {
     double *M;                       // the block's unit triangular factors, M[t][lane]: see UnitFactor
     double *sc;                      // ... and the reciprocals of R's and U's diagonal
     int *flag, *kexp;                // kexp: exponents of the column norms
+    int raise;                       // what an ill-conditioned panel writes to *flag
+    int keep;                        // batch: *flag is the matrix's, clear at the start; a raised one skips the rest
+    int tb;                          // batch: T's blocks of width tb alone (0: the whole T)
 };
+
+// The panels of one launch: by value, or (blockIdx.y: which) a list in device memory.
+template <class Real>
+struct GramList {
+    GramArgs<Real> one;
+    const GramArgs<Real> *list;
+};
+template <class Real>
+__device__ __forceinline__ const GramArgs<Real> &nth_panel(const GramList<Real> &g) {
+    return g.list ? g.list[blockIdx.y] : g.one;
+}
 
 template <class Real>
 __device__ __forceinline__ double g_at(const GramArgs<Real> &p, int i, int j, int k) {
@@ -104,12 +121,13 @@ enum UnitFactor { UF_CHOL = 0, UF_L = 1, UF_U = 2 };
 // warp 0's sub-partition, stays idle, so that the chain's instructions do not
 // queue behind it.
 template <class Real>
-__global__ void __launch_bounds__(kThreads) gram_diag_kernel(const GramArgs<Real> p, int k) {
+__global__ void __launch_bounds__(kThreads) gram_diag_kernel(const __grid_constant__ GramList<Real> args, int k) {
     __shared__ double S[GB][GB + 1], Rb[GB][GB + 1];     // [column][row]; Rb: R(row, column)
     __shared__ double cb[2][GB], ub[2][GB], rb[2], rd[GB], sg[GB];
     __shared__ int bad;
+    const GramArgs<Real> p = nth_panel(args);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, b0 = k * GB;
-    if (k > 0 && *(volatile int *)p.flag) return;
+    if (k >= p.nblk || ((k > 0 || p.keep) && *(volatile int *)p.flag)) return;
     double a1[GB / 8];                                   // the LU's block, loaded behind the Cholesky's
 #pragma unroll
     for (int q = 0; q < GB / 8; ++q) {
@@ -161,10 +179,10 @@ __global__ void __launch_bounds__(kThreads) gram_diag_kernel(const GramArgs<Real
     }
     __syncthreads();
     if (bad) {
-        if (tid == 0) *p.flag = 1;
+        if (tid == 0) *p.flag = p.raise;
         return;
     }
-    if (k == 0 && tid == 0) *p.flag = 0;
+    if (k == 0 && tid == 0 && !p.keep) *p.flag = 0;
 #pragma unroll
     for (int q = 0; q < GB / 8; ++q) {
         // row t = c of the factor, lane = i
@@ -288,9 +306,10 @@ __device__ __forceinline__ void load_unit(double (*M)[GB + 1], const double *src
 // U_kk^{-1}, YR_l = R_lk R_kk^{-1} and YL_l = sum_j L_kj LI_jl.
 // blockIdx.x = task * 8 + column (row) group.
 template <class Real>
-__global__ void __launch_bounds__(GT) gram_row_kernel(const GramArgs<Real> p, int k) {
+__global__ void __launch_bounds__(GT) gram_row_kernel(const __grid_constant__ GramList<Real> args, int k) {
     __shared__ double sA[GB][GB + 1], sB[4][GB];
-    if (*(volatile int *)p.flag) return;
+    const GramArgs<Real> p = nth_panel(args);
+    if (k >= p.nblk || *(volatile int *)p.flag) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int task = blockIdx.x >> 3;
     const int c0 = (blockIdx.x & 7) * 4, rest = p.nblk - k - 1, c = c0 + warp;
@@ -328,13 +347,14 @@ __global__ void __launch_bounds__(GT) gram_row_kernel(const GramArgs<Real> p, in
             y *= rinv;
             blk(p.RI, k, k)[c + lane * GLD] = y;
             // the row is scaled by the norm of column b0 + c of the panel
-            if (!(y * y * __ldcg(p.gd + k * GB + c) <= kGramBound2)) *(volatile int *)p.flag = 1;
+            if (!(y * y * __ldcg(p.gd + k * GB + c) <= kGramBound2)) *(volatile int *)p.flag = p.raise;
         } else {
             blk(p.LI, k, k)[lane + c * GLD] = y;
         }
         return;
     }
     const int e = task - 3, l = e / 3, what = e % 3;
+    if (l >= k) return;
     if (what < 2) {
         const double a = __ldcg(blk(what == 0 ? p.U : p.R, l, k) + c + lane * GLD);   // row c
         load_unit(sA, p.M, what == 0 ? UF_U : UF_CHOL);
@@ -357,9 +377,10 @@ __global__ void __launch_bounds__(GT) gram_row_kernel(const GramArgs<Real> p, in
 // Trailing blocks of G (upper) and A1, then for l < k: X_lk = -sum X_lj YX_j,
 // RI_lk = -sum RI_lj YR_j, LI_kl = -LI_kk YL_l.
 template <class Real>
-__global__ void __launch_bounds__(GT) gram_trail_kernel(const GramArgs<Real> p, int k) {
+__global__ void __launch_bounds__(GT) gram_trail_kernel(const __grid_constant__ GramList<Real> args, int k) {
     __shared__ double sA[GB][GB + 1], sB[4][GB];
-    if (*(volatile int *)p.flag) return;
+    const GramArgs<Real> p = nth_panel(args);
+    if (k >= p.nblk || *(volatile int *)p.flag) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Tile tl{sA, sB, warp, lane};
     const int c0 = (blockIdx.x & 7) * 4, rest = p.nblk - k - 1, c = c0 + warp;
@@ -377,6 +398,7 @@ __global__ void __launch_bounds__(GT) gram_trail_kernel(const GramArgs<Real> p, 
         return;
     }
     const int e = task - 2 * rest * rest, l = e / 3, what = e % 3;
+    if (l >= k) return;
     double acc = 0.0;
     if (what == 2) {
         tl.load_a(blk(p.LI, k, k), false);
@@ -394,21 +416,22 @@ __global__ void __launch_bounds__(GT) gram_trail_kernel(const GramArgs<Real> p, 
         acc = tl.dot(acc);
     }
     blk(what == 0 ? p.X : p.RI, l, k)[lane + c * GLD] = -acc;
-    if (what == 1 && !(acc * acc * __ldcg(p.gd + l * GB + lane) <= kGramBound2)) *(volatile int *)p.flag = 1;
+    if (what == 1 && !(acc * acc * __ldcg(p.gd + l * GB + lane) <= kGramBound2)) *(volatile int *)p.flag = p.raise;
 }
 
 // Z = X T = -R+^{-1} S V1^{-T} (step 0), then T = U Z, the top block of Y = V T
 // = (A - [R; 0]) Z and V1 \\ R over the panel's top block (step 1).  A CTA
 // takes 32 x 2 outputs of block (i, j), a warp one column and the even or odd
 // 32-wide steps; all operands are staged at once.  blockIdx.x = block * 16 +
-// column pair, blockIdx.y = 1: Y.
+// column pair, blockIdx.z = 1: Y.
 template <class Real>
-__global__ void __launch_bounds__(GT) gram_t_kernel(const GramArgs<Real> p, int step) {
+__global__ void __launch_bounds__(GT) gram_t_kernel(const __grid_constant__ GramList<Real> args, int step) {
     __shared__ double sA[4][GB][GB + 1], sB[2][4 * GB], part[2][GB];
-    if (*(volatile int *)p.flag) return;
+    const GramArgs<Real> p = nth_panel(args);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, col = warp & 1, half = warp >> 1;
     const int c0 = (blockIdx.x & 15) * 2, c = c0 + col, task = blockIdx.x >> 4;
-    const bool top = blockIdx.y == 1;
+    const bool top = blockIdx.z == 1;
+    if (task >= p.nblk * p.nblk || (top && !p.Y) || *(volatile int *)p.flag) return;
     const int i = task % p.nblk, j = task / p.nblk, l0 = top ? 0 : i;
     const int gi = i * GB + lane, gj = j * GB + c;
     double acc = 0.0;
@@ -447,15 +470,38 @@ __global__ void __launch_bounds__(GT) gram_t_kernel(const GramArgs<Real> p, int 
         }
         return;
     }
-    if (gi >= p.w || gj >= p.w) return;
+    if (gj >= p.w) return;
+    if (p.tb && !top && gi / p.tb == gj / p.tb)        // rows past the last block's width are zeroed too
+        p.Tout[gi % p.tb + (int64_t)gj * p.ldt] = gi <= gj && gi < p.w ? (Real)acc : Real(0);
+    if (gi >= p.w) return;
     if (top) {
         p.Y[gi + (int64_t)gj * p.ldy] = (Real)acc;
         return;
     }
-    p.Tout[gi + (int64_t)gj * p.ldt] = gi <= gj ? (Real)acc : Real(0);
+    if (!p.tb) p.Tout[gi + (int64_t)gj * p.ldt] = gi <= gj ? (Real)acc : Real(0);
     p.A[gi + (int64_t)gj * p.lda] =
         (Real)(gi <= gj ? __ldcg(p.sgn + gi) * __ldcg(p.R + gi + gj * GLD) : __ldcg(p.L + gi + gj * GLD));
 }
+
+}  // namespace
+
+namespace {
+
+// Points p's arrays into `work` (gram_work_elems() doubles).
+template <class Real>
+void gram_carve(GramArgs<Real> &p, double *work) {
+    double **slots[] = {&p.G, &p.R, &p.RI, &p.A1, &p.L, &p.U, &p.LI, &p.X, &p.YX, &p.YR, &p.YL, &p.B1, &p.Z};
+    double *at = work;
+    for (double **s : slots) { *s = at; at += (size_t)GLD * GLD; }
+    p.M = at;
+    p.sc = p.M + 3 * GB * GB;
+    p.sgn = p.sc + 2 * GB;
+    p.gd = p.sgn + GLD;
+    p.kexp = (int *)(p.gd + GLD);
+}
+
+int gram_row_blocks(int nblk, int k) { return (2 * (nblk - k - 1) + 3 + 3 * k) * 8; }
+int gram_trail_blocks(int nblk, int k) { return (2 * (nblk - k - 1) * (nblk - k - 1) + 3 * k) * 8; }
 
 }  // namespace
 
@@ -494,18 +540,13 @@ template <class Real>
 gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, Real *A, int64_t lda, Real *T, int64_t ldt, Real *Y, int64_t ldy,
                     double *work, int *flag, const OzScratch &oz) {
     constexpr int D = oz_digits<Real>();
-    GramArgs<Real> p{};
+    GramList<Real> gl{};
+    GramArgs<Real> &p = gl.one;
     p.A = A; p.lda = lda; p.Tout = T; p.ldt = ldt; p.Y = Y; p.ldy = ldy;
     p.w = (int)w; p.nblk = (int)((w + GB - 1) / GB);
-    double **slots[] = {&p.G, &p.R, &p.RI, &p.A1, &p.L, &p.U, &p.LI, &p.X, &p.YX, &p.YR, &p.YL, &p.B1, &p.Z};
-    double *at = work;
-    for (double **s : slots) { *s = at; at += (size_t)GLD * GLD; }
-    p.M = at;
-    p.sc = p.M + 3 * GB * GB;
-    p.sgn = p.sc + 2 * GB;
-    p.gd = p.sgn + GLD;
+    gram_carve(p, work);
     p.flag = flag;
-    p.kexp = (int *)(p.gd + GLD);
+    p.raise = 1;
     const GramScratch sc = gram_scratch(D, m, w, Y != nullptr);
     if (sc.total > oz.bytes) return GBQR_ENOMEM;
     char *base = (char *)oz.base;
@@ -527,21 +568,21 @@ gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, Real *A, int64_t lda, 
     const double f3 = 2.0 * GB * GB * GB;
     for (int k = 0; k < p.nblk; ++k) {
         trace_begin(ex, FAM_OTHER);
-        gram_diag_kernel<Real><<<1, kThreads, 0, ex.stream>>>(p, k);
+        gram_diag_kernel<Real><<<1, kThreads, 0, ex.stream>>>(gl, k);
         TRY_ST(mark(f3));
-        const int rest = p.nblk - k - 1, row = 2 * rest + 3 + 3 * k, trail = 2 * rest * rest + 3 * k;
+        const int row = gram_row_blocks(p.nblk, k), trail = gram_trail_blocks(p.nblk, k);
         trace_begin(ex, FAM_OTHER);
-        gram_row_kernel<Real><<<row * 8, GT, 0, ex.stream>>>(p, k);
-        TRY_ST(mark(row * f3));
+        gram_row_kernel<Real><<<row, GT, 0, ex.stream>>>(gl, k);
+        TRY_ST(mark(row / 8 * f3));
         if (trail) {
             trace_begin(ex, FAM_OTHER);
-            gram_trail_kernel<Real><<<trail * 8, GT, 0, ex.stream>>>(p, k);
-            TRY_ST(mark(trail * f3));
+            gram_trail_kernel<Real><<<trail, GT, 0, ex.stream>>>(gl, k);
+            TRY_ST(mark(trail / 8 * f3));
         }
     }
     for (int step = 0; step < 2; ++step) {
         trace_begin(ex, FAM_OTHER);
-        gram_t_kernel<Real><<<dim3(p.nblk * p.nblk * 16, step == 1 && Y ? 2 : 1), GT, 0, ex.stream>>>(p, step);
+        gram_t_kernel<Real><<<dim3(p.nblk * p.nblk * 16, 1, step == 1 && Y ? 2 : 1), GT, 0, ex.stream>>>(gl, step);
         TRY_ST(mark(p.nblk * p.nblk * f3));
     }
     if (m > w) {
@@ -583,5 +624,531 @@ template gbqr_status gram_qr(const Exec &, int64_t, int64_t, double *, int64_t, 
                              double *, int *, const OzScratch &);
 template gbqr_status gram_qr(const Exec &, int64_t, int64_t, float *, int64_t, float *, int64_t, float *, int64_t,
                              double *, int *, const OzScratch &);
+
+
+// ------------------------------------------------------------------ batches
+// The panels of many matrices in lockstep: every launch above over a list of
+// panels.  A plan holds the lists of all launches as one blob whose pointers
+// are offsets (into the workspace, or into a matrix's A or T); a call copies
+// the blob into the workspace and relocates it there, so a plan serves any
+// buffers.  Matrices go in groups whose scratch fits kGroupBytes.
+namespace {
+
+constexpr size_t kGroupBytes = (size_t)6 << 30;
+constexpr int kBatchTb = 16;                     // width of a batch's T blocks
+constexpr int kGroupPanels = 4;
+
+enum RelocBase { RB_WS = 0, RB_A = 1, RB_T = 2 };
+struct Reloc { uint64_t off; uint32_t word; int mat; int base; int pad; };
+
+enum StepKind { ST_SLICE, ST_SLICE64, ST_MMA, ST_REDUCE, ST_REQUANT, ST_DIAG, ST_ROW, ST_TRAIL, ST_T };
+struct GroupStep {
+    StepKind kind;
+    size_t list = 0;          // the list's place in the blob
+    int n = 0;                // its length
+    int grid = 0;             // CTAs (slice), items (MMA), blocks per panel, columns (requant)
+    int k = 0;                // block (diag, row, trail) or step (T)
+    int z = 1;                // T: 2 where Y is wanted
+    bool tall = false;
+    double elems = 0.0;
+};
+
+template <class P>
+__global__ void __launch_bounds__(256) reloc_kernel(const Reloc *r, int n, uint64_t *blob, char *ws, const char *mats,
+                                                    int stride) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    const Reloc x = r[i];
+    uint64_t base = (uint64_t)ws;
+    if (x.base != RB_WS) {
+        // the matrix table starts with its pointers A and T
+        const P *p = reinterpret_cast<const P *>(mats + (size_t)x.mat * stride);
+        base = (uint64_t)p[x.base == RB_A ? 0 : 1];
+    }
+    blob[x.word] = base + x.off;
+}
+
+}  // namespace
+
+struct GroupPlan {
+    int D = 7;
+    size_t blob_off = 0, status_off = 0, total = 0;      // workspace layout, from its start
+    std::vector<uint8_t> blob;
+    std::vector<Reloc> relocs;
+    std::vector<GroupStep> steps;
+    std::vector<int> width;                              // per matrix: its panels' width, 0 = not grouped
+    uint8_t *d_blob = nullptr;                           // device copies (batch_group_upload)
+    Reloc *d_relocs = nullptr;
+};
+
+void group_plan_free(GroupPlan *g) {
+    if (!g) return;
+    cudaFree(g->d_blob);
+    cudaFree(g->d_relocs);
+    delete g;
+}
+size_t group_plan_bytes(const GroupPlan *g) { return g ? g->total : 0; }
+const int *group_widths(const GroupPlan *g) { return g->width.data(); }
+size_t group_status_offset(const GroupPlan *g) { return g->status_off; }
+
+namespace {
+
+// The panel width of an m x n matrix: equal panels of at most 128 columns, a
+// multiple of T's block width, each with 4 rows a column.  Shorter matrices
+// take narrower panels, up to kGroupPanels of them; 0 beyond that.
+int group_width(int64_t m, int64_t n) {
+    if (n < kGramMinW || m > (1 << 28)) return 0;
+    const int64_t np0 = (n + kGramMaxW - 1) / kGramMaxW;
+    for (int64_t np = np0; np <= std::max<int64_t>(np0, kGroupPanels); ++np) {
+        const int64_t w = ((n + np - 1) / np + kBatchTb - 1) / kBatchTb * kBatchTb;
+        if (w > kGramMaxW) continue;
+        bool fits = true;
+        for (int64_t j = 0; j < n; j += w) fits = fits && m - j >= 4 * std::min(w, n - j);
+        if (fits) return (int)w;
+    }
+    return 0;
+}
+
+template <class Real>
+struct GroupBuilder {
+    GroupPlan *g;
+    size_t arena = 0, peak = 0;
+    int D = oz_digits<Real>();
+
+    static size_t al(size_t x) { return (x + 255) / 256 * 256; }
+    size_t take(size_t bytes) {
+        const size_t o = arena;
+        arena += al(std::max<size_t>(bytes, 16));
+        peak = std::max(peak, arena);
+        return o;
+    }
+    // appends a list to the blob; fix(entry, place of the entry) adds relocations
+    template <class E>
+    size_t put(const std::vector<E> &v) {
+        size_t at = (g->blob.size() + 255) / 256 * 256;
+        g->blob.resize(at + v.size() * sizeof(E), 0);
+        memcpy(g->blob.data() + at, v.data(), v.size() * sizeof(E));
+        return at;
+    }
+    template <class F>
+    void rel(size_t at, const void *entry, const F *field, int base, int mat, uint64_t off) {
+        const size_t byte = at + (size_t)((const char *)field - (const char *)entry);
+        g->relocs.push_back({off, (uint32_t)(byte / 8), mat, base, 0});
+    }
+    template <class F>
+    void rel_flag(size_t at, const void *entry, const F *field, size_t flag) {
+        rel(at, entry, field, RB_WS, 0, flag);
+        g->relocs.back().pad = 1;                  // a place outside the arena
+    }
+    template <class Src>
+    void places(size_t at, const OzOperand<Src> &o, int base, int mat, uint64_t x, size_t digits, int64_t R, int64_t K,
+                size_t flag, size_t kexp) {
+        rel(at, &o, &o.X, base, mat, x);
+        rel(at, &o, &o.dst, RB_WS, 0, digits);
+        rel(at, &o, &o.exps, RB_WS, 0, exps_of(digits, R, K, o.rt));
+        rel_flag(at, &o, &o.skip, flag);
+        if (kexp) rel(at, &o, &o.kexp, RB_WS, 0, kexp);
+    }
+    size_t exps_of(size_t digits, int64_t R, int64_t K, int rt) const {
+        return digits + oz_digit_bytes(D, R, K, rt) - al((size_t)R * 4);
+    }
+};
+
+// Arena of one panel of one matrix, in bytes from the workspace's start.
+struct PanelPlaces { size_t work, p, x, z, part, y, vd, yd, c, wd, wf; };
+
+}  // namespace
+
+template <class Real>
+GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const int64_t *lda, const int64_t *ldt,
+                            int num_sms, size_t ws_off) {
+    std::vector<int> mats;
+    std::vector<int> width(count, 0);
+    for (int i = 0; i < count; ++i) {
+        width[i] = group_width(m[i], n[i]);
+        if (width[i]) mats.push_back(i);
+    }
+    if (mats.empty()) return nullptr;
+    GroupPlan *g = new (std::nothrow) GroupPlan();
+    if (!g) return nullptr;
+    constexpr int D = oz_digits<Real>();
+    g->D = D;
+    g->width = width;
+    GroupBuilder<Real> b{g};
+    g->status_off = GroupBuilder<Real>::al(ws_off);
+    // the arena's place depends on the blob's size: offsets are relative to
+    // the arena while building, and shifted at the end
+    auto flag_of = [&](int i) { return g->status_off + (size_t)i * 4; };
+    const size_t work_bytes = gram_work_elems() * 8;
+    // scratch of matrix i (its first panel is its largest)
+    auto need = [&](int i) {
+        const int64_t w = std::min<int64_t>(width[i], n[i]), nc = n[i] - w;
+        const size_t splits = oz_ktiles(m[i]);
+        size_t s = work_bytes + std::max(oz_digit_bytes(D, w, m[i], kOzTileA), oz_digit_bytes(D, m[i], w, kOzTileA)) +
+                   2 * oz_digit_bytes(D, w, w, kOzTileB) + std::min<size_t>(splits, 40) * w * w * 8;
+        if (nc > 0)
+            s += (size_t)m[i] * w * sizeof(Real) + oz_digit_bytes(D, m[i], w, kOzTileA) + oz_digit_bytes(D, w, m[i], kOzTileA) +
+                 oz_digit_bytes(D, nc, m[i], kOzTileB) + oz_digit_bytes(D, nc, w, kOzTileB) + (size_t)w * nc * sizeof(Real) +
+                 (splits / 16 + 1) * w * nc * 8;
+        return s + 16 * 256;
+    };
+    size_t at = 0;
+    while (at < mats.size()) {
+        size_t end = at, bytes = 0;
+        while (end < mats.size() && (end == at || bytes + need(mats[end]) <= kGroupBytes) && end - at < 60000) bytes += need(mats[end++]);
+        int64_t panels = 0;
+        for (size_t q = at; q < end; ++q) panels = std::max<int64_t>(panels, (n[mats[q]] + width[mats[q]] - 1) / width[mats[q]]);
+        for (int64_t pn = 0; pn < panels; ++pn) {
+            b.arena = 0;
+            std::vector<int> act;
+            for (size_t q = at; q < end; ++q)
+                if ((int64_t)width[mats[q]] * pn < n[mats[q]]) act.push_back(mats[q]);
+            const int na = (int)act.size();
+            std::vector<PanelPlaces> pl(na);
+            std::vector<OzOperand<Real>> sp(na), sa, sv;
+            std::vector<OzOperand<double>> sx;
+            std::vector<OzProblem<Real>> pg(na), pv, p1, p2;
+            std::vector<GramArgs<Real>> ga(na);
+            std::vector<int> trailing;
+            auto W = [&](int i) { return std::min<int64_t>(width[i], n[i] - width[i] * pn); };
+            auto J = [&](int i) { return (int64_t)width[i] * pn; };
+            auto M = [&](int i) { return m[i] - J(i); };
+            auto NC = [&](int i) { return n[i] - J(i) - W(i); };
+            auto Aoff = [&](int i, int64_t r, int64_t c) { return (uint64_t)((r + c * lda[i]) * (int64_t)sizeof(Real)); };
+            for (int q = 0; q < na; ++q) {
+                const int i = act[q];
+                PanelPlaces &s = pl[q];
+                s.work = b.take(work_bytes);
+                s.p = b.take(std::max(oz_digit_bytes(D, W(i), M(i), kOzTileA), oz_digit_bytes(D, M(i), W(i), kOzTileA)));
+                s.x = b.take(oz_digit_bytes(D, W(i), W(i), kOzTileB));
+                s.z = b.take(oz_digit_bytes(D, W(i), W(i), kOzTileB));
+                if (NC(i) > 0) {
+                    trailing.push_back(q);
+                    s.y = b.take((size_t)M(i) * W(i) * sizeof(Real));
+                    s.vd = b.take(oz_digit_bytes(D, M(i), W(i), kOzTileA));
+                    s.yd = b.take(oz_digit_bytes(D, W(i), M(i), kOzTileA));
+                    s.c = b.take(oz_digit_bytes(D, NC(i), M(i), kOzTileB));
+                    s.wd = b.take(oz_digit_bytes(D, NC(i), W(i), kOzTileB));
+                    s.wf = b.take((size_t)W(i) * NC(i) * sizeof(Real));
+                }
+            }
+            // ---- digits of P, G = P^T P
+            bool tall = false;
+            unsigned blocks = 0;
+            int items = 0;
+            size_t largest = 0;
+            double elems = 0.0, prods = 0.0;
+            for (int i : act) tall = tall || M(i) > 8192;
+            for (int q = 0; q < na; ++q) {
+                const int i = act[q];
+                sp[q] = oz_operand(D, (const Real *)nullptr, lda[i], W(i), M(i), false, MASK_NONE, kOzTileA, nullptr);
+                sp[q].first = blocks;
+                blocks += oz_slice_blocks(sp[q], tall);
+                elems += (double)W(i) * M(i);
+                pg[q] = oz_problem<Real>(sp[q], sp[q]);
+                // a full GPU of matrices needs no fine splits: 1024 k an item (FP64: 512)
+                pg[q].kt_per = std::max(1, std::min(pg[q].KT, sizeof(Real) == 8 ? 16 : 32));
+                if (na < num_sms) pg[q].kt_per = std::max(1, std::min(pg[q].kt_per, (pg[q].KT * na + num_sms - 1) / num_sms));
+                pg[q].kt_per = std::max(pg[q].kt_per, (pg[q].KT + 39) / 40);
+                pg[q].S = (pg[q].KT + pg[q].kt_per - 1) / pg[q].kt_per;
+                pg[q].ldc = GLD;
+                pg[q].first = items;
+                items += oz_items((int)W(i), (int)W(i), pg[q].S);
+                largest = std::max(largest, (size_t)W(i) * W(i));
+                prods += (double)W(i) * W(i) * M(i);
+                pl[q].part = b.take((size_t)pg[q].S * W(i) * W(i) * 8);
+                GramArgs<Real> &p = ga[q];
+                p = GramArgs<Real>{};
+                p.lda = lda[i]; p.ldt = ldt[i]; p.ldy = M(i);
+                p.w = (int)W(i); p.nblk = (int)((W(i) + GB - 1) / GB);
+                p.raise = 1 + (int)pn; p.keep = 1; p.tb = kBatchTb;
+            }
+            size_t L = b.put(sp);
+            for (int q = 0; q < na; ++q) {
+                const int i = act[q];
+                const size_t e = L + q * sizeof(sp[0]);
+                b.places(e, sp[q], RB_A, i, Aoff(i, J(i), J(i)), pl[q].p, W(i), M(i), flag_of(i), 0);
+            }
+            g->steps.push_back({ST_SLICE, L, na, (int)blocks, 0, 1, tall, elems});
+            L = b.put(pg);
+            const size_t gram_list = b.put(ga);
+            for (int q = 0; q < na; ++q) {
+                const int i = act[q];
+                const size_t e = L + q * sizeof(pg[0]);
+                const OzProblem<Real> &p = pg[q];
+                b.rel(e, &p, &p.a, RB_WS, 0, pl[q].p);
+                b.rel(e, &p, &p.b, RB_WS, 0, pl[q].p);
+                b.rel(e, &p, &p.ea, RB_WS, 0, b.exps_of(pl[q].p, W(i), M(i), kOzTileA));
+                b.rel(e, &p, &p.eb, RB_WS, 0, b.exps_of(pl[q].p, W(i), M(i), kOzTileA));
+                b.rel(e, &p, &p.partial, RB_WS, 0, pl[q].part);
+                b.rel_flag(e, &p, &p.skip, flag_of(i));
+                // the panel's arrays: carved from a null base, so that the fields hold their offsets
+                GramArgs<Real> c = ga[q];
+                gram_carve(c, (double *)nullptr);
+                b.rel(e, &p, &p.Cd, RB_WS, 0, pl[q].work + (size_t)(char *)c.G);
+                const size_t ge = gram_list + q * sizeof(ga[0]);
+                const GramArgs<Real> &a = ga[q];
+                double *GramArgs<Real>::*const f[] = {&GramArgs<Real>::G, &GramArgs<Real>::R, &GramArgs<Real>::RI, &GramArgs<Real>::A1,
+                    &GramArgs<Real>::L, &GramArgs<Real>::U, &GramArgs<Real>::LI, &GramArgs<Real>::X, &GramArgs<Real>::YX, &GramArgs<Real>::YR,
+                    &GramArgs<Real>::YL, &GramArgs<Real>::B1, &GramArgs<Real>::Z, &GramArgs<Real>::sgn, &GramArgs<Real>::gd,
+                    &GramArgs<Real>::M, &GramArgs<Real>::sc};
+                for (auto fp : f) b.rel(ge, &a, &(a.*fp), RB_WS, 0, pl[q].work + (size_t)(char *)(c.*fp));
+                b.rel(ge, &a, &a.kexp, RB_WS, 0, pl[q].work + (size_t)(char *)c.kexp);
+                b.rel_flag(ge, &a, &a.flag, flag_of(i));
+                b.rel(ge, &a, &a.A, RB_A, i, Aoff(i, J(i), J(i)));
+                b.rel(ge, &a, &a.Tout, RB_T, i, (uint64_t)(J(i) * ldt[i] * (int64_t)sizeof(Real)));
+                if (NC(i) > 0) b.rel(ge, &a, &a.Y, RB_WS, 0, pl[q].y);
+            }
+            g->steps.push_back({ST_MMA, L, na, items, 0, 1, false, prods});
+            g->steps.push_back({ST_REDUCE, L, na, (int)((largest + kThreads - 1) / kThreads), 0, 1, false, 0.0});
+            int nblk = 1;
+            for (auto &p : ga) nblk = std::max(nblk, p.nblk);
+            for (int k = 0; k < nblk; ++k) {
+                int row = 0, trail = 0;
+                for (auto &p : ga)
+                    if (k < p.nblk) {
+                        row = std::max(row, gram_row_blocks(p.nblk, k));
+                        trail = std::max(trail, gram_trail_blocks(p.nblk, k));
+                    }
+                g->steps.push_back({ST_DIAG, gram_list, na, 1, k, 1, false, 0.0});
+                g->steps.push_back({ST_ROW, gram_list, na, row, k, 1, false, 0.0});
+                if (trail) g->steps.push_back({ST_TRAIL, gram_list, na, trail, k, 1, false, 0.0});
+            }
+            for (int k = 0; k < 2; ++k)
+                g->steps.push_back({ST_T, gram_list, na, nblk * nblk * 16, k, k == 1 && !trailing.empty() ? 2 : 1, false, 0.0});
+            // ---- digits of A2, X, Z; V2 = A2 X, Y2 = A2 Z
+            blocks = 0;
+            unsigned xblocks = 0;
+            items = 0;
+            elems = prods = 0.0;
+            double xelems = 0.0;
+            struct Fix { int q; int what; };   // what: 0 A2, 1 X, 2 Z
+            std::vector<Fix> fa, fx, fv;
+            auto place_of = [&](int q, int what) { return what == 0 ? pl[q].p : (what == 1 ? pl[q].x : pl[q].z); };
+            for (int q = 0; q < na; ++q) {
+                const int i = act[q];
+                if (M(i) <= W(i)) continue;
+                OzOperand<Real> a2 = oz_operand(D, (const Real *)nullptr, lda[i], M(i) - W(i), W(i), true, MASK_NONE, kOzTileA, nullptr);
+                a2.ksign = -1;
+                a2.first = blocks;
+                blocks += oz_slice_blocks(a2, false);
+                elems += (double)(M(i) - W(i)) * W(i);
+                sa.push_back(a2);
+                fa.push_back({q, 0});
+                for (int y = 0; y < (NC(i) > 0 ? 2 : 1); ++y) {
+                    OzOperand<double> x = oz_operand(D, (const double *)nullptr, GLD, W(i), W(i), false, MASK_UPPER, kOzTileB, nullptr);
+                    x.ksign = 1;
+                    x.first = xblocks;
+                    xblocks += oz_slice_blocks(x, false);
+                    xelems += (double)W(i) * W(i);
+                    sx.push_back(x);
+                    fx.push_back({q, 1 + y});
+                    OzProblem<Real> p = oz_problem<Real>(a2, x);
+                    p.ldc = y == 0 ? lda[i] : M(i);
+                    p.first = items;
+                    items += oz_items((int)(M(i) - W(i)), (int)W(i), 1);
+                    prods += (double)(M(i) - W(i)) * W(i) * W(i);
+                    pv.push_back(p);
+                    fv.push_back({q, 1 + y});
+                }
+            }
+            if (!sa.empty()) {
+                GramArgs<Real> c{};
+                gram_carve(c, (double *)nullptr);
+                L = b.put(sa);
+                for (size_t e = 0; e < sa.size(); ++e) {
+                    const int q = fa[e].q, i = act[q];
+                    b.places(L + e * sizeof(sa[0]), sa[e], RB_A, i, Aoff(i, J(i) + W(i), J(i)), pl[q].p, M(i) - W(i), W(i), flag_of(i),
+                             pl[q].work + (size_t)(char *)c.kexp);
+                }
+                g->steps.push_back({ST_SLICE, L, (int)sa.size(), (int)blocks, 0, 1, false, elems});
+                L = b.put(sx);
+                for (size_t e = 0; e < sx.size(); ++e) {
+                    const int q = fx[e].q, i = act[q];
+                    b.places(L + e * sizeof(sx[0]), sx[e], RB_WS, 0, pl[q].work + (size_t)(char *)(fx[e].what == 1 ? c.X : c.Z),
+                             place_of(q, fx[e].what), W(i), W(i), flag_of(i), pl[q].work + (size_t)(char *)c.kexp);
+                }
+                g->steps.push_back({ST_SLICE64, L, (int)sx.size(), (int)xblocks, 0, 1, false, xelems});
+                L = b.put(pv);
+                for (size_t e = 0; e < pv.size(); ++e) {
+                    const int q = fv[e].q, i = act[q];
+                    const size_t pe = L + e * sizeof(pv[0]), xp = place_of(q, fv[e].what);
+                    const OzProblem<Real> &p = pv[e];
+                    b.rel(pe, &p, &p.a, RB_WS, 0, pl[q].p);
+                    b.rel(pe, &p, &p.ea, RB_WS, 0, b.exps_of(pl[q].p, M(i) - W(i), W(i), kOzTileA));
+                    b.rel(pe, &p, &p.b, RB_WS, 0, xp);
+                    b.rel(pe, &p, &p.eb, RB_WS, 0, b.exps_of(xp, W(i), W(i), kOzTileB));
+                    b.rel_flag(pe, &p, &p.skip, flag_of(i));
+                    if (fv[e].what == 1) b.rel(pe, &p, &p.C, RB_A, i, Aoff(i, J(i) + W(i), J(i)));
+                    else b.rel(pe, &p, &p.C, RB_WS, 0, pl[q].y + (size_t)W(i) * sizeof(Real));
+                }
+                g->steps.push_back({ST_MMA, L, (int)pv.size(), items, 0, 1, false, prods});
+            }
+            if (!trailing.empty()) {
+                // ---- C -= V (Y^T C)
+                blocks = 0;
+                elems = prods = 0.0;
+                items = 0;
+                int items2 = 0, widest = 0;
+                for (int q : trailing) {
+                    const int i = act[q];
+                    OzOperand<Real> v = oz_operand(D, (const Real *)nullptr, lda[i], M(i), W(i), true, MASK_UNIT_LOWER, kOzTileA, nullptr);
+                    OzOperand<Real> y = oz_operand(D, (const Real *)nullptr, M(i), W(i), M(i), false, MASK_NONE, kOzTileA, nullptr);
+                    OzOperand<Real> c = oz_operand(D, (const Real *)nullptr, lda[i], NC(i), M(i), false, MASK_NONE, kOzTileB, nullptr);
+                    const OzOperand<Real> wq = oz_operand(D, (const Real *)nullptr, 1, NC(i), W(i), false, MASK_NONE, kOzTileB, nullptr);
+                    for (OzOperand<Real> *o : {&v, &y, &c}) {
+                        o->first = blocks;
+                        blocks += oz_slice_blocks(*o, tall);
+                        elems += (double)o->R * o->K;
+                        sv.push_back(*o);
+                    }
+                    OzProblem<Real> p = oz_problem<Real>(y, c);
+                    p.kt_per = std::max(1, std::min(p.KT, 16));
+                    if ((int)trailing.size() < num_sms)
+                        p.kt_per = std::max(1, std::min(p.kt_per, (int)((p.KT * trailing.size() + num_sms - 1) / num_sms)));
+                    p.kt_per = std::max(p.kt_per, (p.KT + 39) / 40);
+                    p.S = (p.KT + p.kt_per - 1) / p.kt_per;
+                    p.ldc = W(i);
+                    p.first = items;
+                    items += oz_items((int)W(i), (int)NC(i), p.S);
+                    pl[q].part = b.take((size_t)p.S * W(i) * NC(i) * 8);
+                    p1.push_back(p);
+                    widest = std::max(widest, (int)NC(i));
+                    prods += (double)W(i) * NC(i) * M(i);
+                    OzProblem<Real> u = oz_problem<Real>(v, wq);
+                    u.ldc = lda[i];
+                    u.alpha = Real(-1);
+                    u.beta = Real(1);
+                    u.ldadd = W(i);
+                    u.add_rows = (int)W(i);
+                    u.first = items2;
+                    items2 += oz_items((int)M(i), (int)NC(i), 1);
+                    p2.push_back(u);
+                }
+                L = b.put(sv);
+                const size_t L1 = b.put(p1), L2 = b.put(p2);
+                for (size_t t = 0; t < trailing.size(); ++t) {
+                    const int q = trailing[t], i = act[q];
+                    const uint64_t ctop = Aoff(i, J(i), J(i) + W(i));
+                    const size_t e = L + 3 * t * sizeof(sv[0]);
+                    b.places(e, sv[3 * t], RB_A, i, Aoff(i, J(i), J(i)), pl[q].vd, M(i), W(i), flag_of(i), 0);
+                    b.places(e + sizeof(sv[0]), sv[3 * t + 1], RB_WS, 0, pl[q].y, pl[q].yd, W(i), M(i), flag_of(i), 0);
+                    b.places(e + 2 * sizeof(sv[0]), sv[3 * t + 2], RB_A, i, ctop, pl[q].c, NC(i), M(i), flag_of(i), 0);
+                    const size_t e1 = L1 + t * sizeof(p1[0]), e2 = L2 + t * sizeof(p2[0]);
+                    const OzProblem<Real> &p = p1[t], &u = p2[t];
+                    b.rel(e1, &p, &p.a, RB_WS, 0, pl[q].yd);
+                    b.rel(e1, &p, &p.ea, RB_WS, 0, b.exps_of(pl[q].yd, W(i), M(i), kOzTileA));
+                    b.rel(e1, &p, &p.b, RB_WS, 0, pl[q].c);
+                    b.rel(e1, &p, &p.eb, RB_WS, 0, b.exps_of(pl[q].c, NC(i), M(i), kOzTileB));
+                    b.rel(e1, &p, &p.partial, RB_WS, 0, pl[q].part);
+                    b.rel_flag(e1, &p, &p.skip, flag_of(i));
+                    b.rel(e1, &p, &p.C, RB_WS, 0, pl[q].wf);
+                    b.rel(e1, &p, &p.qdst, RB_WS, 0, pl[q].wd);
+                    b.rel(e1, &p, &p.qexp, RB_WS, 0, b.exps_of(pl[q].wd, NC(i), W(i), kOzTileB));
+                    b.rel(e2, &u, &u.a, RB_WS, 0, pl[q].vd);
+                    b.rel(e2, &u, &u.ea, RB_WS, 0, b.exps_of(pl[q].vd, M(i), W(i), kOzTileA));
+                    b.rel(e2, &u, &u.b, RB_WS, 0, pl[q].wd);
+                    b.rel(e2, &u, &u.eb, RB_WS, 0, b.exps_of(pl[q].wd, NC(i), W(i), kOzTileB));
+                    b.rel_flag(e2, &u, &u.skip, flag_of(i));
+                    b.rel(e2, &u, &u.add, RB_WS, 0, pl[q].wf);
+                    b.rel(e2, &u, &u.C, RB_A, i, ctop);
+                }
+                g->steps.push_back({ST_SLICE, L, (int)sv.size(), (int)blocks, 0, 1, tall, elems});
+                g->steps.push_back({ST_MMA, L1, (int)p1.size(), items, 0, 1, false, prods});
+                g->steps.push_back({ST_REQUANT, L1, (int)p1.size(), widest, 0, 1, false, 0.0});
+                g->steps.push_back({ST_MMA, L2, (int)p2.size(), items2, 0, 1, false, prods});
+            }
+        }
+        at = end;
+    }
+    // workspace: [... | status | blob | arena]; arena offsets are shifted to
+    // their place (status places are absolute already)
+    g->blob_off = GroupBuilder<Real>::al(g->status_off + (size_t)count * 4);
+    const size_t arena0 = GroupBuilder<Real>::al(g->blob_off + g->blob.size());
+    for (Reloc &r : g->relocs)
+        if (r.base == RB_WS && !r.pad) r.off += arena0;
+    g->total = arena0 + b.peak;
+    return g;
+}
+
+// Device copies of the plan's blob and relocations (not during a capture).
+gbqr_status group_plan_upload(GroupPlan *g) {
+    if (!g || g->d_blob) return GBQR_OK;
+    if (cudaMalloc((void **)&g->d_blob, g->blob.size()) != cudaSuccess ||
+        cudaMalloc((void **)&g->d_relocs, g->relocs.size() * sizeof(Reloc)) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(g->d_blob);
+        g->d_blob = nullptr;
+        return GBQR_ENOMEM;
+    }
+    if (cudaMemcpy(g->d_blob, g->blob.data(), g->blob.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(g->d_relocs, g->relocs.data(), g->relocs.size() * sizeof(Reloc), cudaMemcpyHostToDevice) != cudaSuccess)
+        return GBQR_ECUDA;
+    return GBQR_OK;
+}
+
+// Enqueues the grouped factorizations; mats: the matrix table in device
+// memory (A and T first).  status[i] stays 0 for a grouped matrix that is
+// done, else 1 + the panel it stopped at.
+template <class Real>
+gbqr_status group_enqueue(const Exec &ex, const GroupPlan *g, char *ws, const void *mats, int stride, int count, int *err) {
+    if (!g->d_blob || g->D != oz_digits<Real>()) return GBQR_EINVAL;
+    uint8_t *blob = (uint8_t *)ws + g->blob_off;
+    if (cudaMemsetAsync(ws + g->status_off, 0, (size_t)count * 4, ex.stream) != cudaSuccess ||
+        cudaMemcpyAsync(blob, g->d_blob, g->blob.size(), cudaMemcpyDeviceToDevice, ex.stream) != cudaSuccess)
+        return GBQR_ECUDA;
+    const int nr = (int)g->relocs.size();
+    trace_begin(ex, FAM_OTHER);
+    reloc_kernel<Real *><<<(nr + 255) / 256, 256, 0, ex.stream>>>(g->d_relocs, nr, (uint64_t *)blob, ws, (const char *)mats, stride);
+    TRY_ST(trace_end(ex, FAM_OTHER, 0.0, 0.0));
+    for (const GroupStep &s : g->steps) {
+        switch (s.kind) {
+            case ST_SLICE: {
+                OzSliceArgs<Real> a{};
+                a.list = reinterpret_cast<const OzOperand<Real> *>(blob + s.list);
+                a.n = s.n;
+                TRY_ST(oz_slice_launch(ex, g->D, a, (unsigned)s.grid, s.tall, s.elems));
+                break;
+            }
+            case ST_SLICE64: {
+                OzSliceArgs<double> a{};
+                a.list = reinterpret_cast<const OzOperand<double> *>(blob + s.list);
+                a.n = s.n;
+                TRY_ST(oz_slice_launch(ex, g->D, a, (unsigned)s.grid, s.tall, s.elems));
+                break;
+            }
+            case ST_MMA:
+            case ST_REDUCE:
+            case ST_REQUANT: {
+                OzMmaArgs<Real> a{};
+                a.list = reinterpret_cast<const OzProblem<Real> *>(blob + s.list);
+                a.n = s.n;
+                a.items = s.grid;
+                a.err = err;
+                if (s.kind == ST_MMA) TRY_ST(oz_mma_launch(ex, a, s.elems));
+                else if (s.kind == ST_REDUCE) TRY_ST(oz_reduce_launch(ex, a, (size_t)s.grid * kThreads));
+                else TRY_ST(oz_requant_launch(ex, a, s.grid));
+                break;
+            }
+            default: {
+                GramList<Real> gl{};
+                gl.list = reinterpret_cast<const GramArgs<Real> *>(blob + s.list);
+                trace_begin(ex, FAM_OTHER);
+                const dim3 grid((unsigned)s.grid, (unsigned)s.n, (unsigned)s.z);
+                if (s.kind == ST_DIAG) gram_diag_kernel<Real><<<grid, kThreads, 0, ex.stream>>>(gl, s.k);
+                else if (s.kind == ST_ROW) gram_row_kernel<Real><<<grid, GT, 0, ex.stream>>>(gl, s.k);
+                else if (s.kind == ST_TRAIL) gram_trail_kernel<Real><<<grid, GT, 0, ex.stream>>>(gl, s.k);
+                else gram_t_kernel<Real><<<grid, GT, 0, ex.stream>>>(gl, s.k);
+                TRY_ST(trace_end(ex, FAM_OTHER, 0.0, 0.0));
+            }
+        }
+    }
+    return GBQR_OK;
+}
+
+template GroupPlan *group_plan_build<double>(int, const int64_t *, const int64_t *, const int64_t *, const int64_t *, int, size_t);
+template GroupPlan *group_plan_build<float>(int, const int64_t *, const int64_t *, const int64_t *, const int64_t *, int, size_t);
+template gbqr_status group_enqueue<double>(const Exec &, const GroupPlan *, char *, const void *, int, int, int *);
+template gbqr_status group_enqueue<float>(const Exec &, const GroupPlan *, char *, const void *, int, int, int *);
 
 }  // namespace gbqr

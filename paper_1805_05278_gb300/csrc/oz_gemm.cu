@@ -174,10 +174,10 @@ __device__ __forceinline__ Real oz_load(const OzOperand<Real> &o, int64_t r, int
     if (o.mask == MASK_UNIT_LOWER && i <= j) return i == j && o.unit ? Real(1) : Real(0);
     if (o.mask == MASK_UPPER && i > j) return Real(0);
     const Real x = o.X[i + j * o.ld];
-    return o.kexp ? mul_pow2(x, o.ksign * __ldcg(o.kexp + k)) : x;
+    return o.kexp ? mul_pow2(x, o.ksign * o.kexp[k]) : x;
 }
 
-// Digits of the NV = 4 or 16 consecutive entries v of operand row r from k0.
+// Digits of the NV = 4 or 8 consecutive entries v of operand row r from k0.
 template <int D, class Real, int NV>
 __device__ __forceinline__ void store_digits(uint8_t *dst, int KT, int rt, int64_t r, int64_t k0, const Real (&v)[NV],
                                              int exmax) {
@@ -229,14 +229,14 @@ __device__ __forceinline__ void store_exp(const OzOperand<Real> &o, int64_t r, i
 // CTAs [first[i], first[i + 1]).  Bound by HBM (8 bytes read, 14 written per
 // entry) and, for few rows, by latency, so every entry is read once where
 // registers hold the row between the search for its maximum and the split:
-// NT threads keep NQ quads each (256 x 8: rows of 8192; 1024 x 4: 16384; what
+// NT threads keep NQ quads each (256 x 8: rows of 8192; 512 x 8: 16384; what
 // lies beyond is read again).
 //   by column: a warp per operand row (K <= 1024) or a CTA per row; a thread
 //              takes 4 consecutive k (8-byte stores, 64 bytes a row tile).
-//   by row:    a CTA takes 32 rows, lane = row, a warp 16 consecutive k (reads
-//              are coalesced along the rows, stores are 16 bytes).
+//   by row:    eight warps take 32 rows, lane = row, a warp 16 consecutive k
+//              (reads are coalesced along the rows, stores are 16 bytes).
 template <class Real, int D, int NT, int NQ>
-__global__ void __launch_bounds__(NT) oz_slice_kernel(const __grid_constant__ OzSliceArgs<Real> args) {
+__global__ void __launch_bounds__(NT, 512 / NT) oz_slice_kernel(const __grid_constant__ OzSliceArgs<Real> args) {
     __shared__ int red[NT / 32][32];
     constexpr int NW = NT / 32, INF = ExpOf<Real>::INF;
     int which = 0;
@@ -258,29 +258,53 @@ __global__ void __launch_bounds__(NT) oz_slice_kernel(const __grid_constant__ Oz
     const int64_t kpad = (int64_t)o.KT * OZ_BK;
     int ex = 0;
     if (o.by_row) {
-        const int64_t r = blk * 32 + lane;
-        Real v[16];
-        for (int64_t k0 = warp * 16; k0 < o.K; k0 += 16 * NW) {
+        const int sub = warp >> 3, w8 = warp & 7;
+        const int64_t r0 = blk * (4 * NW) + sub * 32, r = r0 + lane;
+        // rows that no mask touches (a V basis below its triangle) are read directly
+        const bool direct = o.mask == MASK_NONE || (o.mask == MASK_UNIT_LOWER && r0 >= o.K);
+        auto load16 = [&](int64_t k0, Real (&v)[16]) {
+            if (direct && k0 + 16 <= o.K) {
+                const Real *x = o.X + r + k0 * o.ld;
 #pragma unroll
-            for (int q = 0; q < 16; ++q) v[q] = oz_load(o, r, k0 + q);
+                for (int q = 0; q < 16; ++q) v[q] = r < o.R ? x[q * o.ld] : Real(0);
+                if (o.kexp) {
+                    const int ke = o.ksign * o.kexp[k0 + (lane & 15)];
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) v[q] = mul_pow2(v[q], __shfl_sync(0xffffffffu, ke, q));
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < 16; ++q) v[q] = oz_load(o, r, k0 + q);
+            }
+        };
+        Real v[16];
+        for (int64_t k0 = w8 * 16; k0 < o.K; k0 += 128) {
+            load16(k0, v);
 #pragma unroll
             for (int q = 0; q < 16; ++q) ex = max(ex, exp_field(v[q]));
         }
         red[warp][lane] = ex;
         __syncthreads();
 #pragma unroll
-        for (int w = 0; w < NW; ++w) ex = max(ex, red[w][lane]);
+        for (int w = 0; w < 8; ++w) ex = max(ex, red[sub * 8 + w][lane]);
         ex = max(ex, 1);
-        if (r >= o.R) return;
-        if (warp == 0) store_exp(o, r, ex);
-        const bool kept = o.K <= 16 * NW;                       // v holds this warp's only 16 k
-        for (int64_t k0 = warp * 16; k0 < kpad; k0 += 16 * NW) {
+        if (w8 == 0 && r < o.R) store_exp(o, r, ex);
+        const bool kept = o.K <= 128;                           // v holds this warp's only 16 k
+        for (int64_t k0 = w8 * 16; k0 < kpad; k0 += 128) {
+            if (!kept) load16(k0, v);
+            if (ex == INF || (kept && k0 >= o.K)) {
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                if (ex == INF || (kept && k0 >= o.K)) v[q] = Real(0);
-                else if (!kept) v[q] = oz_load(o, r, k0 + q);
+                for (int q = 0; q < 16; ++q) v[q] = Real(0);
             }
-            store_digits<D>(o.dst, o.KT, o.rt, r, k0, v, ex);
+            if (r < o.R) {
+                Real h[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) h[q] = v[q];
+                store_digits<D>(o.dst, o.KT, o.rt, r, k0, h, ex);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) h[q] = v[8 + q];
+                store_digits<D>(o.dst, o.KT, o.rt, r, k0 + 8, h, ex);
+            }
         }
         return;
     }
@@ -636,7 +660,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_mma_kernel(const __grid_cons
             } else if (ok) {
                 // compared once: an FP64 comparison costs as much as an addition
                 const bool minus = p.beta == Real(1) && p.alpha == Real(-1), read = p.beta != Real(0), plain = p.alpha == Real(1);
-                if (minus && t.m0 >= p.add_rows && t.m0 + OZ_BM <= p.M && nb + OZ_COLS <= p.N) {
+                const bool whole = t.m0 >= p.add_rows && t.m0 + OZ_BM <= p.M && nb + OZ_COLS <= p.N;
+                if (whole && minus) {
                     // a whole tile of C -= V W
                     Real *cp = p.C + m + (int64_t)nb * p.ldc;
 #pragma unroll
@@ -648,6 +673,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_mma_kernel(const __grid_cons
                         for (int c = 0; c < 8; ++c, cp += p.ldc)
                             *cp = cv[c] - scaled(X[g + c], ea + __shfl_sync(0xffffffffu, eb, g + c) - 14 - Tr::UNIT, Real(0));
                     }
+                } else if (whole && !read && plain) {
+                    // a whole tile of C = A X
+                    Real *cp = p.C + m + (int64_t)nb * p.ldc;
+#pragma unroll
+                    for (int c = 0; c < OZ_COLS; ++c, cp += p.ldc)
+                        *cp = scaled(X[c], ea + __shfl_sync(0xffffffffu, eb, c) - 14 - Tr::UNIT, Real(0));
                 } else {
                     Real *cp = p.C + m + (int64_t)nb * p.ldc;
                     const Real *ap = m < min(p.add_rows, p.M) ? p.add + m + (int64_t)nb * p.ldadd : nullptr;
@@ -808,8 +839,8 @@ template OzOperand<float> oz_operand(int, const float *, int64_t, int64_t, int64
 
 template <class Real>
 unsigned oz_slice_blocks(const OzOperand<Real> &o, bool tall) {
-    const int warps = tall ? 32 : 8;
-    return (unsigned)(o.by_row ? (o.R + 31) / 32 : (o.K > 1024 ? o.R : (o.R + warps - 1) / warps));
+    const int warps = tall ? 16 : 8;
+    return (unsigned)(o.by_row ? (o.R + 4 * warps - 1) / (4 * warps) : (o.K > 1024 ? o.R : (o.R + warps - 1) / warps));
 }
 template unsigned oz_slice_blocks(const OzOperand<double> &, bool);
 template unsigned oz_slice_blocks(const OzOperand<float> &, bool);
@@ -820,10 +851,10 @@ gbqr_status oz_slice_launch(const Exec &ex, int D, const OzSliceArgs<Src> &args,
     if (D != kD32 && (D != kD64 || std::is_same<Src, float>::value)) return GBQR_EINVAL;
     trace_begin(ex, FAM_OTHER);
     if (D == kD32) {
-        if (tall) oz_slice_kernel<Src, kD32, 1024, 4><<<blocks, 1024, 0, ex.stream>>>(args);
+        if (tall) oz_slice_kernel<Src, kD32, 512, 8><<<blocks, 512, 0, ex.stream>>>(args);
         else oz_slice_kernel<Src, kD32, kThreads, 8><<<blocks, kThreads, 0, ex.stream>>>(args);
     } else if constexpr (std::is_same<Src, double>::value) {
-        if (tall) oz_slice_kernel<Src, kD64, 1024, 4><<<blocks, 1024, 0, ex.stream>>>(args);
+        if (tall) oz_slice_kernel<Src, kD64, 512, 8><<<blocks, 512, 0, ex.stream>>>(args);
         else oz_slice_kernel<Src, kD64, kThreads, 8><<<blocks, kThreads, 0, ex.stream>>>(args);
     }
     return trace_end(ex, FAM_OTHER, 0.0, ((double)sizeof(Src) + 2.0 * D) * elems);
