@@ -986,6 +986,10 @@ static bool oz_plan(const GemmOpT<Real> &op, const OzScratch &sc, int num_sms, O
     }
     const size_t digits = oz_digit_bytes(OzTraits<Real>::D, op.M, op.K, OZ_BM) + oz_digit_bytes(OzTraits<Real>::D, nc, op.K, OZ_BN);
     if (digits > sc.bytes) return false;
+    // a chunk of a masked B starts off B's diagonal: below it a unit lower
+    // trapezoid is one again (oz_gemm), the others are not cut
+    if (nc < op.N && op.maskB != MASK_NONE &&
+        !(op.maskB == MASK_UNIT_LOWER && op.maskA == MASK_NONE && op.K >= op.N + 64)) return false;
     if ((size_t)op.M * nc >= ((size_t)1 << 32) || oz_items((int)op.M, (int)nc, 1) < 0) return false;
     plan->nc = nc;
     plan->split = oz_split<Real>(op.M, nc, op.K, num_sms, (sc.bytes - digits) / 8, false);
@@ -1050,7 +1054,13 @@ gbqr_status oz_gemm(const Exec &ex, const GemmOpT<Real> &op, const OzScratch &sc
         c.N = std::min(pl.nc, op.N - j);
         c.B = op.B + j * op.ldb;
         c.C = op.C + j * op.ldc;
-        TRY_ST(oz_chunk(ex, c, sc, j == 0));
+        const bool below = j > 0 && op.maskB == MASK_UNIT_LOWER;   // the rows above the chunk's diagonal are zero
+        if (below) {
+            c.K = op.K - j;
+            c.A = op.ta ? op.A + j : op.A + j * op.lda;
+            c.B += j;
+        }
+        TRY_ST(oz_chunk(ex, c, sc, j == 0 || below));
     }
     return GBQR_OK;
 }
