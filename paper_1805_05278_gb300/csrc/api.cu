@@ -92,6 +92,8 @@ struct Params {
     bool oz = true;        // scratch for digit-split FP64 products (off: a caller's workspace without room for it)
 };
 
+bool gram_room(const Params &r) { return r.b == kDefaultCutoff && r.leaf_rows == 0 && !r.dmma; }
+
 bool resolve(const gbqr_opts *o, int64_t m, int64_t n, Params *p) {
     Params r;
     r.nb = gbqr_default_panel_nb(m, n);
@@ -114,7 +116,7 @@ bool resolve(const gbqr_opts *o, int64_t m, int64_t n, Params *p) {
     }
     r.nb = std::max<int64_t>(1, r.nb);
     // a caller who sets the TSQR's parameters gets the TSQR
-    r.gram = r.b == kDefaultCutoff && r.leaf_rows == 0 && r.fanout == kDefaultFanout && !r.dmma;
+    r.gram = gram_room(r) && r.fanout == kDefaultFanout;
     *p = r;
     return true;
 }
@@ -148,9 +150,18 @@ Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num
                            std::max(gemm_partial_elems_min(num_sms),
                                     (size_t)std::max<int64_t>(m, 1) * (size_t)std::max<int64_t>(n, 1) / 4));
     L.n_gcount = gemm_counters_max(num_sms);
-    const bool gram = pr.gram && pr.oz && n >= kGramMinW && m >= 4 * kGramMinW;
-    const int w = (int)std::max<int64_t>(1, std::min<int64_t>(gram ? std::max(pr.b, kGramFallbackB) : pr.b, n));
+    // one size for every fan-out, whether its panels are Gram-matrix ones or not
+    const bool gram = gram_room(pr) && pr.oz && n >= kGramMinW && m >= 4 * kGramMinW;
+    const int w = (int)std::max<int64_t>(1, std::min<int64_t>(pr.b, n));
     L.tsqr = tsqr_plan_bound(std::max<int64_t>(m, 1), w, pr.leaf_rows, pr.fanout, num_sms);
+    if (gram) {
+        const TsqrPlan f = tsqr_plan_bound(m, (int)std::min<int64_t>(kGramFallbackB, n), 0, kDefaultFanout, num_sms);
+        L.tsqr.nR = std::max(L.tsqr.nR, f.nR);
+        L.tsqr.nT = std::max(L.tsqr.nT, f.nT);
+        L.tsqr.nY = std::max(L.tsqr.nY, f.nY);
+        L.tsqr.nX = std::max(L.tsqr.nX, f.nX);
+        L.tsqr.ncount = std::max(L.tsqr.ncount, f.ncount);
+    }
     const int64_t nb = std::min<int64_t>(pr.nb, std::max<int64_t>(n, 1));
     // temporaries of the update / T-assembly products and of applying Q
     size_t nM = (size_t)((n + 1) / 2) * (size_t)(n / 2 + 1);
@@ -197,9 +208,9 @@ Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num
         L.n_oz = pr.nsplit > 0 ? oz_gemm_scratch_bytes<double>(kv, nn, kv)
                                : std::max(need(std::min(nn, kOzChunkCols)), std::min(need(nn), kOzMainBytes));
         // a panel: its Gram matrix, V and Y, or the products of its halves
-        const int64_t h = gram ? std::min<int64_t>(nb, kGramMaxW) : std::max<int64_t>((nb + 1) / 2, 1);
-        const size_t panel = gram ? std::max(gram_scratch_bytes<double>(mm, h), oz_gemm_scratch_bytes<double>(mm, h, h))
-                                  : std::max(oz_gemm_scratch_bytes<double>(h, h, mm), oz_gemm_scratch_bytes<double>(mm, h, h));
+        const int64_t h = std::max<int64_t>((nb + 1) / 2, 1), hg = std::min<int64_t>(nb, kGramMaxW);
+        size_t panel = std::max(oz_gemm_scratch_bytes<double>(h, h, mm), oz_gemm_scratch_bytes<double>(mm, h, h));
+        if (gram) panel = std::max({panel, gram_scratch_bytes<double>(mm, hg), oz_gemm_scratch_bytes<double>(mm, hg, hg)});
         if (gram || !pr.lookahead) L.n_oz = std::max(L.n_oz, panel);
         L.oz = take(L.n_oz);
         L.n_oz2 = pr.lookahead && nn > nb ? panel : 0;
@@ -440,10 +451,10 @@ void carve_work(gbqr_ctx *cx, char *base, const Layout &L, const Params &pr, con
     w->gs2.counters = (unsigned *)(base + w->L.gcount2);
     w->gs2.ncounters = w->L.n_gcount;
     w->gs2.oz = {w->L.n_oz2 ? (void *)(base + w->L.oz2) : nullptr, w->L.n_oz2, &cx->dinfo->timeout};
-    w->gram = w->L.n_gram ? (double *)(base + w->L.gram) : nullptr;
-    w->Y = w->L.n_vy ? (double *)(base + w->L.Y) : nullptr;
-    w->vy = w->L.n_vy ? base + w->L.vy : nullptr;
-    w->gram_flag = w->L.n_gram ? (int *)(w->gram + w->L.n_gram) : nullptr;
+    w->gram = pr.gram && w->L.n_gram ? (double *)(base + w->L.gram) : nullptr;
+    w->Y = pr.gram && w->L.n_vy ? (double *)(base + w->L.Y) : nullptr;
+    w->vy = pr.gram && w->L.n_vy ? base + w->L.vy : nullptr;
+    w->gram_flag = w->gram ? (int *)(w->gram + w->L.n_gram) : nullptr;
     w->M1b = (double *)(base + w->L.M1b);
     w->M2b = (double *)(base + w->L.M2b);
     w->tcs.base = w->L.n_tc ? (void *)(base + w->L.tc) : nullptr;
