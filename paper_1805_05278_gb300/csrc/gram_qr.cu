@@ -516,7 +516,8 @@ GramScratch gram_scratch(int D, int64_t m, int64_t w, bool with_y) {
     GramScratch s;
     s.p = std::max(oz_digit_bytes(D, w, m, kOzTileA), oz_digit_bytes(D, m, w, kOzTileA));
     s.xz = oz_digit_bytes(D, w, w, kOzTileB) * (with_y ? 2 : 1);
-    const size_t splits = std::min<size_t>(oz_ktiles(m), 128);
+    // a split has at most 16 K tiles (512 rows), and up to 128 splits fill the GPU
+    const size_t kt = oz_ktiles(m), splits = std::max<size_t>(std::min<size_t>(kt, 128), (kt + 15) / 16);
     s.total = s.p + std::max(s.xz, splits * w * w * 8);
     return s;
 }

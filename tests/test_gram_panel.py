@@ -83,3 +83,14 @@ def test_zero_and_nan_columns(gb, ctx):
     st, info = ctx.sync()
     assert st == gb.GBQR_ENONFINITE and info.nonfinite
     assert not np.isfinite(VR[:, 39]).all()
+
+
+@pytest.mark.parametrize("m,n", [(65537, 16), (70001, 130), (140000, 40)])
+def test_panels_taller_than_the_usual_split(gb, ctx, m, n):
+    """More rows than 128 splits of 512 hold: the Gram matrix's partials have
+    their room (a valid QR, Q applied to the identity's columns by the panels)."""
+    a = workloads.gaussian(m, n, 95)
+    VR, T, nb = _gpu.factor_gpu(ctx, a, gb.GBQR_T_PANEL)
+    Q = _gpu.q_from_panels(VR, T, nb)
+    assert np.linalg.norm(a - Q @ np.triu(VR[:n])) <= 1e-13 * np.linalg.norm(a)
+    assert np.linalg.norm(Q.T @ Q - np.eye(n)) <= 1e-13 * n
