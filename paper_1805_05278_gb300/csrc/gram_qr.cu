@@ -38,7 +38,7 @@
 // per 76 on this part, so diag is bound by its 64 dependent pivots (a
 // reciprocal, a multiply-add and a barrier each) and does nothing else: with
 // the block's inverses formed in it by augmented columns, it took 75 us, the
-// columns' FP64 issue delaying the chain; without them 20 us.  A 32^3 product
+// columns' FP64 issue delaying the chain; without them 33 us.  A 32^3 product
 // on one SM would take 9 us, so row and trail spread every block over 8 CTAs;
 // a triangular solve with a unit diagonal is 32 shuffles and multiply-adds,
 // no longer than a product with the inverse.
@@ -786,7 +786,7 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
         const int64_t w = std::min<int64_t>(width[i], n[i]), nc = n[i] - w;
         const size_t splits = oz_ktiles(m[i]);
         size_t s = work_bytes + std::max(oz_digit_bytes(D, w, m[i], kOzTileA), oz_digit_bytes(D, m[i], w, kOzTileA)) +
-                   2 * oz_digit_bytes(D, w, w, kOzTileB) + std::min<size_t>(splits, 40) * w * w * 8;
+                   2 * oz_digit_bytes(D, w, w, kOzTileB) + std::max(std::min<size_t>(splits, 40), splits / 16 + 1) * w * w * 8;
         if (nc > 0)
             s += (size_t)m[i] * w * sizeof(Real) + oz_digit_bytes(D, m[i], w, kOzTileA) + oz_digit_bytes(D, w, m[i], kOzTileA) +
                  oz_digit_bytes(D, nc, m[i], kOzTileB) + oz_digit_bytes(D, nc, w, kOzTileB) + (size_t)w * nc * sizeof(Real) +
@@ -850,7 +850,7 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                 // a full GPU of matrices needs no fine splits: 1024 k an item (FP64: 512)
                 pg[q].kt_per = std::max(1, std::min(pg[q].KT, sizeof(Real) == 8 ? 16 : 32));
                 if (na < num_sms) pg[q].kt_per = std::max(1, std::min(pg[q].kt_per, (pg[q].KT * na + num_sms - 1) / num_sms));
-                pg[q].kt_per = std::max(pg[q].kt_per, (pg[q].KT + 39) / 40);
+                pg[q].kt_per = std::max(pg[q].kt_per, std::min((pg[q].KT + 39) / 40, oz_max_ktiles<Real>()));
                 pg[q].S = (pg[q].KT + pg[q].kt_per - 1) / pg[q].kt_per;
                 pg[q].ldc = GLD;
                 pg[q].first = items;
@@ -1007,7 +1007,7 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                     p.kt_per = std::max(1, std::min(p.KT, 16));
                     if ((int)trailing.size() < num_sms)
                         p.kt_per = std::max(1, std::min(p.kt_per, (int)((p.KT * trailing.size() + num_sms - 1) / num_sms)));
-                    p.kt_per = std::max(p.kt_per, (p.KT + 39) / 40);
+                    p.kt_per = std::max(p.kt_per, std::min((p.KT + 39) / 40, oz_max_ktiles<Real>()));
                     p.S = (p.KT + p.kt_per - 1) / p.kt_per;
                     p.ldc = W(i);
                     p.first = items;

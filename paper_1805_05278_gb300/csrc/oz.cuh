@@ -58,6 +58,9 @@ struct OzMmaArgs {
 
 int oz_ktiles(int64_t K);
 int oz_items(int M, int N, int S);
+// K tiles of one item: what its 64-bit integer sums hold for any digits
+// (leading products of 2^14, FP64 in units of 2^-40, FP32 of 2^-24).
+template <class Real> constexpr int oz_max_ktiles() { return sizeof(Real) == 8 ? 16 : 64; }
 constexpr int kOzDigits64 = 7, kOzDigits32 = 4;   // digits of an operand of FP64 and FP32 products
 template <class Real> constexpr int oz_digits() { return sizeof(Real) == 8 ? kOzDigits64 : kOzDigits32; }
 // bytes of an operand's digits and exponents, 256-aligned

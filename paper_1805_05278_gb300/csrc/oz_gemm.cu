@@ -96,6 +96,7 @@ template <class Real> constexpr int oz_products() {
         for (int j = 1; j <= OzTraits<Real>::D; ++j) n += i + j <= OzTraits<Real>::TOP;
     return n;
 }
+static_assert(OzTraits<double>::MAX_KT == oz_max_ktiles<double>() && OzTraits<float>::MAX_KT == oz_max_ktiles<float>(), "item sizes");
 static_assert(kD64 == kOzDigits64 && kD32 == kOzDigits32, "digits");
 static_assert(oz_products<double>() == 34 && oz_products<float>() == 10, "digit products");
 
