@@ -14,7 +14,7 @@ path); the reported value is the flops of all ranks over the slowest rank's
 time.
 
 The timed region runs with launch tracing off.  The roofline of the dominant
-kernel (the FP64 GEMM family) comes from a separate traced pass of the same
+kernel family (the digit products, or the FP64 FMA products) comes from a separate traced pass of the same
 factorization with the look-ahead off, so that every launch runs alone and
 its event-bracketed duration is its own (with look-ahead the side stream's
 panel shares the SMs and stretches the GEMMs it overlaps).
@@ -64,6 +64,17 @@ DGEMM_TRAFFIC_RATIO = {
     ("graded_4096x4096", 128, 16, "dfma"): 0.780,
 }
 DGEMM_TRAFFIC_SOURCE = "ncu: all dgemm launches of graded 4096x4096 (nb 128, b 16, DFMA), dram read+write / algorithmic"
+
+
+def bf16_peak():
+    """The measured cuBLAS BF16 rate of this machine type, TFLOP/s."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["bf16_tflops"]), "measured: cuBLAS bf16 GEMM, burst"
+    except (OSError, KeyError, ValueError, TypeError):
+        return 1900.0, "fallback: an earlier cuBLAS bf16 measurement"
+
+
 METRIC = "QR TFLOP/s (2mn^2-2n^3/3) vs peak; LS solves/s, p99 ms: mixed vs FP64"
 
 
@@ -255,8 +266,7 @@ def _time_batch_graph(gb, ctx, stream, buf, pristine, As, Ts, o, steps):
 def measure_batched(gb, dev, args):
     """The batched tall-skinny workload: args.batched matrices, m log-uniform
     in [256, 16384], n uniform in [16, 256], factored by gbqr_factor_batched
-    (FP64: one persistent kernel launch for the whole batch, captured in a
-    graph with its table upload), then the same matrices rounded to FP32 by
+    (captured in a graph with its table upload), then the same matrices rounded to FP32 by
     gbqr_factor_batched_f32.  Each timed step restores the inputs with one
     device copy (untimed), then launches the graph."""
     import torch
@@ -275,14 +285,22 @@ def measure_batched(gb, dev, args):
             o, tune_ms = ctx.autotune_batched(shapes, gb.GBQR_FP64, args.batched_autotune_ms)
         tuned = gb.opts_dict(o)
     ms = _time_batch_graph(gb, ctx, stream, buf, pristine, As, Ts, o, args.batched_steps)
+
+    def kernel_launches(As_, Ts_, o_):
+        before = ctx.launch_count()
+        ctx.factor_batched(As_, Ts_, o_)
+        return ctx.launch_count() - before
+
+    launches = kernel_launches(As, Ts, o)
     st, _ = ctx.sync()
     out = {"workload": f"{len(shapes)} matrices, m log-uniform [256, 16384], n uniform [16, 256], "
                        f"iid N(0,1), seed {workloads.BATCHED_SEED}",
            "total_flops": flops, "ms_per_batch": ms, "tflops": flops / (ms * 1e-3) / 1e12,
            "frac_of_fp64_peak": flops / (ms * 1e-3) / 1e12 / FP64_PEAK_TFLOPS,
            "matrices_per_s": len(shapes) / (ms * 1e-3), "graph_launches_per_batch": 1, "status": int(st),
-           "engine": "one persistent kernel launch (panel and update tasks, list-scheduled), captured in a graph",
-           "kernel_launches_per_batch": 1, "cutoff_b": o.cutoff_b or 16,
+           "engine": "grouped Gram-matrix panels and digit products in lockstep; one persistent kernel launch "
+                     "(panel and update tasks, list-scheduled) for the other matrices; captured in a graph",
+           "kernel_launches_per_batch": launches, "cutoff_b": o.cutoff_b or 16,
            "tuned": tuned, "tuned_ms": tune_ms, "dtype": "f64"}
     del As, Ts, buf, pristine
     # FP32: the same matrices rounded to float32, FP32 arithmetic throughout
@@ -293,10 +311,11 @@ def measure_batched(gb, dev, args):
     Ts32 = [torch.empty((n, min(128, n)), dtype=torch.float32, device=f"cuda:{dev}").T for (m, n) in shapes]
     o32 = gb.opts(cutoff_b=args.batched_cutoff32, batch_streams=args.batched_streams)
     ms32 = _time_batch_graph(gb, ctx, stream, buf32, pristine32, As32, Ts32, o32, args.batched_steps)
+    launches32 = kernel_launches(As32, Ts32, o32)
     st32, _ = ctx.sync()
     out["fp32"] = {"ms_per_batch": ms32, "tflops": flops / (ms32 * 1e-3) / 1e12,
                    "matrices_per_s": len(shapes) / (ms32 * 1e-3), "status": int(st32), "dtype": "f32",
-                   "cutoff_b": args.batched_cutoff32 or 16, "kernel_launches_per_batch": 1}
+                   "cutoff_b": args.batched_cutoff32 or 16, "kernel_launches_per_batch": launches32}
     ctx.close()
     return out
 
@@ -729,31 +748,40 @@ def run_gbqr(args):
     batched = measure_batched(gb, dev, args) if (args.batched > 0 and rank == 0) else None
     serving = measure_serving(gb, dev, args) if (args.serving > 0 and rank == 0) else None
 
-    gemm = trace.get("gemm", {})
+    # the dominant product family: the digit products on the tensor cores
+    # (their BF16 flops, 34 per FP64 multiply-add), or the FMA kernels' own
+    digit = trace.get("tc_gemm", {}).get("ms", 0.0) >= trace.get("gemm", {}).get("ms", 0.0)
+    gemm = trace.get("tc_gemm" if digit else "gemm", {})
     achieved = gemm["flops"] / (gemm["ms"] * 1e-3) / 1e12 if gemm.get("ms") else None
     share = (gemm.get("ms", 0.0) / serial_ms) if serial_ms else None
     if share is not None and share > 1.0:
         raise RuntimeError(f"GEMM family time exceeds the step in the serial pass (share {share:.3f})")
     alg_bytes = (gemm["bytes"] / gemm["launches"]) if gemm.get("launches") else None
-    ratio = DGEMM_TRAFFIC_RATIO.get(
+    ratio = None if digit else DGEMM_TRAFFIC_RATIO.get(
         (w.name, nb if layout == gb.GBQR_T_PANEL else 0, o.cutoff_b or 16, "dmma" if o.fp64_gemm == gb.GBQR_GEMM_DMMA else "dfma"))
+    peak, peak_source = bf16_peak() if digit else (
+        FP64_PEAK_TFLOPS, "derived: 152 SMs x 4 FP64 flop/clk x 2.070 GHz (nominal 1.25 TFLOP/s FP64); "
+                          "measured DFMA probe 1.06, DMMA probe 1.10, largest update launch 1.22 TFLOP/s")
     roofline = {
-        "bound": "alu", "kernel": "dgemm_kernel (update / T-assembly products)",
-        "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-        "frac": (achieved / FP64_PEAK_TFLOPS) if achieved else None,
-        "peak_source": "derived: 152 SMs x 4 FP64 flop/clk x 2.070 GHz (nominal 1.25 TFLOP/s FP64); "
-                       "measured DFMA probe 1.06, DMMA probe 1.10, largest update launch 1.22 TFLOP/s",
-        "how": f"algorithmic flops / summed CUDA-event durations of every GEMM launch in {args.roofline_steps} "
+        "bound": "tensor" if digit else "alu",
+        "kernel": "oz_mma_kernel (digit products of the update, Gram-matrix and panel products)" if digit
+                  else "dgemm_kernel (update / T-assembly products)",
+        "achieved": achieved, "peak": peak, "unit": "TFLOP/s (BF16)" if digit else "TFLOP/s",
+        "frac": (achieved / peak) if achieved else None,
+        "peak_source": peak_source,
+        "how": f"{'BF16 flops of the digit products' if digit else 'algorithmic flops'} / summed CUDA-event durations "
+               f"of every launch of the family in {args.roofline_steps} "
                f"traced factorizations with the look-ahead off (launches run alone)",
         "traffic": (ratio * alg_bytes) if (ratio and alg_bytes) else None,
         "traffic_unit": "bytes per launch (dram read + write): ncu ratio to algorithmic bytes x this pass's "
                         "algorithmic bytes per launch",
         "traffic_ratio_ncu": ratio,
         "traffic_source": DGEMM_TRAFFIC_SOURCE if ratio else None,
-        "algorithmic_bytes_per_launch": alg_bytes,
+        "algorithmic_bytes_per_launch": alg_bytes if not digit else None,
         "launches": gemm.get("launches"), "share_of_step": share,
         "serial_ms_per_step": serial_ms / max(1, args.roofline_steps),
         "step_frac": value / world / FP64_PEAK_TFLOPS,
+        "step_frac_of": "the FP64 pipe's derived peak (above 1: the products run as exact BF16 digit products)",
     }
     fams = {k: {"launches": v["launches"] / max(1, args.roofline_steps),
                 "ms_per_step": v["ms"] / max(1, args.roofline_steps),

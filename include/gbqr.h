@@ -186,7 +186,11 @@ GBQR_API gbqr_status gbqr_sync(gbqr_ctx *ctx, gbqr_info *info);
  * (Algorithm 2).  Base case (n <= b): TSQR with leaf QR per CTA, a fan-out-k
  * tree of structured R merges, the downsweep that forms the leading columns
  * W of Q, and the Householder reconstruction X + S = LU, T = U S L^{-T},
- * R = -S R_tree, V = W U^{-1} (Appendix C).
+ * R = -S R_tree, V = W U^{-1} (Appendix C).  With the default cutoff, leaf
+ * height, fan-out and GEMM engine, well-conditioned panels of 16 to 128
+ * columns and at least four rows a column get the same (V, T, R) from their
+ * Gram matrix (Cholesky, then that reconstruction); a check on the device
+ * hands the others to the TSQR.
  * A and T may instead both be HOST pointers (pageable or pinned): the call
  * then stages them through device workspace, copies the results back and
  * returns after the stream has synchronised.  With page-locked buffers and
@@ -205,8 +209,9 @@ GBQR_API gbqr_status gbqr_factor(gbqr_ctx *ctx, int64_t m, int64_t n, double *A,
                         double *T, int64_t ldt, int t_layout, const gbqr_opts *opts);
 
 /* gbqr_factor in FP32: A (m x n, m >= n) and T are float DEVICE arrays and
- * every step computes in FP32 with the float instantiations of the same
- * kernels (TSQR, tiled GEMM); same layouts, options and look-ahead.
+ * every step computes in FP32 or better with the float instantiations of the
+ * same kernels (TSQR, tiled GEMM, digit products; a panel's Gram matrix is
+ * decomposed in FP64); same layouts, options and look-ahead.
  * opts->update_prec must be GBQR_FP64 / 0 (no tensor-core updates); the
  * autotuner's cache is not used.  Errors: EINVAL (m < n, lda, ldt, opts),
  * EUNSUPPORTED (host pointers), ENOMEM, ECUDA. */
@@ -222,13 +227,20 @@ GBQR_API int64_t gbqr_default_panel_nb(int64_t m, int64_t n);
  * for each matrix): A[i] (m[i] x n[i], lda[i], device) is factored in place
  * exactly as gbqr_factor does with GBQR_T_PANEL, T[i] (ldt[i] x n[i]) receives
  * its panel kernels.  m, n, A, lda, T, ldt are HOST arrays of count entries.
- * The matrices are spread over opts->batch_streams (default 128) internal streams (largest first, to
- * the least loaded stream), forked from and joined back to the context's
- * stream by events, so a capture of the context's stream (gbqr_graph_begin /
- * gbqr_graph_end) turns the whole batch into one graph launch.  Each stream
- * has its own workspace slice (gbqr_batched_workspace_bytes in total); the
- * first call creates the streams and grows library-owned workspace, so make
- * it before any capture.  opts apply to every matrix (panel_nb per matrix is
+ * By default (cutoff 16, panel_nb at most the cutoff) matrices of 16 columns
+ * or more with about four rows a column are factored group by group from
+ * their panels' Gram matrices, in lockstep launches over lists of panels;
+ * the others, and those that the condition check hands back, by one launch
+ * of a persistent kernel.  A caller's workspace without room for the groups
+ * gets the persistent kernel alone.  With panel_nb above the cutoff, a cutoff
+ * above 32 or a mixed update_prec, the matrices are spread over
+ * opts->batch_streams (default 128) internal streams (largest first, to
+ * the least loaded stream), each with its own workspace slice.  Internal
+ * streams are forked from and joined back to the context's stream by events,
+ * so a capture of the context's stream (gbqr_graph_begin / gbqr_graph_end)
+ * turns the whole batch into one graph launch (gbqr_batched_workspace_bytes
+ * in total).  The first call plans the batch, creates the streams and grows
+ * library-owned workspace, so make it before any capture.  opts apply to every matrix (panel_nb per matrix is
  * min(opts->panel_nb or 128, n[i]); the cutoff b defaults to 16 here).
  * Errors: EINVAL, ENOMEM, ECUDA. */
 GBQR_API gbqr_status gbqr_factor_batched(gbqr_ctx *ctx, int count, const int64_t *m, const int64_t *n,

@@ -1,5 +1,9 @@
-// Persistent batched QR: thousands of independent, uneven QR factorizations
-// in ONE kernel launch (the 1D-CAQR-EG instance of Section 6 for each
+// Persistent batched QR: independent, uneven QR factorizations in ONE kernel
+// launch.  In a default batch it takes the matrices that the grouped path
+// (gram_qr.cu) does not: those of fewer than 16 columns or less than about
+// four rows a column, beside the groups on a few SMs (bound by their chains
+// of steps), and, after them, what their condition check handed back.  (The
+// 1D-CAQR-EG instance of Section 6 for each
 // matrix: a right-looking top level over panels of width b, Section 8.4,
 // each panel factored by TSQR, Section 5 / Appendix C).
 //

@@ -49,8 +49,10 @@ struct Record {
 };
 
 // GBQR_PREC_AUTO: the tensor-core updates only pay off where the update
-// GEMMs dominate the solve.  Measured single-solve speed-ups of the mixed
-// path over FP64 (graded columns, kappa ~ 1e4, two GMRES steps each):
+// GEMMs dominate the solve.  The line is where it was measured with FP64
+// products on FMA units and TSQR panels (with digit products the two paths
+// are within 10 % of each other on large problems, and FP64 is the faster on
+// most).  Single-solve speed-ups of the mixed path over FP64 then (graded columns, kappa ~ 1e4, two GMRES steps each):
 // 3.19x at 65536 x 1024, 1.96x at 65536 x 512, 1.88x at 16384 x 1024,
 // 1.36x at 16384 x 512, 1.32x at 65536 x 256, 1.12x at 8192 x 512, 1.08x
 // at 16384 x 256, 1.01x at 2048 x 1024 (all m n^2 >= 1e9); slower below
