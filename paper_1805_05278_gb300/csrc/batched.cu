@@ -1,11 +1,11 @@
 // Persistent batched QR: independent, uneven QR factorizations in ONE kernel
-// launch.  In a default batch it takes the matrices that the grouped path
+// launch (the 1D-CAQR-EG instance of Section 6 for each matrix: a
+// right-looking top level over panels of width b, Section 8.4, each panel
+// factored by TSQR, Section 5 / Appendix C).  FP32 batches are all its own.
+// In a default FP64 batch it takes the matrices that the grouped path
 // (gram_qr.cu) does not: those of fewer than 16 columns or less than about
 // four rows a column, beside the groups on a few SMs (bound by their chains
-// of steps), and, after them, what their condition check handed back.  (The
-// 1D-CAQR-EG instance of Section 6 for each
-// matrix: a right-looking top level over panels of width b, Section 8.4,
-// each panel factored by TSQR, Section 5 / Appendix C).
+// of steps), and, after them, what their condition check handed back.
 //
 // Work decomposition.  Matrix i (m_i x n_i) is cut into column blocks of
 // width b.  Its tasks are
@@ -661,7 +661,7 @@ struct BatchPlan {
     std::vector<int> state0;     // each matrix's first column-block counter
     std::vector<unsigned char> stage;   // pageable staging of the table for uncaptured calls
     double est_ms = 0.0;         // the list schedule's estimated makespan
-    GroupPlan *group = nullptr;  // the grouped part (b = 16), its workspace behind `total`
+    GroupPlan *group = nullptr;  // the grouped part (FP64, b = 16), its workspace behind `total`
 };
 
 void batch_plan_free(BatchPlan *pl) {
@@ -838,7 +838,11 @@ gbqr_status batched_plan(BatchPlan **cache, int device, int num_sms, int count, 
     pl->smem = smem;
     pl->grid = per_sm * num_sms;
     if (!build_plan(pl, count, m, n, b, pl->grid, sizeof(Real), sizeof(BMat<Real>))) return GBQR_ENOMEM;
-    if (b == 16) pl->group = group_plan_build<Real>(count, m, n, lda, ldt, num_sms, pl->total);
+    // FP64 only.  The persistent kernel's FP32 pivots carry their own rounding,
+    // and where one is zero to that rounding it decides the reflection's sign,
+    // hence a row of R and a column of V: from a Gram matrix the signs of such
+    // columns, and with them the results, would be others.
+    if (b == 16 && sizeof(Real) == 8) pl->group = group_plan_build(count, m, n, lda, ldt, num_sms, pl->total);
     pl->nalone = pl->ntasks;
     if (pl->group) {
         const int *width = group_widths(pl->group);
@@ -924,7 +928,7 @@ gbqr_status batched_enqueue(const Exec &ex, BatchPlan *pl, Real *const *A, Real 
         TRY_ST(launch(q, std::min(pl->grid, kBesideCtas), side.stream));
         if (cudaEventRecord(side.join, side.stream) != cudaSuccess) return GBQR_ECUDA;
     }
-    TRY_ST(group_enqueue<Real>(ex, pl->group, ws, ws, (int)sizeof(BMat<Real>), pl->count, timeout_flag));
+    TRY_ST(group_enqueue(ex, pl->group, ws, ws, (int)sizeof(BMat<Real>), pl->count, timeout_flag));
     if (beside && cudaStreamWaitEvent(ex.stream, side.join, 0) != cudaSuccess) return GBQR_ECUDA;
     p.status = reinterpret_cast<const int *>(ws + group_status_offset(pl->group));
     p.tasks += pl->nalone;

@@ -187,11 +187,10 @@ template <class Real>
 gbqr_status batched_plan(BatchPlan **cache, int device, int num_sms, int count, const int64_t *m,
                          const int64_t *n, const int64_t *lda, const int64_t *ldt, int b, bool may_build,
                          BatchPlan **out);
-// Grouped part of a batch (gram_qr.cu): the well-shaped matrices' panels from
+// Grouped part of an FP64 batch (gram_qr.cu): the well-shaped matrices' panels from
 // their Gram matrices, all matrices of a group in lockstep; the persistent
 // kernel then does the other matrices, and what stopped as ill-conditioned.
 struct GroupPlan;
-template <class Real>
 GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const int64_t *lda, const int64_t *ldt,
                             int num_sms, size_t ws_off);
 void group_plan_free(GroupPlan *g);
@@ -199,7 +198,6 @@ size_t group_plan_bytes(const GroupPlan *g);           // workspace, from its st
 const int *group_widths(const GroupPlan *g);           // per matrix, 0 = not grouped
 size_t group_status_offset(const GroupPlan *g);
 gbqr_status group_plan_upload(GroupPlan *g);
-template <class Real>
 gbqr_status group_enqueue(const Exec &ex, const GroupPlan *g, char *ws, const void *mats, int stride, int count, int *err);
 // The plan's workspace without the grouped part, and the upload of that part
 // (outside captures).

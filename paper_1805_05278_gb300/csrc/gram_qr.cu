@@ -642,7 +642,7 @@ constexpr int kGroupPanels = 4;
 enum RelocBase { RB_WS = 0, RB_A = 1, RB_T = 2 };
 struct Reloc { uint64_t off; uint32_t word; int mat; int base; int pad; };
 
-enum StepKind { ST_SLICE, ST_SLICE64, ST_MMA, ST_REDUCE, ST_REQUANT, ST_DIAG, ST_ROW, ST_TRAIL, ST_T };
+enum StepKind { ST_SLICE, ST_MMA, ST_REDUCE, ST_REQUANT, ST_DIAG, ST_ROW, ST_TRAIL, ST_T };
 struct GroupStep {
     StepKind kind;
     size_t list = 0;          // the list's place in the blob
@@ -654,7 +654,6 @@ struct GroupStep {
     double elems = 0.0;
 };
 
-template <class P>
 __global__ void __launch_bounds__(256) reloc_kernel(const Reloc *r, int n, uint64_t *blob, char *ws, const char *mats,
                                                     int stride) {
     const int i = blockIdx.x * 256 + threadIdx.x;
@@ -663,7 +662,7 @@ __global__ void __launch_bounds__(256) reloc_kernel(const Reloc *r, int n, uint6
     uint64_t base = (uint64_t)ws;
     if (x.base != RB_WS) {
         // the matrix table starts with its pointers A and T
-        const P *p = reinterpret_cast<const P *>(mats + (size_t)x.mat * stride);
+        double *const *p = reinterpret_cast<double *const *>(mats + (size_t)x.mat * stride);
         base = (uint64_t)p[x.base == RB_A ? 0 : 1];
     }
     blob[x.word] = base + x.off;
@@ -672,13 +671,12 @@ __global__ void __launch_bounds__(256) reloc_kernel(const Reloc *r, int n, uint6
 }  // namespace
 
 struct GroupPlan {
-    int D = 7;
     size_t blob_off = 0, status_off = 0, total = 0;      // workspace layout, from its start
     std::vector<uint8_t> blob;
     std::vector<Reloc> relocs;
     std::vector<GroupStep> steps;
     std::vector<int> width;                              // per matrix: its panels' width, 0 = not grouped
-    uint8_t *d_blob = nullptr;                           // device copies (batch_group_upload)
+    uint8_t *d_blob = nullptr;                           // device copies (group_plan_upload)
     Reloc *d_relocs = nullptr;
 };
 
@@ -710,11 +708,10 @@ int group_width(int64_t m, int64_t n) {
     return 0;
 }
 
-template <class Real>
 struct GroupBuilder {
     GroupPlan *g;
     size_t arena = 0, peak = 0;
-    int D = oz_digits<Real>();
+    static constexpr int D = kOzDigits64;
 
     static size_t al(size_t x) { return (x + 255) / 256 * 256; }
     size_t take(size_t bytes) {
@@ -741,8 +738,7 @@ struct GroupBuilder {
         rel(at, entry, field, RB_WS, 0, flag);
         g->relocs.back().pad = 1;                  // a place outside the arena
     }
-    template <class Src>
-    void places(size_t at, const OzOperand<Src> &o, int base, int mat, uint64_t x, size_t digits, int64_t R, int64_t K,
+    void places(size_t at, const OzOperand<double> &o, int base, int mat, uint64_t x, size_t digits, int64_t R, int64_t K,
                 size_t flag, size_t kexp) {
         rel(at, &o, &o.X, base, mat, x);
         rel(at, &o, &o.dst, RB_WS, 0, digits);
@@ -760,7 +756,6 @@ struct PanelPlaces { size_t work, p, x, z, part, y, vd, yd, c, wd, wf; };
 
 }  // namespace
 
-template <class Real>
 GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const int64_t *lda, const int64_t *ldt,
                             int num_sms, size_t ws_off) {
     std::vector<int> mats;
@@ -772,11 +767,10 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
     if (mats.empty()) return nullptr;
     GroupPlan *g = new (std::nothrow) GroupPlan();
     if (!g) return nullptr;
-    constexpr int D = oz_digits<Real>();
-    g->D = D;
+    constexpr int D = kOzDigits64;
     g->width = width;
-    GroupBuilder<Real> b{g};
-    g->status_off = GroupBuilder<Real>::al(ws_off);
+    GroupBuilder b{g};
+    g->status_off = GroupBuilder::al(ws_off);
     // the arena's place depends on the blob's size: offsets are relative to
     // the arena while building, and shifted at the end
     auto flag_of = [&](int i) { return g->status_off + (size_t)i * 4; };
@@ -788,8 +782,8 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
         size_t s = work_bytes + std::max(oz_digit_bytes(D, w, m[i], kOzTileA), oz_digit_bytes(D, m[i], w, kOzTileA)) +
                    2 * oz_digit_bytes(D, w, w, kOzTileB) + std::max(std::min<size_t>(splits, 40), splits / 16 + 1) * w * w * 8;
         if (nc > 0)
-            s += (size_t)m[i] * w * sizeof(Real) + oz_digit_bytes(D, m[i], w, kOzTileA) + oz_digit_bytes(D, w, m[i], kOzTileA) +
-                 oz_digit_bytes(D, nc, m[i], kOzTileB) + oz_digit_bytes(D, nc, w, kOzTileB) + (size_t)w * nc * sizeof(Real) +
+            s += (size_t)m[i] * w * 8 + oz_digit_bytes(D, m[i], w, kOzTileA) + oz_digit_bytes(D, w, m[i], kOzTileA) +
+                 oz_digit_bytes(D, nc, m[i], kOzTileB) + oz_digit_bytes(D, nc, w, kOzTileB) + (size_t)w * nc * 8 +
                  (splits / 16 + 1) * w * nc * 8;
         return s + 16 * 256;
     };
@@ -806,16 +800,15 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                 if ((int64_t)width[mats[q]] * pn < n[mats[q]]) act.push_back(mats[q]);
             const int na = (int)act.size();
             std::vector<PanelPlaces> pl(na);
-            std::vector<OzOperand<Real>> sp(na), sa, sv;
-            std::vector<OzOperand<double>> sx;
-            std::vector<OzProblem<Real>> pg(na), pv, p1, p2;
-            std::vector<GramArgs<Real>> ga(na);
+            std::vector<OzOperand<double>> sp(na), sa, sv, sx;
+            std::vector<OzProblem<double>> pg(na), pv, p1, p2;
+            std::vector<GramArgs<double>> ga(na);
             std::vector<int> trailing;
             auto W = [&](int i) { return std::min<int64_t>(width[i], n[i] - width[i] * pn); };
             auto J = [&](int i) { return (int64_t)width[i] * pn; };
             auto M = [&](int i) { return m[i] - J(i); };
             auto NC = [&](int i) { return n[i] - J(i) - W(i); };
-            auto Aoff = [&](int i, int64_t r, int64_t c) { return (uint64_t)((r + c * lda[i]) * (int64_t)sizeof(Real)); };
+            auto Aoff = [&](int i, int64_t r, int64_t c) { return (uint64_t)((r + c * lda[i]) * 8); };
             for (int q = 0; q < na; ++q) {
                 const int i = act[q];
                 PanelPlaces &s = pl[q];
@@ -825,12 +818,12 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                 s.z = b.take(oz_digit_bytes(D, W(i), W(i), kOzTileB));
                 if (NC(i) > 0) {
                     trailing.push_back(q);
-                    s.y = b.take((size_t)M(i) * W(i) * sizeof(Real));
+                    s.y = b.take((size_t)M(i) * W(i) * 8);
                     s.vd = b.take(oz_digit_bytes(D, M(i), W(i), kOzTileA));
                     s.yd = b.take(oz_digit_bytes(D, W(i), M(i), kOzTileA));
                     s.c = b.take(oz_digit_bytes(D, NC(i), M(i), kOzTileB));
                     s.wd = b.take(oz_digit_bytes(D, NC(i), W(i), kOzTileB));
-                    s.wf = b.take((size_t)W(i) * NC(i) * sizeof(Real));
+                    s.wf = b.take((size_t)W(i) * NC(i) * 8);
                 }
             }
             // ---- digits of P, G = P^T P
@@ -842,15 +835,15 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
             for (int i : act) tall = tall || M(i) > 8192;
             for (int q = 0; q < na; ++q) {
                 const int i = act[q];
-                sp[q] = oz_operand(D, (const Real *)nullptr, lda[i], W(i), M(i), false, MASK_NONE, kOzTileA, nullptr);
+                sp[q] = oz_operand(D, (const double *)nullptr, lda[i], W(i), M(i), false, MASK_NONE, kOzTileA, nullptr);
                 sp[q].first = blocks;
                 blocks += oz_slice_blocks(sp[q], tall);
                 elems += (double)W(i) * M(i);
-                pg[q] = oz_problem<Real>(sp[q], sp[q]);
-                // a full GPU of matrices needs no fine splits: 1024 k an item (FP64: 512)
-                pg[q].kt_per = std::max(1, std::min(pg[q].KT, sizeof(Real) == 8 ? 16 : 32));
+                pg[q] = oz_problem<double>(sp[q], sp[q]);
+                // a full GPU of matrices needs no fine splits: 512 k an item
+                pg[q].kt_per = std::max(1, std::min(pg[q].KT, 16));
                 if (na < num_sms) pg[q].kt_per = std::max(1, std::min(pg[q].kt_per, (pg[q].KT * na + num_sms - 1) / num_sms));
-                pg[q].kt_per = std::max(pg[q].kt_per, std::min((pg[q].KT + 39) / 40, oz_max_ktiles<Real>()));
+                pg[q].kt_per = std::max(pg[q].kt_per, std::min((pg[q].KT + 39) / 40, oz_max_ktiles<double>()));
                 pg[q].S = (pg[q].KT + pg[q].kt_per - 1) / pg[q].kt_per;
                 pg[q].ldc = GLD;
                 pg[q].first = items;
@@ -858,8 +851,8 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                 largest = std::max(largest, (size_t)W(i) * W(i));
                 prods += (double)W(i) * W(i) * M(i);
                 pl[q].part = b.take((size_t)pg[q].S * W(i) * W(i) * 8);
-                GramArgs<Real> &p = ga[q];
-                p = GramArgs<Real>{};
+                GramArgs<double> &p = ga[q];
+                p = GramArgs<double>{};
                 p.lda = lda[i]; p.ldt = ldt[i]; p.ldy = M(i);
                 p.w = (int)W(i); p.nblk = (int)((W(i) + GB - 1) / GB);
                 p.raise = 1 + (int)pn; p.keep = 1; p.tb = kBatchTb;
@@ -876,7 +869,7 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
             for (int q = 0; q < na; ++q) {
                 const int i = act[q];
                 const size_t e = L + q * sizeof(pg[0]);
-                const OzProblem<Real> &p = pg[q];
+                const OzProblem<double> &p = pg[q];
                 b.rel(e, &p, &p.a, RB_WS, 0, pl[q].p);
                 b.rel(e, &p, &p.b, RB_WS, 0, pl[q].p);
                 b.rel(e, &p, &p.ea, RB_WS, 0, b.exps_of(pl[q].p, W(i), M(i), kOzTileA));
@@ -884,20 +877,20 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                 b.rel(e, &p, &p.partial, RB_WS, 0, pl[q].part);
                 b.rel_flag(e, &p, &p.skip, flag_of(i));
                 // the panel's arrays: carved from a null base, so that the fields hold their offsets
-                GramArgs<Real> c = ga[q];
+                GramArgs<double> c = ga[q];
                 gram_carve(c, (double *)nullptr);
                 b.rel(e, &p, &p.Cd, RB_WS, 0, pl[q].work + (size_t)(char *)c.G);
                 const size_t ge = gram_list + q * sizeof(ga[0]);
-                const GramArgs<Real> &a = ga[q];
-                double *GramArgs<Real>::*const f[] = {&GramArgs<Real>::G, &GramArgs<Real>::R, &GramArgs<Real>::RI, &GramArgs<Real>::A1,
-                    &GramArgs<Real>::L, &GramArgs<Real>::U, &GramArgs<Real>::LI, &GramArgs<Real>::X, &GramArgs<Real>::YX, &GramArgs<Real>::YR,
-                    &GramArgs<Real>::YL, &GramArgs<Real>::B1, &GramArgs<Real>::Z, &GramArgs<Real>::sgn, &GramArgs<Real>::gd,
-                    &GramArgs<Real>::M, &GramArgs<Real>::sc};
+                const GramArgs<double> &a = ga[q];
+                double *GramArgs<double>::*const f[] = {&GramArgs<double>::G, &GramArgs<double>::R, &GramArgs<double>::RI, &GramArgs<double>::A1,
+                    &GramArgs<double>::L, &GramArgs<double>::U, &GramArgs<double>::LI, &GramArgs<double>::X, &GramArgs<double>::YX, &GramArgs<double>::YR,
+                    &GramArgs<double>::YL, &GramArgs<double>::B1, &GramArgs<double>::Z, &GramArgs<double>::sgn, &GramArgs<double>::gd,
+                    &GramArgs<double>::M, &GramArgs<double>::sc};
                 for (auto fp : f) b.rel(ge, &a, &(a.*fp), RB_WS, 0, pl[q].work + (size_t)(char *)(c.*fp));
                 b.rel(ge, &a, &a.kexp, RB_WS, 0, pl[q].work + (size_t)(char *)c.kexp);
                 b.rel_flag(ge, &a, &a.flag, flag_of(i));
                 b.rel(ge, &a, &a.A, RB_A, i, Aoff(i, J(i), J(i)));
-                b.rel(ge, &a, &a.Tout, RB_T, i, (uint64_t)(J(i) * ldt[i] * (int64_t)sizeof(Real)));
+                b.rel(ge, &a, &a.Tout, RB_T, i, (uint64_t)(J(i) * ldt[i] * 8));
                 if (NC(i) > 0) b.rel(ge, &a, &a.Y, RB_WS, 0, pl[q].y);
             }
             g->steps.push_back({ST_MMA, L, na, items, 0, 1, false, prods});
@@ -929,7 +922,7 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
             for (int q = 0; q < na; ++q) {
                 const int i = act[q];
                 if (M(i) <= W(i)) continue;
-                OzOperand<Real> a2 = oz_operand(D, (const Real *)nullptr, lda[i], M(i) - W(i), W(i), true, MASK_NONE, kOzTileA, nullptr);
+                OzOperand<double> a2 = oz_operand(D, (const double *)nullptr, lda[i], M(i) - W(i), W(i), true, MASK_NONE, kOzTileA, nullptr);
                 a2.ksign = -1;
                 a2.first = blocks;
                 blocks += oz_slice_blocks(a2, false);
@@ -944,7 +937,7 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                     xelems += (double)W(i) * W(i);
                     sx.push_back(x);
                     fx.push_back({q, 1 + y});
-                    OzProblem<Real> p = oz_problem<Real>(a2, x);
+                    OzProblem<double> p = oz_problem<double>(a2, x);
                     p.ldc = y == 0 ? lda[i] : M(i);
                     p.first = items;
                     items += oz_items((int)(M(i) - W(i)), (int)W(i), 1);
@@ -954,7 +947,7 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                 }
             }
             if (!sa.empty()) {
-                GramArgs<Real> c{};
+                GramArgs<double> c{};
                 gram_carve(c, (double *)nullptr);
                 L = b.put(sa);
                 for (size_t e = 0; e < sa.size(); ++e) {
@@ -969,19 +962,19 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                     b.places(L + e * sizeof(sx[0]), sx[e], RB_WS, 0, pl[q].work + (size_t)(char *)(fx[e].what == 1 ? c.X : c.Z),
                              place_of(q, fx[e].what), W(i), W(i), flag_of(i), pl[q].work + (size_t)(char *)c.kexp);
                 }
-                g->steps.push_back({ST_SLICE64, L, (int)sx.size(), (int)xblocks, 0, 1, false, xelems});
+                g->steps.push_back({ST_SLICE, L, (int)sx.size(), (int)xblocks, 0, 1, false, xelems});
                 L = b.put(pv);
                 for (size_t e = 0; e < pv.size(); ++e) {
                     const int q = fv[e].q, i = act[q];
                     const size_t pe = L + e * sizeof(pv[0]), xp = place_of(q, fv[e].what);
-                    const OzProblem<Real> &p = pv[e];
+                    const OzProblem<double> &p = pv[e];
                     b.rel(pe, &p, &p.a, RB_WS, 0, pl[q].p);
                     b.rel(pe, &p, &p.ea, RB_WS, 0, b.exps_of(pl[q].p, M(i) - W(i), W(i), kOzTileA));
                     b.rel(pe, &p, &p.b, RB_WS, 0, xp);
                     b.rel(pe, &p, &p.eb, RB_WS, 0, b.exps_of(xp, W(i), W(i), kOzTileB));
                     b.rel_flag(pe, &p, &p.skip, flag_of(i));
                     if (fv[e].what == 1) b.rel(pe, &p, &p.C, RB_A, i, Aoff(i, J(i) + W(i), J(i)));
-                    else b.rel(pe, &p, &p.C, RB_WS, 0, pl[q].y + (size_t)W(i) * sizeof(Real));
+                    else b.rel(pe, &p, &p.C, RB_WS, 0, pl[q].y + (size_t)W(i) * 8);
                 }
                 g->steps.push_back({ST_MMA, L, (int)pv.size(), items, 0, 1, false, prods});
             }
@@ -993,21 +986,21 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                 int items2 = 0, widest = 0;
                 for (int q : trailing) {
                     const int i = act[q];
-                    OzOperand<Real> v = oz_operand(D, (const Real *)nullptr, lda[i], M(i), W(i), true, MASK_UNIT_LOWER, kOzTileA, nullptr);
-                    OzOperand<Real> y = oz_operand(D, (const Real *)nullptr, M(i), W(i), M(i), false, MASK_NONE, kOzTileA, nullptr);
-                    OzOperand<Real> c = oz_operand(D, (const Real *)nullptr, lda[i], NC(i), M(i), false, MASK_NONE, kOzTileB, nullptr);
-                    const OzOperand<Real> wq = oz_operand(D, (const Real *)nullptr, 1, NC(i), W(i), false, MASK_NONE, kOzTileB, nullptr);
-                    for (OzOperand<Real> *o : {&v, &y, &c}) {
+                    OzOperand<double> v = oz_operand(D, (const double *)nullptr, lda[i], M(i), W(i), true, MASK_UNIT_LOWER, kOzTileA, nullptr);
+                    OzOperand<double> y = oz_operand(D, (const double *)nullptr, M(i), W(i), M(i), false, MASK_NONE, kOzTileA, nullptr);
+                    OzOperand<double> c = oz_operand(D, (const double *)nullptr, lda[i], NC(i), M(i), false, MASK_NONE, kOzTileB, nullptr);
+                    const OzOperand<double> wq = oz_operand(D, (const double *)nullptr, 1, NC(i), W(i), false, MASK_NONE, kOzTileB, nullptr);
+                    for (OzOperand<double> *o : {&v, &y, &c}) {
                         o->first = blocks;
                         blocks += oz_slice_blocks(*o, tall);
                         elems += (double)o->R * o->K;
                         sv.push_back(*o);
                     }
-                    OzProblem<Real> p = oz_problem<Real>(y, c);
+                    OzProblem<double> p = oz_problem<double>(y, c);
                     p.kt_per = std::max(1, std::min(p.KT, 16));
                     if ((int)trailing.size() < num_sms)
                         p.kt_per = std::max(1, std::min(p.kt_per, (int)((p.KT * trailing.size() + num_sms - 1) / num_sms)));
-                    p.kt_per = std::max(p.kt_per, std::min((p.KT + 39) / 40, oz_max_ktiles<Real>()));
+                    p.kt_per = std::max(p.kt_per, std::min((p.KT + 39) / 40, oz_max_ktiles<double>()));
                     p.S = (p.KT + p.kt_per - 1) / p.kt_per;
                     p.ldc = W(i);
                     p.first = items;
@@ -1016,10 +1009,10 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                     p1.push_back(p);
                     widest = std::max(widest, (int)NC(i));
                     prods += (double)W(i) * NC(i) * M(i);
-                    OzProblem<Real> u = oz_problem<Real>(v, wq);
+                    OzProblem<double> u = oz_problem<double>(v, wq);
                     u.ldc = lda[i];
-                    u.alpha = Real(-1);
-                    u.beta = Real(1);
+                    u.alpha = -1.0;
+                    u.beta = 1.0;
                     u.ldadd = W(i);
                     u.add_rows = (int)W(i);
                     u.first = items2;
@@ -1036,7 +1029,7 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                     b.places(e + sizeof(sv[0]), sv[3 * t + 1], RB_WS, 0, pl[q].y, pl[q].yd, W(i), M(i), flag_of(i), 0);
                     b.places(e + 2 * sizeof(sv[0]), sv[3 * t + 2], RB_A, i, ctop, pl[q].c, NC(i), M(i), flag_of(i), 0);
                     const size_t e1 = L1 + t * sizeof(p1[0]), e2 = L2 + t * sizeof(p2[0]);
-                    const OzProblem<Real> &p = p1[t], &u = p2[t];
+                    const OzProblem<double> &p = p1[t], &u = p2[t];
                     b.rel(e1, &p, &p.a, RB_WS, 0, pl[q].yd);
                     b.rel(e1, &p, &p.ea, RB_WS, 0, b.exps_of(pl[q].yd, W(i), M(i), kOzTileA));
                     b.rel(e1, &p, &p.b, RB_WS, 0, pl[q].c);
@@ -1064,8 +1057,8 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
     }
     // workspace: [... | status | blob | arena]; arena offsets are shifted to
     // their place (status places are absolute already)
-    g->blob_off = GroupBuilder<Real>::al(g->status_off + (size_t)count * 4);
-    const size_t arena0 = GroupBuilder<Real>::al(g->blob_off + g->blob.size());
+    g->blob_off = GroupBuilder::al(g->status_off + (size_t)count * 4);
+    const size_t arena0 = GroupBuilder::al(g->blob_off + g->blob.size());
     for (Reloc &r : g->relocs)
         if (r.base == RB_WS && !r.pad) r.off += arena0;
     g->total = arena0 + b.peak;
@@ -1091,38 +1084,30 @@ gbqr_status group_plan_upload(GroupPlan *g) {
 // Enqueues the grouped factorizations; mats: the matrix table in device
 // memory (A and T first).  status[i] stays 0 for a grouped matrix that is
 // done, else 1 + the panel it stopped at.
-template <class Real>
 gbqr_status group_enqueue(const Exec &ex, const GroupPlan *g, char *ws, const void *mats, int stride, int count, int *err) {
-    if (!g->d_blob || g->D != oz_digits<Real>()) return GBQR_EINVAL;
+    if (!g->d_blob) return GBQR_EINVAL;
     uint8_t *blob = (uint8_t *)ws + g->blob_off;
     if (cudaMemsetAsync(ws + g->status_off, 0, (size_t)count * 4, ex.stream) != cudaSuccess ||
         cudaMemcpyAsync(blob, g->d_blob, g->blob.size(), cudaMemcpyDeviceToDevice, ex.stream) != cudaSuccess)
         return GBQR_ECUDA;
     const int nr = (int)g->relocs.size();
     trace_begin(ex, FAM_OTHER);
-    reloc_kernel<Real *><<<(nr + 255) / 256, 256, 0, ex.stream>>>(g->d_relocs, nr, (uint64_t *)blob, ws, (const char *)mats, stride);
+    reloc_kernel<<<(nr + 255) / 256, 256, 0, ex.stream>>>(g->d_relocs, nr, (uint64_t *)blob, ws, (const char *)mats, stride);
     TRY_ST(trace_end(ex, FAM_OTHER, 0.0, 0.0));
     for (const GroupStep &s : g->steps) {
         switch (s.kind) {
             case ST_SLICE: {
-                OzSliceArgs<Real> a{};
-                a.list = reinterpret_cast<const OzOperand<Real> *>(blob + s.list);
-                a.n = s.n;
-                TRY_ST(oz_slice_launch(ex, g->D, a, (unsigned)s.grid, s.tall, s.elems));
-                break;
-            }
-            case ST_SLICE64: {
                 OzSliceArgs<double> a{};
                 a.list = reinterpret_cast<const OzOperand<double> *>(blob + s.list);
                 a.n = s.n;
-                TRY_ST(oz_slice_launch(ex, g->D, a, (unsigned)s.grid, s.tall, s.elems));
+                TRY_ST(oz_slice_launch(ex, kOzDigits64, a, (unsigned)s.grid, s.tall, s.elems));
                 break;
             }
             case ST_MMA:
             case ST_REDUCE:
             case ST_REQUANT: {
-                OzMmaArgs<Real> a{};
-                a.list = reinterpret_cast<const OzProblem<Real> *>(blob + s.list);
+                OzMmaArgs<double> a{};
+                a.list = reinterpret_cast<const OzProblem<double> *>(blob + s.list);
                 a.n = s.n;
                 a.items = s.grid;
                 a.err = err;
@@ -1132,24 +1117,19 @@ gbqr_status group_enqueue(const Exec &ex, const GroupPlan *g, char *ws, const vo
                 break;
             }
             default: {
-                GramList<Real> gl{};
-                gl.list = reinterpret_cast<const GramArgs<Real> *>(blob + s.list);
+                GramList<double> gl{};
+                gl.list = reinterpret_cast<const GramArgs<double> *>(blob + s.list);
                 trace_begin(ex, FAM_OTHER);
                 const dim3 grid((unsigned)s.grid, (unsigned)s.n, (unsigned)s.z);
-                if (s.kind == ST_DIAG) gram_diag_kernel<Real><<<grid, kThreads, 0, ex.stream>>>(gl, s.k);
-                else if (s.kind == ST_ROW) gram_row_kernel<Real><<<grid, GT, 0, ex.stream>>>(gl, s.k);
-                else if (s.kind == ST_TRAIL) gram_trail_kernel<Real><<<grid, GT, 0, ex.stream>>>(gl, s.k);
-                else gram_t_kernel<Real><<<grid, GT, 0, ex.stream>>>(gl, s.k);
+                if (s.kind == ST_DIAG) gram_diag_kernel<double><<<grid, kThreads, 0, ex.stream>>>(gl, s.k);
+                else if (s.kind == ST_ROW) gram_row_kernel<double><<<grid, GT, 0, ex.stream>>>(gl, s.k);
+                else if (s.kind == ST_TRAIL) gram_trail_kernel<double><<<grid, GT, 0, ex.stream>>>(gl, s.k);
+                else gram_t_kernel<double><<<grid, GT, 0, ex.stream>>>(gl, s.k);
                 TRY_ST(trace_end(ex, FAM_OTHER, 0.0, 0.0));
             }
         }
     }
     return GBQR_OK;
 }
-
-template GroupPlan *group_plan_build<double>(int, const int64_t *, const int64_t *, const int64_t *, const int64_t *, int, size_t);
-template GroupPlan *group_plan_build<float>(int, const int64_t *, const int64_t *, const int64_t *, const int64_t *, int, size_t);
-template gbqr_status group_enqueue<double>(const Exec &, const GroupPlan *, char *, const void *, int, int, int *);
-template gbqr_status group_enqueue<float>(const Exec &, const GroupPlan *, char *, const void *, int, int, int *);
 
 }  // namespace gbqr
