@@ -267,7 +267,10 @@ typedef struct gbqr_graph gbqr_graph;
 /* Begin capturing the context's stream into a CUDA graph (relaxed capture
  * mode).  Every library call until gbqr_graph_end is recorded, not run; the
  * calls must not need new workspace or streams (make one uncaptured call
- * first).  Tracing must be off.  Errors: EINVAL, EBUSY, ECUDA. */
+ * first).  The graph keeps the tables and lists it reads, and refers to the
+ * workspace that the context had: it may be launched after other calls as
+ * long as none of them made the workspace grow.  Tracing must be off.
+ * Errors: EINVAL, EBUSY, ECUDA. */
 GBQR_API gbqr_status gbqr_graph_begin(gbqr_ctx *ctx);
 /* End the capture and instantiate it; *out receives the graph. */
 GBQR_API gbqr_status gbqr_graph_end(gbqr_ctx *ctx, gbqr_graph **out);

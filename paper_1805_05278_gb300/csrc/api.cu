@@ -264,7 +264,7 @@ struct gbqr_ctx {
     mutable std::mutex tuned_mu;           // autotuner results (gbqr_autotune*)
     std::unordered_map<uint64_t, gbqr_opts> tuned;
     gbqr::BatchPlan *bplan[2] = {nullptr, nullptr};   // persistent batched engine: FP64, FP32 plans
-    std::vector<void *> capture_owned;    // page-locked tables a capture in progress refers to
+    std::vector<std::shared_ptr<void>> capture_owned;   // tables and lists a capture in progress refers to
 
     Exec exec() {
         Exec e;
@@ -304,10 +304,7 @@ bool ctx_lookup_tuned(const gbqr_ctx *cx, uint64_t key, gbqr_opts *o) {
     *o = it->second;
     return true;
 }
-void ctx_free_capture_owned(gbqr_ctx *cx) {
-    for (void *h : cx->capture_owned) cudaFreeHost(h);
-    cx->capture_owned.clear();
-}
+void ctx_free_capture_owned(gbqr_ctx *cx) { cx->capture_owned.clear(); }
 void ctx_copy_tuned(const gbqr_ctx *from, gbqr_ctx *to) {
     std::unordered_map<uint64_t, gbqr_opts> copy;
     {
@@ -1478,14 +1475,11 @@ gbqr_status gbqr::factor_batched_untuned(gbqr_ctx *cx, int count, const int64_t 
         if (!cx->ws_owned && cx->ws_bytes < bytes) bytes = batched_plan_bytes_plain(pl);
         if (capturing && cx->ws_bytes < bytes) return GBQR_EBUSY;
         TRY(ensure_workspace(cx, bytes));
-        if (!capturing) TRY(batched_plan_upload(pl));
+        if (!capturing) TRY(batched_plan_upload(pl, cx->stream));
         if (prepare_only) return GBQR_OK;
-        void *owned = nullptr;
-        const gbqr_status st = batched_enqueue<Real>(cx->exec(), pl, A, T, m, n, lda, ldt, cx->ws, cx->ws_bytes,
-                                                     &cx->dinfo->timeout, &cx->dinfo->nonfinite, capturing, &owned,
-                                                     BatchSide{cx->side, cx->ev_fork, cx->ev_panel});
-        if (owned) cx->capture_owned.push_back(owned);
-        return st;
+        return batched_enqueue<Real>(cx->exec(), pl, A, T, m, n, lda, ldt, cx->ws, cx->ws_bytes, &cx->dinfo->timeout,
+                                     &cx->dinfo->nonfinite, capturing ? &cx->capture_owned : nullptr,
+                                     BatchSide{cx->side, cx->ev_fork, cx->ev_panel});
     }
     int64_t mmax = 1, nmax = 1;
     std::vector<double> cost(count);
@@ -1609,7 +1603,7 @@ size_t gbqr_batched_workspace_bytes(int count, const int64_t *m, const int64_t *
 struct gbqr_graph {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    std::vector<void *> owned;   // page-locked tables its memcpy nodes read at every launch
+    std::vector<std::shared_ptr<void>> owned;   // page-locked tables and device lists its nodes read at every launch
 };
 
 gbqr_status gbqr_graph_begin(gbqr_ctx *cx) {
@@ -1648,7 +1642,6 @@ gbqr_status gbqr_graph_destroy(gbqr_graph *g) {
     if (!g) return GBQR_EINVAL;
     if (g->exec) cudaGraphExecDestroy(g->exec);
     if (g->graph) cudaGraphDestroy(g->graph);
-    for (void *h : g->owned) cudaFreeHost(h);
     delete g;
     return GBQR_OK;
 }

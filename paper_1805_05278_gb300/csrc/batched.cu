@@ -672,7 +672,7 @@ void batch_plan_free(BatchPlan *pl) {
 double batch_plan_estimate_ms(const BatchPlan *pl) { return pl ? pl->est_ms : 0.0; }
 size_t batched_plan_bytes_plain(const BatchPlan *pl) { return pl ? pl->total : 0; }
 size_t batched_plan_bytes(const BatchPlan *pl) { return pl ? std::max(pl->total, group_plan_bytes(pl->group)) : 0; }
-gbqr_status batched_plan_upload(BatchPlan *pl) { return group_plan_upload(pl->group); }
+gbqr_status batched_plan_upload(BatchPlan *pl, cudaStream_t stream) { return group_plan_upload(pl->group, stream); }
 
 namespace {
 
@@ -857,9 +857,8 @@ gbqr_status batched_plan(BatchPlan **cache, int device, int num_sms, int count, 
 template <class Real>
 gbqr_status batched_enqueue(const Exec &ex, BatchPlan *pl, Real *const *A, Real *const *T, const int64_t *m,
                             const int64_t *n, const int64_t *lda, const int64_t *ldt, char *ws, size_t ws_bytes,
-                            int *timeout_flag, unsigned long long *nonfinite, bool capturing, void **owned,
+                            int *timeout_flag, unsigned long long *nonfinite, std::vector<std::shared_ptr<void>> *keep,
                             const BatchSide &side) {
-    *owned = nullptr;
     if (!pl || pl->real != sizeof(Real) || ws_bytes < pl->total) return GBQR_EINVAL;
     if (pl->ntasks == 0) return GBQR_OK;
     for (int i = 0; i < pl->count; ++i)
@@ -870,9 +869,10 @@ gbqr_status batched_enqueue(const Exec &ex, BatchPlan *pl, Real *const *A, Real 
     // returns), from page-locked memory that the captured graph keeps when
     // capturing
     unsigned char *host = nullptr;
-    if (capturing) {
+    if (keep) {
         if (cudaMallocHost((void **)&host, pl->table_bytes) != cudaSuccess) { cudaGetLastError(); return GBQR_ENOMEM; }
-        *owned = host;
+        keep->emplace_back(host, [](void *h) { cudaFreeHost(h); });
+        if (group) keep->push_back(group_plan_lists(pl->group));
     } else {
         pl->stage.resize(pl->table_bytes);
         host = pl->stage.data();
@@ -947,10 +947,12 @@ template gbqr_status batched_plan<float>(BatchPlan **, int, int, int, const int6
                                          const int64_t *, const int64_t *, int, bool, BatchPlan **);
 template gbqr_status batched_enqueue<double>(const Exec &, BatchPlan *, double *const *, double *const *,
                                              const int64_t *, const int64_t *, const int64_t *, const int64_t *,
-                                             char *, size_t, int *, unsigned long long *, bool, void **, const BatchSide &);
+                                             char *, size_t, int *, unsigned long long *, std::vector<std::shared_ptr<void>> *,
+                                             const BatchSide &);
 template gbqr_status batched_enqueue<float>(const Exec &, BatchPlan *, float *const *, float *const *,
                                             const int64_t *, const int64_t *, const int64_t *, const int64_t *,
-                                            char *, size_t, int *, unsigned long long *, bool, void **, const BatchSide &);
+                                            char *, size_t, int *, unsigned long long *, std::vector<std::shared_ptr<void>> *,
+                                            const BatchSide &);
 
 }  // namespace gbqr
 

@@ -6,6 +6,9 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <memory>
+#include <vector>
+
 #include "../../include/gbqr.h"
 
 namespace gbqr {
@@ -197,19 +200,20 @@ void group_plan_free(GroupPlan *g);
 size_t group_plan_bytes(const GroupPlan *g);           // workspace, from its start
 const int *group_widths(const GroupPlan *g);           // per matrix, 0 = not grouped
 size_t group_status_offset(const GroupPlan *g);
-gbqr_status group_plan_upload(GroupPlan *g);
+gbqr_status group_plan_upload(GroupPlan *g, cudaStream_t stream);
+std::shared_ptr<void> group_plan_lists(const GroupPlan *g);   // what a captured graph has to keep
 gbqr_status group_enqueue(const Exec &ex, const GroupPlan *g, char *ws, const void *mats, int stride, int count, int *err);
 // The plan's workspace without the grouped part, and the upload of that part
 // (outside captures).
 size_t batched_plan_bytes_plain(const BatchPlan *pl);
-gbqr_status batched_plan_upload(BatchPlan *pl);
+gbqr_status batched_plan_upload(BatchPlan *pl, cudaStream_t stream);
 // Enqueues the table upload, the counter reset and the launch on ex.stream.
-// capturing: the table is staged in page-locked memory returned in *owned,
-// which the captured graph must keep alive.
+// keep: null, or (capturing) receives what the captured graph must keep alive:
+// the table's page-locked staging, and the grouped part's lists.
 template <class Real>
 gbqr_status batched_enqueue(const Exec &ex, BatchPlan *pl, Real *const *A, Real *const *T, const int64_t *m,
                             const int64_t *n, const int64_t *lda, const int64_t *ldt, char *ws, size_t ws_bytes,
-                            int *timeout_flag, unsigned long long *nonfinite, bool capturing, void **owned,
+                            int *timeout_flag, unsigned long long *nonfinite, std::vector<std::shared_ptr<void>> *keep,
                             const BatchSide &side);
 
 // ------------------------------------------------------------ small kernels

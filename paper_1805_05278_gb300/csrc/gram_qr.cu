@@ -48,6 +48,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -670,22 +671,28 @@ __global__ void __launch_bounds__(256) reloc_kernel(const Reloc *r, int n, uint6
 
 }  // namespace
 
+// Device copies of a plan's blob and relocations.  A captured graph reads them
+// at every launch, so it shares them with the plan: whichever goes last frees
+// them.
+struct GroupLists {
+    uint8_t *blob = nullptr;
+    Reloc *relocs = nullptr;
+    ~GroupLists() {
+        cudaFree(blob);
+        cudaFree(relocs);
+    }
+};
+
 struct GroupPlan {
     size_t blob_off = 0, status_off = 0, total = 0;      // workspace layout, from its start
     std::vector<uint8_t> blob;
     std::vector<Reloc> relocs;
     std::vector<GroupStep> steps;
     std::vector<int> width;                              // per matrix: its panels' width, 0 = not grouped
-    uint8_t *d_blob = nullptr;                           // device copies (group_plan_upload)
-    Reloc *d_relocs = nullptr;
+    std::shared_ptr<GroupLists> lists;                   // device copies (group_plan_upload)
 };
 
-void group_plan_free(GroupPlan *g) {
-    if (!g) return;
-    cudaFree(g->d_blob);
-    cudaFree(g->d_relocs);
-    delete g;
-}
+void group_plan_free(GroupPlan *g) { delete g; }
 size_t group_plan_bytes(const GroupPlan *g) { return g ? g->total : 0; }
 const int *group_widths(const GroupPlan *g) { return g->width.data(); }
 size_t group_status_offset(const GroupPlan *g) { return g->status_off; }
@@ -1066,33 +1073,37 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
 }
 
 // Device copies of the plan's blob and relocations (not during a capture).
-gbqr_status group_plan_upload(GroupPlan *g) {
-    if (!g || g->d_blob) return GBQR_OK;
-    if (cudaMalloc((void **)&g->d_blob, g->blob.size()) != cudaSuccess ||
-        cudaMalloc((void **)&g->d_relocs, g->relocs.size() * sizeof(Reloc)) != cudaSuccess) {
+// Waits for them: the calls that read them may be on another stream.
+gbqr_status group_plan_upload(GroupPlan *g, cudaStream_t stream) {
+    if (!g || g->lists) return GBQR_OK;
+    std::shared_ptr<GroupLists> l(new (std::nothrow) GroupLists());
+    if (!l) return GBQR_ENOMEM;
+    const size_t nb = g->blob.size(), nr = g->relocs.size() * sizeof(Reloc);
+    if (cudaMalloc((void **)&l->blob, nb) != cudaSuccess || cudaMalloc((void **)&l->relocs, nr) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(g->d_blob);
-        g->d_blob = nullptr;
         return GBQR_ENOMEM;
     }
-    if (cudaMemcpy(g->d_blob, g->blob.data(), g->blob.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(g->d_relocs, g->relocs.data(), g->relocs.size() * sizeof(Reloc), cudaMemcpyHostToDevice) != cudaSuccess)
+    if (cudaMemcpyAsync(l->blob, g->blob.data(), nb, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+        cudaMemcpyAsync(l->relocs, g->relocs.data(), nr, cudaMemcpyHostToDevice, stream) != cudaSuccess ||
+        cudaStreamSynchronize(stream) != cudaSuccess)
         return GBQR_ECUDA;
+    g->lists = std::move(l);
     return GBQR_OK;
 }
+std::shared_ptr<void> group_plan_lists(const GroupPlan *g) { return g->lists; }
 
 // Enqueues the grouped factorizations; mats: the matrix table in device
 // memory (A and T first).  status[i] stays 0 for a grouped matrix that is
 // done, else 1 + the panel it stopped at.
 gbqr_status group_enqueue(const Exec &ex, const GroupPlan *g, char *ws, const void *mats, int stride, int count, int *err) {
-    if (!g->d_blob) return GBQR_EINVAL;
+    if (!g->lists) return GBQR_EINVAL;
     uint8_t *blob = (uint8_t *)ws + g->blob_off;
     if (cudaMemsetAsync(ws + g->status_off, 0, (size_t)count * 4, ex.stream) != cudaSuccess ||
-        cudaMemcpyAsync(blob, g->d_blob, g->blob.size(), cudaMemcpyDeviceToDevice, ex.stream) != cudaSuccess)
+        cudaMemcpyAsync(blob, g->lists->blob, g->blob.size(), cudaMemcpyDeviceToDevice, ex.stream) != cudaSuccess)
         return GBQR_ECUDA;
     const int nr = (int)g->relocs.size();
     trace_begin(ex, FAM_OTHER);
-    reloc_kernel<<<(nr + 255) / 256, 256, 0, ex.stream>>>(g->d_relocs, nr, (uint64_t *)blob, ws, (const char *)mats, stride);
+    reloc_kernel<<<(nr + 255) / 256, 256, 0, ex.stream>>>(g->lists->relocs, nr, (uint64_t *)blob, ws, (const char *)mats, stride);
     TRY_ST(trace_end(ex, FAM_OTHER, 0.0, 0.0));
     for (const GroupStep &s : g->steps) {
         switch (s.kind) {

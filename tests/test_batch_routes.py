@@ -1,6 +1,8 @@
 """Which path a batch takes, and that what it computes does not depend on
 things the caller did not ask for."""
 
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -18,6 +20,11 @@ def _device(mats, dtype):
 def _kernels(gb, mats, dtype):
     import torch
     return [torch.zeros((a.shape[1], min(16, a.shape[1])), dtype=dtype, device="cuda").T for a in mats]
+
+
+def _need(gb, shapes):
+    I64 = ctypes.c_int64 * len(shapes)
+    return gb.gbqr_batched_workspace_bytes(len(shapes), I64(*[s[0] for s in shapes]), I64(*[s[1] for s in shapes]), None)
 
 
 def test_fp32_batch_does_not_depend_on_the_workspace(gb):
@@ -39,3 +46,43 @@ def test_fp32_batch_does_not_depend_on_the_workspace(gb):
         assert torch.equal(A, B)
     for (A, B) in zip(*[o[1] for o in out]):
         assert torch.equal(A, B)
+
+
+def test_graphs_of_several_shape_sets_on_one_context(gb):
+    """A captured batch keeps what it reads: after the context has planned
+    other batches it replays to the bits that eager calls gave.  (The
+    workspace is the caller's, so that nothing moves it.)"""
+    import torch
+    sets = [[(2000, 256), (900, 40), (5003, 128)], [(700, 64), (1300, 250), (600, 300), (64, 16)], [(4096, 96), (100, 60)]]
+    stream = torch.cuda.Stream()
+    with gb.Context(0, stream) as ctx:
+        ws = torch.empty(1 << 30, dtype=torch.uint8, device="cuda")
+        ctx.set_workspace(ws)
+        assert max(_need(gb, s) for s in sets) <= ws.numel()     # (room for the grouped path)
+        want, graphs, held = [], [], []
+        for k, shapes in enumerate(sets):
+            mats = [workloads.gaussian(m, n, 520 + 10 * k + i) for i, (m, n) in enumerate(shapes)]
+            A, T = _device(mats, torch.float64), _kernels(gb, mats, torch.float64)
+            torch.cuda.synchronize()
+            ctx.factor_batched(A, T)
+            torch.cuda.synchronize()
+            want.append((A, T))
+            A, T = _device(mats, torch.float64), _kernels(gb, mats, torch.float64)
+            fresh = [a.clone() for a in A]
+            torch.cuda.synchronize()
+            graphs.append(ctx.capture(lambda: ctx.factor_batched(A, T)))
+            held.append((A, T, fresh))
+        for k in (0, 2, 1, 0):
+            A, T, fresh = held[k]
+            for a, t, f in zip(A, T, fresh):
+                a.copy_(f)
+                t.zero_()
+            torch.cuda.synchronize()
+            graphs[k].launch()
+            torch.cuda.synchronize()
+            assert ctx.sync()[0] == gb.GBQR_OK
+            for got, exp in zip(A + T, want[k][0] + want[k][1]):
+                assert torch.equal(got, exp)
+        for g in graphs:
+            g.close()
+        ctx.set_workspace(None)
