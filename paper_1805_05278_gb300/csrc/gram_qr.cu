@@ -98,6 +98,14 @@ __device__ __forceinline__ double a1_at(const GramArgs<Real> &p, int i, int j, i
     return (i < p.w && j < p.w) ? (double)p.A[i + (int64_t)j * p.lda] : (i == j ? 1.0 : 0.0);
 }
 
+// Whether the panel was given up: read once for the whole CTA, since another
+// CTA of the same launch may raise the flag meanwhile, and threads of one CTA
+// that saw different values would part ahead of a barrier.
+template <class Real>
+__device__ __forceinline__ bool given_up(const GramArgs<Real> &p) {
+    return __syncthreads_or(threadIdx.x == 0 && *(volatile int *)p.flag);
+}
+
 // 1/d by the reciprocal approximation and one third-order Newton step
 // (r + r (e + e^2), e = 1 - d r): three dependent FP64 instructions, where
 // the correctly rounded reciprocal takes about twice as long.
@@ -310,7 +318,7 @@ template <class Real>
 __global__ void __launch_bounds__(GT) gram_row_kernel(const __grid_constant__ GramList<Real> args, int k) {
     __shared__ double sA[GB][GB + 1], sB[4][GB];
     const GramArgs<Real> p = nth_panel(args);
-    if (k >= p.nblk || *(volatile int *)p.flag) return;
+    if (k >= p.nblk || given_up(p)) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int task = blockIdx.x >> 3;
     const int c0 = (blockIdx.x & 7) * 4, rest = p.nblk - k - 1, c = c0 + warp;
@@ -381,7 +389,7 @@ template <class Real>
 __global__ void __launch_bounds__(GT) gram_trail_kernel(const __grid_constant__ GramList<Real> args, int k) {
     __shared__ double sA[GB][GB + 1], sB[4][GB];
     const GramArgs<Real> p = nth_panel(args);
-    if (k >= p.nblk || *(volatile int *)p.flag) return;
+    if (k >= p.nblk || given_up(p)) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Tile tl{sA, sB, warp, lane};
     const int c0 = (blockIdx.x & 7) * 4, rest = p.nblk - k - 1, c = c0 + warp;
@@ -432,7 +440,7 @@ __global__ void __launch_bounds__(GT) gram_t_kernel(const __grid_constant__ Gram
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, col = warp & 1, half = warp >> 1;
     const int c0 = (blockIdx.x & 15) * 2, c = c0 + col, task = blockIdx.x >> 4;
     const bool top = blockIdx.z == 1;
-    if (task >= p.nblk * p.nblk || (top && !p.Y) || *(volatile int *)p.flag) return;
+    if (task >= p.nblk * p.nblk || (top && !p.Y) || given_up(p)) return;
     const int i = task % p.nblk, j = task / p.nblk, l0 = top ? 0 : i;
     const int gi = i * GB + lane, gj = j * GB + c;
     double acc = 0.0;

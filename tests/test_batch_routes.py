@@ -86,3 +86,28 @@ def test_graphs_of_several_shape_sets_on_one_context(gb):
         for g in graphs:
             g.close()
         ctx.set_workspace(None)
+
+
+def test_panels_given_up_at_every_place(gb):
+    """Matrices whose panels fail the condition check at different columns, in
+    one batch: whichever CTA finds out first, the results are the same, and
+    those of a workspace that only the persistent kernel fits."""
+    import torch
+    n, mats = 128, []
+    for j in range(1, n, 3):
+        a = workloads.gaussian(600 + j, n, 560 + j)
+        a[:, j] = a[:, j // 2] + 1e-9 * a[:, j]
+        mats.append(a)
+    with gb.Context(0) as ctx:
+        out = []
+        for ws in (None, None, None, torch.empty(64 << 20, dtype=torch.uint8, device="cuda")):
+            A, T = _device(mats, torch.float64), _kernels(gb, mats, torch.float64)
+            if ws is not None:
+                ctx.set_workspace(ws)
+            ctx.factor_batched(A, T)
+            assert ctx.sync()[0] == gb.GBQR_OK
+            out.append(A + T)
+        ctx.set_workspace(None)
+    for other in out[1:]:
+        for p, q in zip(out[0], other):
+            assert torch.equal(p, q)
