@@ -1,5 +1,5 @@
 // Householder QR of a well-conditioned m x w panel (w <= 128, m >= 4 w) from
-// its Gram matrix, the fast base case of QR-EG in FP64.
+// its Gram matrix, the fast base case of QR-EG in FP64 and FP32.
 //
 // The TSQR base case (tsqr.cu) is a serial chain of w Householder steps per
 // tree level, about 12 us a column, whatever the number of rows.  A panel
@@ -20,13 +20,12 @@
 // signs.  It is the reconstruction of Appendix C.2 with A R^{-1} for W
 // (Ballard, Demmel, Grigori, Jacquelin, Nguyen, Solomonik 2014, who note
 // that it is the less stable variant: errors grow with the panel's
-// condition).  So it is taken only where the condition allows: every entry
-// of R+^{-1}, its rows scaled by the column norms, has to stay at or below 4
-// in magnitude (1 on the diagonal and 0 off it for orthogonal columns).  Then
-// the Cholesky's few u are amplified by a small factor, and V, T and R agree
-// with the TSQR's to rounding.  Otherwise a device flag is raised, the panel
-// is left untouched, and the caller's TSQR launches, which return at once
-// while the flag is zero, factor it.
+// condition).  So it is taken only where the condition allows: no column may
+// be nearly a combination of the others (gram_bound).  Then orthogonality and
+// backward error are at or below the TSQR's, and V, T and R agree with its to
+// rounding.  Otherwise a device flag is raised, the panel is left untouched,
+// and the caller's TSQR launches, which return at once while the flag is zero,
+// factor it.
 //
 // The w x w work runs in 32-wide blocks, three launches a block:
 //   diag   one CTA: Cholesky and LU of the diagonal block
@@ -59,7 +58,19 @@ namespace {
 constexpr int GB = 32;               // block width
 constexpr int GLD = kGramMaxW;       // leading dimension of every w x w array
 constexpr int GT = 128;              // threads of the row / trail kernels: 32 x 4 outputs
-constexpr double kGramBound2 = 16.0; // largest accepted (R^-1)_ij^2 g_ii
+
+// Largest accepted g_ii (G^-1)_ii = sum_j (R^-1)_ij^2 g_ii of a panel of w
+// columns: how far column i's part orthogonal to all the others is below its
+// length, squared (1 for orthogonal columns).  The loss of orthogonality grows
+// with it and with the number of columns that share a direction.  FP64: at
+// sqrt(360 / w) - 1.7 for 128 columns, 2.4 for 64, 4.7 for 16 - it is below
+// Householder's for every kind of columns tried (a common mean, a common
+// factor, chains and pairs of correlated ones; at 2 and 128 columns with a
+// mean it is 1.3 times Householder's, at 16 thirty times), and no panel of
+// Gaussian columns with 4 rows a column is refused (1.55 the largest of 100
+// at 128, 2.2 of 300 at 16).  FP32: the same in FP64 costs no accuracy up to 16.
+template <class Real>
+double gram_bound(int w) { return sizeof(Real) == 8 ? std::sqrt(360.0 / w) : 16.0; }
 
 template <class Real>
 struct GramArgs {
@@ -74,6 +85,7 @@ struct GramArgs {
     int raise;                       // what an ill-conditioned panel writes to *flag
     int keep;                        // batch: *flag is the matrix's, clear at the start; a raised one skips the rest
     int tb;                          // batch: T's blocks of width tb alone (0: the whole T)
+    double bound;                    // gram_bound()
 };
 
 // The panels of one launch: by value, or (blockIdx.y: which) a list in device memory.
@@ -99,8 +111,8 @@ __device__ __forceinline__ double a1_at(const GramArgs<Real> &p, int i, int j, i
 }
 
 // Whether the panel was given up: read once for the whole CTA, since another
-// CTA of the same launch may raise the flag meanwhile, and threads of one CTA
-// that saw different values would part ahead of a barrier.
+// CTA of the same launch (of gram_t's first step) may raise the flag meanwhile,
+// and threads of one CTA that saw different values would part ahead of a barrier.
 template <class Real>
 __device__ __forceinline__ bool given_up(const GramArgs<Real> &p) {
     return __syncthreads_or(threadIdx.x == 0 && *(volatile int *)p.flag);
@@ -180,8 +192,10 @@ __global__ void __launch_bounds__(kThreads) gram_diag_kernel(const __grid_consta
     }
     // R = D^{1/2} Lc^T; column t of S holds d_t Lc(:, t)
     if (warp == 0) {
+        // (the pivot's own share of the sum that gram_t bounds: most panels that
+        // will not do stop here)
         const double d = S[lane][lane];
-        if (!(d > 0.0 && d < 1e300)) bad = 1;
+        if (!(d > 0.0 && d < 1e300 && d * p.bound >= __ldcg(p.gd + b0 + lane))) bad = 1;
         const double s = sqrt(d);
         sg[lane] = s;
         p.sc[lane] = s * rd[lane];                       // 1 / r_tt
@@ -318,7 +332,7 @@ template <class Real>
 __global__ void __launch_bounds__(GT) gram_row_kernel(const __grid_constant__ GramList<Real> args, int k) {
     __shared__ double sA[GB][GB + 1], sB[4][GB];
     const GramArgs<Real> p = nth_panel(args);
-    if (k >= p.nblk || given_up(p)) return;
+    if (k >= p.nblk || *(volatile int *)p.flag) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int task = blockIdx.x >> 3;
     const int c0 = (blockIdx.x & 7) * 4, rest = p.nblk - k - 1, c = c0 + warp;
@@ -353,10 +367,7 @@ __global__ void __launch_bounds__(GT) gram_row_kernel(const __grid_constant__ Gr
         if (task == 0) {
             blk(p.X, k, k)[c + lane * GLD] = y * uinv;
         } else if (task == 1) {
-            y *= rinv;
-            blk(p.RI, k, k)[c + lane * GLD] = y;
-            // the row is scaled by the norm of column b0 + c of the panel
-            if (!(y * y * __ldcg(p.gd + k * GB + c) <= kGramBound2)) *(volatile int *)p.flag = p.raise;
+            blk(p.RI, k, k)[c + lane * GLD] = y * rinv;
         } else {
             blk(p.LI, k, k)[lane + c * GLD] = y;
         }
@@ -389,7 +400,7 @@ template <class Real>
 __global__ void __launch_bounds__(GT) gram_trail_kernel(const __grid_constant__ GramList<Real> args, int k) {
     __shared__ double sA[GB][GB + 1], sB[4][GB];
     const GramArgs<Real> p = nth_panel(args);
-    if (k >= p.nblk || given_up(p)) return;
+    if (k >= p.nblk || *(volatile int *)p.flag) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Tile tl{sA, sB, warp, lane};
     const int c0 = (blockIdx.x & 7) * 4, rest = p.nblk - k - 1, c = c0 + warp;
@@ -425,17 +436,16 @@ __global__ void __launch_bounds__(GT) gram_trail_kernel(const __grid_constant__ 
         acc = tl.dot(acc);
     }
     blk(what == 0 ? p.X : p.RI, l, k)[lane + c * GLD] = -acc;
-    if (what == 1 && !(acc * acc * __ldcg(p.gd + l * GB + lane) <= kGramBound2)) *(volatile int *)p.flag = p.raise;
 }
 
-// Z = X T = -R+^{-1} S V1^{-T} (step 0), then T = U Z, the top block of Y = V T
+// Z = X T = -R+^{-1} S V1^{-T} and the condition check (step 0), then T = U Z, the top block of Y = V T
 // = (A - [R; 0]) Z and V1 \\ R over the panel's top block (step 1).  A CTA
 // takes 32 x 2 outputs of block (i, j), a warp one column and the even or odd
 // 32-wide steps; all operands are staged at once.  blockIdx.x = block * 16 +
 // column pair, blockIdx.z = 1: Y.
 template <class Real>
 __global__ void __launch_bounds__(GT) gram_t_kernel(const __grid_constant__ GramList<Real> args, int step) {
-    __shared__ double sA[4][GB][GB + 1], sB[2][4 * GB], part[2][GB];
+    __shared__ double sA[4][GB][GB + 1], sB[2][4 * GB], part[4][GB];
     const GramArgs<Real> p = nth_panel(args);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, col = warp & 1, half = warp >> 1;
     const int c0 = (blockIdx.x & 15) * 2, c = c0 + col, task = blockIdx.x >> 4;
@@ -456,6 +466,18 @@ __global__ void __launch_bounds__(GT) gram_t_kernel(const __grid_constant__ Gram
                               : __ldcg(blk(p.Z, l, j) + lane + c * GLD);
         }
         __syncthreads();
+        if (step == 0 && j == p.nblk - 1 && c0 == 0) {
+            // block row i of R^{-1} is here whole: rows' sums of squares, times g_ii
+            double q = 0.0;
+            for (int l = 0; l <= j - i; ++l)
+#pragma unroll
+                for (int kk = 0; kk < GB; kk += 4) q = rfma(sA[l][kk + warp][lane], sA[l][kk + warp][lane], q);
+            part[warp][lane] = q;
+            __syncthreads();
+            q = part[0][lane] + part[1][lane] + part[2][lane] + part[3][lane];
+            if (warp == 0 && !(q * __ldcg(p.gd + gi) <= p.bound)) *(volatile int *)p.flag = p.raise;
+            __syncthreads();
+        }
         double a0 = 0.0, a1 = 0.0;
         for (int l = half; l <= j - l0; l += 2)
 #pragma unroll
@@ -557,6 +579,7 @@ gbqr_status gram_qr(const Exec &ex, int64_t m, int64_t w, Real *A, int64_t lda, 
     gram_carve(p, work);
     p.flag = flag;
     p.raise = 1;
+    p.bound = gram_bound<Real>((int)w);
     const GramScratch sc = gram_scratch(D, m, w, Y != nullptr);
     if (sc.total > oz.bytes) return GBQR_ENOMEM;
     char *base = (char *)oz.base;
@@ -871,6 +894,7 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                 p.lda = lda[i]; p.ldt = ldt[i]; p.ldy = M(i);
                 p.w = (int)W(i); p.nblk = (int)((W(i) + GB - 1) / GB);
                 p.raise = 1 + (int)pn; p.keep = 1; p.tb = kBatchTb;
+                p.bound = gram_bound<double>(p.w);
             }
             size_t L = b.put(sp);
             for (int q = 0; q < na; ++q) {
