@@ -18,8 +18,8 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libgbqr.so")
 ROOT = os.path.dirname(HERE)
 
-SOURCES = ["api.cu", "gemm.cu", "tsqr.cu", "aux_kernels.cu", "probe.cu", "noalloc.cu", "tc_gemm.cu", "oz_gemm.cu", "gram_qr.cu", "server.cu", "tune.cu", "batched.cu", "applyvec.cu", "trsvchain.cu"]
-HEADERS = ["common.cuh", "tsqr_dev.cuh", "tc_ptx.cuh", "oz.cuh"]
+SOURCES = ["api.cu", "gemm.cu", "tsqr.cu", "aux_kernels.cu", "probe.cu", "noalloc.cu", "tc_gemm.cu", "oz_gemm.cu", "gram_qr.cu", "panel_chain.cu", "server.cu", "tune.cu", "batched.cu", "applyvec.cu", "trsvchain.cu"]
+HEADERS = ["common.cuh", "tsqr_dev.cuh", "tc_ptx.cuh", "oz.cuh", "tsqr_block.cuh", "gemm_tile.cuh", "panel_chain.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
               "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]

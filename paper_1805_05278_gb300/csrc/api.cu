@@ -9,6 +9,7 @@
 // on the host.
 #include "common.cuh"
 #include "oz.cuh"
+#include "panel_chain.cuh"
 
 #include <algorithm>
 #include <climits>
@@ -36,7 +37,6 @@ constexpr int kMaxBatchLanes = 128;
 constexpr size_t kOzMainBytes = (size_t)384 << 20;   // digit scratch of the trailing updates (8192^2: up to three column chunks)
 constexpr int64_t kOzChunkCols = 512;              // ... never less than this many columns' worth
 constexpr int64_t kFusedMinRows = 256;             // shorter matrices update by separate products
-constexpr int kGramFallbackB = 64;   // TSQR width behind a Gram-matrix panel: few launches, which mostly return at once
 
 struct DeviceInfo {
     unsigned long long nonfinite;
@@ -123,7 +123,7 @@ bool resolve(const gbqr_opts *o, int64_t m, int64_t n, Params *p) {
 
 // Workspace regions (bytes, 256-aligned) for an m x n problem.
 struct Layout {
-    size_t partial = 0, gcount = 0, tR = 0, tT = 0, tY = 0, tX = 0, tcount = 0;
+    size_t partial = 0, gcount = 0, tR = 0, tT = 0, tY = 0, tX = 0, tcount = 0, ccount = 0;
     size_t M1 = 0, M2 = 0, bigA = 0, bigT = 0, vec = 0;
     size_t partial2 = 0, gcount2 = 0, M1b = 0, M2b = 0;   // second lane (look-ahead panel stream)
     size_t tc = 0, n_tc = 0;                              // tensor-core slices (mixed updates)
@@ -155,7 +155,7 @@ Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num
     const int w = (int)std::max<int64_t>(1, std::min<int64_t>(pr.b, n));
     L.tsqr = tsqr_plan_bound(std::max<int64_t>(m, 1), w, pr.leaf_rows, pr.fanout, num_sms);
     if (gram) {
-        const TsqrPlan f = tsqr_plan_bound(m, (int)std::min<int64_t>(kGramFallbackB, n), 0, kDefaultFanout, num_sms);
+        const TsqrPlan f = tsqr_plan_bound(m, (int)std::min<int64_t>(kChainMaxW, n), 0, kDefaultFanout, num_sms);
         L.tsqr.nR = std::max(L.tsqr.nR, f.nR);
         L.tsqr.nT = std::max(L.tsqr.nT, f.nT);
         L.tsqr.nY = std::max(L.tsqr.nY, f.nY);
@@ -172,9 +172,12 @@ Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num
     L.n_bigA = staging ? (size_t)std::max<int64_t>(m, 1) * (size_t)std::max<int64_t>(n, 1) : 1;
     L.n_bigT = staging ? (size_t)std::max<int64_t>(n, 1) * (size_t)std::max<int64_t>(n, 1) : 1;
     L.partial = take(L.n_partial * 8);
-    L.counter_bytes = align_up(L.n_gcount * 4, 16) + L.tsqr.ncount * 4;
+    L.tcount = align_up(L.n_gcount * 4, 16);
+    L.ccount = L.tcount + align_up(L.tsqr.ncount * 4, 16);
+    L.counter_bytes = gram ? L.ccount + 16 : L.tcount + L.tsqr.ncount * 4;
     L.gcount = take(L.counter_bytes);
-    L.tcount = L.gcount + align_up(L.n_gcount * 4, 16);
+    L.tcount += L.gcount;
+    L.ccount += L.gcount;
     L.tR = take(L.tsqr.nR * 8);
     L.tT = take(L.tsqr.nT * 8);
     L.tY = take(L.tsqr.nY * 8);
@@ -359,6 +362,7 @@ struct Work {
     double *M1b, *M2b;
     double *gram = nullptr;          // Gram-matrix panels: work, and the flag behind it (null: TSQR only)
     int *gram_flag = nullptr;
+    unsigned *chain_ctr = nullptr;   // counters of the launch behind a Gram-matrix panel
     double *Y = nullptr;             // fused updates (null: none)
     char *vy = nullptr;
 
@@ -452,6 +456,7 @@ void carve_work(gbqr_ctx *cx, char *base, const Layout &L, const Params &pr, con
     w->Y = pr.gram && w->L.n_vy ? (double *)(base + w->L.Y) : nullptr;
     w->vy = pr.gram && w->L.n_vy ? base + w->L.vy : nullptr;
     w->gram_flag = w->gram ? (int *)(w->gram + w->L.n_gram) : nullptr;
+    w->chain_ctr = (unsigned *)(base + w->L.ccount);
     w->M1b = (double *)(base + w->L.M1b);
     w->M2b = (double *)(base + w->L.M2b);
     w->tcs.base = w->L.n_tc ? (void *)(base + w->L.tc) : nullptr;
@@ -570,27 +575,25 @@ gbqr_status form_y(const Exec &ex, const GemmScratchT<Real> &gs, int64_t m, int6
 }
 
 // A panel from its Gram matrix.  Where that is too ill-conditioned the flag is
-// up and A as it was, and the recursion on FMA products and wide TSQRs, whose
-// launches return at once while the flag is zero, does it.  Y: V T, or null.
+// up and A as it was, and the recursion on FMA products and TSQRs, one launch
+// that returns at once while the flag is zero, does it.  Y: V T, or null.
 template <class Real>
 gbqr_status gram_or_tsqr(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, Real *T, int64_t ldt, Real *Y, int64_t ldy) {
     TRY(gram_qr(w.ex, m, n, A, lda, T, ldt, Y, ldy, w.gram, w.gram_flag, w.gs.oz));
+    ChainRecorder rec;
     Work f = w;
-    f.ex.pred = w.gram_flag;
-    TsqrPlan pl;
-    const int64_t n1 = n <= kGramFallbackB ? n : n / 2;
-    const bool wide = tsqr_plan(m, (int)n1, 0, 0, w.ex.num_sms, &pl) &&
-                      (n1 == n || tsqr_plan(m - n1, (int)(n - n1), 0, 0, w.ex.num_sms, &pl));
-    f.pr.b = wide ? kGramFallbackB : kGramFallbackB / 2;
+    f.ex.chain = &rec;
+    f.pr.b = kChainMaxW;
     TRY(qr_eg(f, m, n, A, lda, T, ldt));
-    return Y ? form_y(f.ex, f.gsr<Real>(), m, n, A, lda, T, ldt, Y, ldy) : GBQR_OK;
+    if (Y) TRY(form_y(f.ex, f.gsr<Real>(), m, n, A, lda, T, ldt, Y, ldy));
+    return chain_launch<Real>(w.ex, rec, w.gram_flag, w.chain_ctr, &w.cx->dinfo->timeout);
 }
 
 // Algorithm 2: (V, T, R) = QR-EG(A, b), V\R in place over A, T (n x n) at T.
 template <class Real>
 gbqr_status qr_eg(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, Real *T, int64_t ldt) {
     if (n <= 0) return GBQR_OK;
-    if (w.gram && !w.ex.pred && gram_qr_fits<Real>(w.gs.oz, m, n))
+    if (w.gram && !w.ex.chain && gram_qr_fits<Real>(w.gs.oz, m, n))
         return gram_or_tsqr<Real>(w, m, n, A, lda, T, ldt, nullptr, 0);
     if (n <= w.pr.b) return base_qr(w, m, n, A, lda, T, ldt);
     const int64_t n1 = n / 2, n2 = n - n1;
@@ -602,7 +605,7 @@ gbqr_status qr_eg(Work &w, int64_t m, int64_t n, Real *A, int64_t lda, Real *T, 
     // two tall products go to the tensor cores once they are large enough to
     // beat the FP64 kernel's latency (the T-assembly below stays FP64, so T
     // stays consistent with V and Q = I - V T V^T orthogonal to FP64 accuracy).
-    const int nsplit_in = (w.pr.nsplit > 0 && !w.ex.pred && n1 >= kInPanelTcMinCols && m >= kInPanelTcMinRows) ? w.pr.nsplit : 0;
+    const int nsplit_in = (w.pr.nsplit > 0 && !w.ex.chain && n1 >= kInPanelTcMinCols && m >= kInPanelTcMinRows) ? w.pr.nsplit : 0;
     TRY(apply_block(w, true, m, n2, n1, A, lda, T, ldt, AR, lda, nsplit_in));
     // right recursion on B22
     Real *TR = T + n1 + n1 * ldt;

@@ -26,6 +26,8 @@ struct Tracer {
     virtual ~Tracer() {}
 };
 
+struct ChainRecorder;
+
 // Everything a launcher needs besides its operands.
 struct Exec {
     cudaStream_t stream = nullptr;
@@ -34,7 +36,7 @@ struct Exec {
     int num_sms = 152;
     int device = 0;
     bool dmma = false;          // 64 x 64 FP64 GEMM tiles on the FP64 tensor cores (else DFMA)
-    const int *pred = nullptr;  // device flag: the kernels of gemm() and tsqr_run() return at once while it is zero
+    ChainRecorder *chain = nullptr;   // gemm() and tsqr_run() put their work here instead of launching it
 };
 
 inline void trace_begin(const Exec &ex, Family f) {
@@ -42,7 +44,7 @@ inline void trace_begin(const Exec &ex, Family f) {
 }
 inline gbqr_status trace_end(const Exec &ex, Family f, double flops, double bytes) {
     if (ex.launches) ++*ex.launches;
-    if (ex.tracer) ex.tracer->end(ex.stream, f, ex.pred ? 0.0 : flops, ex.pred ? 0.0 : bytes);
+    if (ex.tracer) ex.tracer->end(ex.stream, f, flops, bytes);
     return cudaPeekAtLastError() == cudaSuccess ? GBQR_OK : GBQR_ECUDA;
 }
 

@@ -15,7 +15,7 @@
 // (Section 4, Lemma 3).  The partial tiles are summed by a fixed-shape tree
 // of "last CTA to arrive" reductions (fan-in 8): no CTA ever waits on
 // another, and the summation order is fixed, so results are deterministic.
-#include "common.cuh"
+#include "gemm_tile.cuh"
 
 #include <algorithm>
 #include <type_traits>
@@ -23,176 +23,11 @@
 namespace gbqr {
 namespace {
 
-constexpr int BK = 16;
-constexpr int kGroup = 8;   // fan-in of the split-K reduction tree
-
-template <class Real>
-struct GemmParamsT {
-    int64_t M, N, K;
-    const Real *A; int64_t lda; int maskA;
-    const Real *B; int64_t ldb; int maskB;
-    Real *C; int64_t ldc;
-    Real alpha, beta;
-    Real *partial;            // per tile: slots_per_tile * BM*BN elements
-    unsigned *counters;       // per tile: counters_per_tile
-    int slots_per_tile, counters_per_tile;
-    const int *pred;          // non-null: run only while *pred != 0
-};
-using GemmParams = GemmParamsT<double>;
-
-__device__ __forceinline__ double rfma(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float rfma(float a, float b, float c) { return fmaf(a, b, c); }
-
-template <class Real>
-__device__ __forceinline__ Real masked(const Real *X, int64_t ld, int64_t r, int64_t c, int mask) {
-    if (mask == MASK_UNIT_LOWER) {
-        if (r < c) return Real(0);
-        if (r == c) return Real(1);
-    } else if (mask == MASK_UPPER) {
-        if (r > c) return Real(0);
-    }
-    return X[r + c * ld];
-}
-
-// K range [kb, ke) outside which op(A)(i, k) or op(B)(k, j) is structurally
-// zero for every i in [m0, m0+BM) and j in [n0, n0+BN).
-template <class P>
-__device__ __forceinline__ void k_range(const P &p, bool ta, int64_t m0, int64_t n0,
-                                        int BM, int BN, int64_t &kb, int64_t &ke) {
-    kb = 0; ke = p.K;
-    if (p.maskA == MASK_UNIT_LOWER) {
-        if (!ta) ke = min(ke, m0 + BM);   // A(i,k) != 0 needs k <= i
-        else kb = max(kb, m0);            // A(k,i) != 0 needs k >= i
-    } else if (p.maskA == MASK_UPPER) {
-        if (!ta) kb = max(kb, m0);        // A(i,k) != 0 needs k >= i
-        else ke = min(ke, m0 + BM);       // A(k,i) != 0 needs k <= i
-    }
-    if (p.maskB == MASK_UNIT_LOWER) kb = max(kb, n0);       // B(k,j) != 0 needs k >= j
-    else if (p.maskB == MASK_UPPER) ke = min(ke, n0 + BN);  // B(k,j) != 0 needs k <= j
-}
-
 template <class Real, int BM, int BN, bool TA>
 __global__ void __launch_bounds__(kThreads) dgemm_kernel(GemmParamsT<Real> p) {
-    constexpr int RM = BM / 16, RN = BN / 16;
     __shared__ Real As[BK][BM + 1];
     __shared__ Real Bs[BK][BN + 1];
-    __shared__ int s_last;
-    if (p.pred && *(volatile const int *)p.pred == 0) return;
-
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int64_t m0 = (int64_t)blockIdx.x * BM, n0 = (int64_t)blockIdx.y * BN;
-    const int S = gridDim.z, z = blockIdx.z;
-
-    int64_t kb, ke;
-    k_range(p, TA, m0, n0, BM, BN, kb, ke);
-    int64_t k_lo = kb, k_hi = kb;
-    if (ke > kb) {
-        int64_t chunk = (ke - kb + S - 1) / S;
-        chunk = (chunk + BK - 1) / BK * BK;
-        k_lo = kb + (int64_t)z * chunk;
-        k_hi = min(ke, k_lo + chunk);
-    }
-
-    Real acc[RM][RN];
-#pragma unroll
-    for (int r = 0; r < RM; ++r)
-#pragma unroll
-        for (int c = 0; c < RN; ++c) acc[r][c] = Real(0);
-
-    for (int64_t k0 = k_lo; k0 < k_hi; k0 += BK) {
-        // op(A) tile: rows m0.., k0..
-#pragma unroll
-        for (int idx = tid; idx < BM * BK; idx += kThreads) {
-            int i, kk;
-            if (!TA) { i = idx % BM; kk = idx / BM; }   // coalesced along rows of stored A
-            else     { kk = idx % BK; i = idx / BK; }   // coalesced along rows of stored A (= k)
-            const int64_t gi = m0 + i, gk = k0 + kk;
-            Real v = Real(0);
-            if (gi < p.M && gk < k_hi) v = TA ? masked(p.A, p.lda, gk, gi, p.maskA)
-                                              : masked(p.A, p.lda, gi, gk, p.maskA);
-            As[kk][i] = v;
-        }
-        // B tile: stored K x N, coalesced along k
-#pragma unroll
-        for (int idx = tid; idx < BK * BN; idx += kThreads) {
-            const int kk = idx % BK, j = idx / BK;
-            const int64_t gk = k0 + kk, gj = n0 + j;
-            Real v = Real(0);
-            if (gj < p.N && gk < k_hi) v = masked(p.B, p.ldb, gk, gj, p.maskB);
-            Bs[kk][j] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            Real a[RM], b[RN];
-#pragma unroll
-            for (int r = 0; r < RM; ++r) a[r] = As[kk][tx + 16 * r];
-#pragma unroll
-            for (int c = 0; c < RN; ++c) b[c] = Bs[kk][ty + 16 * c];
-#pragma unroll
-            for (int r = 0; r < RM; ++r)
-#pragma unroll
-                for (int c = 0; c < RN; ++c) acc[r][c] = rfma(a[r], b[c], acc[r][c]);
-        }
-        __syncthreads();
-    }
-
-    if (S > 1) {
-        // Split-K: deterministic tree of last-arriver reductions.
-        const int64_t tile = blockIdx.x + (int64_t)blockIdx.y * gridDim.x;
-        Real *tp = p.partial + (size_t)tile * p.slots_per_tile * (BM * BN);
-        unsigned *tc = p.counters + (size_t)tile * p.counters_per_tile;
-        int slot = z, Sl = S, base = 0, cbase = 0;
-        for (;;) {
-            Real *dst = tp + (size_t)(base + slot) * (BM * BN);
-#pragma unroll
-            for (int r = 0; r < RM; ++r)
-#pragma unroll
-                for (int c = 0; c < RN; ++c) dst[(tx + 16 * r) + (ty + 16 * c) * BM] = acc[r][c];
-            const int group = slot / kGroup, first = group * kGroup;
-            const int cnt = min(kGroup, Sl - first);
-            const int Snext = (Sl + kGroup - 1) / kGroup;
-            __threadfence();
-            __syncthreads();
-            if (tid == 0) {
-                unsigned prev = atomicAdd(&tc[cbase + group], 1u);
-                s_last = (prev == (unsigned)(cnt - 1));
-            }
-            __syncthreads();
-            if (!s_last) return;
-            __threadfence();
-            if (tid == 0) tc[cbase + group] = 0u;   // leave the counter zero for the next launch
-#pragma unroll
-            for (int r = 0; r < RM; ++r)
-#pragma unroll
-                for (int c = 0; c < RN; ++c) {
-                    Real s = Real(0);
-                    for (int q = 0; q < cnt; ++q)
-                        s += __ldcg(tp + (size_t)(base + first + q) * (BM * BN) + (tx + 16 * r) + (ty + 16 * c) * BM);
-                    acc[r][c] = s;
-                }
-            if (Snext == 1) break;
-            base += Sl;
-            cbase += Snext;
-            slot = group;
-            Sl = Snext;
-        }
-    }
-
-#pragma unroll
-    for (int c = 0; c < RN; ++c) {
-        const int64_t gj = n0 + ty + 16 * c;
-        if (gj >= p.N) continue;
-#pragma unroll
-        for (int r = 0; r < RM; ++r) {
-            const int64_t gi = m0 + tx + 16 * r;
-            if (gi >= p.M) continue;
-            Real *cp = p.C + gi + gj * p.ldc;
-            Real v = p.alpha * acc[r][c];
-            if (p.beta != Real(0)) v = rfma(p.beta, *cp, v);
-            *cp = v;
-        }
-    }
+    gemm_tile<Real, BM, BN, TA, false>(p, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.x, gridDim.z, As, Bs);
 }
 
 // 64 x 64 tiles on the FP64 tensor cores: mma.sync m8n8k4 (DMMA).  Same
@@ -207,14 +42,13 @@ __device__ __forceinline__ void dmma_8x8x4(double &d0, double &d1, double a, dou
 }
 
 template <bool TA>
-__global__ void __launch_bounds__(kThreads) dgemm_dmma_kernel(GemmParams p) {
+__global__ void __launch_bounds__(kThreads) dgemm_dmma_kernel(GemmParamsT<double> p) {
     constexpr int BM = 64, BN = 64;
     // Row stride 68 = 4 (mod 16) doubles: the fragment loads (4 k-rows x 8
     // consecutive columns per warp) then touch 16 distinct bank pairs per half-warp.
     __shared__ double As[BK][BM + 4];
     __shared__ double Bs[BK][BN + 4];
     __shared__ int s_last;
-    if (p.pred && *(volatile const int *)p.pred == 0) return;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wm = warp & 1, wn = warp >> 1;
@@ -339,18 +173,6 @@ __global__ void __launch_bounds__(kThreads) dgemm_dmma_kernel(GemmParams p) {
 
 int tile_for(int64_t d) { return d <= 16 ? 16 : (d <= 32 ? 32 : 64); }
 
-// Slots and counters per tile of the reduction tree for S splits.
-void tree_shape(int S, int *slots, int *counters) {
-    int s = 0, c = 0, Sl = S;
-    while (Sl > 1) {
-        s += Sl;
-        Sl = (Sl + kGroup - 1) / kGroup;
-        c += Sl;
-    }
-    *slots = std::max(s, 1);
-    *counters = std::max(c, 1);
-}
-
 template <class Real, int BM, int BN>
 cudaError_t launch_bm_bn(const GemmParamsT<Real> &p, bool ta, dim3 grid, cudaStream_t st) {
     if (ta) dgemm_kernel<Real, BM, BN, true><<<grid, kThreads, 0, st>>>(p);
@@ -410,7 +232,8 @@ gbqr_status gemm(const Exec &ex, const GemmOpT<Real> &op, const GemmScratchT<Rea
     if (op.K <= 0) {
         if (op.beta == Real(1)) return GBQR_OK;
     }
-    if (!ex.dmma && !ex.pred && oz_gemm_wanted(op, sc.oz, ex.num_sms)) return oz_gemm(ex, op, sc.oz);
+    if (ex.chain) return chain_gemm(ex, op, sc);
+    if (!ex.dmma && oz_gemm_wanted(op, sc.oz, ex.num_sms)) return oz_gemm(ex, op, sc.oz);
     // A small output (the T products of Algorithm 2 are 64 x 64 x 64 at the
     // panel's top node) on 64 x 64 tiles would run on a handful of SMs at one
     // SM's FP64 rate (2 FMA/clock: ~60 us for 64^3): shrink the tiles until
@@ -460,7 +283,6 @@ gbqr_status gemm(const Exec &ex, const GemmOpT<Real> &op, const GemmScratchT<Rea
     p.C = op.C; p.ldc = op.ldc; p.alpha = op.alpha; p.beta = op.beta;
     p.partial = sc.partial; p.counters = sc.counters;
     p.slots_per_tile = 1; p.counters_per_tile = 1;
-    p.pred = ex.pred;
     if (S > 1) {
         tree_shape(S, &p.slots_per_tile, &p.counters_per_tile);
         size_t need_p = (size_t)tiles * p.slots_per_tile * BM * BN;

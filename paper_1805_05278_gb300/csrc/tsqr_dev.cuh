@@ -490,7 +490,7 @@ __device__ void unit_lower_inverse(const Real *L, Real *Li, Real *M, int w) {
 // Z (over M) = T (V1^T B) for a leaf: V1 = the unit lower top w x w block of
 // the leaf's V (entry (l, i), l > i, at V1[l * ld1v + i * ldv]), T upper (in
 // M on entry), B upper; C is w x w scratch.  Z is upper triangular.
-template <class Real>
+template <int MaxW, class Real>
 __device__ void leaf_z(const Real *V1, int64_t ldv, const Real *B, Real *C, Real *M, int w) {
     const int tid = threadIdx.x, nthr = blockDim.x;
     for (int idx = tid; idx < w * w; idx += nthr) {          // C = V1^T B (upper)
@@ -503,7 +503,7 @@ __device__ void leaf_z(const Real *V1, int64_t ldv, const Real *B, Real *C, Real
         C[idx] = s;
     }
     __syncthreads();
-    Real z2[(kMaxPanel * kMaxPanel + kThreads - 1) / kThreads];   // Z = T C, then over M
+    Real z2[(MaxW * MaxW + kThreads - 1) / kThreads];   // Z = T C, then over M
     int q = 0;
     for (int idx = tid; idx < w * w; idx += nthr, ++q) {
         const int i = idx % w, c = idx / w;
