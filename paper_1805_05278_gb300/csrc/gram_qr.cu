@@ -72,6 +72,13 @@ constexpr int GT = 128;              // threads of the row / trail kernels: 32 x
 template <class Real>
 double gram_bound(int w) { return sizeof(Real) == 8 ? std::sqrt(360.0 / w) : 16.0; }
 
+// Squared column norms a panel may have.  The factorizations multiply two
+// entries of the Gram matrix (fourth powers of the norms), and what such a
+// product loses to underflow has to lie below the rounding of the smallest:
+// at 2^-250 the norms 2^-75 of it do.  FP32: R's entries stay finite.
+constexpr double kGramLeast = 0x1p-500;
+template <class Real> __device__ constexpr double gram_most() { return sizeof(Real) == 8 ? 0x1p500 : 0x1p250; }
+
 template <class Real>
 struct GramArgs {
     Real *A; int64_t lda;            // panel
@@ -195,7 +202,7 @@ __global__ void __launch_bounds__(kThreads) gram_diag_kernel(const __grid_consta
         // (the pivot's own share of the sum that gram_t bounds: most panels that
         // will not do stop here)
         const double d = S[lane][lane];
-        if (!(d > 0.0 && d < 1e300 && d * p.bound >= __ldcg(p.gd + b0 + lane))) bad = 1;
+        if (!(d > kGramLeast && d < gram_most<Real>() && d * p.bound >= __ldcg(p.gd + b0 + lane))) bad = 1;
         const double s = sqrt(d);
         sg[lane] = s;
         p.sc[lane] = s * rd[lane];                       // 1 / r_tt
