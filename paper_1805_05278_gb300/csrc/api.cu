@@ -422,6 +422,19 @@ gbqr_status ensure_workspace(gbqr_ctx *cx, size_t bytes) {
     return GBQR_OK;
 }
 
+// Whether the workspace has or can be given this many bytes.  What can do with
+// less asks first, so that a library-owned workspace is not freed for an
+// allocation that fails, nor touched during a capture.
+bool room_for(gbqr_ctx *cx, size_t bytes) {
+    if (bytes <= cx->ws_bytes) return true;
+    if (!cx->ws_owned) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cx->ws && (cudaStreamIsCapturing(cx->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)) return false;
+    size_t avail = 0, total = 0;
+    if (cudaMemGetInfo(&avail, &total) != cudaSuccess) { cudaGetLastError(); return false; }
+    return bytes <= avail + cx->ws_bytes;
+}
+
 // Point w's buffers into the workspace region at `base` laid out as L.
 void carve_work(gbqr_ctx *cx, char *base, const Layout &L, const Params &pr, const Exec &ex, Work *w) {
     w->cx = cx;
@@ -479,13 +492,15 @@ gbqr_status begin_work(gbqr_ctx *cx, int64_t m, int64_t n, int t_layout, const P
                        size_t min_M = 0) {
     if (cudaSetDevice(cx->device) != cudaSuccess) return GBQR_ECUDA;
     Layout L = make_layout(m, n, t_layout, pr, cx->num_sms, true, min_M);
-    if (!cx->ws_owned && L.total > cx->ws_bytes) {
-        // a caller's workspace without room for the digits: FMA products only
+    gbqr_status st = GBQR_ENOMEM;
+    if (!pr.oz || room_for(cx, L.total)) st = ensure_workspace(cx, L.total);
+    if (st == GBQR_ENOMEM && pr.oz) {
+        // a caller's workspace, or a GPU, without room for the digits: FMA products only
         Params p0 = pr;
         p0.oz = false;
         L = make_layout(m, n, t_layout, p0, cx->num_sms, true, min_M);
+        st = ensure_workspace(cx, L.total);
     }
-    gbqr_status st = ensure_workspace(cx, L.total);
     if (st != GBQR_OK) return st;
     carve_work(cx, cx->ws, L, pr, cx->exec(), w);
     return zero_counters(*w, cx->stream);
@@ -1473,12 +1488,14 @@ gbqr_status gbqr::factor_batched_untuned(gbqr_ctx *cx, int count, const int64_t 
         BatchPlan *pl = nullptr;
         TRY(batched_plan<Real>(&cx->bplan[sizeof(Real) == 8 ? 0 : 1], cx->device, cx->num_sms, count, m, n, lda, ldt,
                                b, !capturing, &pl));
-        // a caller's workspace without room for the grouped part: the persistent kernel alone
-        size_t bytes = batched_plan_bytes(pl);
-        if (!cx->ws_owned && cx->ws_bytes < bytes) bytes = batched_plan_bytes_plain(pl);
-        if (capturing && cx->ws_bytes < bytes) return GBQR_EBUSY;
-        TRY(ensure_workspace(cx, bytes));
-        if (!capturing) TRY(batched_plan_upload(pl, cx->stream));
+        // a caller's workspace, or a GPU, without room for the grouped part:
+        // the persistent kernel alone
+        const size_t bytes = batched_plan_bytes(pl), plain = batched_plan_bytes_plain(pl);
+        gbqr_status st = GBQR_ENOMEM;
+        if (bytes == plain || room_for(cx, bytes)) st = capturing && cx->ws_bytes < bytes ? GBQR_EBUSY : ensure_workspace(cx, bytes);
+        if (st == GBQR_ENOMEM && bytes > plain) st = capturing && cx->ws_bytes < plain ? GBQR_EBUSY : ensure_workspace(cx, plain);
+        if (st == GBQR_OK && !capturing) st = batched_plan_upload(pl, cx->stream);
+        if (st != GBQR_OK) return st;
         if (prepare_only) return GBQR_OK;
         return batched_enqueue<Real>(cx->exec(), pl, A, T, m, n, lda, ldt, cx->ws, cx->ws_bytes, &cx->dinfo->timeout,
                                      &cx->dinfo->nonfinite, capturing ? &cx->capture_owned : nullptr,

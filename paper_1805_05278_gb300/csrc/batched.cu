@@ -672,7 +672,10 @@ void batch_plan_free(BatchPlan *pl) {
 double batch_plan_estimate_ms(const BatchPlan *pl) { return pl ? pl->est_ms : 0.0; }
 size_t batched_plan_bytes_plain(const BatchPlan *pl) { return pl ? pl->total : 0; }
 size_t batched_plan_bytes(const BatchPlan *pl) { return pl ? std::max(pl->total, group_plan_bytes(pl->group)) : 0; }
-gbqr_status batched_plan_upload(BatchPlan *pl, cudaStream_t stream) { return group_plan_upload(pl->group, stream); }
+gbqr_status batched_plan_upload(BatchPlan *pl, cudaStream_t stream) {
+    const gbqr_status st = group_plan_upload(pl->group, stream);
+    return st == GBQR_ENOMEM ? GBQR_OK : st;             // then no groups: batched_enqueue looks
+}
 
 namespace {
 
@@ -863,7 +866,7 @@ gbqr_status batched_enqueue(const Exec &ex, BatchPlan *pl, Real *const *A, Real 
     if (pl->ntasks == 0) return GBQR_OK;
     for (int i = 0; i < pl->count; ++i)
         if (n[i] > 0 && (!A[i] || !T[i])) return GBQR_EINVAL;
-    const bool group = pl->group && ws_bytes >= batched_plan_bytes(pl);
+    const bool group = pl->group && group_plan_lists(pl->group) && ws_bytes >= batched_plan_bytes(pl);
     // the matrix table and the task list, uploaded on the stream: from
     // pageable staging when running now (the copy is staged before the call
     // returns), from page-locked memory that the captured graph keeps when

@@ -805,20 +805,7 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                             int num_sms, size_t ws_off) {
     std::vector<int> mats;
     std::vector<int> width(count, 0);
-    for (int i = 0; i < count; ++i) {
-        width[i] = group_width(m[i], n[i]);
-        if (width[i]) mats.push_back(i);
-    }
-    if (mats.empty()) return nullptr;
-    GroupPlan *g = new (std::nothrow) GroupPlan();
-    if (!g) return nullptr;
     constexpr int D = kOzDigits64;
-    g->width = width;
-    GroupBuilder b{g};
-    g->status_off = GroupBuilder::al(ws_off);
-    // the arena's place depends on the blob's size: offsets are relative to
-    // the arena while building, and shifted at the end
-    auto flag_of = [&](int i) { return g->status_off + (size_t)i * 4; };
     const size_t work_bytes = gram_work_elems() * 8;
     // scratch of matrix i (its first panel is its largest)
     auto need = [&](int i) {
@@ -832,10 +819,24 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
                  (splits / 16 + 1) * w * nc * 8;
         return s + 16 * 256;
     };
+    for (int i = 0; i < count; ++i) {
+        width[i] = group_width(m[i], n[i]);
+        if (width[i] && need(i) > kGroupBytes) width[i] = 0;       // a group of its own would not hold it
+        if (width[i]) mats.push_back(i);
+    }
+    if (mats.empty()) return nullptr;
+    GroupPlan *g = new (std::nothrow) GroupPlan();
+    if (!g) return nullptr;
+    g->width = width;
+    GroupBuilder b{g};
+    g->status_off = GroupBuilder::al(ws_off);
+    // the arena's place depends on the blob's size: offsets are relative to
+    // the arena while building, and shifted at the end
+    auto flag_of = [&](int i) { return g->status_off + (size_t)i * 4; };
     size_t at = 0;
     while (at < mats.size()) {
         size_t end = at, bytes = 0;
-        while (end < mats.size() && (end == at || bytes + need(mats[end]) <= kGroupBytes) && end - at < 60000) bytes += need(mats[end++]);
+        while (end < mats.size() && bytes + need(mats[end]) <= kGroupBytes && end - at < 60000) bytes += need(mats[end++]);
         int64_t panels = 0;
         for (size_t q = at; q < end; ++q) panels = std::max<int64_t>(panels, (n[mats[q]] + width[mats[q]] - 1) / width[mats[q]]);
         for (int64_t pn = 0; pn < panels; ++pn) {

@@ -1,0 +1,84 @@
+"""Calls that fit without the scratch of the digit products and groups run
+where that scratch does not fit: little free memory on the GPU, or matrices
+whose digits alone would fill it."""
+
+import ctypes
+
+import numpy as np
+import pytest
+
+import workloads
+from tests import _gpu
+
+pytestmark = pytest.mark.gpu
+
+
+class _Held:
+    """All free memory of the GPU but `leave` bytes."""
+
+    def __init__(self, leave):
+        import torch
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        self.t = torch.empty(torch.cuda.mem_get_info()[0] - leave, dtype=torch.uint8, device="cuda")
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *exc):
+        import torch
+        del self.t
+        torch.cuda.empty_cache()
+
+
+def _plain(gb, m, n):
+    return gb.workspace_bytes(m, n, gb.GBQR_T_PANEL, gb.opts(fp64_gemm=gb.GBQR_GEMM_DMMA))
+
+
+def test_factor_without_room_for_digits(gb):
+    import torch
+    m, n = 2_000_000, 64
+    with gb.Context(0) as roomy:
+        a = torch.empty((n, m), dtype=torch.float64, device="cuda").normal_(generator=torch.Generator("cuda").manual_seed(1))
+        A, B = a.clone().T, a.T
+        T, U = gb.colmajor(n, n, fill=0.0), gb.colmajor(n, n, fill=0.0)
+        roomy.factor(A, T, gb.GBQR_T_PANEL)
+        assert roomy.sync()[0] == gb.GBQR_OK
+    leave = _plain(gb, m, n) + (1 << 30)
+    assert leave < gb.workspace_bytes(m, n)
+    with gb.Context(0) as ctx, _Held(leave):
+        ctx.factor(B, U, gb.GBQR_T_PANEL)
+        assert ctx.sync()[0] == gb.GBQR_OK
+    s = float(np.sqrt(m))
+    assert float((torch.tril(A, -1) - torch.tril(B, -1)).abs().max()) <= 1e-11
+    assert float((torch.triu(A[:n]) - torch.triu(B[:n])).abs().max()) <= 1e-11 * s
+    assert float((T - U).abs().max()) <= 1e-11
+
+
+def test_batch_without_room_for_groups(gb):
+    import torch
+    mats = [workloads.gaussian(4000, 128, 900 + i % 4) for i in range(200)]
+    dev = lambda: [torch.from_numpy(np.ascontiguousarray(a.T)).cuda().T for a in mats]
+    out = []
+    with gb.Context(0) as ctx:
+        I64 = ctypes.c_int64 * 200
+        assert gb.gbqr_batched_workspace_bytes(200, I64(*[4000] * 200), I64(*[128] * 200), None) > 1 << 30
+        ctx.set_workspace(torch.empty(64 << 20, dtype=torch.uint8, device="cuda"))
+        A, T = dev(), [gb.colmajor(16, 128, fill=0.0) for _ in mats]
+        ctx.factor_batched(A, T)
+        assert ctx.sync()[0] == gb.GBQR_OK
+        out.append(A + T)
+        ctx.set_workspace(None)
+        A, T = dev(), [gb.colmajor(16, 128, fill=0.0) for _ in mats]
+        with _Held(1 << 30):
+            ctx.factor_batched(A, T)
+            assert ctx.sync()[0] == gb.GBQR_OK
+        out.append(A + T)
+    for p, q in zip(*out):
+        assert torch.equal(p, q)
+
+
+def test_groups_hold_their_matrices(gb):
+    """A matrix whose digits alone exceed a group's scratch is not grouped."""
+    I64 = ctypes.c_int64 * 2
+    assert gb.gbqr_batched_workspace_bytes(2, I64(20_000_000, 2000), I64(16, 64), None) < 8 << 30
