@@ -36,6 +36,7 @@ constexpr int64_t kInPanelTcMinRows = 2048;   // ... and m >= 2048
 constexpr int kMaxBatchLanes = 128;
 constexpr size_t kOzMainBytes = (size_t)384 << 20;   // digit scratch of the trailing updates (8192^2: up to three column chunks)
 constexpr int64_t kOzChunkCols = 512;              // ... never less than this many columns' worth
+constexpr size_t kOzMostBytes = (size_t)64 << 30;  // all digit scratch of a call: a quarter of the GPU (9e6 rows of panels of 128)
 constexpr int64_t kFusedMinRows = 256;             // shorter matrices update by separate products
 
 struct DeviceInfo {
@@ -138,8 +139,7 @@ struct Layout {
     TsqrPlan tsqr;
 };
 
-Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num_sms, bool staging = true,
-                   size_t min_M = 0) {
+Layout lay_out(int64_t m, int64_t n, int t_layout, const Params &pr, int num_sms, bool staging, size_t min_M) {
     Layout L;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + std::max<size_t>(bytes, 16), 256); return o; };
@@ -151,7 +151,7 @@ Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num
                                     (size_t)std::max<int64_t>(m, 1) * (size_t)std::max<int64_t>(n, 1) / 4));
     L.n_gcount = gemm_counters_max(num_sms);
     // one size for every fan-out, whether its panels are Gram-matrix ones or not
-    const bool gram = gram_room(pr) && pr.oz && n >= kGramMinW && m >= 4 * kGramMinW;
+    const bool gram = gram_room(pr) && pr.oz && n >= kGramMinW && m >= 4 * kGramMinW && m <= kOzMaxRows;
     const int w = (int)std::max<int64_t>(1, std::min<int64_t>(pr.b, n));
     L.tsqr = tsqr_plan_bound(std::max<int64_t>(m, 1), w, pr.leaf_rows, pr.fanout, num_sms);
     if (gram) {
@@ -243,6 +243,17 @@ Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num
     }
     L.total = off;
     return L;
+}
+
+// ... with digits, unless these alone would take more than kOzMostBytes.
+Layout make_layout(int64_t m, int64_t n, int t_layout, const Params &pr, int num_sms, bool staging = true,
+                   size_t min_M = 0) {
+    const Layout L = lay_out(m, n, t_layout, pr, num_sms, staging, min_M);
+    if (!pr.oz || L.total <= kOzMostBytes) return L;
+    Params p0 = pr;
+    p0.oz = false;
+    const Layout L0 = lay_out(m, n, t_layout, p0, num_sms, staging, min_M);
+    return L.total - L0.total > kOzMostBytes ? L0 : L;
 }
 
 }  // namespace

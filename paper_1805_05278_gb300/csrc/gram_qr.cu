@@ -569,7 +569,7 @@ template size_t gram_scratch_bytes<float>(int64_t, int64_t);
 
 template <class Real>
 bool gram_qr_fits(const OzScratch &oz, int64_t m, int64_t w) {
-    return w >= kGramMinW && w <= kGramMaxW && m >= 4 * w && m <= (1 << 30) && oz.base &&
+    return w >= kGramMinW && w <= kGramMaxW && m >= 4 * w && m <= kOzMaxRows && oz.base &&
            gram_scratch(oz_digits<Real>(), m, w, true).total <= oz.bytes;
 }
 template bool gram_qr_fits<double>(const OzScratch &, int64_t, int64_t);

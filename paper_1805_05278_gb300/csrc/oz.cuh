@@ -8,6 +8,8 @@ namespace gbqr {
 constexpr int kOzTileA = 128, kOzTileB = 64;   // rows of a digit tile of the M and N side of a product
 constexpr int kOzOps = 4;            // operands or problems passed by value
 constexpr int kOzItemsPerCta = 4;
+constexpr int kOzMaxSplits = 65535;
+constexpr int64_t kOzMaxRows = (int64_t)kOzMaxSplits * 512;   // longest K of a product that sums integers of 512 k each
 
 // One operand to split: R rows of K entries each, from the columns (by_row ==
 // 0: row r is column r of X) or the rows of the column-major X.

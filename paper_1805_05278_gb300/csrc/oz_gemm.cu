@@ -807,7 +807,7 @@ OzSplit oz_split(int64_t M, int64_t N, int64_t K, int num_sms, size_t part_cap_e
     OzSplit best{0, 0, 1e30};
     for (int per = 1; per <= std::min(kt, OzTraits<Real>::MAX_KT); ++per) {
         const int S = (kt + per - 1) / per;
-        if ((S > 1 || force_partial) && ((size_t)S * M * N > part_cap_elems || S > 65535)) continue;
+        if ((S > 1 || force_partial) && ((size_t)S * M * N > part_cap_elems || S > kOzMaxSplits)) continue;
         const double item = 1000.0 + step * per + 3500.0 * ((per + OZ_CHUNK - 1) / OZ_CHUNK) + (S == 1 && !force_partial ? 3000.0 : 1500.0);
         double clk = 4000.0 + std::ceil((double)tiles * S / num_sms) * item;
         if (S > 1) clk += 6000.0 + (double)S * M * N * 16.0 / 2500.0;

@@ -79,6 +79,28 @@ def test_batch_without_room_for_groups(gb):
 
 
 def test_groups_hold_their_matrices(gb):
-    """A matrix whose digits alone exceed a group's scratch is not grouped."""
+    """A matrix whose digits alone exceed a group's scratch (36 GB here) is not
+    grouped: it asks for what one of 15 columns does, which never is."""
     I64 = ctypes.c_int64 * 2
-    assert gb.gbqr_batched_workspace_bytes(2, I64(20_000_000, 2000), I64(16, 64), None) < 8 << 30
+    need = [gb.gbqr_batched_workspace_bytes(2, I64(20_000_000, 2000), I64(n, 64), None) for n in (16, 15)]
+    assert need[0] <= need[1] + (1 << 30)
+
+
+def test_more_rows_than_one_sum_splits(gb):
+    """2^25 rows, more than a digit product sums in 65535 splits: the TSQR."""
+    import torch
+    m, n = 1 << 25, 16
+    a = torch.empty((n, m), dtype=torch.float64, device="cuda").normal_(generator=torch.Generator("cuda").manual_seed(3))
+    G = a @ a.T
+    T = gb.colmajor(n, n, fill=0.0)
+    with gb.Context(0) as ctx:
+        ctx.factor(a.T, T, gb.GBQR_T_PANEL)
+        assert ctx.sync()[0] == gb.GBQR_OK
+    R = torch.triu(a.T[:n])
+    assert float((R.T @ R - G).norm() / G.norm()) <= 1e-13
+
+
+def test_digits_leave_room(gb):
+    """The digits' share of the workspace is bounded, whatever the rows."""
+    for m, n in [(100_000_000, 16), (20_000_000, 256)]:
+        assert gb.workspace_bytes(m, n) - _plain(gb, m, n) <= 64 << 30
