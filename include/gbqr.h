@@ -429,14 +429,17 @@ typedef struct {
  * each with a private context and stream, so admitted requests overlap on
  * the device; at most mem_cap_bytes of request footprint in flight.  A
  * request's footprint is its workspace (gbqr_workspace_bytes of its shape
- * and precision, + 1 MiB) plus its own A, b and x.  A queued request is
+ * and precision, + 1 MiB) plus its own A, b and x; one that exceeds the cap
+ * only by the scratch of the digit products is served without them, and so is
+ * one whose workspace the device cannot hold otherwise.  A queued request is
  * admitted (first fit, in arrival order) when a worker is free and its
  * footprint fits under the cap beside the running ones; at most 8 later
  * requests may be admitted ahead of a waiting one, after which it blocks the
  * queue until it fits (at the latest when nothing else runs).  Its workspace
  * comes from the stream-ordered allocator and returns on completion.  Each request runs
  * gbqr_ls_solve (Section 2.1 least squares through the QR); the kernels are
- * deterministic, so a result does not depend on what else is in flight.
+ * deterministic, so a result does not depend on what else is in flight (with
+ * enough device memory for the cap).
  * Errors: EINVAL, EBUSY (already started), ENOMEM, ECUDA. */
 GBQR_API gbqr_status gbqr_server_start(gbqr_ctx *ctx, int device, int workers, size_t mem_cap_bytes);
 /* Queue a request; *id receives its handle.  The request's buffers must stay

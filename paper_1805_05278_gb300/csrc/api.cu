@@ -1067,11 +1067,14 @@ gbqr_status gbqr_set_workspace(gbqr_ctx *cx, void *ptr, size_t bytes) {
     return GBQR_OK;
 }
 
-size_t gbqr_workspace_bytes(int64_t m, int64_t n, int t_layout, const gbqr_opts *opts) {
+}  // extern "C"
+
+size_t gbqr::workspace_bytes(int64_t m, int64_t n, int t_layout, const gbqr_opts *opts, bool digits) {
     if (m < 0 || n < 0) return 0;
     if (t_layout != GBQR_T_FULL && t_layout != GBQR_T_PANEL) return 0;
     Params pr;
     if (!resolve(opts, m, n, &pr)) return 0;
+    pr.oz = digits;
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) {
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); sms = 152; }
@@ -1084,6 +1087,12 @@ size_t gbqr_workspace_bytes(int64_t m, int64_t n, int t_layout, const gbqr_opts 
                            (size_t)(t_layout == GBQR_T_FULL ? m : nbp) * (size_t)(n - m)).total;
     }
     return make_layout(m, n, t_layout, pr, sms).total;
+}
+
+extern "C" {
+
+size_t gbqr_workspace_bytes(int64_t m, int64_t n, int t_layout, const gbqr_opts *opts) {
+    return gbqr::workspace_bytes(m, n, t_layout, opts, true);
 }
 
 gbqr_status gbqr_sync(gbqr_ctx *cx, gbqr_info *info) {

@@ -285,6 +285,8 @@ bool ctx_lookup_tuned(const gbqr_ctx *cx, uint64_t key, gbqr_opts *o);
 void ctx_copy_tuned(const gbqr_ctx *from, gbqr_ctx *to);
 // frees the page-locked tables recorded by a capture (after its graph is gone)
 void ctx_free_capture_owned(gbqr_ctx *cx);
+// gbqr_workspace_bytes, with or without room for the digit products.
+size_t workspace_bytes(int64_t m, int64_t n, int t_layout, const gbqr_opts *opts, bool digits);
 // gbqr_factor / gbqr_factor_batched without the tuner cache (the tuner's own
 // measurements must see exactly the options it passes)
 gbqr_status factor_untuned(gbqr_ctx *cx, int64_t m, int64_t n, double *A, int64_t lda, double *T, int64_t ldt,

@@ -70,15 +70,21 @@ size_t operand_bytes(const gbqr_request &r) {
 // HBM a request holds while it runs: the workspace of gbqr_ls_solve for its
 // shape and precision (with the serving context's autotuned parameters where
 // it has some - the workers carry a copy of that cache, so they size their
-// work the same way), plus its own A (lda x n), b (m) and x (n).
-size_t footprint_of(const gbqr_ctx *cx, const gbqr_request &r, int prec) {
+// work the same way), plus its own A (lda x n), b (m) and x (n).  Without
+// `digits`: the least that serves it, by FMA products.
+size_t footprint_of(const gbqr_ctx *cx, const gbqr_request &r, int prec, bool digits) {
     gbqr_opts o;
     memset(&o, 0, sizeof o);
     if (gbqr::ctx_lookup_tuned(cx, gbqr::tune_key(GBQR_TUNE_FACTOR, r.m, r.n, GBQR_T_PANEL, prec), &o)) {
         o.batch_streams = 0;
     }
     o.update_prec = prec;
-    return gbqr_workspace_bytes(r.m, r.n, GBQR_T_PANEL, &o) + ((size_t)1 << 20) + operand_bytes(r);
+    return gbqr::workspace_bytes(r.m, r.n, GBQR_T_PANEL, &o, digits) + ((size_t)1 << 20) + operand_bytes(r);
+}
+// AUTO may fall back to FP64 inside the same workspace: size for both.
+size_t footprint_of(const gbqr_ctx *cx, const gbqr_request &r, bool digits) {
+    if (r.prec != GBQR_PREC_AUTO) return footprint_of(cx, r, r.prec, digits);
+    return std::max(footprint_of(cx, r, auto_precision(r.m, r.n), digits), footprint_of(cx, r, GBQR_FP64, digits));
 }
 
 }  // namespace
@@ -141,8 +147,14 @@ void worker_loop(gbqr_server *sv, int wi) {
         int used = r.prec;
         bool fell_back = false;
         void *ws = nullptr;
-        const size_t ws_bytes = rec->footprint - operand_bytes(r);   // the rest is the caller's A, b, x
-        if (cudaMallocAsync(&ws, ws_bytes, st) != cudaSuccess) {
+        size_t ws_bytes = rec->footprint - operand_bytes(r);   // the rest is the caller's A, b, x
+        cudaError_t got = cudaMallocAsync(&ws, ws_bytes, st);
+        if (got != cudaSuccess) {
+            cudaGetLastError();
+            const size_t least = footprint_of(cx, r, false) - operand_bytes(r);
+            if (least < ws_bytes) got = cudaMallocAsync(&ws, ws_bytes = least, st);
+        }
+        if (got != cudaSuccess) {
             cudaGetLastError();
             status = GBQR_ENOMEM;
         } else {
@@ -243,10 +255,8 @@ GBQR_API gbqr_status gbqr_submit(gbqr_ctx *ctx, const gbqr_request *req, uint64_
         return GBQR_EINVAL;
     Record rec;
     rec.req = r;
-    // AUTO may fall back to FP64 inside the same workspace: size for both
-    rec.footprint = (r.prec == GBQR_PREC_AUTO)
-                        ? std::max(footprint_of(ctx, r, auto_precision(r.m, r.n)), footprint_of(ctx, r, GBQR_FP64))
-                        : footprint_of(ctx, r, r.prec);
+    rec.footprint = footprint_of(ctx, r, true);
+    if (rec.footprint > sv->cap) rec.footprint = footprint_of(ctx, r, false);
     if (rec.footprint > sv->cap) return GBQR_ENOMEM;
     rec.t_submit = Clock::now();
     {

@@ -104,3 +104,24 @@ def test_digits_leave_room(gb):
     """The digits' share of the workspace is bounded, whatever the rows."""
     for m, n in [(100_000_000, 16), (20_000_000, 256)]:
         assert gb.workspace_bytes(m, n) - _plain(gb, m, n) <= 64 << 30
+
+
+def test_server_cap_without_room_for_digits(gb, orc):
+    """A cap that holds a request only without the digit products admits it."""
+    import torch
+    m, n = 20000, 300
+    a, _, b = workloads.ls_problem(m, n, 2.0, 910)
+    A, bd, x = _gpu.device_matrix(a), torch.from_numpy(b).cuda(), torch.zeros(n, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    cap = _plain(gb, m, n) + (1 << 20) + 8 * (m * n + m + n)
+    assert cap < gb.workspace_bytes(m, n)
+    with gb.Context(0) as ctx:
+        ctx.serve(2, cap)
+        r = ctx.poll(ctx.submit(A, bd, x, gb.GBQR_FP64), wait=True)
+        with pytest.raises(gb.GbqrError):
+            ctx.submit(_gpu.device_matrix(workloads.gaussian(m, n + 8, 911)), bd,
+                       torch.zeros(n + 8, dtype=torch.float64, device="cuda"), gb.GBQR_FP64)
+        ctx.stop_serving()
+    assert r.status == gb.GBQR_OK and r.footprint_bytes == cap
+    x_o, _ = orc.ls_solve(a, b)
+    assert np.linalg.norm(x.cpu().numpy() - x_o) <= 1e-11 * np.linalg.norm(x_o)
