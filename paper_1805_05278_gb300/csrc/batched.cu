@@ -4,8 +4,8 @@
 // factored by TSQR, Section 5 / Appendix C).  FP32 batches are all its own.
 // In a default FP64 batch it takes the matrices that the grouped path
 // (gram_qr.cu) does not: those of fewer than 16 columns or less than about
-// four rows a column, beside the groups on a few SMs (bound by their chains
-// of steps), and, after them, what their condition check handed back.
+// four rows a column, beside the groups on some SMs or before them, and, after
+// them, what their condition check handed back.
 //
 // Work decomposition.  Matrix i (m_i x n_i) is cut into column blocks of
 // width b.  Its tasks are
@@ -49,8 +49,6 @@ namespace gbqr {
 namespace {
 
 constexpr int kUpdCols = 64;    // columns of an update task (the look-ahead block excepted)
-
-constexpr int kBesideCtas = 32;  // CTAs of the launch beside the grouped part: two per SM
 
 constexpr size_t kSmemBudget = 110 * 1024;   // two CTAs per SM
 
@@ -654,6 +652,8 @@ struct BatchPlan {
     size_t real = 8;
     int b = 16, hblk = 0, hup = 64, ldS = 0, grid = 0, ntasks = 0, nstate = 0, tscr_blocks = 0, count = 0;
     int nalone = 0;              // the first tasks: those of ungrouped matrices
+    int beside = 0;              // CTAs that do them beside the grouped part; 0: the whole grid before it
+    std::vector<double> work_ms, span_ms;   // per matrix, one CTA's: all its tasks, its longest chain
     size_t smem = 0;
     size_t off_tasks = 0, off_state = 0, off_tscr = 0, total = 0, table_bytes = 0, state_bytes = 0;
     size_t tscr_stride = 0;
@@ -678,6 +678,8 @@ gbqr_status batched_plan_upload(BatchPlan *pl, cudaStream_t stream) {
 }
 
 namespace {
+
+constexpr double kCyclesPerMs = 2.07e6;
 
 // Task list of the batch in list-schedule order: tasks are started on G
 // simulated workers as workers free up, highest bottom level (longest path
@@ -739,10 +741,14 @@ bool build_plan(BatchPlan *pl, int count, const int64_t *m, const int64_t *n, in
     }
     if (tk.size() > (size_t)(INT32_MAX / 2)) return false;
     // bottom levels (creation order is topological)
+    pl->work_ms.assign(count, 0.0);
+    pl->span_ms.assign(count, 0.0);
     for (int t = (int)tk.size() - 1; t >= 0; --t) {
         double best = 0.0;
         for (int s2 : tk[t].succ) best = std::max(best, tk[s2].bl);
         tk[t].bl = tk[t].dur + best;
+        pl->work_ms[tk[t].mat] += tk[t].dur / kCyclesPerMs;
+        pl->span_ms[tk[t].mat] = std::max(pl->span_ms[tk[t].mat], tk[t].bl / kCyclesPerMs);
     }
     // list schedule on `grid` workers
     auto cmp = [&](int a, int c) { return tk[a].bl < tk[c].bl || (tk[a].bl == tk[c].bl && a > c); };
@@ -772,7 +778,7 @@ bool build_plan(BatchPlan *pl, int count, const int64_t *m, const int64_t *n, in
             if (--tk[s2].npred == 0) ready.push(s2);
     }
     if (pl->order.size() != tk.size()) return false;
-    pl->est_ms = now / 2.07e6;
+    pl->est_ms = now / kCyclesPerMs;
     pl->ntasks = (int)pl->order.size();
     pl->nstate = nstate;
     pl->tscr_blocks = maxP;
@@ -788,6 +794,28 @@ bool build_plan(BatchPlan *pl, int count, const int64_t *m, const int64_t *n, in
     pl->tscr_stride = (size_t)maxP * b * b;
     pl->total = al(pl->off_tscr + real * pl->tscr_stride * (size_t)grid);
     return true;
+}
+
+// CTAs for the ungrouped matrices beside the grouped part (`group_ms`), one
+// per SM, where those SMs then hold no product of the groups; or 0: all CTAs
+// before it.  `work`, `span`: the ungrouped matrices' (ms of one CTA that
+// shares its SM with another; alone it is 1.7 times as fast, measured from 32
+// CTAs against 304).  Few and small, they are bound by their chains and cost
+// least on a few SMs (the 85 of 2000 benchmark matrices: 2 ms of 109 on 32
+// CTAs); 999 of 400 x 300 beside one 2000 x 64 took 327 ms there, 58 on all.
+int ctas_beside(double work, double span, double group_ms, int num_sms, int grid) {
+    // (more CTAs only where they are estimated 10 % better: the estimates are no closer)
+    double best = 1e300;
+    int ctas = 0;
+    auto take = [&](int c, double ms) {
+        if (ms < 0.9 * best) { best = ms; ctas = c; }
+    };
+    for (int c = 32; c < num_sms; c += 32) {
+        const double t = std::max(work / (1.7 * c), span);
+        take(c, t + std::max(0.0, group_ms - t * (1.0 - (double)c / num_sms)));
+    }
+    take(0, std::max(work / grid, span) + group_ms);
+    return ctas;
 }
 
 }  // namespace
@@ -851,6 +879,13 @@ gbqr_status batched_plan(BatchPlan **cache, int device, int num_sms, int count, 
         const int *width = group_widths(pl->group);
         auto mid = std::stable_partition(pl->order.begin(), pl->order.end(), [&](const int4 &t) { return width[t.x] == 0; });
         pl->nalone = (int)(mid - pl->order.begin());
+        double work = 0.0, span = 0.0;
+        for (int i = 0; i < count; ++i)
+            if (!width[i]) {
+                work += pl->work_ms[i];
+                span = std::max(span, pl->span_ms[i]);
+            }
+        pl->beside = ctas_beside(work, span, group_plan_ms(pl->group), num_sms, pl->grid);
     }
     pl->key = key;
     *out = pl;
@@ -919,17 +954,19 @@ gbqr_status batched_enqueue(const Exec &ex, BatchPlan *pl, Real *const *A, Real 
         return trace_end(e, FAM_BATCHED, 0.0, 0.0);
     };
     if (!group) return launch(p, pl->grid, ex.stream);
-    // the ungrouped matrices (few and small: bound by their chains of steps)
-    // beside the grouped ones, on a few SMs; then whatever the grouped part
-    // left, with a T scratch of its own (the first launch is over by then)
-    const bool beside = pl->nalone > 0;
+    // the ungrouped matrices beside the grouped ones or before them; then
+    // whatever the grouped part left, with a T scratch of its own (the first
+    // launch is over by then)
+    const bool beside = pl->nalone > 0 && pl->beside > 0;
+    BParams<Real> q = p;
+    q.ntasks = pl->nalone;
     if (beside) {
-        BParams<Real> q = p;
-        q.ntasks = pl->nalone;
         if (cudaEventRecord(side.fork, ex.stream) != cudaSuccess || cudaStreamWaitEvent(side.stream, side.fork, 0) != cudaSuccess)
             return GBQR_ECUDA;
-        TRY_ST(launch(q, std::min(pl->grid, kBesideCtas), side.stream));
+        TRY_ST(launch(q, std::min(pl->grid, pl->beside), side.stream));
         if (cudaEventRecord(side.join, side.stream) != cudaSuccess) return GBQR_ECUDA;
+    } else if (pl->nalone > 0) {
+        TRY_ST(launch(q, pl->grid, ex.stream));
     }
     TRY_ST(group_enqueue(ex, pl->group, ws, ws, (int)sizeof(BMat<Real>), pl->count, timeout_flag));
     if (beside && cudaStreamWaitEvent(ex.stream, side.join, 0) != cudaSuccess) return GBQR_ECUDA;

@@ -202,6 +202,7 @@ void group_plan_free(GroupPlan *g);
 size_t group_plan_bytes(const GroupPlan *g);           // workspace, from its start
 const int *group_widths(const GroupPlan *g);           // per matrix, 0 = not grouped
 size_t group_status_offset(const GroupPlan *g);
+double group_plan_ms(const GroupPlan *g);              // estimated time
 gbqr_status group_plan_upload(GroupPlan *g, cudaStream_t stream);
 std::shared_ptr<void> group_plan_lists(const GroupPlan *g);   // what a captured graph has to keep
 gbqr_status group_enqueue(const Exec &ex, const GroupPlan *g, char *ws, const void *mats, int stride, int count, int *err);

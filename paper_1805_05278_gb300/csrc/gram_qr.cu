@@ -727,6 +727,7 @@ struct GroupPlan {
     std::vector<Reloc> relocs;
     std::vector<GroupStep> steps;
     std::vector<int> width;                              // per matrix: its panels' width, 0 = not grouped
+    double est_ms = 0.0;
     std::shared_ptr<GroupLists> lists;                   // device copies (group_plan_upload)
 };
 
@@ -734,6 +735,7 @@ void group_plan_free(GroupPlan *g) { delete g; }
 size_t group_plan_bytes(const GroupPlan *g) { return g ? g->total : 0; }
 const int *group_widths(const GroupPlan *g) { return g->width.data(); }
 size_t group_status_offset(const GroupPlan *g) { return g->status_off; }
+double group_plan_ms(const GroupPlan *g) { return g->est_ms; }
 
 namespace {
 
@@ -839,6 +841,13 @@ GroupPlan *group_plan_build(int count, const int64_t *m, const int64_t *n, const
         while (end < mats.size() && bytes + need(mats[end]) <= kGroupBytes && end - at < 60000) bytes += need(mats[end++]);
         int64_t panels = 0;
         for (size_t q = at; q < end; ++q) panels = std::max<int64_t>(panels, (n[mats[q]] + width[mats[q]] - 1) / width[mats[q]]);
+        // a panel's chain, and 4 TFLOP/s: 200 of 2000 x 128 take 4.5 ms, the
+        // 2000 benchmark matrices (351 GFLOP) 109
+        g->est_ms += 0.4 * panels;
+        for (size_t q = at; q < end; ++q) {
+            const double mm = (double)m[mats[q]], nn = (double)n[mats[q]];
+            g->est_ms += (2.0 * mm * nn * nn - 2.0 / 3.0 * nn * nn * nn) / 4e9;
+        }
         for (int64_t pn = 0; pn < panels; ++pn) {
             b.arena = 0;
             std::vector<int> act;

@@ -111,3 +111,25 @@ def test_panels_given_up_at_every_place(gb):
     for other in out[1:]:
         for p, q in zip(out[0], other):
             assert torch.equal(p, q)
+
+
+@pytest.mark.parametrize("few,many", [((300, 280), (2000, 64)), ((2000, 64), (300, 280))])
+def test_ungrouped_matrices_beside_and_before_the_groups(gb, orc, few, many):
+    """Few ungrouped matrices run beside the groups, many before them."""
+    import torch
+    shapes = [few] * 2 + [many] * 90
+    mats = [workloads.gaussian(m, n, 580 + i % 5) for i, (m, n) in enumerate(shapes)]
+    with gb.Context(0) as ctx:
+        out = []
+        for ws in (None, torch.empty(64 << 20, dtype=torch.uint8, device="cuda")):
+            A, T = _device(mats, torch.float64), _kernels(gb, mats, torch.float64)
+            ctx.set_workspace(ws)
+            ctx.factor_batched(A, T)
+            assert ctx.sync()[0] == gb.GBQR_OK
+            out.append((A, T))
+        ctx.set_workspace(None)
+    for i in (0, 1, 2, 91):
+        a = mats[i]
+        _gpu.compare_factor(a, gb.to_numpy(out[0][0][i]), gb.to_numpy(out[0][1][i]), gb.GBQR_T_PANEL, 16, orc, f"{a.shape}")
+        if a.shape[0] == 300:       # the persistent kernel's, in either place
+            assert torch.equal(out[0][0][i], out[1][0][i]) and torch.equal(out[0][1][i], out[1][1][i])
