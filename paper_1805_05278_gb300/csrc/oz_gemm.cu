@@ -12,24 +12,28 @@
 // two to magnitude < 1 and written as a 55-bit fixed-point number, cut into
 // 7 balanced base-256 digits d_1 ... d_7, |d| <= 128, each exact in BF16 and
 // stored with its weight 256^-(i-1).  A digit product is an integer of at
-// most 2^14 times its weight, so the tensor cores' FP32 accumulators hold a
-// sum of products of equal weight exactly while fewer than 2^24 / 2^14 =
-// 1024 of them meet.  The weights i + j = 2 ... 7 (1 to 6 products per k)
-// have an accumulator each, i + j = 8 and 9 share one; i + j >= 10 (below
-// 2^-62 of the row and column maxima) is left out.  Every 256 k the
-// accumulators are drained into a 64-bit integer per output (unit 2^-40 of a
-// leading digit product), and the integer is rounded to FP64 once.  Sums over
-// more than 512 k are integer partials, so neither the split nor the order
-// changes a bit of the result.
+// most 2^14 times its weight, so an FP32 accumulator of the tensor cores holds
+// a sum of products of equal weight exactly while it stays below 2^24 of them.
+// The weights i + j = 2 ... 7 (1 to 6 products per k) have an accumulator
+// each, i + j = 8 and 9 share one; i + j >= 10 (below 2^-62 of the row and
+// column maxima) is left out.  Every 256 k the accumulators are drained into a
+// 64-bit integer per output (unit 2^-40 of a leading digit product), and the
+// integer is rounded to FP64 once.  Sums over more than 512 k are integer
+// partials, which add without rounding in any order.
 //
-// Error.  Entries within a factor 4 of the row (column) maximum are exact,
-// the others lose what lies below 2^-56 of it; the sums are exact but for
-// the FP32 rounding of the shared accumulator (2^-24 of a weight 2^-48).
-// Measured on whole factorizations, backward error and orthogonality are at
-// or below the FMA kernel's, which rounds at every k (graded 8192^2: backward
-// error 6.6e-16, FMA 8.4e-16; Gaussian 4096^2: 1.8e-15, 2.3e-15).  Sharing
-// one accumulator among i + j = 6, 7, 8 instead cost a digit and a half: the
-// tensor cores' accumulation truncates, and its bias grows with K.
+// Error.  Entries within a factor 4 of the row (column) maximum are exact, the
+// others lose what lies below 2^-56 of it.  A drain's 256 k are 1280 products
+// of weight 6 and 1536 of weight 7: these sums leave the exact range only where
+// the products of their digits average more than 114^2 or 104^2 of 128^2, all
+// of one sign; the steps past 2^24 then truncate, at worst (every digit 127)
+// 32 units of 2^-32 and 64 of 2^-40, 2^-48.6 of sum |a_ik b_kj| (the FMA
+// kernel's bound over 256 k is 2^-45).  The shared accumulator truncates at
+// 2^-59 of it.  Where none of this happens a result does not depend on the
+// split.  Measured on whole factorizations, backward error and orthogonality
+// are at or below the FMA kernel's, which rounds at every k (graded 8192^2:
+// backward error 6.6e-16, FMA 8.4e-16; Gaussian 4096^2: 1.8e-15, 2.3e-15).
+// Sharing one accumulator among i + j = 6, 7, 8 instead cost a digit and a
+// half: the tensor cores' accumulation truncates, and its bias grows with K.
 //
 // Kernels of one product:
 //   oz_slice_kernel   digits of the operands (HBM: 8 B read, 14 written per
@@ -48,9 +52,9 @@
 // swizzle the MMA descriptors name, so a stage is filled by one bulk copy an
 // operand and a product needs no tensor map.
 //
-// Measured (one factorization with the FMA kernel against this one): graded
-// 8192^2 687 -> 157 ms, 32768 x 2048 256 -> 65 ms; the thin Q of 16001 x 1000
-// 31.3 -> 3.3 ms.
+// Measured with the FMA kernel against this one, all else as it was then (TSQR
+// panels): graded 8192^2 687 -> 157 ms, 32768 x 2048 256 -> 65 ms; the thin Q
+// of 16001 x 1000 31.3 -> 3.2 ms.
 #include "oz.cuh"
 #include "tc_ptx.cuh"
 
@@ -67,7 +71,7 @@ constexpr int OZ_BM = 128;
 constexpr int OZ_BN = 64;
 constexpr int OZ_BK = 32;            // one 64-byte row of BF16
 constexpr uint32_t OZ_PIECE = 4096;  // bytes per bulk copy
-constexpr int OZ_CHUNK = 8;          // K tiles per drain (256 k: the accumulators stay exact)
+constexpr int OZ_CHUNK = 8;          // K tiles per drain (256 k; see the error above)
 constexpr int OZ_EPI_WARPS = 16;
 constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;
 constexpr int OZ_COLS = OZ_BN / (OZ_EPI_WARPS / 4);   // columns per epilogue thread
@@ -481,7 +485,7 @@ __device__ __forceinline__ OzItem oz_item(const OzMmaArgs<Real> &args, int item,
     return t;
 }
 
-// 10 warps per CTA: bulk-copy producer (per 32-k step all digits of a tile of
+// 18 warps per CTA: bulk-copy producer (per 32-k step all digits of a tile of
 // A, 56 KB in FP64, and of one of B, 28 KB), MMA issuer (two instructions
 // per digit product and stage), 16 epilogue warps (warp w reads TMEM lanes 32
 // (w % 4) .. + 31 and a quarter of the columns; with 8 warps the epilogue, a

@@ -55,3 +55,24 @@ def test_mixed_least_squares_with_given_up_panels(gb, ctx, orc):
     assert st == gb.GBQR_OK
     # columns' condition about 1 / 3e-2, times the square for a residual near zero
     assert np.linalg.norm(xd.cpu().numpy() - x) <= 1e-11 * np.linalg.norm(x)
+
+
+def test_given_up_panels_in_a_graph(gb):
+    import torch
+    a = _near_pairs(3000, 300, 750, 3e-2)
+    stream = torch.cuda.Stream()
+    with gb.Context(0, stream) as ctx:
+        A, T = _gpu.device_matrix(a), gb.colmajor(128, 300, fill=0.0)
+        torch.cuda.synchronize()
+        ctx.factor(A, T, gb.GBQR_T_PANEL)
+        torch.cuda.synchronize()
+        B, U, fresh = _gpu.device_matrix(a), gb.colmajor(128, 300, fill=0.0), _gpu.device_matrix(a)
+        torch.cuda.synchronize()
+        graph = ctx.capture(lambda: ctx.factor(B, U, gb.GBQR_T_PANEL))
+        for _ in range(2):
+            B.copy_(fresh)
+            torch.cuda.synchronize()
+            graph.launch()
+            torch.cuda.synchronize()
+            assert torch.equal(A, B) and torch.equal(T, U)
+        graph.close()
