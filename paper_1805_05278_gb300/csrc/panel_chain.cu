@@ -10,7 +10,7 @@
 // persistent CTAs take the steps' CTAs in order from a ticket: a CTA waits
 // until all earlier steps are done.  It waits only for tasks taken before its
 // own, by CTAs that are running, so however few CTAs are resident, every wait
-// ends (and is bounded).  One CTA per SM: the leaves' FP64 chains slow each
+// ends (and is bounded).  One CTA per SM in FP64: the leaves' chains slow each
 // other down on a shared one (1024 x 128 1934 us with two CTAs, 1780 with
 // one); the products then load a K tile ahead (32768 x 128 4447 -> 3888).
 //
@@ -119,6 +119,10 @@ __global__ void __launch_bounds__(kThreads) panel_chain_kernel(const __grid_cons
         for (int i = 0; i < 4; ++i) a.ctr[i] = 0u;
 }
 
+// Persistent CTAs per SM: FP64 chains slow each other down on a shared SM, FP32
+// ones hide each other's latencies (32768 x 128 of close pairs 2098 -> 1910 us).
+template <class Real> constexpr int chain_per_sm() { return sizeof(Real) == 8 ? 1 : 2; }
+
 constexpr size_t kChainSmemCap = 200 * 1024;     // as the TSQR's plans
 
 template <class Real>
@@ -157,9 +161,8 @@ template <class Real>
 gbqr_status chain_gemm(const Exec &ex, const GemmOpT<Real> &op, const GemmScratchT<Real> &sc) {
     const int BM = !op.ta && op.M >= (int64_t)64 * ex.num_sms ? 64 : 16;
     const int64_t tm = (op.M + BM - 1) / BM, tn = (op.N + 15) / 16, tiles = tm * tn, kt = (op.K + BK - 1) / BK;
-    int64_t S = 1;
-    if (tiles < (int64_t)ex.num_sms)
-        S = std::max<int64_t>(1, std::min<int64_t>({kt / (kt >= 32 ? 4 : 1), (int64_t)ex.num_sms / tiles, 512}));
+    const int64_t ctas = (int64_t)chain_per_sm<Real>() * ex.num_sms;
+    int64_t S = std::max<int64_t>(1, std::min<int64_t>({kt / (kt >= 32 ? 4 : 1), ctas / tiles, 512}));
     int slots = 1, counters = 1;
     for (; S > 1; --S) {
         tree_shape((int)S, &slots, &counters);
@@ -202,7 +205,7 @@ gbqr_status chain_launch(const Exec &ex, ChainRecorder &rec, const int *flag, un
     a.ctr = ctr;
     a.timeout = timeout;
     trace_begin(ex, FAM_OTHER);
-    panel_chain_kernel<Real><<<std::min(rec.widest, ex.num_sms), kThreads, rec.smem, ex.stream>>>(a);
+    panel_chain_kernel<Real><<<std::min(rec.widest, chain_per_sm<Real>() * ex.num_sms), kThreads, rec.smem, ex.stream>>>(a);
     return trace_end(ex, FAM_OTHER, 0.0, 0.0);
 }
 template gbqr_status chain_launch<double>(const Exec &, ChainRecorder &, const int *, unsigned *, int *);
