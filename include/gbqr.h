@@ -189,8 +189,9 @@ GBQR_API gbqr_status gbqr_sync(gbqr_ctx *ctx, gbqr_info *info);
  * R = -S R_tree, V = W U^{-1} (Appendix C).  With the default cutoff, leaf
  * height, fan-out and GEMM engine, well-conditioned panels of 16 to 128
  * columns and at least four rows a column get the same (V, T, R) from their
- * Gram matrix (Cholesky, then that reconstruction); a check on the device
- * hands the others to the TSQR.
+ * Gram matrix (Cholesky, then that reconstruction) as accurately; a check on
+ * the device hands the others, columns that nearly depend on each other, to
+ * the recursion on TSQRs.
  * A and T may instead both be HOST pointers (pageable or pinned): the call
  * then stages them through device workspace, copies the results back and
  * returns after the stream has synchronised.  With page-locked buffers and
@@ -211,7 +212,9 @@ GBQR_API gbqr_status gbqr_factor(gbqr_ctx *ctx, int64_t m, int64_t n, double *A,
 /* gbqr_factor in FP32: A (m x n, m >= n) and T are float DEVICE arrays and
  * every step computes in FP32 or better with the float instantiations of the
  * same kernels (TSQR, tiled GEMM, digit products; a panel's Gram matrix is
- * decomposed in FP64); same layouts, options and look-ahead.
+ * decomposed in FP64); same layouts, options and look-ahead.  Where a pivot
+ * is zero to FP32 rounding, the reflection may take either sign, and with it
+ * a row of R and a column of V.
  * opts->update_prec must be GBQR_FP64 / 0 (no tensor-core updates); the
  * autotuner's cache is not used.  Errors: EINVAL (m < n, lda, ldt, opts),
  * EUNSUPPORTED (host pointers), ENOMEM, ECUDA. */
@@ -230,8 +233,8 @@ GBQR_API int64_t gbqr_default_panel_nb(int64_t m, int64_t n);
  * By default (cutoff 16, panel_nb at most the cutoff) matrices of 16 columns
  * or more with about four rows a column are factored group by group from
  * their panels' Gram matrices, in lockstep launches over lists of panels;
- * the others, and those that the condition check hands back, by one launch
- * of a persistent kernel.  A caller's workspace without room for the groups
+ * the others, and those that the condition check hands back, by a persistent
+ * kernel.  A caller's workspace, or a device, without room for the groups
  * gets the persistent kernel alone.  With panel_nb above the cutoff, a cutoff
  * above 32 or a mixed update_prec, the matrices are spread over
  * opts->batch_streams (default 128) internal streams (largest first, to
@@ -251,8 +254,8 @@ GBQR_API gbqr_status gbqr_factor_batched(gbqr_ctx *ctx, int count, const int64_t
  * leaves, merges, reconstruction and the QR-EG update and T-assembly products
  * - computes in FP32 with the same kernels instantiated for float (this part
  * issues FP32 at 64x its FP64 rate, and the TSQR reflector chains shorten
- * accordingly).  Same layout, scheduling, streams, workspace and graph
- * capture rules as gbqr_factor_batched; opts->update_prec must be GBQR_FP64
+ * accordingly), by the persistent kernel alone.  Same layout, scheduling,
+ * streams, workspace and graph capture rules as gbqr_factor_batched; opts->update_prec must be GBQR_FP64
  * (meaning: no tensor-core updates) or zero; the autotuner's cache is not
  * used.  Errors: EINVAL, ENOMEM, ECUDA. */
 GBQR_API gbqr_status gbqr_factor_batched_f32(gbqr_ctx *ctx, int count, const int64_t *m, const int64_t *n,

@@ -24,8 +24,8 @@
 // be nearly a combination of the others (gram_bound).  Then orthogonality and
 // backward error are at or below the TSQR's, and V, T and R agree with its to
 // rounding.  Otherwise a device flag is raised, the panel is left untouched,
-// and the caller's TSQR launches, which return at once while the flag is zero,
-// factor it.
+// and the launch that the caller puts behind (panel_chain.cu), which returns at
+// once while the flag is zero, factors it.
 //
 // The w x w work runs in 32-wide blocks, three launches a block:
 //   diag   one CTA: Cholesky and LU of the diagonal block
