@@ -433,14 +433,15 @@ gbqr_status ensure_workspace(gbqr_ctx *cx, size_t bytes) {
     return GBQR_OK;
 }
 
-// Whether the workspace has or can be given this many bytes.  What can do with
-// less asks first, so that a library-owned workspace is not freed for an
-// allocation that fails, nor touched during a capture.
+// Whether to try for this many bytes of workspace, where a call can do with
+// less: a library-owned workspace is not given up for an allocation that
+// fails, nor touched during a capture.  A first one is simply tried.
 bool room_for(gbqr_ctx *cx, size_t bytes) {
     if (bytes <= cx->ws_bytes) return true;
     if (!cx->ws_owned) return false;
+    if (!cx->ws) return true;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cx->ws && (cudaStreamIsCapturing(cx->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)) return false;
+    if (cudaStreamIsCapturing(cx->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
     size_t avail = 0, total = 0;
     if (cudaMemGetInfo(&avail, &total) != cudaSuccess) { cudaGetLastError(); return false; }
     return bytes <= avail + cx->ws_bytes;
